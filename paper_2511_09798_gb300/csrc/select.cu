@@ -1,7 +1,7 @@
 // Parameter choice and projected solves (Algorithms 2 and 4), lift alpha = Z_l y.
 //
 // Grid: lambda_t = s~_1 10^{t}, t = t_lo + (t_hi - t_lo) * idx / (J - 1).
-// For each grid point (one thread each):
+// For each grid point (one warp each):
 //   q_i = lambda^2 / (s~_i^2 + lambda^2)         (= 1 - phi~_i)
 //   rho^2 = sum_i q_i^2 f~_i^2 + f~_{l+1}^2         (eq. rho_proj)
 //   eta^2 = sum_i (s~_i f~_i / (s~_i^2 + lambda^2))^2 (eq. eta_proj)
@@ -23,19 +23,24 @@ namespace {
 
 __device__ __forceinline__ int sel_l(const ProjDims& d, int b) { return d.l_arr ? d.l_arr[b] : d.l; }
 
-__global__ void k_grid_terms(ProjDims d, const double* __restrict__ sigma_all, const double* __restrict__ ftil_all,
-                             int J, double t_lo, double t_hi, double* __restrict__ gcv_all,
-                             double* __restrict__ xr_all, double* __restrict__ ye_all) {
+// One warp per grid point, lanes along the singular values (one thread per
+// point spent its time in a chain of l IEEE divisions: 82 -> 10 us at l = 150).
+constexpr int GT_WARPS = 4;
+
+__global__ void __launch_bounds__(GT_WARPS * 32)
+    k_grid_terms(ProjDims d, const double* __restrict__ sigma_all, const double* __restrict__ ftil_all, int J,
+                 double t_lo, double t_hi, double* __restrict__ gcv_all, double* __restrict__ xr_all,
+                 double* __restrict__ ye_all) {
     const int b = blockIdx.y;
     const int l = sel_l(d, b);
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int t = blockIdx.x * GT_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (t >= J || l < 1) return;
     const double* sigma = sigma_all + (size_t)b * d.L;
     const double* ftil = ftil_all + (size_t)b * (d.L + 1);
     const double lam = sigma[0] * exp10(grid_t(t, J, t_lo, t_hi));
     const double lam2 = lam * lam;
-    double rho2 = 0.0, eta2 = 0.0, den = 1.0;
-    for (int i = 0; i < l; ++i) {
+    double rho2 = 0.0, eta2 = 0.0, den = 0.0;
+    for (int i = lane; i < l; i += 32) {
         const double s = sigma[i], f = ftil[i];
         const double inv = 1.0 / fma(s, s, lam2);
         const double q = lam2 * inv;
@@ -44,28 +49,74 @@ __global__ void k_grid_terms(ProjDims d, const double* __restrict__ sigma_all, c
         eta2 = fma(g, g, eta2);
         den += q;
     }
-    rho2 = fma(ftil[l], ftil[l], rho2);
-    gcv_all[(size_t)b * J + t] = rho2 / (den * den);
-    xr_all[(size_t)b * J + t] = 0.5 * log(rho2);
-    ye_all[(size_t)b * J + t] = 0.5 * log(eta2);
+    rho2 = warp_sum(rho2);
+    eta2 = warp_sum(eta2);
+    den = 1.0 + warp_sum(den);
+    if (lane == 0) {
+        rho2 = fma(ftil[l], ftil[l], rho2);
+        gcv_all[(size_t)b * J + t] = rho2 / (den * den);
+        xr_all[(size_t)b * J + t] = 0.5 * log(rho2);
+        ye_all[(size_t)b * J + t] = 0.5 * log(eta2);
+    }
+}
+
+constexpr int CH_T = 256;  // threads of the choice kernels
+
+// The block's best (value, index): the largest or smallest value,
+// lowest index on ties, in every thread.
+__device__ __forceinline__ void block_best(double& v, int& idx, bool largest) {
+    __shared__ double bv[CH_T / 32];
+    __shared__ int bi[CH_T / 32];
+    auto take = [&](double ov, int oi) {
+        if ((largest ? ov > v : ov < v) || (ov == v && oi < idx)) {
+            v = ov;
+            idx = oi;
+        }
+    };
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        take(__shfl_xor_sync(RBF_FULL_MASK, v, o), __shfl_xor_sync(RBF_FULL_MASK, idx, o));
+    const int warp = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0) {
+        bv[warp] = v;
+        bi[warp] = idx;
+    }
+    __syncthreads();
+    for (int w = 0; w < CH_T / 32; ++w) take(bv[w], bi[w]);
+    __syncthreads();
+}
+
+// The block's sums of two values, in thread 0.
+__device__ __forceinline__ void block_sum2(double& a, double& b) {
+    __shared__ double ra[CH_T / 32], rb[CH_T / 32];
+    a = warp_sum(a);
+    b = warp_sum(b);
+    if ((threadIdx.x & 31) == 0) {
+        ra[threadIdx.x >> 5] = a;
+        rb[threadIdx.x >> 5] = b;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        a = b = 0.0;
+        for (int w = 0; w < CH_T / 32; ++w) {
+            a += ra[w];
+            b += rb[w];
+        }
+    }
+    __syncthreads();
 }
 
 // Choose lambda (rule 0 GCV, 1 L-curve, 2 fixed, 3 fixed t: lambda = s~_1
 // 10^lambda_in) and form the coefficient vector cvec_i = s_i f_i / (s_i^2 +
 // lambda^2); eta = |cvec| and rho (eq. rho_proj) at that lambda go to the
 // state (instance 0).  One block per instance.
-__global__ void k_choose_lambda(ProjDims d, const double* __restrict__ sigma_all,
-                                const double* __restrict__ ftil_all, int J, double t_lo, double t_hi,
-                                int rule0, double lambda0, const int* __restrict__ rule_arr,
-                                const double* __restrict__ lam_arr, const double* __restrict__ gcv_all,
-                                const double* __restrict__ xr_all, const double* __restrict__ ye_all,
-                                double* __restrict__ curve_all, double* __restrict__ cvec_all,
-                                double* __restrict__ lam_out, int* __restrict__ idx_out,
-                                rbf_dev_state* __restrict__ stt) {
-    __shared__ double bv[1024];
-    __shared__ double gcv_red[1024];
-    __shared__ int bi[1024];
-    __shared__ double lam_s;
+__global__ void __launch_bounds__(CH_T)
+    k_choose_lambda(ProjDims d, const double* __restrict__ sigma_all, const double* __restrict__ ftil_all, int J,
+                    double t_lo, double t_hi, int rule0, double lambda0, const int* __restrict__ rule_arr,
+                    const double* __restrict__ lam_arr, const double* __restrict__ gcv_all,
+                    const double* __restrict__ xr_all, const double* __restrict__ ye_all,
+                    double* __restrict__ curve_all, double* __restrict__ cvec_all, double* __restrict__ lam_out,
+                    int* __restrict__ idx_out, rbf_dev_state* __restrict__ stt) {
     const int b = blockIdx.x;
     const int l = sel_l(d, b);
     if (l < 1) return;
@@ -79,7 +130,7 @@ __global__ void k_choose_lambda(ProjDims d, const double* __restrict__ sigma_all
     double* curve = curve_all ? curve_all + (size_t)b * J : nullptr;
     double* cvec = cvec_all + (size_t)b * d.L;
     const double h = (t_hi - t_lo) / (double)(J - 1);
-    // per-thread best over a strided subset, then a tree with lowest-index tie-break
+    // per-thread best over a strided subset, then over the block with lowest-index tie-break
     double best = rule == 1 ? -INFINITY : INFINITY;
     int besti = 0x7fffffff;
     if (rule < 2) {
@@ -106,39 +157,20 @@ __global__ void k_choose_lambda(ProjDims d, const double* __restrict__ sigma_all
                 if (v > best || (v == best && t < besti)) { best = v; besti = t; }
             }
         }
+        block_best(best, besti, rule == 1);
     }
-    bv[threadIdx.x] = best;
-    bi[threadIdx.x] = besti;
-    __syncthreads();
-    for (int off = blockDim.x / 2; off > 0; off >>= 1) {
-        if ((int)threadIdx.x < off) {
-            const double ov = bv[threadIdx.x + off];
-            const int oi = bi[threadIdx.x + off];
-            const double mv = bv[threadIdx.x];
-            const int mi = bi[threadIdx.x];
-            const bool take = rule == 1 ? (ov > mv || (ov == mv && oi < mi)) : (ov < mv || (ov == mv && oi < mi));
-            if (take) {
-                bv[threadIdx.x] = ov;
-                bi[threadIdx.x] = oi;
-            }
-        }
-        __syncthreads();
+    double lam;
+    int idx = -1;
+    if (rule == 2) {
+        lam = lambda_in;
+    } else if (rule == 3) {
+        lam = sigma[0] * exp10(lambda_in);
+    } else {
+        idx = besti;
+        if (idx < 0 || idx >= J) idx = 0;
+        lam = sigma[0] * exp10(grid_t(idx, J, t_lo, t_hi));
     }
     if (threadIdx.x == 0) {
-        double lam;
-        int idx;
-        if (rule == 2) {
-            lam = lambda_in;
-            idx = -1;
-        } else if (rule == 3) {
-            lam = sigma[0] * exp10(lambda_in);
-            idx = -1;
-        } else {
-            idx = bi[0];
-            if (idx < 0 || idx >= J) idx = 0;
-            lam = sigma[0] * exp10(grid_t(idx, J, t_lo, t_hi));
-        }
-        lam_s = lam;
         if (lam_out) lam_out[b] = lam;
         if (idx_out) idx_out[b] = idx;
         if (stt && b == 0) {
@@ -147,8 +179,7 @@ __global__ void k_choose_lambda(ProjDims d, const double* __restrict__ sigma_all
             stt->info[IN_INDEX] = idx;
         }
     }
-    __syncthreads();
-    const double lam2 = lam_s * lam_s;
+    const double lam2 = lam * lam;
     double e2 = 0.0, r2 = 0.0;
     for (int i = threadIdx.x; i < l; i += blockDim.x) {
         const double s = sigma[i];
@@ -160,30 +191,22 @@ __global__ void k_choose_lambda(ProjDims d, const double* __restrict__ sigma_all
         r2 = fma(q, q, r2);
     }
     if (stt && b == 0) {
-        __syncthreads();
-        bv[threadIdx.x] = e2;
-        gcv_red[threadIdx.x] = r2;
-        __syncthreads();
-        for (int off = blockDim.x / 2; off > 0; off >>= 1) {
-            if ((int)threadIdx.x < off) {
-                bv[threadIdx.x] += bv[threadIdx.x + off];
-                gcv_red[threadIdx.x] += gcv_red[threadIdx.x + off];
-            }
-            __syncthreads();
-        }
+        block_sum2(e2, r2);
         if (threadIdx.x == 0) {
-            stt->scal[SC_ETA] = sqrt(bv[0]);
-            stt->scal[SC_RHO] = sqrt(fma(ftil[l], ftil[l], gcv_red[0]));
+            stt->scal[SC_ETA] = sqrt(e2);
+            stt->scal[SC_RHO] = sqrt(fma(ftil[l], ftil[l], r2));
         }
     }
 }
 
 // Ine-TSVD rank by GCV_l(k) (or the given rank) and cvec_i = f_i / s_i, i <= k.
-__global__ void k_choose_rank(ProjDims d, const double* __restrict__ sigma_all,
-                              const double* __restrict__ ftil_all, int rank_in, double* __restrict__ curve_all,
-                              double* __restrict__ cvec_all, double* __restrict__ work_all,
-                              int* __restrict__ rank_out, rbf_dev_state* __restrict__ stt) {
-    __shared__ int k_s;
+// The suffix sums S_k = sum_{i>k} f_i^2 + f_{l+1}^2 by a block scan from the end
+// (one thread summing them took 95 us at l = 140).
+__global__ void __launch_bounds__(CH_T)
+    k_choose_rank(ProjDims d, const double* __restrict__ sigma_all, const double* __restrict__ ftil_all, int rank_in,
+                  double* __restrict__ curve_all, double* __restrict__ cvec_all, int* __restrict__ rank_out,
+                  rbf_dev_state* __restrict__ stt) {
+    __shared__ double wsum[CH_T / 32];
     const int b = blockIdx.x;
     const int l = sel_l(d, b);
     if (l < 1) return;
@@ -191,75 +214,114 @@ __global__ void k_choose_rank(ProjDims d, const double* __restrict__ sigma_all,
     const double* ftil = ftil_all + (size_t)b * (d.L + 1);
     double* curve = curve_all ? curve_all + (size_t)b * d.L : nullptr;
     double* cvec = cvec_all + (size_t)b * d.L;
-    double* work = work_all + (size_t)b * (d.L + 2);
-    if (threadIdx.x == 0) {
-        const double s1 = sigma[0];
-        int r = 0;
-        for (int i = 0; i < l; ++i) r += sigma[i] > (double)(l + 1) * DBL_EPSILON * s1 ? 1 : 0;
-        int k = rank_in;
-        if (k <= 0) {
-            // suffix sums S_k = sum_{i=k+1}^{l} f_i^2 + f_{l+1}^2 (1-based i), k = l..1
-            double acc = ftil[l] * ftil[l];
-            for (int kk = l; kk >= 1; --kk) {
-                work[kk] = acc;       // S_kk
-                acc = fma(ftil[kk - 1], ftil[kk - 1], acc);
-            }
-            double best = INFINITY;
-            k = 1;
-            for (int kk = 1; kk <= r; ++kk) {
-                const double dd = (double)(l + 1 - kk);
-                const double gv = work[kk] / (dd * dd);
-                if (curve) curve[kk - 1] = gv;
-                if (gv < best) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const double s1 = sigma[0];
+    const double thr = (double)(l + 1) * DBL_EPSILON * s1;
+    int k = rank_in;
+    if (k <= 0) {
+        // thread t: the terms l - t per - per .. l - t per - 1 (0-based), summed
+        // downwards after the terms of the threads before it and f_{l+1}^2
+        const int per = (l + CH_T - 1) / CH_T;
+        const int i1 = max(0, l - (int)threadIdx.x * per), i0 = max(0, i1 - per);
+        double run = 0.0;
+        for (int i = i1 - 1; i >= i0; --i) run = fma(ftil[i], ftil[i], run);
+        double pre = run;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double t = __shfl_up_sync(RBF_FULL_MASK, pre, o);
+            if (lane >= o) pre += t;
+        }
+        if (lane == 31) wsum[warp] = pre;
+        __syncthreads();
+        double acc = pre - run;
+        for (int w = 0; w < warp; ++w) acc += wsum[w];
+        acc = fma(ftil[l], ftil[l], acc);
+        double best = INFINITY;
+        int besti = 0x7fffffff;
+        for (int i = i1 - 1; i >= i0; --i) {  // acc = S_{i+1}: the terms past the first i + 1
+            if (sigma[i] > thr) {
+                const double dd = (double)(l - i);
+                const double gv = acc / (dd * dd);
+                if (curve) curve[i] = gv;
+                if (gv < best || (gv == best && i + 1 < besti)) {
                     best = gv;
-                    k = kk;
+                    besti = i + 1;
                 }
             }
-            if (r == 0) k = 1;
+            acc = fma(ftil[i], ftil[i], acc);
         }
-        if (k > l) k = l;
-        k_s = k;
+        block_best(best, besti, false);
+        k = best < INFINITY ? besti : 1;
+    }
+    if (k > l) k = l;
+    double e2 = 0.0, r2 = 0.0;
+    for (int i = threadIdx.x; i < l; i += blockDim.x) {
+        const double f = ftil[i];
+        const double cv = i < k ? f / sigma[i] : 0.0;
+        cvec[i] = cv;
+        if (i < k) e2 = fma(cv, cv, e2);
+        else r2 = fma(f, f, r2);
+    }
+    if (stt && b == 0) block_sum2(e2, r2);
+    if (threadIdx.x == 0) {
         if (rank_out) rank_out[b] = k;
         if (stt && b == 0) {
-            double e2 = 0.0, r2 = ftil[l] * ftil[l];
-            for (int i = 0; i < l; ++i) {
-                if (i < k) {
-                    const double cv = ftil[i] / sigma[i];
-                    e2 = fma(cv, cv, e2);
-                } else {
-                    r2 = fma(ftil[i], ftil[i], r2);
-                }
-            }
             stt->info[IN_RANK] = k;
             stt->scal[SC_SIGMA1] = s1;
             stt->scal[SC_ETA] = sqrt(e2);
-            stt->scal[SC_RHO] = sqrt(r2);
+            stt->scal[SC_RHO] = sqrt(fma(ftil[l], ftil[l], r2));
         }
     }
+}
+
+// Column-major products out = M c: 32 rows x 8 column groups per CTA, four
+// chains each (with 4 groups and one chain of loads and FMAs per thread: V c at
+// l = 150 69 -> 9 us, Z y at n = 8000, l = 150 22 -> 10 us).
+constexpr int CM_GROUPS = 8;
+
+__device__ __forceinline__ double col_product(const double* __restrict__ M, int64_t ld, const double* __restrict__ c,
+                                              int l, int64_t row, bool ok, double (*red)[32]) {
+    const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
+    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+    if (ok) {
+        const double* p = M + row;
+        int m = grp;
+        for (; m + 3 * CM_GROUPS < l; m += 4 * CM_GROUPS) {
+            a0 = fma(p[(int64_t)m * ld], c[m], a0);
+            a1 = fma(p[(int64_t)(m + CM_GROUPS) * ld], c[m + CM_GROUPS], a1);
+            a2 = fma(p[(int64_t)(m + 2 * CM_GROUPS) * ld], c[m + 2 * CM_GROUPS], a2);
+            a3 = fma(p[(int64_t)(m + 3 * CM_GROUPS) * ld], c[m + 3 * CM_GROUPS], a3);
+        }
+        for (; m < l; m += CM_GROUPS) a0 = fma(p[(int64_t)m * ld], c[m], a0);
+    }
+    red[grp][lane] = (a0 + a1) + (a2 + a3);
     __syncthreads();
-    const int k = k_s;
-    for (int i = threadIdx.x; i < l; i += blockDim.x) cvec[i] = i < k ? ftil[i] / sigma[i] : 0.0;
+    double t = 0.0;
+    if (grp == 0)
+#pragma unroll
+        for (int g = 0; g < CM_GROUPS; ++g) t += red[g][lane];
+    return t;  // valid in the first warp
 }
 
 // y = V cvec (V column-major l x l, ld ldv), per instance
-__global__ void k_vmul(ProjDims d, const double* __restrict__ V_all, int64_t ldv,
-                       const double* __restrict__ cvec_all, double* __restrict__ y_all) {
+__global__ void __launch_bounds__(CM_GROUPS * 32)
+    k_vmul(ProjDims d, const double* __restrict__ V_all, int64_t ldv, const double* __restrict__ cvec_all,
+           double* __restrict__ y_all) {
+    __shared__ double red[CM_GROUPS][32];
     const int b = blockIdx.y;
     const int l = sel_l(d, b);
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= l) return;
-    const double* V = V_all + (size_t)b * d.L * ldv;
-    const double* cvec = cvec_all + (size_t)b * d.L;
-    double acc = 0.0;
-    for (int i = 0; i < l; ++i) acc = fma(V[(int64_t)i * ldv + r], cvec[i], acc);
-    y_all[(size_t)b * d.L + r] = acc;
+    const int r = blockIdx.x * 32 + (threadIdx.x & 31);
+    if ((int)blockIdx.x * 32 >= l) return;
+    const double t = col_product(V_all + (size_t)b * d.L * ldv, ldv, cvec_all + (size_t)b * d.L, l, r, r < l, red);
+    if (threadIdx.x < 32 && r < l) y_all[(size_t)b * d.L + r] = t;
 }
 
-// coef = Z y (Z column-major n x l, ld ldz): 32 rows x 4 column groups per CTA.
-// Batched: instance b = blockIdx.y with n, Z offset, ld and coef offset from tables.
-__global__ void __launch_bounds__(128) k_lift(ProjDims d, const double* __restrict__ Z_all, LiftDims ld,
-                                              const double* __restrict__ y_all, double* __restrict__ coef_all) {
-    __shared__ double red[4][32];
+// coef = Z y (Z column-major n x l, ld ldz).  Batched: instance b = blockIdx.y
+// with n, Z offset, ld and coef offset from tables.
+__global__ void __launch_bounds__(CM_GROUPS * 32)
+    k_lift(ProjDims d, const double* __restrict__ Z_all, LiftDims ld, const double* __restrict__ y_all,
+           double* __restrict__ coef_all) {
+    __shared__ double red[CM_GROUPS][32];
     __shared__ double ys[1024];
     const int b = blockIdx.y;
     const int l = sel_l(d, b);
@@ -269,17 +331,12 @@ __global__ void __launch_bounds__(128) k_lift(ProjDims d, const double* __restri
     const double* Z = Z_all + (ld.zoff ? ld.zoff[b] : 0);
     double* coef = coef_all + (ld.coff ? ld.coff[b] : 0);
     const double* y = y_all + (size_t)b * d.L;
-    for (int m = threadIdx.x; m < l; m += 128)
+    for (int m = threadIdx.x; m < l; m += CM_GROUPS * 32)
         if (RBF_IN_RANGE(m, 1024)) ys[m] = y[m];  // the projected dimension fits the shared copy
     __syncthreads();
-    const int row = threadIdx.x & 31, grp = threadIdx.x >> 5;
-    const int64_t i = (int64_t)blockIdx.x * 32 + row;
-    double acc = 0.0;
-    if (i < n)
-        for (int m = grp; m < l; m += 4) acc = fma(Z[(int64_t)m * ldz + i], ys[m], acc);
-    red[grp][row] = acc;
-    __syncthreads();
-    if (grp == 0 && i < n) coef[i] = (red[0][row] + red[1][row]) + (red[2][row] + red[3][row]);
+    const int64_t i = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31);
+    const double t = col_product(Z, ldz, ys, l, i, i < n, red);
+    if (threadIdx.x < 32 && i < n) coef[i] = t;
 }
 
 }  // namespace
@@ -301,7 +358,6 @@ rbf_status launch_select_batch(rbf_ctx* ctx, ProjDims d, int method, int rule, d
     double* ye = wc.take<double>((size_t)J * B);
     double* cvec = wc.take<double>((size_t)L * B);
     double* y = wc.take<double>((size_t)L * B);
-    double* work = wc.take<double>((size_t)(L + 2) * B);
     void* svd = (void*)wc.take<char>(svd_ws_bytes_batch(L, B));
     cudaStream_t s = ctx->stream;
     rbf_dev_state* stt = single ? ctx->d_state : nullptr;
@@ -311,23 +367,23 @@ rbf_status launch_select_batch(rbf_ctx* ctx, ProjDims d, int method, int rule, d
     rbf_timer_start(ctx);
     if (method == 0) {
         if (rule == RBF_GCV || rule == RBF_LCURVE || rule_arr) {
-            k_grid_terms<<<dim3((J + 31) / 32, B), 32, 0, s>>>(d, sigma, ftil, J, tlo, thi, gcv, xr, ye);
+            k_grid_terms<<<dim3((J + GT_WARPS - 1) / GT_WARPS, B), GT_WARPS * 32, 0, s>>>(d, sigma, ftil, J, tlo, thi, gcv, xr, ye);
             RBF_LAUNCHED(ctx, "k_grid_terms");
         }
-        k_choose_lambda<<<B, 1024, 0, s>>>(d, sigma, ftil, J, tlo, thi, rule, lambda_in, rule_arr, lam_arr, gcv, xr,
+        k_choose_lambda<<<B, CH_T, 0, s>>>(d, sigma, ftil, J, tlo, thi, rule, lambda_in, rule_arr, lam_arr, gcv, xr,
                                            ye, curve, cvec, lam_out, idx_out, stt);
         RBF_LAUNCHED(ctx, "k_choose_lambda");
     } else {
-        k_choose_rank<<<B, 256, 0, s>>>(d, sigma, ftil, rank, curve, cvec, work, rank_out, stt);
+        k_choose_rank<<<B, CH_T, 0, s>>>(d, sigma, ftil, rank, curve, cvec, rank_out, stt);
         RBF_LAUNCHED(ctx, "k_choose_rank");
     }
-    k_vmul<<<dim3((L + 127) / 128, B), 128, 0, s>>>(d, V, L, cvec, y);
+    k_vmul<<<dim3((L + 31) / 32, B), CM_GROUPS * 32, 0, s>>>(d, V, L, cvec, y);
     RBF_LAUNCHED(ctx, "k_vmul");
     ctx->tim.select_ms = rbf_timer_stop(ctx);
     rbf_timer_start(ctx);
     const int64_t nmax = ld.nmax;
     if (coef) {
-        k_lift<<<dim3((unsigned)((nmax + 31) / 32), B), 128, 0, s>>>(d, Z, ld, y, coef);
+        k_lift<<<dim3((unsigned)((nmax + 31) / 32), B), CM_GROUPS * 32, 0, s>>>(d, Z, ld, y, coef);
         RBF_LAUNCHED(ctx, "k_lift");
     }
     ctx->tim.lift_ms = rbf_timer_stop(ctx);
