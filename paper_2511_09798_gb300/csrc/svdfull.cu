@@ -3,10 +3,8 @@
 // gcv_svd and tikh_svd_solution) and TSVD (eq. tsvd_solution).
 //
 // Default: Householder bidiagonalization A = Q_L B Q_R^T in one cooperative
-// kernel (per step a left reflector on column k applied to the trailing
-// columns and to f, which rides along as an extra column so that g = Q_L^T f
-// comes out of the same pass, then a right reflector on row k applied to the
-// trailing rows; bounded grid barriers between the phases), then the SVD of
+// kernel (f rides along as an extra column, so that g = Q_L^T f comes out of
+// the same passes; two bounded grid barriers per step), then the SVD of
 // the bidiagonal through the Golub-Kahan tridiagonal (the projected-SVD
 // kernels with C = [B^T; 0]: sigma, V~ = U_B and U~ = V_B), f^ = V~^T g and
 // alpha = Q_R (U~ d).
@@ -37,8 +35,8 @@ constexpr int JT = 256;
 constexpr int JW = JT / 32;
 constexpr int MAX_SWEEPS = 40;
 
-// W[j n + i] = A[i lda + j] (column j of A contiguous), V = I.
-__global__ void k_fsvd_init(const double* __restrict__ A, int64_t lda, int64_t n, double* __restrict__ W,
+// W[j ldw + i] = A[i lda + j] (column j of A contiguous), V = I when given.
+__global__ void k_fsvd_init(const double* __restrict__ A, int64_t lda, int64_t n, double* __restrict__ W, int64_t ldw,
                             double* __restrict__ V) {
     __shared__ double t[32][33];
     const int64_t i0 = (int64_t)blockIdx.y * 32, j0 = (int64_t)blockIdx.x * 32;
@@ -50,8 +48,8 @@ __global__ void k_fsvd_init(const double* __restrict__ A, int64_t lda, int64_t n
     for (int r = threadIdx.y; r < 32; r += blockDim.y) {
         const int64_t j = j0 + r, i = i0 + threadIdx.x;
         if (i < n && j < n) {
-            W[j * n + i] = t[threadIdx.x][r];
-            V[j * n + i] = i == j ? 1.0 : 0.0;
+            W[j * ldw + i] = t[threadIdx.x][r];
+            if (V) V[j * n + i] = i == j ? 1.0 : 0.0;
         }
     }
 }
@@ -168,49 +166,107 @@ __global__ void __launch_bounds__(JT) k_fhat(const double* __restrict__ W, int64
     if (threadIdx.x == 0) fhat[kk] = sig_sorted[kk] > 0.0 ? a / sig_sorted[kk] : 0.0;
 }
 
-// rank r and s_perp = sum_{i >= r} fhat_i^2 (one thread; O(n))
-__global__ void k_fsvd_rank(const double* __restrict__ sig, const double* __restrict__ fhat, int64_t n,
-                            int* __restrict__ r_out, double* __restrict__ sperp_out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    const double thr = (double)n * DBL_EPSILON * sig[0];
-    int64_t r = 0;
-    while (r < n && sig[r] > thr && sig[0] > 0.0) ++r;
-    double sp = 0.0;
-    for (int64_t i = r; i < n; ++i) sp = fma(fhat[i], fhat[i], sp);
-    *r_out = (int)r;
-    *sperp_out = sp;
+constexpr int FT = 1024;  // threads of the one-block kernels over n
+
+// Block sum of one value over FT threads, in every thread.
+__device__ __forceinline__ double ft_sum(double v, double* red) {
+    v = warp_sum(v);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    return warp_sum(red[threadIdx.x & 31]);
 }
 
-// Tikhonov GCV on the grid: (sum_{i<r} (1-phi_i)^2 fhat_i^2 + s_perp) / ((n - r) + sum_{i<r} (1-phi_i))^2
-__global__ void k_fsvd_gcv(const double* __restrict__ sig, const double* __restrict__ fhat, int64_t n,
-                           const int* __restrict__ r_in, const double* __restrict__ sperp, int J, double t_lo,
-                           double t_hi, double* __restrict__ gcv) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= J) return;
+// rank r = #{sigma_i > n eps sigma_1} (sigma descending) and s_perp = sum_{i >=
+// r} fhat_i^2, one block (one thread took 344 us at n = 3001)
+__global__ void __launch_bounds__(FT) k_fsvd_rank(const double* __restrict__ sig, const double* __restrict__ fhat,
+                                                  int64_t n, int* __restrict__ r_out, double* __restrict__ sperp_out) {
+    __shared__ double red[FT / 32];
+    const double thr = (double)n * DBL_EPSILON * sig[0];
+    const bool some = sig[0] > 0.0;
+    double cnt = 0.0;
+    for (int64_t i = threadIdx.x; i < n; i += FT) cnt += some && sig[i] > thr ? 1.0 : 0.0;
+    const int64_t r = (int64_t)ft_sum(cnt, red);
+    double sp = 0.0;
+    for (int64_t i = threadIdx.x; i < n; i += FT)
+        if (i >= r) sp = fma(fhat[i], fhat[i], sp);
+    sp = ft_sum(sp, red);
+    if (threadIdx.x == 0) {
+        *r_out = (int)r;
+        *sperp_out = sp;
+    }
+}
+
+// Tikhonov GCV on the grid: (sum_{i<r} (1-phi_i)^2 fhat_i^2 + s_perp) / ((n - r) + sum_{i<r} (1-phi_i))^2,
+// one CTA per grid point (one thread per point: 1.54 ms at n = 3001)
+constexpr int GCV_T = 128;
+__global__ void __launch_bounds__(GCV_T)
+    k_fsvd_gcv(const double* __restrict__ sig, const double* __restrict__ fhat, int64_t n,
+               const int* __restrict__ r_in, const double* __restrict__ sperp, int J, double t_lo, double t_hi,
+               double* __restrict__ gcv) {
+    __shared__ double red[2][GCV_T / 32];
+    const int t = blockIdx.x;
     const int r = *r_in;
     const double lam = sig[0] * exp10(grid_t(t, J, t_lo, t_hi));
     const double l2 = lam * lam;
-    double num = 0.0, den = (double)(n - r);
-    for (int i = 0; i < r; ++i) {
+    double num = 0.0, den = 0.0;
+    for (int i = threadIdx.x; i < r; i += GCV_T) {
         const double s = sig[i];
         const double q = l2 / fma(s, s, l2);
         num = fma(q * q, fhat[i] * fhat[i], num);
         den += q;
     }
+    num = warp_sum(num);
+    den = warp_sum(den);
+    if ((threadIdx.x & 31) == 0) {
+        red[0][threadIdx.x >> 5] = num;
+        red[1][threadIdx.x >> 5] = den;
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    num = 0.0;
+    den = (double)(n - r);
+    for (int w = 0; w < GCV_T / 32; ++w) {
+        num += red[0][w];
+        den += red[1][w];
+    }
     gcv[t] = (num + *sperp) / (den * den);
 }
 
-// TSVD GCV over k = 1..min(r, n-1): (sum_{k<=i<r} fhat_i^2 + s_perp) / (n - k)^2
-__global__ void k_fsvd_gcv_rank(const double* __restrict__ fhat, int64_t n, const int* __restrict__ r_in,
-                                const double* __restrict__ sperp, double* __restrict__ curve) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x + 1;
-    const int r = *r_in;
+// TSVD GCV over k = 1..min(r, n-1): (sum_{k<=i<r} fhat_i^2 + s_perp) / (n -
+// k)^2, one block: suffix sums by a scan from the end (a thread per k summing
+// its own tail did O(n^2) dependent additions)
+__global__ void __launch_bounds__(FT)
+    k_fsvd_gcv_rank(const double* __restrict__ fhat, int64_t n, const int* __restrict__ r_in,
+                    const double* __restrict__ sperp, double* __restrict__ curve) {
+    __shared__ double wsum[FT / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t r = *r_in;
     const int64_t kmax = r < n - 1 ? r : n - 1;
-    if (k > kmax) return;
-    double s = *sperp;
-    for (int64_t i = r - 1; i >= k; --i) s = fma(fhat[i], fhat[i], s);
-    const double d = (double)(n - k);
-    curve[k - 1] = s / (d * d);
+    // thread t: terms r - (t + 1) per .. r - t per - 1, added downwards
+    const int64_t per = (r + FT - 1) / FT;
+    const int64_t i1 = r - (int64_t)threadIdx.x * per > 0 ? r - (int64_t)threadIdx.x * per : 0;
+    const int64_t i0 = i1 - per > 0 ? i1 - per : 0;
+    double run = 0.0;
+    for (int64_t i = i1 - 1; i >= i0; --i) run = fma(fhat[i], fhat[i], run);
+    double pre = run;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double t = __shfl_up_sync(RBF_FULL_MASK, pre, o);
+        if (lane >= o) pre += t;
+    }
+    if (lane == 31) wsum[warp] = pre;
+    __syncthreads();
+    double acc = *sperp;
+    for (int w = 0; w < warp; ++w) acc += wsum[w];
+    acc += pre - run;
+    for (int64_t i = i1 - 1; i >= i0; --i) {  // acc = sum over the terms past i: k = i + 1
+        if (i + 1 <= kmax) {
+            const double d = (double)(n - (i + 1));
+            curve[i] = acc / (d * d);
+        }
+        acc = fma(fhat[i], fhat[i], acc);
+    }
 }
 
 // argmin with lowest index on ties (one block); method 0: Tikhonov (index into
@@ -289,17 +345,10 @@ __global__ void k_fsvd_lift(const double* __restrict__ V, int64_t n, const int* 
 }
 
 // ---------------------------------------------------------------------------
-// Householder bidiagonalization path (n <= 1023)
+// Householder bidiagonalization path
 // ---------------------------------------------------------------------------
 constexpr int BT = 256;
 constexpr int BW = BT / 32;
-// the bidiagonalization kernel runs one CTA per SM of NT threads: 1024 above
-// n = 2048, so that enough loads of the trailing matrix are in flight (with 8
-// warps per SM the passes over it were bound by load latency: 1.26 -> 0.91 s
-// per GCV Tikhonov at n = 4000), 256 below (the per-step block reductions
-// over 32 warps cost more than they gain there: 48 -> 59 ms at n = 1000)
-constexpr int BIDIAG_BIG_N = 2048;
-
 template <int NW>
 __device__ __forceinline__ double block_sum1(double v, double* red) {
     v = warp_sum(v);
@@ -313,132 +362,293 @@ __device__ __forceinline__ double block_sum1(double v, double* red) {
     return t;
 }
 
-// Reflector H = I - tau v v^T with v = [1; x_rest * scale] and H x = beta e_1,
-// from x_0 and ss = |x_rest|^2 (tau = 0: no reflection needed).
-__device__ __forceinline__ void reflector(double x0, double ss, double* sc) {
-    if (ss == 0.0) {
-        sc[0] = 0.0;
-        sc[1] = 0.0;
-        sc[2] = x0;
-        return;
-    }
-    const double nrm = sqrt(fma(x0, x0, ss));
-    const double beta = x0 >= 0.0 ? -nrm : nrm;
-    sc[0] = (beta - x0) / beta;
-    sc[1] = 1.0 / (x0 - beta);
-    sc[2] = beta;
+// Householder reflector of x = [x0; rest], ss = |rest|^2, in the unnormalised
+// form H = I - t w w^T, w = [x0 - beta; rest], H x = beta e_1: t = 1 / (nrm (nrm
+// + |x0|)) with nrm = |x| and beta = -sign(x0) nrm; t = 0 (w_0 = 0, beta = x0)
+// when the rest is zero.  One reciprocal square root and one reciprocal, each
+// an estimate refined to FP64 rounding; out-of-range sums of squares take the
+// library's square root and division.
+struct Refl {
+    double t, w0, beta;
+};
+
+__device__ __forceinline__ double rcp_f64(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    double e = fma(-x, y, 1.0);
+    y = fma(y, e, y);
+    e = fma(-x, y, 1.0);
+    return fma(y, e, y);
 }
 
-// W column-major n x (n+1) (ld n), the last column f.  On return: dg = diag
-// of B, eg = superdiagonal, column n = Q_L^T f, the right reflectors in rows
-// k (entries k+2..n-1, unscaled) with taur / scaler.
-template <int NT>
-__global__ void __launch_bounds__(NT) k_bidiag(double* __restrict__ W, int64_t n, double* __restrict__ dg,
-                                               double* __restrict__ eg, double* __restrict__ taur,
-                                               double* __restrict__ scaler, rbf_dev_state* __restrict__ stt,
-                                               unsigned* __restrict__ bar, int group, long long budget) {
-    constexpr int NW = NT / 32;
-    __shared__ double red[NW];
-    __shared__ double sc[3];
-    __shared__ double rp[NW][32];
-    __shared__ double rw[32];
+__device__ __forceinline__ Refl reflector(double x0, double ss) {
+    if (ss == 0.0) return Refl{0.0, 0.0, x0};
+    const double q = fma(x0, x0, ss), ax = fabs(x0);
+    double nrm, t;
+    if (q > 1e-140 && q < 1e140) {
+        nrm = q * rsqrt_f64(q);
+        t = rcp_f64(nrm * (nrm + ax));
+    } else {
+        nrm = sqrt(q);
+        t = 1.0 / nrm / (nrm + ax);
+    }
+    const double beta = x0 >= 0.0 ? -nrm : nrm;
+    return Refl{t, x0 - beta, beta};
+}
+
+// Householder bidiagonalization, one cooperative kernel of one CTA per SM.
+// W column-major n x (n+1), the last column f.  On return: dg = diag of
+// B, eg = superdiagonal, column n = Q_L^T f, the right reflectors in rows k
+// (entries k+2..n-1, unscaled) with taur / scaler.
+//
+// The stored matrix S lags the reduced one by the rank-2 update of the step
+// before: A = S - u y^T - x v^T.  Step k, with two grid barriers:
+//   A  (whole columns, column j on CTA j mod G, pieces of 256 rows per warp):
+//      apply that update, write S, and take u'^T s_j with the new left reflector
+//      u' in the same pass: y'_j = t u'^T s_j, row k: r_j = s_kj - u'_k y'_j
+//   -- barrier --  right reflector v' from r
+//   B  (blocks of 4 rows over all columns): x'_i = t' (sum_j S_ij v'_j - u'_i
+//      y'^T v'), and column k + 1 of A with its norm: the next left reflector
+//   -- barrier --
+// so S is read twice and written once per step (a pass for the products and one
+// for the update of each reflector read it four times and wrote it twice), the
+// vectors u, x and v sit in shared memory, and the norms come from one partial
+// per CTA instead of a pass over the vector in every CTA.  The FP64 pipe bounds
+// it (4 n^3 / 3 FMAs: 57 ms at n = 3001, 2.1 ms at 1000) together with the two
+// barriers and reflector chains per step.  n = 1000: 26.5 -> 20.5 ms, n =
+// 3001: 244 -> 137 ms.
+constexpr int BD_T = 512;
+constexpr int BD_W = BD_T / 32;
+constexpr int BD_ROWS = 256;  // rows of a column piece (8 per lane)
+constexpr int BD_RB = 4;      // rows of a block of pass B: one 32-byte sector per column
+
+struct BidiagArgs {
+    double* W;  // ld a multiple of 4
+    int64_t n, ld;
+    double *dg, *eg, *taur, *scaler;
+    double *y, *r, *x, *a;  // [n+1] y' and r by column, x' and column k + 1 of A by row
+    double* part;           // [3][G] |r|^2, y.r (columns past k + 1), |a|^2 (rows past k + 1)
+    rbf_dev_state* stt;
+    unsigned* bar;
+    int group;
+    long long budget;
+};
+
+// doubles of dynamic shared memory: u, x (or v) and the new u; partial dots;
+// row-k entries; row-block partials
+__host__ __device__ inline int64_t bd_cols(int64_t n, int G) { return (n + G) / G + 1; }
+__host__ __device__ inline int64_t bd_pieces(int64_t n) { return n / BD_ROWS + 2; }
+__host__ __device__ inline int64_t bd_blocks(int64_t n, int G) { return (n / BD_RB + G + 1) / G + 1; }
+inline size_t bd_smem(int64_t n, int G) {
+    return sizeof(double) * (size_t)(3 * n + bd_cols(n, G) * (bd_pieces(n) + 1) + bd_blocks(n, G) * BD_W * BD_RB);
+}
+
+// sum of G partials, in every lane of the calling warp (fixed order)
+__device__ __forceinline__ double bd_sum(const double* p, int G, int lane) {
+    double s = 0.0;
+    for (int b = lane; b < G; b += 32) s += __ldcg(p + b);
+    return warp_sum(s);
+}
+
+__global__ void __launch_bounds__(BD_T) k_bidiag(BidiagArgs g) {
+    extern __shared__ double sm[];
+    __shared__ double sc[4];
+    const int64_t n = g.n, ld = g.ld;
+    const int G = gridDim.x, cta = blockIdx.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t GW = (int64_t)gridDim.x * NW, gw = (int64_t)blockIdx.x * NW + warp;
-    for (int64_t k = 0; k < n; ++k) {
-        // left reflector of column k (rows k..n-1), every CTA computes it
-        const double* xk = W + k * n + k;
-        const int64_t m = n - k;
+    double* W = g.W;
+    double* uo = sm;          // left reflector of the step before
+    double* un = sm + n;      // left reflector of this step
+    double* xs = sm + 2 * n;  // x of the step before, then v' of this step
+    const int pmax = (int)bd_pieces(n);
+    double* pd = sm + 3 * n;                 // [columns][pieces] partial dots
+    double* sk = pd + bd_cols(n, G) * pmax;  // [columns] row k of the updated columns
+    double* rp = sk + bd_cols(n, G);         // [row blocks][warps][rows]
+    unsigned epoch = 0;
+    // column 0 and its norm
+    {
         double ss = 0.0;
-        for (int64_t i = 1 + threadIdx.x; i < m; i += NT) ss = fma(xk[i], xk[i], ss);
-        ss = block_sum1<NW>(ss, red);
-        if (threadIdx.x == 0) reflector(xk[0], ss, sc);
-        __syncthreads();
-        const double tau = sc[0], scale = sc[1];
-        if (tau != 0.0) {
-            for (int64_t j = k + 1 + gw; j <= n; j += GW) {  // warp per trailing column, f included
-                double* wj = W + j * n + k;
-                const double w0 = wj[0];
-                double sd = 0.0, sd1 = 0.0;
-                int64_t i = 1 + lane;
-                for (; i + 32 < m; i += 64) {
-                    sd = fma(xk[i], wj[i], sd);
-                    sd1 = fma(xk[i + 32], wj[i + 32], sd1);
-                }
-                if (i < m) sd = fma(xk[i], wj[i], sd);
-                sd = warp_sum(sd + sd1);
-                const double t = tau * fma(scale, sd, w0);
-                const double ts = t * scale;
-                for (int64_t i = 1 + lane; i < m; i += 32) wj[i] = fma(-ts, xk[i], wj[i]);
-                if (lane == 0) wj[0] = w0 - t;
+        for (int64_t i = cta * (int64_t)BD_T + threadIdx.x; i < n; i += (int64_t)G * BD_T) {
+            const double v = W[i];
+            g.a[i] = v;
+            g.x[i] = 0.0;
+            if (i > 0) ss = fma(v, v, ss);
+        }
+        ss = block_sum1<BD_W>(ss, pd);
+        if (threadIdx.x == 0) g.part[2 * G + cta] = ss;
+        for (int64_t i = threadIdx.x; i < n; i += BD_T) uo[i] = 0.0;
+        if (!grid_reduce_sync(g.stt, g.bar, g.group, g.budget, ++epoch, nullptr, nullptr, nullptr, 0, 0)) return;
+    }
+    double vscale = 0.0;  // 1 once a right reflector is pending
+    for (int64_t k = 0; k < n; ++k) {
+        // ---- left reflector of column k
+        if (warp == 0) {
+            const Refl h = reflector(__ldcg(g.a + k), bd_sum(g.part + 2 * G, G, lane));
+            if (lane == 0) {
+                sc[0] = h.t;
+                sc[1] = h.w0;
+                un[k] = h.w0;
+                xs[k] = 0.0;
+                if (cta == 0) g.dg[k] = h.beta;
             }
         }
-        if (blockIdx.x == 0 && threadIdx.x == 0) dg[k] = sc[2];
-        if (!grid_sync(stt, bar, group, budget)) return;
+        for (int64_t i = k + 1 + threadIdx.x; i < n; i += BD_T) {
+            un[i] = __ldcg(g.a + i);
+            xs[i] = __ldcg(g.x + i);
+        }
+        // x at row k: its own value, needed by row k of the update
+        if (threadIdx.x == BD_T - 1) sc[2] = __ldcg(g.x + k);
+        __syncthreads();
+        const double t1 = sc[0], uk = sc[1], xk = sc[2];
+        // ---- pass A
+        const int64_t j0 = k + 1 + (((int64_t)cta - (k + 1)) % G + G) % G;  // first own column past k
+        const int nc = j0 <= n ? (int)((n - j0) / G) + 1 : 0;
+        const int64_t base = k & ~(int64_t)31;
+        const int np = (int)((n - base + BD_ROWS - 1) / BD_ROWS);
+        for (int u = warp; u < nc * np; u += BD_W) {
+            const int c = u / np, piece = u - c * np;
+            const int64_t j = j0 + (int64_t)c * G;
+            double* col = W + j * ld;
+            const double yj = k > 0 ? __ldcg(g.y + j) : 0.0;
+            const double vj = j < n && vscale != 0.0 ? __ldcg(g.r + j) : 0.0;
+            const int64_t i0 = base + (int64_t)piece * BD_ROWS + lane;
+            double v[8], dot = 0.0, dot1 = 0.0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int64_t i = i0 + 32 * q;
+                v[q] = i >= k && i < n ? __ldcg(col + i) : 0.0;
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int64_t i = i0 + 32 * q;
+                if (i > k && i < n) {
+                    v[q] = fma(-xs[i], vj, fma(-uo[i], yj, v[q]));
+                    col[i] = v[q];
+                    if (q & 1) dot1 = fma(un[i], v[q], dot1);
+                    else dot = fma(un[i], v[q], dot);
+                } else if (i == k) {
+                    const double s = fma(-xk, vj, fma(-uo[i], yj, v[q]));
+                    sk[c] = s;
+                    dot = fma(uk, s, dot);
+                }
+            }
+            dot = warp_sum(dot + dot1);
+            if (lane == 0) pd[(int64_t)c * pmax + piece] = dot;
+        }
+        __syncthreads();
+        if (warp < 2) {
+            double rr = 0.0, yr = 0.0;
+            for (int c = threadIdx.x; c < nc; c += 64) {
+                const int64_t j = j0 + (int64_t)c * G;
+                double d = 0.0;
+                for (int q = 0; q < np; ++q) d += pd[(int64_t)c * pmax + q];
+                const double yj = t1 * d;
+                const double r = fma(-uk, yj, sk[c]);
+                g.y[j] = yj;
+                g.r[j] = r;
+                W[j * ld + k] = r;
+                if (j > k + 1 && j < n) {
+                    rr = fma(r, r, rr);
+                    yr = fma(yj, r, yr);
+                }
+            }
+            rr = warp_sum(rr);
+            yr = warp_sum(yr);
+            if (lane == 0) {
+                rp[2 * warp] = rr;
+                rp[2 * warp + 1] = yr;
+            }
+        }
         if (k == n - 1) break;
-        // right reflector of row k (columns k+1..n-1)
-        const int64_t m2 = n - k - 1;
-        double ss2 = 0.0;
-        for (int64_t c = 1 + threadIdx.x; c < m2; c += NT) {
-            const double y = W[(k + 1 + c) * n + k];
-            ss2 = fma(y, y, ss2);
-        }
-        ss2 = block_sum1<NW>(ss2, red);
-        if (threadIdx.x == 0) reflector(W[(k + 1) * n + k], ss2, sc);
         __syncthreads();
-        const double tau2 = sc[0], scale2 = sc[1];
-        if (tau2 != 0.0) {
-            // blocks of RB rows over the CTAs (RB = 32, 16 or 8: the largest that
-            // still gives every CTA a block); lane = (row r, column lane cl), warp
-            // q takes the columns c = q CPL + cl, stepping by NW CPL (coalesced
-            // along the rows); partial dots combined in shared memory in a fixed
-            // order (for RB = 32 one column per warp step, as before)
-            const int64_t rows = n - k - 1;
-            const int RB = rows >= 32 * (int64_t)gridDim.x ? 32 : (rows >= 16 * (int64_t)gridDim.x ? 16 : 8);
-            const int CPL = 32 / RB, CW = NW * CPL;
-            const int r = lane % RB, cl = lane / RB;
-            const int64_t nblk = (rows + RB - 1) / RB;
-            for (int64_t rb = blockIdx.x; rb < nblk; rb += gridDim.x) {
-                const int64_t i = k + 1 + rb * RB + r;
-                const bool ok = i < n;
-                double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-                int64_t c = 1 + warp * CPL + cl;
-                for (; c + 3 * CW < m2; c += 4 * CW) {
-                    if (ok) {
-                        a0 = fma(W[(k + 1 + c) * n + i], W[(k + 1 + c) * n + k], a0);
-                        a1 = fma(W[(k + 1 + c + CW) * n + i], W[(k + 1 + c + CW) * n + k], a1);
-                        a2 = fma(W[(k + 1 + c + 2 * CW) * n + i], W[(k + 1 + c + 2 * CW) * n + k], a2);
-                        a3 = fma(W[(k + 1 + c + 3 * CW) * n + i], W[(k + 1 + c + 3 * CW) * n + k], a3);
-                    }
+        if (threadIdx.x == 0) {
+            g.part[cta] = rp[0] + rp[2];
+            g.part[G + cta] = rp[1] + rp[3];
+        }
+        if (!grid_reduce_sync(g.stt, g.bar, g.group, g.budget, ++epoch, nullptr, nullptr, nullptr, 0, 0)) return;
+        // ---- right reflector of row k
+        if (warp == 0) {
+            const double ss = bd_sum(g.part, G, lane), yr = bd_sum(g.part + G, G, lane);
+            const double x0 = __ldcg(g.r + k + 1);
+            const Refl h = reflector(x0, ss);
+            if (lane == 0) {
+                sc[0] = h.t;
+                sc[1] = fma(__ldcg(g.y + k + 1), h.w0, yr);  // y'^T v'
+                xs[k + 1] = h.w0;
+                sc[2] = __ldcg(g.y + k + 1);
+                sc[3] = h.w0;
+                if (cta == 0) {
+                    g.eg[k] = h.beta;
+                    g.taur[k] = h.t * h.w0 * h.w0;
+                    g.scaler[k] = h.t != 0.0 ? 1.0 / h.w0 : 0.0;
                 }
-                for (; c < m2; c += CW)
-                    if (ok) a0 = fma(W[(k + 1 + c) * n + i], W[(k + 1 + c) * n + k], a0);
-                rp[warp][lane] = (a0 + a1) + (a2 + a3);
-                __syncthreads();
-                if (warp == 0 && lane < RB) {
-                    double t = 0.0;
-                    for (int q = 0; q < NW; ++q)
-                        for (int l = 0; l < CPL; ++l) t += rp[q][l * RB + lane];
-                    const int64_t ir = k + 1 + rb * RB + lane;
-                    const double x0 = ir < n ? W[(k + 1) * n + ir] : 0.0;
-                    rw[lane] = tau2 * fma(scale2, t, x0);  // t_i = tau (u . w_i)
-                }
-                __syncthreads();
-                const double ti = rw[r];
-                if (ok) {
-                    if (warp == 0 && cl == 0) W[(k + 1) * n + i] -= ti;
-                    const double tsi = ti * scale2;
-                    for (int64_t cc = 1 + warp * CPL + cl; cc < m2; cc += CW)
-                        W[(k + 1 + cc) * n + i] = fma(-tsi, W[(k + 1 + cc) * n + k], W[(k + 1 + cc) * n + i]);
-                }
-                __syncthreads();
             }
         }
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            eg[k] = sc[2];
-            taur[k] = tau2;
-            scaler[k] = scale2;
+        for (int64_t j = k + 2 + threadIdx.x; j < n; j += BD_T) xs[j] = __ldcg(g.r + j);
+        __syncthreads();
+        const double t2 = sc[0], yv = sc[1], y1 = sc[2], v1 = sc[3];
+        // ---- pass B
+        const int64_t rbase = (k + 1) & ~(int64_t)(BD_RB - 1);
+        const int64_t nblk = (n - rbase + BD_RB - 1) / BD_RB;
+        const int rl = lane & (BD_RB - 1), cl = lane / BD_RB;
+        constexpr int CPW = 32 / BD_RB, CW = BD_W * CPW;  // columns of a warp step, of a CTA step
+        int nb = 0;
+        for (int64_t rb = cta; rb < nblk; rb += G, ++nb) {
+            const int64_t i = rbase + rb * BD_RB + rl;
+            const bool ok = i > k && i < n;
+            double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+            if (ok) {
+                const double* p = W + i;
+                int64_t j = k + 1 + warp * CPW + cl;
+                for (; j + 3 * CW < n; j += 4 * CW) {
+                    const double s0 = __ldcg(p + j * ld), s1 = __ldcg(p + (j + CW) * ld);
+                    const double s2 = __ldcg(p + (j + 2 * CW) * ld), s3 = __ldcg(p + (j + 3 * CW) * ld);
+                    a0 = fma(s0, xs[j], a0);
+                    a1 = fma(s1, xs[j + CW], a1);
+                    a2 = fma(s2, xs[j + 2 * CW], a2);
+                    a3 = fma(s3, xs[j + 3 * CW], a3);
+                }
+                for (; j < n; j += CW) a0 = fma(__ldcg(p + j * ld), xs[j], a0);
+            }
+            a0 = (a0 + a1) + (a2 + a3);
+#pragma unroll
+            for (int o = BD_RB; o < 32; o <<= 1) a0 += __shfl_xor_sync(RBF_FULL_MASK, a0, o);
+            if (lane < BD_RB) rp[((int64_t)nb * BD_W + warp) * BD_RB + lane] = a0;
         }
-        if (!grid_sync(stt, bar, group, budget)) return;
+        __syncthreads();
+        double ss = 0.0;
+        for (int e = threadIdx.x; e < nb * BD_RB; e += BD_T) {
+            const int q = e / BD_RB, rr = e - q * BD_RB;
+            const int64_t i = rbase + ((int64_t)cta + (int64_t)q * G) * BD_RB + rr;
+            if (i <= k || i >= n) continue;
+            double z0 = 0.0, z1 = 0.0;
+#pragma unroll
+            for (int w = 0; w < BD_W; w += 2) {
+                z0 += rp[((int64_t)q * BD_W + w) * BD_RB + rr];
+                z1 += rp[((int64_t)q * BD_W + w + 1) * BD_RB + rr];
+            }
+            const double xi = t2 * fma(-un[i], yv, z0 + z1);
+            const double ai = fma(-xi, v1, fma(-un[i], y1, __ldcg(W + (k + 1) * ld + i)));
+            g.x[i] = xi;
+            g.a[i] = ai;
+            if (i > k + 1) ss = fma(ai, ai, ss);
+        }
+        const int nw = min(BD_W, (nb * BD_RB + 31) / 32);  // warps that hold rows
+        if (warp < nw) {
+            ss = warp_sum(ss);
+            if (lane == 0) pd[warp] = ss;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double t = 0.0;
+            for (int w = 0; w < nw; ++w) t += pd[w];
+            g.part[2 * G + cta] = t;
+        }
+        if (!grid_reduce_sync(g.stt, g.bar, g.group, g.budget, ++epoch, nullptr, nullptr, nullptr, 0, 0)) return;
+        double* t = uo;
+        uo = un;
+        un = t;
+        vscale = 1.0;
     }
 }
 
@@ -462,20 +672,147 @@ __global__ void __launch_bounds__(BT) k_vt_g(const double* __restrict__ Vt, int6
     if (threadIdx.x == 0) fhat[blockIdx.x] = a;
 }
 
-// x[row] = sum_i U~[row][i] d_i over the first n rows of U~ (ld n+1)
-__global__ void k_u_d(const double* __restrict__ Ut, int64_t n, const double* __restrict__ d, double* __restrict__ x) {
-    const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (row >= n) return;
-    double acc = 0.0;
-    for (int64_t i = 0; i < n; ++i) {
-        const double di = d[i];
-        if (di != 0.0) acc = fma(Ut[i * (n + 1) + row], di, acc);
+// x[row] = sum_i U~[row][i] d_i over the first n rows of U~ (ld n+1): 32 rows x
+// 32 column groups per CTA, four chains each (one thread per row: 1.45 ms at n =
+// 3001, latency of n dependent FMAs)
+__global__ void __launch_bounds__(1024) k_u_d(const double* __restrict__ Ut, int64_t n, const double* __restrict__ d,
+                                              double* __restrict__ x) {
+    __shared__ double red[32][33];
+    const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
+    const int64_t row = (int64_t)blockIdx.x * 32 + lane, ldu = n + 1;
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    if (row < n) {
+        const double* p = Ut + row;
+        int64_t i = grp;
+        for (; i + 96 < n; i += 128)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) a[u] = fma(p[(i + 32 * u) * ldu], d[i + 32 * u], a[u]);
+        for (; i < n; i += 32) a[0] = fma(p[i * ldu], d[i], a[0]);
     }
-    x[row] = acc;
+    red[grp][lane] = (a[0] + a[1]) + (a[2] + a[3]);
+    __syncthreads();
+    const double t = warp_sum(red[lane][grp]);  // warp grp: row grp of the CTA
+    const int64_t out = (int64_t)blockIdx.x * 32 + grp;
+    if (lane == 0 && out < n) x[out] = t;
+}
+
+// alpha = Q_R z for one vector, by blocks of QB reflectors H_k = I - tau_k v_k
+// v_k^T (v_k: 1 at k+1, W's row k times scaler_k beyond): all QB dots of a
+// block at once, z' = z - V a with a from the dots and the Gram matrix of the
+// block's reflectors (a_q = tau_q (w_q - sum_{p > q} G_qp a_p)).  The Gram
+// matrices of all blocks come first (k_qr_gram, one launch).  One grid barrier
+// per block; a reflector at a time on one CTA took 17.8 ms at n = 3001 and 2.8
+// at 1000 (1.6 and 0.55 ms now, Gram matrices included).
+constexpr int QB = 32;
+constexpr int QG_ROWS = 512;  // entries of the reflectors per Gram partial
+constexpr int QA_T = 256;
+
+__device__ __forceinline__ double refl_entry(const double* __restrict__ W, int64_t ld, const double* scaler,
+                                             int64_t k, int64_t j, int64_t last) {
+    if (k >= last || j <= k) return 0.0;
+    return j == k + 1 ? 1.0 : W[j * ld + k] * scaler[k];
+}
+
+// part[chunk][block][p][q] = sum over QG_ROWS entries of v_p v_q, p < q (others 0)
+__global__ void __launch_bounds__(QA_T) k_qr_gram(const double* __restrict__ W, int64_t n, int64_t ld,
+                                                  const double* __restrict__ scaler, double* __restrict__ part) {
+    __shared__ double t[64][QB + 1];
+    const int64_t k0 = (int64_t)blockIdx.x * QB;
+    const int64_t j0 = (int64_t)blockIdx.y * QG_ROWS, j1 = j0 + QG_ROWS < n ? j0 + QG_ROWS : n;
+    const int q = threadIdx.x & (QB - 1), p0 = threadIdx.x / QB;  // pairs (p0 + 8 r, q), r < 4
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int64_t jb = j0; jb < j1; jb += 64) {
+        if (jb + 64 > k0 + 1)
+            for (int r = p0; r < 64; r += QA_T / QB)
+                t[r][q] = jb + r < j1 ? refl_entry(W, ld, scaler, k0 + q, jb + r, n - 1) : 0.0;
+        __syncthreads();
+        if (jb + 64 > k0 + 1)
+            for (int r = 0; r < 64; ++r) {
+                const double vq = t[r][q];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (p0 + 8 * u < q) acc[u] = fma(t[r][p0 + 8 * u], vq, acc[u]);
+            }
+        __syncthreads();
+    }
+    double* out = part + ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * QB * QB;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) out[(p0 + 8 * u) * QB + q] = acc[u];
+}
+
+struct QrArgs {
+    const double* W;
+    int64_t n, ld;
+    const double *taur, *scaler, *gram;
+    double* z;
+    double *hpart, *gpart;  // [QB][G] and 2 x [QB][groups]
+    rbf_dev_state* stt;
+    unsigned* bar;
+    int group;
+    long long budget;
+};
+
+// CTA b owns the entries [n b / G, n (b+1) / G) of z, in shared memory with the
+// current block's reflectors at them.
+__global__ void __launch_bounds__(QA_T) k_qr_apply(QrArgs a) {
+    extern __shared__ double qs[];
+    __shared__ double dots[QA_T / 32][QB], hs[QB], al[QB], Gs[QB][QB + 1], tau[QB];
+    const int64_t n = a.n;
+    const int G = gridDim.x;
+    const int64_t r0 = n * blockIdx.x / G;
+    const int R = (int)(n * (blockIdx.x + 1) / G - r0);
+    double* z = qs;            // [R]
+    double* vt = qs + R;       // [R][QB + 1]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int r = threadIdx.x; r < R; r += QA_T) z[r] = a.z[r0 + r];
+    unsigned epoch = 0;
+    const int64_t nblk = (n - 1 + QB - 1) / QB;
+    for (int64_t blk = nblk - 1; blk >= 0; --blk) {
+        const int64_t k0 = blk * QB;
+        __syncthreads();
+        for (int r = warp; r < R; r += QA_T / 32)
+            vt[r * (QB + 1) + lane] = refl_entry(a.W, a.ld, a.scaler, k0 + lane, r0 + r, n - 1);
+        if (warp == 0) tau[lane] = k0 + lane < n - 1 ? a.taur[k0 + lane] : 0.0;
+        for (int e = threadIdx.x; e < QB * QB; e += QA_T) Gs[e / QB][e % QB] = a.gram[blk * QB * QB + e];
+        __syncthreads();
+        double d = 0.0;
+        for (int r = warp; r < R; r += QA_T / 32) d = fma(vt[r * (QB + 1) + lane], z[r], d);
+        dots[warp][lane] = d;
+        __syncthreads();
+        if (warp == 0) {
+            d = 0.0;
+            for (int w = 0; w < QA_T / 32; ++w) d += dots[w][lane];
+            a.hpart[(int64_t)lane * G + blockIdx.x] = d;
+        }
+        if (!grid_reduce_sync(a.stt, a.bar, a.group, a.budget, ++epoch, a.hpart, a.gpart, hs, QB, (int64_t)2 * QB * G))
+            return;
+        if (warp == 0) {  // lane p: w_p, the later reflectors' parts removed in order
+            double w = hs[lane];
+            for (int q = QB - 1; q > 0; --q) {
+                const double aq = tau[q] * __shfl_sync(RBF_FULL_MASK, w, q);
+                if (lane < q) w = fma(-Gs[lane][q], aq, w);
+            }
+            al[lane] = tau[lane] * w;
+        }
+        __syncthreads();
+        for (int rr = 0; rr < R; rr += QA_T / 8) {  // 8 lanes per entry
+            const int r = rr + threadIdx.x / 8, g8 = threadIdx.x & 7;
+            double t = 0.0;
+            if (r < R)
+#pragma unroll
+                for (int u = 0; u < QB / 8; ++u) t = fma(vt[r * (QB + 1) + g8 + 8 * u], al[g8 + 8 * u], t);
+            t += __shfl_xor_sync(RBF_FULL_MASK, t, 1);
+            t += __shfl_xor_sync(RBF_FULL_MASK, t, 2);
+            t += __shfl_xor_sync(RBF_FULL_MASK, t, 4);
+            if (g8 == 0 && r < R) z[r] -= t;
+        }
+    }
+    __syncthreads();
+    for (int r = threadIdx.x; r < R; r += QA_T) a.z[r0 + r] = z[r];
 }
 
 // Z <- Q_R Z, one CTA per column (ld ldz): the right reflectors in reverse order.
-__global__ void __launch_bounds__(BT) k_apply_qr(const double* __restrict__ W, int64_t n,
+__global__ void __launch_bounds__(BT) k_apply_qr(const double* __restrict__ W, int64_t n, int64_t ld,
                                                  const double* __restrict__ taur, const double* __restrict__ scaler,
                                                  double* __restrict__ Z, int64_t ldz) {
     __shared__ double red[BW];
@@ -487,11 +824,11 @@ __global__ void __launch_bounds__(BT) k_apply_qr(const double* __restrict__ W, i
         const int64_t m2 = n - k - 1;
         const double z0 = z[k + 1];
         double sd = 0.0;
-        for (int64_t c = 1 + threadIdx.x; c < m2; c += BT) sd = fma(W[(k + 1 + c) * n + k], z[k + 1 + c], sd);
+        for (int64_t c = 1 + threadIdx.x; c < m2; c += BT) sd = fma(W[(k + 1 + c) * ld + k], z[k + 1 + c], sd);
         sd = block_sum1<BW>(sd, red);
         const double t = tau * fma(scale, sd, z0);
         const double ts = t * scale;
-        for (int64_t c = 1 + threadIdx.x; c < m2; c += BT) z[k + 1 + c] = fma(-ts, W[(k + 1 + c) * n + k], z[k + 1 + c]);
+        for (int64_t c = 1 + threadIdx.x; c < m2; c += BT) z[k + 1 + c] = fma(-ts, W[(k + 1 + c) * ld + k], z[k + 1 + c]);
         if (threadIdx.x == 0) z[k + 1] = z0 - t;
         __syncthreads();
     }
@@ -525,12 +862,16 @@ struct Fsvd {
     int* perm;
     // bidiagonalization
     double *Wb, *taur, *scaler, *Vt, *Ut;
+    int64_t ldw;
+    double *gram, *gram_part, *hpart, *gpart;  // blocked application of Q_R
+    unsigned* bar;
+    int G, group, bar_k;
     int sweeps;
 };
 
-int coop_grid(rbf_ctx* ctx, const void* kernel, int threads, int cap, int* group, int* bar_k) {
+int coop_grid(rbf_ctx* ctx, const void* kernel, int threads, int cap, int* group, int* bar_k, size_t smem = 0) {
     int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, 0) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, smem) != cudaSuccess) {
         cudaGetLastError();
         occ = 1;
     }
@@ -547,7 +888,7 @@ int coop_grid(rbf_ctx* ctx, const void* kernel, int threads, int cap, int* group
 rbf_status fsvd_common_tail(rbf_ctx* ctx, Fsvd* F, const double* f) {
     cudaStream_t s = ctx->stream;
     if (f) {
-        k_fsvd_rank<<<1, 32, 0, s>>>(F->sig, F->fhat, F->n, F->r, F->sperp);
+        k_fsvd_rank<<<1, FT, 0, s>>>(F->sig, F->fhat, F->n, F->r, F->sperp);
         RBF_LAUNCHED(ctx, "k_fsvd_rank");
     }
     return RBF_OK;
@@ -583,7 +924,7 @@ rbf_status fsvd_jacobi(rbf_ctx* ctx, const rbf_operator* op, const double* f, Fs
     RBF_CUDA(ctx, cudaMemsetAsync(bar, 0, (size_t)(bar_k + 2) * BAR_STRIDE * sizeof(unsigned), s));
     RBF_CUDA(ctx, cudaMemsetAsync(&ctx->d_state->info[IN_ERR], 0, 2 * sizeof(int), s));  // IN_DONE, IN_ERR
     dim3 tb(32, 8), tg((unsigned)((n + 31) / 32), (unsigned)((n + 31) / 32));
-    k_fsvd_init<<<tg, tb, 0, s>>>((const double*)op->d_A, op->lda, n, F->W, F->V);
+    k_fsvd_init<<<tg, tb, 0, s>>>((const double*)op->d_A, op->lda, n, F->W, n, F->V);
     RBF_LAUNCHED(ctx, "k_fsvd_init");
     double tol = sqrt((double)n) * DBL_EPSILON;
     long long budget = ctx->opt.wait_budget;
@@ -628,23 +969,28 @@ rbf_status fsvd_jacobi(rbf_ctx* ctx, const rbf_operator* op, const double* f, Fs
 // Bidiagonalization path
 rbf_status fsvd_bidiag(rbf_ctx* ctx, const rbf_operator* op, const double* f, Fsvd* F) {
     const int64_t n = op->n;
-    int group, bar_k;
-    const bool big = n > BIDIAG_BIG_N;
-    const void* kbid = big ? (const void*)k_bidiag<1024> : (const void*)k_bidiag<256>;
-    const int nt = big ? 1024 : 256;
-    const int G = coop_grid(ctx, kbid, nt, ctx->sm_count, &group, &bar_k);
     const int J = ctx->opt.grid_j;
     const int L = (int)n;
-    const size_t need = ws_align((size_t)n * (n + 1) * 8) + ws_align((size_t)n * n * 8) +
-                        ws_align((size_t)(n + 1) * n * 8) + 8 * ws_align((size_t)(n + 2) * 8) +
+    const size_t smem = bd_smem(n, ctx->sm_count);
+    if (smem > 48 * 1024)
+        RBF_CUDA(ctx, cudaFuncSetAttribute(k_bidiag, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    F->G = coop_grid(ctx, (const void*)k_bidiag, BD_T, ctx->sm_count, &F->group, &F->bar_k, smem);
+    const int G = F->G;
+    if (G != ctx->sm_count) return rbf_fail(ctx, RBF_ERR_INTERNAL, "bidiagonalization grid of %d CTAs", G);
+    const int64_t qblk = (n - 1 + QB - 1) / QB, qchunk = (n + QG_ROWS - 1) / QG_ROWS;
+    F->ldw = (n + 3) & ~(int64_t)3;
+    const size_t need = ws_align((size_t)F->ldw * (n + 1) * 8) + ws_align((size_t)n * n * 8) +
+                        ws_align((size_t)(n + 1) * n * 8) + 14 * ws_align((size_t)(n + 2) * 8) +
                         ws_align((size_t)(J > n ? J : n) * 8) + ws_align(8) + ws_align(4) +
-                        ws_align((size_t)(bar_k + 2) * BAR_STRIDE * 4) + svd_ws_bytes(L) + 4096;
+                        ws_align((size_t)3 * G * 8) + ws_align((size_t)3 * QB * G * 8) +
+                        ws_align((size_t)(qchunk + 1) * qblk * QB * QB * 8) + ws_align((size_t)2 * QB * G * 8) +
+                        2 * ws_align((size_t)(F->bar_k + 2) * BAR_STRIDE * 4) + svd_ws_bytes(L) + 4096;
     RBF_TRY(rbf_ws_reserve(ctx, need));
     WsCarve wc(ctx->ws);
     F->tgk = true;
     F->n = n;
     F->sweeps = 0;
-    F->Wb = wc.take<double>((size_t)n * (n + 1));
+    F->Wb = wc.take<double>((size_t)F->ldw * (n + 1));
     F->Vt = wc.take<double>((size_t)n * n);
     F->Ut = wc.take<double>((size_t)(n + 1) * n);
     double* dg = wc.take<double>((size_t)n + 2);
@@ -657,34 +1003,37 @@ rbf_status fsvd_bidiag(rbf_ctx* ctx, const rbf_operator* op, const double* f, Fs
     F->sig = wc.take<double>((size_t)n + 2);
     F->fhat = wc.take<double>((size_t)n + 2);
     F->d = wc.take<double>((size_t)n + 2);
+    double* vec[4];
+    for (double*& v : vec) v = wc.take<double>((size_t)n + 2);
     F->curve = wc.take<double>((size_t)(J > n ? J : n));
     F->sperp = wc.take<double>(1);
     F->r = wc.take<int>(1);
-    unsigned* bar = wc.take<unsigned>((size_t)(bar_k + 2) * BAR_STRIDE);
+    double* part = wc.take<double>((size_t)3 * G);
+    F->hpart = wc.take<double>((size_t)QB * G);
+    F->gpart = wc.take<double>((size_t)2 * QB * G);
+    F->gram_part = wc.take<double>((size_t)qchunk * qblk * QB * QB);
+    F->gram = wc.take<double>((size_t)qblk * QB * QB);
+    unsigned* bar = wc.take<unsigned>((size_t)(F->bar_k + 2) * BAR_STRIDE);
+    F->bar = wc.take<unsigned>((size_t)(F->bar_k + 2) * BAR_STRIDE);
     void* svd = (void*)wc.take<char>(svd_ws_bytes(L));
     cudaStream_t s = ctx->stream;
-    RBF_CUDA(ctx, cudaMemsetAsync(bar, 0, (size_t)(bar_k + 2) * BAR_STRIDE * sizeof(unsigned), s));
+    const size_t bar_bytes = (size_t)(F->bar_k + 2) * BAR_STRIDE * sizeof(unsigned);
+    RBF_CUDA(ctx, cudaMemsetAsync(bar, 0, bar_bytes, s));
+    RBF_CUDA(ctx, cudaMemsetAsync(F->bar, 0, bar_bytes, s));
     RBF_CUDA(ctx, cudaMemsetAsync(&ctx->d_state->info[IN_ERR], 0, 2 * sizeof(int), s));
     RBF_CUDA(ctx, cudaMemsetAsync(F->taur, 0, sizeof(double) * (n + 2), s));
-    // W = [A f] column-major (V is only a scratch target of the init kernel here)
+    // W = [A f] column-major
     dim3 tb(32, 8), tg((unsigned)((n + 31) / 32), (unsigned)((n + 31) / 32));
-    k_fsvd_init<<<tg, tb, 0, s>>>((const double*)op->d_A, op->lda, n, F->Wb, F->Vt);
+    k_fsvd_init<<<tg, tb, 0, s>>>((const double*)op->d_A, op->lda, n, F->Wb, F->ldw, nullptr);
     RBF_LAUNCHED(ctx, "k_fsvd_init");
-    if (f) RBF_CUDA(ctx, cudaMemcpyAsync(F->Wb + n * n, f, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
-    else RBF_CUDA(ctx, cudaMemsetAsync(F->Wb + n * n, 0, sizeof(double) * n, s));
+    double* g = F->Wb + n * F->ldw;  // f, then Q_L^T f
+    if (f) RBF_CUDA(ctx, cudaMemcpyAsync(g, f, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
+    else RBF_CUDA(ctx, cudaMemsetAsync(g, 0, sizeof(double) * n, s));
     {
-        double* Wp = F->Wb;
-        int64_t nn = n;
-        double* dp = dg;
-        double* ep = eg;
-        double* tp = F->taur;
-        double* sp = F->scaler;
-        rbf_dev_state* stt = ctx->d_state;
-        unsigned* bp = bar;
-        int grp = group;
-        long long budget = ctx->opt.wait_budget;
-        void* args[] = {&Wp, &nn, &dp, &ep, &tp, &sp, &stt, &bp, &grp, &budget};
-        RBF_CUDA(ctx, cudaLaunchCooperativeKernel(kbid, dim3(G), dim3(nt), args, 0, s));
+        BidiagArgs a{F->Wb, n,      F->ldw, dg,     eg,   F->taur,      F->scaler, vec[0], vec[1],
+                     vec[2], vec[3], part,   ctx->d_state, bar, F->group, ctx->opt.wait_budget};
+        void* args[] = {&a};
+        RBF_CUDA(ctx, cudaLaunchCooperativeKernel((const void*)k_bidiag, dim3(G), dim3(BD_T), args, smem, s));
         ctx->launches++;
     }
     int err = 0;
@@ -697,10 +1046,27 @@ rbf_status fsvd_bidiag(rbf_ctx* ctx, const rbf_operator* op, const double* f, Fs
     RBF_TRY(launch_projected_svd_batch(ctx, dd, alpha, beta, F->sig, ftil, F->Vt, n, svd, nullptr, nullptr, F->Ut,
                                        n + 1));
     if (f) {
-        k_vt_g<<<(unsigned)n, BT, 0, s>>>(F->Vt, n, F->Wb + n * n, F->fhat);
+        k_vt_g<<<(unsigned)n, BT, 0, s>>>(F->Vt, n, g, F->fhat);
         RBF_LAUNCHED(ctx, "k_vt_g");
     }
     return fsvd_common_tail(ctx, F, f);
+}
+
+// z <- Q_R z for one vector
+rbf_status fsvd_apply_qr(rbf_ctx* ctx, const Fsvd* F, double* z) {
+    const int64_t n = F->n;
+    cudaStream_t s = ctx->stream;
+    const int64_t qblk = (n - 1 + QB - 1) / QB, qchunk = (n + QG_ROWS - 1) / QG_ROWS;
+    k_qr_gram<<<dim3((unsigned)qblk, (unsigned)qchunk), QA_T, 0, s>>>(F->Wb, n, F->ldw, F->scaler, F->gram_part);
+    RBF_LAUNCHED(ctx, "k_qr_gram");
+    RBF_TRY(launch_reduce_partials(ctx, qblk * QB * QB, (int)qchunk, F->gram_part, F->gram));
+    const size_t smem = sizeof(double) * (size_t)((n + F->G - 1) / F->G + 1) * (QB + 2);
+    QrArgs a{F->Wb, n, F->ldw, F->taur, F->scaler, F->gram, z, F->hpart, F->gpart, ctx->d_state, F->bar, F->group,
+             ctx->opt.wait_budget};
+    void* args[] = {&a};
+    RBF_CUDA(ctx, cudaLaunchCooperativeKernel((const void*)k_qr_apply, dim3(F->G), dim3(QA_T), args, smem, s));
+    ctx->launches++;
+    return RBF_OK;
 }
 
 rbf_status fsvd_run(rbf_ctx* ctx, const rbf_operator* op, const double* f, Fsvd* F) {
@@ -721,11 +1087,9 @@ rbf_status fsvd_lift(rbf_ctx* ctx, const Fsvd* F, double* coef) {
         RBF_LAUNCHED(ctx, "k_fsvd_lift");
         return RBF_OK;
     }
-    k_u_d<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(F->Ut, n, F->d, coef);
+    k_u_d<<<(unsigned)((n + 31) / 32), 1024, 0, s>>>(F->Ut, n, F->d, coef);
     RBF_LAUNCHED(ctx, "k_u_d");
-    k_apply_qr<<<1, BT, 0, s>>>(F->Wb, n, F->taur, F->scaler, coef, n);
-    RBF_LAUNCHED(ctx, "k_apply_qr");
-    return RBF_OK;
+    return fsvd_apply_qr(ctx, F, coef);
 }
 
 rbf_status read_state(rbf_ctx* ctx) {
@@ -733,6 +1097,8 @@ rbf_status read_state(rbf_ctx* ctx) {
                                   ctx->stream));
     RBF_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     RBF_CUDA(ctx, cudaGetLastError());
+    if (ctx->h_state->info[IN_ERR] != 0)
+        return rbf_fail(ctx, (rbf_status)ctx->h_state->info[IN_ERR], "a bounded grid barrier of the full SVD gave up");
     return RBF_OK;
 }
 
@@ -753,7 +1119,7 @@ extern "C" rbf_status rbf_svd_full(rbf_ctx* ctx, const rbf_operator* op, const d
         if (F.tgk) {
             k_copy_ut<<<dim3((unsigned)((n + 255) / 256), (unsigned)n), 256, 0, s>>>(F.Ut, n, d_V);
             RBF_LAUNCHED(ctx, "k_copy_ut");
-            k_apply_qr<<<(unsigned)n, BT, 0, s>>>(F.Wb, n, F.taur, F.scaler, d_V, n);
+            k_apply_qr<<<(unsigned)n, BT, 0, s>>>(F.Wb, n, F.ldw, F.taur, F.scaler, d_V, n);
             RBF_LAUNCHED(ctx, "k_apply_qr");
         } else {
             k_gather_cols<<<dim3((unsigned)((n + 255) / 256), (unsigned)n), 256, 0, s>>>(F.V, n, F.perm, d_V);
@@ -780,7 +1146,7 @@ extern "C" rbf_status rbf_tikhonov(rbf_ctx* ctx, const rbf_operator* op, const d
     cudaStream_t s = ctx->stream;
     const double tlo = ctx->opt.grid_t_lo, thi = ctx->opt.grid_t_hi;
     if (rule == RBF_GCV) {
-        k_fsvd_gcv<<<(J + 127) / 128, 128, 0, s>>>(F.sig, F.fhat, n, F.r, F.sperp, J, tlo, thi, F.curve);
+        k_fsvd_gcv<<<J, GCV_T, 0, s>>>(F.sig, F.fhat, n, F.r, F.sperp, J, tlo, thi, F.curve);
         RBF_LAUNCHED(ctx, "k_fsvd_gcv");
     }
     k_fsvd_choose<<<1, 1024, 0, s>>>(F.curve, J, 0, rule == RBF_FIXED, lambda_in, 0, F.sig, F.fhat, F.r, J, tlo, thi,
@@ -813,7 +1179,7 @@ extern "C" rbf_status rbf_tsvd(rbf_ctx* ctx, const rbf_operator* op, const doubl
     const int64_t n = op->n;
     cudaStream_t s = ctx->stream;
     if (rank == 0) {
-        k_fsvd_gcv_rank<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(F.fhat, n, F.r, F.sperp, F.curve);
+        k_fsvd_gcv_rank<<<1, FT, 0, s>>>(F.fhat, n, F.r, F.sperp, F.curve);
         RBF_LAUNCHED(ctx, "k_fsvd_gcv_rank");
     }
     int r = 0;
