@@ -2,11 +2,10 @@
 // forward, backward and Adam kernels; the features it reads from the first GKB
 // steps; a multi-vector reconstruction used to build its training labels.
 //
-// Forward: one CTA of 128 threads per tile of 16 samples, thread j owns hidden
-// unit j; weights are read coalesced (row-major, unit index fastest) and reused
-// across the 16 samples held in shared memory.  Backward: activation gradients
-// per tile, then one thread per parameter sums its gradient over the whole
-// batch in a fixed order (FP64 accumulation, deterministic).
+// A training step is three launches: forward and activation gradients of a few
+// samples per CTA with W2 in shared memory (k_mlp_pass), partial weight
+// gradients over chunks of the batch (k_mlp_wgrad), and the sum of the partials
+// with the Adam update (k_mlp_finish).  All sums are in a fixed order.
 #include <cfloat>
 
 #include "common.cuh"
@@ -15,7 +14,6 @@
 namespace {
 
 constexpr int NI = RBF_MLP_IN, NH = RBF_MLP_HIDDEN, NO = RBF_MLP_OUT;
-constexpr int TS = 16;  // samples per CTA
 constexpr int OFF_W1 = 0, OFF_B1 = OFF_W1 + NI * NH, OFF_W2 = OFF_B1 + NH, OFF_B2 = OFF_W2 + NH * NH,
               OFF_W3 = OFF_B2 + NH, OFF_B3 = OFF_W3 + NH * NO, NPAR = OFF_B3 + NO;
 static_assert(NPAR == RBF_MLP_PARAMS, "parameter layout");
@@ -25,170 +23,311 @@ __device__ __forceinline__ float gelu_grad_f(float z) {
     return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * expf(-0.5f * z * z) * 0.39894228040143268f;
 }
 
-// cache (optional): Z1, H1, Z2, H2 [B][NH]
-__global__ void __launch_bounds__(NH) k_mlp_fwd(const float* __restrict__ P, const float* __restrict__ X, int B,
-                                                float* __restrict__ Y, float* __restrict__ Z1, float* __restrict__ H1,
-                                                float* __restrict__ Z2, float* __restrict__ H2) {
-    __shared__ float xs[TS][NI];
-    __shared__ float h1s[TS][NH];
-    __shared__ float h2s[TS][NH];
-    __shared__ float red[NH / 32][TS][NO];
+// Forward pass and, with TRAIN, the activation gradients of TS samples per CTA
+// of 256 threads: thread (half, j) owns hidden unit j for the samples [half TS /
+// 2, (half + 1) TS / 2).  W2 sits in shared memory for both directions (rows of
+// W2_LD floats: conflict-free reads along a row by 16 bytes and down a column);
+// it arrives by cp.async while layer 1 runs.  Latency bounds it (a network of 19
+// 458 weights): few samples per CTA, so that the batch spreads over the SMs, and
+// no second launch and no cached z.  Forward and activation gradients of 512
+// samples: 27 + 36 us (16 samples per CTA, W2 from L2, read across rows in the
+// backward pass) -> 9.4 us.
+// Writes Y [B][2] and, with TRAIN, H1, H2, DZ1, DZ2 [B][NH] and DY = (Y - T) / B;
+// lpart (optional): squared-error partial per CTA.
+constexpr int MP_T = 2 * NH;
+constexpr int W2_LD = NH + 4;
+
+struct PassArgs {
+    const float *P, *X, *T;
+    int B;
+    float *Y, *H1, *H2, *DZ1, *DZ2, *DY;
+    double* lpart;
+};
+
+template <int TS>
+constexpr size_t mlp_smem() {
+    return sizeof(float) * (size_t)(NH * W2_LD + TS * (NI + 2 * NH));
+}
+
+template <int TS, bool TRAIN>
+__global__ void __launch_bounds__(MP_T) k_mlp_pass(PassArgs a) {
+    constexpr int HS = TS / 2;  // samples per thread
+    extern __shared__ float4 smem4[];
+    float* w2 = (float*)smem4;     // [NH][W2_LD]
+    float* xs = w2 + NH * W2_LD;   // [TS][NI]
+    float* h1s = xs + TS * NI;     // [TS][NH]
+    float* dzs = h1s + TS * NH;    // [TS][NH] dz2
+    __shared__ float red[MP_T / 32][HS][NO];
+    __shared__ float dys[TS][NO];
+    const float* __restrict__ P = a.P;
     const int s0 = blockIdx.x * TS;
-    const int j = threadIdx.x;
-    const int ns = min(TS, B - s0);
-    for (int q = j; q < TS * NI; q += NH) {
-        const int s = q / NI, i = q % NI;
-        xs[s][i] = s < ns ? X[(int64_t)(s0 + s) * NI + i] : 0.f;
+    const int ns = min(TS, a.B - s0);
+    const int j = threadIdx.x & (NH - 1), half = threadIdx.x / NH;
+    for (int q = threadIdx.x; q < NH * NH / 4; q += MP_T) {
+        const int i = q / (NH / 4), c = (q % (NH / 4)) * 4;
+        const unsigned d = (unsigned)__cvta_generic_to_shared(w2 + i * W2_LD + c);
+        // the parameter vector need not be 16-byte aligned
+        if (((uintptr_t)P & 15u) == 0)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(P + OFF_W2 + i * NH + c) : "memory");
+        else
+            for (int e = 0; e < 4; ++e) w2[i * W2_LD + c + e] = P[OFF_W2 + i * NH + c + e];
     }
+    for (int q = threadIdx.x; q < TS * NI; q += MP_T) xs[q] = q / NI < ns ? a.X[(int64_t)s0 * NI + q] : 0.f;
     __syncthreads();
-    float acc[TS];
+    float z1[HS], z2[HS], h2[HS];
+    const float* x = xs + half * HS * NI;
 #pragma unroll
-    for (int s = 0; s < TS; ++s) acc[s] = P[OFF_B1 + j];
+    for (int s = 0; s < HS; ++s) z1[s] = P[OFF_B1 + j];
+#pragma unroll
     for (int i = 0; i < NI; ++i) {
         const float wv = P[OFF_W1 + i * NH + j];
 #pragma unroll
-        for (int s = 0; s < TS; ++s) acc[s] = fmaf(xs[s][i], wv, acc[s]);
+        for (int s = 0; s < HS; ++s) z1[s] = fmaf(x[s * NI + i], wv, z1[s]);
     }
+    float* h1 = h1s + half * HS * NH;
 #pragma unroll
-    for (int s = 0; s < TS; ++s) {
-        const float h = gelu_f(acc[s]);
-        h1s[s][j] = h;
-        if (Z1 && s < ns) {
-            Z1[(int64_t)(s0 + s) * NH + j] = acc[s];
-            H1[(int64_t)(s0 + s) * NH + j] = h;
-        }
+    for (int s = 0; s < HS; ++s) {
+        const float h = gelu_f(z1[s]);
+        h1[s * NH + j] = h;
+        if (TRAIN && half * HS + s < ns) a.H1[(int64_t)(s0 + half * HS + s) * NH + j] = h;
     }
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
     __syncthreads();
 #pragma unroll
-    for (int s = 0; s < TS; ++s) acc[s] = P[OFF_B2 + j];
-    for (int i = 0; i < NH; ++i) {
-        const float wv = P[OFF_W2 + i * NH + j];
+    for (int s = 0; s < HS; ++s) z2[s] = P[OFF_B2 + j];
+#pragma unroll 4
+    for (int i = 0; i < NH; i += 4) {
+        float w[4];
 #pragma unroll
-        for (int s = 0; s < TS; ++s) acc[s] = fmaf(h1s[s][i], wv, acc[s]);
-    }
+        for (int e = 0; e < 4; ++e) w[e] = w2[(i + e) * W2_LD + j];
 #pragma unroll
-    for (int s = 0; s < TS; ++s) {
-        const float h = gelu_f(acc[s]);
-        h2s[s][j] = h;
-        if (Z2 && s < ns) {
-            Z2[(int64_t)(s0 + s) * NH + j] = acc[s];
-            H2[(int64_t)(s0 + s) * NH + j] = h;
+        for (int s = 0; s < HS; ++s) {
+            const float4 h = *reinterpret_cast<const float4*>(h1 + s * NH + i);
+            z2[s] = fmaf(h.w, w[3], fmaf(h.z, w[2], fmaf(h.y, w[1], fmaf(h.x, w[0], z2[s]))));
         }
     }
-    __syncthreads();
-    // output layer: partial products per unit j, reduced across the block
-    const float w30 = P[OFF_W3 + j * NO + 0], w31 = P[OFF_W3 + j * NO + 1];
-    const int warp = j >> 5, lane = j & 31;
+    // output layer: partial products per unit, reduced over the warps of the half
+    const float w30 = P[OFF_W3 + j * NO], w31 = P[OFF_W3 + j * NO + 1];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
-    for (int s = 0; s < TS; ++s) {
-        float p0 = h2s[s][j] * w30, p1 = h2s[s][j] * w31;
-        p0 = warp_sumf(p0);
-        p1 = warp_sumf(p1);
+    for (int s = 0; s < HS; ++s) {
+        h2[s] = gelu_f(z2[s]);
+        if (TRAIN && half * HS + s < ns) a.H2[(int64_t)(s0 + half * HS + s) * NH + j] = h2[s];
+        const float p0 = warp_sumf(h2[s] * w30), p1 = warp_sumf(h2[s] * w31);
         if (lane == 0) {
             red[warp][s][0] = p0;
             red[warp][s][1] = p1;
         }
     }
     __syncthreads();
-    if (j < TS * NO) {
-        const int s = j / NO, o = j % NO;
-        float y = P[OFF_B3 + o];
-        for (int w = 0; w < NH / 32; ++w) y += red[w][s][o];
-        if (s < ns) Y[(int64_t)(s0 + s) * NO + o] = y;
-    }
-}
-
-// dY = (Y - T) / B, dZ2, dZ1 per sample; squared-error partial per tile.
-__global__ void __launch_bounds__(NH) k_mlp_bwd_act(const float* __restrict__ P, const float* __restrict__ Y,
-                                                    const float* __restrict__ T, int B, const float* __restrict__ Z1,
-                                                    const float* __restrict__ Z2, float* __restrict__ DY,
-                                                    float* __restrict__ DZ1, float* __restrict__ DZ2,
-                                                    double* __restrict__ lpart) {
-    __shared__ float dys[TS][NO];
-    __shared__ float dz2s[TS][NH];
-    const int s0 = blockIdx.x * TS;
-    const int i = threadIdx.x;
-    const int ns = min(TS, B - s0);
-    if (i < TS * NO) {
-        const int s = i / NO, o = i % NO;
-        float d = 0.f;
+    if (threadIdx.x < TS * NO) {
+        const int s = threadIdx.x / NO, o = threadIdx.x % NO, hf = s / HS;
+        float y = P[OFF_B3 + o], d = 0.f;
+        double dl = 0.0;
+        for (int w = 0; w < NH / 32; ++w) y += red[hf * (NH / 32) + w][s % HS][o];
         if (s < ns) {
-            d = (Y[(int64_t)(s0 + s) * NO + o] - T[(int64_t)(s0 + s) * NO + o]);
-            DY[(int64_t)(s0 + s) * NO + o] = d / (float)B;
-        }
-        dys[s][o] = d / (float)B;
-    }
-    if (i == 0) {
-        double l = 0.0;
-        for (int s = 0; s < ns; ++s)
-            for (int o = 0; o < NO; ++o) {
-                const double d = (double)Y[(int64_t)(s0 + s) * NO + o] - (double)T[(int64_t)(s0 + s) * NO + o];
-                l += d * d;
+            const int64_t at = (int64_t)(s0 + s) * NO + o;
+            a.Y[at] = y;
+            if (TRAIN) {
+                d = y - a.T[at];
+                dl = (double)y - (double)a.T[at];
+                a.DY[at] = d / (float)a.B;
             }
-        lpart[blockIdx.x] = l;
+        }
+        if (TRAIN) dys[s][o] = d / (float)a.B;
+        if (TRAIN && a.lpart) {  // TS * NO <= 32: one warp
+            double l = dl * dl;
+            for (int q = TS * NO / 2; q > 0; q >>= 1) l += __shfl_xor_sync((1u << (TS * NO)) - 1u, l, q);
+            if (threadIdx.x == 0) a.lpart[blockIdx.x] = l;
+        }
+    }
+    if (!TRAIN) return;
+    __syncthreads();
+    float* dz2 = dzs + half * HS * NH;
+#pragma unroll
+    for (int s = 0; s < HS; ++s) {
+        const int q = half * HS + s;
+        const float dz = (dys[q][0] * w30 + dys[q][1] * w31) * gelu_grad_f(z2[s]);
+        dz2[s * NH + j] = dz;
+        if (q < ns) a.DZ2[(int64_t)(s0 + q) * NH + j] = dz;
     }
     __syncthreads();
-    const float w30 = P[OFF_W3 + i * NO + 0], w31 = P[OFF_W3 + i * NO + 1];
-    for (int s = 0; s < TS; ++s) {
-        float dz = 0.f;
-        if (s < ns) dz = (dys[s][0] * w30 + dys[s][1] * w31) * gelu_grad_f(Z2[(int64_t)(s0 + s) * NH + i]);
-        dz2s[s][i] = dz;
-        if (s < ns) DZ2[(int64_t)(s0 + s) * NH + i] = dz;
-    }
-    __syncthreads();
-    // dh1[s][i] = sum_j dz2[s][j] W2[i][j]
-    float acc[TS];
+    // dh1_j = sum over units u of dz2_u W2[j][u]
+    float acc[HS];
 #pragma unroll
-    for (int s = 0; s < TS; ++s) acc[s] = 0.f;
-    for (int jj = 0; jj < NH; ++jj) {
-        const float wv = P[OFF_W2 + i * NH + jj];
+    for (int s = 0; s < HS; ++s) acc[s] = 0.f;
+    const float* wr = w2 + j * W2_LD;
+#pragma unroll 4
+    for (int u = 0; u < NH; u += 4) {
+        const float4 w = *reinterpret_cast<const float4*>(wr + u);
 #pragma unroll
-        for (int s = 0; s < TS; ++s) acc[s] = fmaf(dz2s[s][jj], wv, acc[s]);
+        for (int s = 0; s < HS; ++s) {
+            const float4 d = *reinterpret_cast<const float4*>(dz2 + s * NH + u);
+            acc[s] = fmaf(d.w, w.w, fmaf(d.z, w.z, fmaf(d.y, w.y, fmaf(d.x, w.x, acc[s]))));
+        }
     }
 #pragma unroll
-    for (int s = 0; s < TS; ++s)
-        if (s < ns) DZ1[(int64_t)(s0 + s) * NH + i] = acc[s] * gelu_grad_f(Z1[(int64_t)(s0 + s) * NH + i]);
+    for (int s = 0; s < HS; ++s)
+        if (half * HS + s < ns) a.DZ1[(int64_t)(s0 + half * HS + s) * NH + j] = acc[s] * gelu_grad_f(z1[s]);
 }
 
-// One thread per parameter: gradient summed over the batch in sample order.
-__global__ void k_mlp_wgrad(const float* __restrict__ X, const float* __restrict__ H1, const float* __restrict__ H2,
-                            const float* __restrict__ DY, const float* __restrict__ DZ1, const float* __restrict__ DZ2,
-                            int B, float* __restrict__ G) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= NPAR) return;
+// Sum of FP32 products as an unevaluated pair s + c (Ogita, Rump and Oishi's
+// Dot2: the product's and the sum's rounding errors, both exact in FP32, are
+// carried in c): the result of a sum in twice FP32's precision.
+struct Pair {
+    float s = 0.f, c = 0.f;
+    __device__ __forceinline__ void two_sum(float p, float e) {
+        const float t = __fadd_rn(s, p), b = __fsub_rn(t, s);
+        const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(p, b));
+        s = t;
+        c = __fadd_rn(c, __fadd_rn(err, e));
+    }
+    __device__ __forceinline__ void dot(float a, float b) {
+        const float p = __fmul_rn(a, b);
+        two_sum(p, __fmaf_rn(a, b, -p));
+    }
+};
+
+// Weight-gradient partials over the samples [chunk c, chunk (c + 1)) of chunk c =
+// blockIdx.x: out[r][j] = sum_s L[s][r] R[s][j], 4 x 4 outputs per thread, 32 rows
+// x 128 columns per CTA.  blockIdx.y: 0..3 W2 (L = H1, R = DZ2); 4 W1 and b1 (L =
+// X and 1, R = DZ1); 5 b2 (L = 1, R = DZ2); 6 W3 transposed (L = DY, R = H2) and b3.
+// An FP64 sum of the products (exact in FP64) runs at 1/64 of the FP32 rate: 10
+// M FP64 FMAs of a 512-sample step are 16 us at best; ten FP32 operations per
+// product in Dot2 give the same FP32 gradients (its error, 2^-47 of the sum of
+// magnitudes, is far below their rounding).  One thread per weight with an FP64
+// chain over the batch: 127 us -> 13.0, and 6.4 for the sum of the partials with the update.
+constexpr int WG_T = 256;
+constexpr int WG_S = 16;  // samples staged at a time
+
+struct GradArgs {
+    const float *X, *H1, *H2, *DY, *DZ1, *DZ2;
+    int B, chunk, chunks;
+    float2* part;  // [chunks][NPAR]
+};
+
+__global__ void __launch_bounds__(WG_T) k_mlp_wgrad(GradArgs a) {
+    __shared__ float Ls[WG_S][32];
+    __shared__ float Rs[WG_S][NH];
+    const int task = blockIdx.y;
+    const int sb = blockIdx.x * a.chunk, se = min(a.B, sb + a.chunk);
+    const int rows = task < 4 ? 32 : (task == 4 ? NI + 1 : (task == 5 ? 1 : NO));
+    const float* __restrict__ Rg = task == 4 ? a.DZ1 : (task == 6 ? a.H2 : a.DZ2);
+    const int r0 = (threadIdx.x >> 5) * 4, c0 = (threadIdx.x & 31) * 4;
+    Pair acc[4][4], b3;
+    for (int s0 = sb; s0 < se; s0 += WG_S) {
+        const int cnt = min(WG_S, se - s0);
+        __syncthreads();
+        for (int q = threadIdx.x; q < WG_S * NH; q += WG_T)
+            Rs[q / NH][q % NH] = q / NH < cnt ? Rg[(int64_t)s0 * NH + q] : 0.f;
+        for (int q = threadIdx.x; q < WG_S * 32; q += WG_T) {
+            const int s = q / 32, r = q % 32;
+            float v = 0.f;
+            if (s < cnt && r < rows) {
+                const int64_t at = s0 + s;
+                if (task < 4) v = a.H1[at * NH + task * 32 + r];
+                else if (task == 4) v = r < NI ? a.X[at * NI + r] : 1.f;
+                else v = task == 5 ? 1.f : a.DY[at * NO + r];
+            }
+            Ls[s][r] = v;
+        }
+        __syncthreads();
+        if (r0 < rows) {
+#pragma unroll 2
+            for (int s = 0; s < cnt; ++s) {
+                const float4 l = *reinterpret_cast<const float4*>(&Ls[s][r0]);
+                const float4 r = *reinterpret_cast<const float4*>(&Rs[s][c0]);
+                const float lv[4] = {l.x, l.y, l.z, l.w}, rv[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) acc[u][v].dot(lv[u], rv[v]);
+            }
+        }
+        if (task == 6 && threadIdx.x >= 32 && threadIdx.x < 32 + NO)
+            for (int s = 0; s < cnt; ++s) b3.two_sum(Ls[s][threadIdx.x - 32], 0.f);
+    }
+    float2* out = a.part + (int64_t)blockIdx.x * NPAR;
+    if (task == 6 && threadIdx.x >= 32 && threadIdx.x < 32 + NO) out[OFF_B3 + threadIdx.x - 32] = make_float2(b3.s, b3.c);
+    if (r0 >= rows) return;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int r = r0 + u;
+        if (r >= rows) break;
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const int c = c0 + v;
+            int at;
+            if (task < 4) at = OFF_W2 + (task * 32 + r) * NH + c;
+            else if (task == 4) at = r < NI ? OFF_W1 + r * NH + c : OFF_B1 + c;
+            else at = task == 5 ? OFF_B2 + c : OFF_W3 + c * NO + r;
+            out[at] = make_float2(acc[u][v].s, acc[u][v].c);
+        }
+    }
+}
+
+// Gradient of one parameter in FP64 over the whole batch: where the paired sum
+// left FP32's range (an infinite or NaN product or sum).
+__device__ float grad_f64(const GradArgs& a, int p) {
     double acc = 0.0;
-    if (p < OFF_B1) {
-        const int i = p / NH, j = p % NH;
-        for (int s = 0; s < B; ++s) acc += (double)X[(int64_t)s * NI + i] * (double)DZ1[(int64_t)s * NH + j];
-    } else if (p < OFF_W2) {
-        const int j = p - OFF_B1;
-        for (int s = 0; s < B; ++s) acc += (double)DZ1[(int64_t)s * NH + j];
-    } else if (p < OFF_B2) {
-        const int q = p - OFF_W2, i = q / NH, j = q % NH;
-        for (int s = 0; s < B; ++s) acc += (double)H1[(int64_t)s * NH + i] * (double)DZ2[(int64_t)s * NH + j];
-    } else if (p < OFF_W3) {
-        const int j = p - OFF_B2;
-        for (int s = 0; s < B; ++s) acc += (double)DZ2[(int64_t)s * NH + j];
-    } else if (p < OFF_B3) {
-        const int q = p - OFF_W3, i = q / NO, o = q % NO;
-        for (int s = 0; s < B; ++s) acc += (double)H2[(int64_t)s * NH + i] * (double)DY[(int64_t)s * NO + o];
-    } else {
-        const int o = p - OFF_B3;
-        for (int s = 0; s < B; ++s) acc += (double)DY[(int64_t)s * NO + o];
+    for (int64_t s = 0; s < a.B; ++s) {
+        double l = 1.0, r;
+        if (p < OFF_B1) {
+            l = a.X[s * NI + p / NH];
+            r = a.DZ1[s * NH + p % NH];
+        } else if (p < OFF_W2) {
+            r = a.DZ1[s * NH + p - OFF_B1];
+        } else if (p < OFF_B2) {
+            l = a.H1[s * NH + (p - OFF_W2) / NH];
+            r = a.DZ2[s * NH + (p - OFF_W2) % NH];
+        } else if (p < OFF_W3) {
+            r = a.DZ2[s * NH + p - OFF_B2];
+        } else if (p < OFF_B3) {
+            l = a.H2[s * NH + (p - OFF_W3) / NO];
+            r = a.DY[s * NO + (p - OFF_W3) % NO];
+        } else {
+            r = a.DY[s * NO + p - OFF_B3];
+        }
+        acc += l * r;
     }
-    G[p] = (float)acc;
+    return (float)acc;
 }
 
-__global__ void k_adam(float* __restrict__ P, float* __restrict__ M, float* __restrict__ V,
-                       const float* __restrict__ G, float lr, float b1, float b2, float c1, float c2, float eps) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+struct AdamArgs {
+    float *P, *M, *V;
+    float lr, b1, b2, c1, c2, eps;
+};
+
+__device__ __forceinline__ void adam_one(const AdamArgs& o, int p, float g) {
+    const float m = o.b1 * o.M[p] + (1.f - o.b1) * g;
+    const float v = o.b2 * o.V[p] + (1.f - o.b2) * g * g;
+    o.M[p] = m;
+    o.V[p] = v;
+    o.P[p] -= o.lr * (m * o.c1) / (sqrtf(v * o.c2) + o.eps);
+}
+
+// G = sum of the chunks' partials in chunk order; with ADAM the update of the
+// parameters by it.
+template <bool ADAM>
+__global__ void __launch_bounds__(128) k_mlp_finish(GradArgs a, float* __restrict__ G, AdamArgs o) {
+    const int p = blockIdx.x * 128 + threadIdx.x;
     if (p >= NPAR) return;
-    const float g = G[p];
-    const float m = b1 * M[p] + (1.f - b1) * g;
-    const float v = b2 * V[p] + (1.f - b2) * g * g;
-    M[p] = m;
-    V[p] = v;
-    P[p] -= lr * (m * c1) / (sqrtf(v * c2) + eps);
+    Pair t;
+    const float2* __restrict__ q = a.part + p;
+#pragma unroll 8
+    for (int c = 0; c < a.chunks; ++c) {
+        const float2 v = q[(int64_t)c * NPAR];
+        t.two_sum(v.x, v.y);
+    }
+    float g = t.s + t.c;
+    if (!isfinite(g)) g = grad_f64(a, p);
+    G[p] = g;
+    if (ADAM) adam_one(o, p, g);
+}
+
+__global__ void __launch_bounds__(128) k_adam(const float* __restrict__ G, AdamArgs o) {
+    const int p = blockIdx.x * 128 + threadIdx.x;
+    if (p < NPAR) adam_one(o, p, G[p]);
 }
 
 __global__ void k_sum_parts(const double* __restrict__ parts, int n, double scale, double* __restrict__ out) {
@@ -313,48 +452,70 @@ __global__ void k_reduce_many(const double* __restrict__ part, int chunks, int64
 }  // namespace
 
 // ---------------------------------------------------------------------------
-static rbf_status mlp_forward_impl(rbf_ctx* ctx, const float* P, const float* X, int B, float* Y, float* cache) {
-    float *Z1 = nullptr, *H1 = nullptr, *Z2 = nullptr, *H2 = nullptr;
-    if (cache) {
-        Z1 = cache;
-        H1 = Z1 + (size_t)B * NH;
-        Z2 = H1 + (size_t)B * NH;
-        H2 = Z2 + (size_t)B * NH;
-    }
-    k_mlp_fwd<<<(B + TS - 1) / TS, NH, 0, ctx->stream>>>(P, X, B, Y, Z1, H1, Z2, H2);
-    RBF_LAUNCHED(ctx, "k_mlp_fwd");
+// Samples per CTA: 4 while that gives at most four waves of CTAs (three fit on an
+// SM), else 8 (each CTA reads W2 once).
+template <bool TRAIN>
+static rbf_status launch_mlp_pass(rbf_ctx* ctx, const PassArgs& a, int* tiles) {
+    const bool small = (int64_t)a.B <= (int64_t)ctx->sm_count * 48;
+    const int ts = small ? 4 : 8;
+    *tiles = (a.B + ts - 1) / ts;
+    const void* k = small ? (const void*)k_mlp_pass<4, TRAIN> : (const void*)k_mlp_pass<8, TRAIN>;
+    const size_t smem = small ? mlp_smem<4>() : mlp_smem<8>();
+    RBF_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (small) k_mlp_pass<4, TRAIN><<<*tiles, MP_T, smem, ctx->stream>>>(a);
+    else k_mlp_pass<8, TRAIN><<<*tiles, MP_T, smem, ctx->stream>>>(a);
+    RBF_LAUNCHED(ctx, "k_mlp_pass");
     return RBF_OK;
 }
 
 extern "C" rbf_status rbf_mlp_forward(rbf_ctx* ctx, const float* d_params, const float* d_x, int batch, float* d_y) {
     if (!ctx) return RBF_ERR_INVALID;
     if (!d_params || !d_x || !d_y || batch < 1) return rbf_fail(ctx, RBF_ERR_INVALID, "rbf_mlp_forward: bad argument");
-    return mlp_forward_impl(ctx, d_params, d_x, batch, d_y, nullptr);
+    PassArgs a{};
+    a.P = d_params;
+    a.X = d_x;
+    a.B = batch;
+    a.Y = d_y;
+    int tiles = 0;
+    return launch_mlp_pass<false>(ctx, a, &tiles);
 }
 
+// Gradient into G and, with `adam`, the update in the same last launch.
 static rbf_status mlp_grad_impl(rbf_ctx* ctx, const float* P, const float* X, const float* T, int B, float* G,
-                                float* h_loss) {
-    const int tiles = (B + TS - 1) / TS;
-    const size_t need = ws_align((size_t)4 * B * NH * 4) + ws_align((size_t)B * NO * 4) * 2 +
-                        ws_align((size_t)2 * B * NH * 4) + ws_align((size_t)(tiles + 1) * 8);
+                                float* h_loss, const AdamArgs* adam) {
+    // chunks of the batch: 16 samples each (32 x 7 CTAs at 512 samples), longer
+    // ones past 64 chunks, where the partials (156 KB per chunk) would cost more
+    // than the shorter sums save
+    int chunk = WG_S;
+    while ((B + chunk - 1) / chunk > 64) chunk += WG_S;
+    const int chunks = (B + chunk - 1) / chunk;
+    const int tiles_max = (B + 3) / 4;
+    const size_t need = 4 * ws_align((size_t)B * NH * 4) + 2 * ws_align((size_t)B * NO * 4) +
+                        ws_align((size_t)chunks * NPAR * sizeof(float2)) + ws_align((size_t)(tiles_max + 1) * 8);
     RBF_TRY(rbf_ws_reserve(ctx, need));
     WsCarve wc(ctx->ws);
-    float* cache = wc.take<float>((size_t)4 * B * NH);
-    float* Y = wc.take<float>((size_t)B * NO);
-    float* DY = wc.take<float>((size_t)B * NO);
-    float* DZ = wc.take<float>((size_t)2 * B * NH);
-    double* lpart = wc.take<double>((size_t)tiles + 1);
-    RBF_TRY(mlp_forward_impl(ctx, P, X, B, Y, cache));
-    const float* Z1 = cache;
-    const float* H1 = Z1 + (size_t)B * NH;
-    const float* Z2 = H1 + (size_t)B * NH;
-    const float* H2 = Z2 + (size_t)B * NH;
-    float* DZ1 = DZ;
-    float* DZ2 = DZ + (size_t)B * NH;
-    k_mlp_bwd_act<<<tiles, NH, 0, ctx->stream>>>(P, Y, T, B, Z1, Z2, DY, DZ1, DZ2, lpart);
-    RBF_LAUNCHED(ctx, "k_mlp_bwd_act");
-    k_mlp_wgrad<<<(NPAR + 255) / 256, 256, 0, ctx->stream>>>(X, H1, H2, DY, DZ1, DZ2, B, G);
+    PassArgs a{};
+    a.P = P;
+    a.X = X;
+    a.T = T;
+    a.B = B;
+    a.H1 = wc.take<float>((size_t)B * NH);
+    a.H2 = wc.take<float>((size_t)B * NH);
+    a.DZ1 = wc.take<float>((size_t)B * NH);
+    a.DZ2 = wc.take<float>((size_t)B * NH);
+    a.Y = wc.take<float>((size_t)B * NO);
+    a.DY = wc.take<float>((size_t)B * NO);
+    float2* part = wc.take<float2>((size_t)chunks * NPAR);
+    double* lpart = wc.take<double>((size_t)tiles_max + 1);
+    a.lpart = h_loss ? lpart : nullptr;
+    int tiles = 0;
+    RBF_TRY(launch_mlp_pass<true>(ctx, a, &tiles));
+    const GradArgs ga{X, a.H1, a.H2, a.DY, a.DZ1, a.DZ2, B, chunk, chunks, part};
+    k_mlp_wgrad<<<dim3(chunks, 7), WG_T, 0, ctx->stream>>>(ga);
     RBF_LAUNCHED(ctx, "k_mlp_wgrad");
+    if (adam) k_mlp_finish<true><<<(NPAR + 127) / 128, 128, 0, ctx->stream>>>(ga, G, *adam);
+    else k_mlp_finish<false><<<(NPAR + 127) / 128, 128, 0, ctx->stream>>>(ga, G, AdamArgs{});
+    RBF_LAUNCHED(ctx, "k_mlp_finish");
     if (h_loss) {
         k_sum_parts<<<1, 32, 0, ctx->stream>>>(lpart, tiles, 1.0 / (2.0 * B), lpart + tiles);
         RBF_LAUNCHED(ctx, "k_sum_parts");
@@ -366,21 +527,24 @@ static rbf_status mlp_grad_impl(rbf_ctx* ctx, const float* P, const float* X, co
     return RBF_OK;
 }
 
+static AdamArgs adam_args(float* P, float* M, float* V, int t, float lr) {
+    const double b1 = 0.9, b2 = 0.999;
+    return AdamArgs{P, M, V, lr, (float)b1, (float)b2, (float)(1.0 / (1.0 - pow(b1, t))),
+                    (float)(1.0 / (1.0 - pow(b2, t))), 1e-8f};
+}
+
 extern "C" rbf_status rbf_mlp_grad(rbf_ctx* ctx, const float* d_params, const float* d_x, const float* d_t, int batch,
                                    float* d_grad, float* h_loss) {
     if (!ctx) return RBF_ERR_INVALID;
     if (!d_params || !d_x || !d_t || !d_grad || batch < 1) return rbf_fail(ctx, RBF_ERR_INVALID, "rbf_mlp_grad: bad argument");
-    return mlp_grad_impl(ctx, d_params, d_x, d_t, batch, d_grad, h_loss);
+    return mlp_grad_impl(ctx, d_params, d_x, d_t, batch, d_grad, h_loss, nullptr);
 }
 
 extern "C" rbf_status rbf_mlp_adam(rbf_ctx* ctx, float* d_params, float* d_m, float* d_v, const float* d_grad, int t,
                                    float lr) {
     if (!ctx) return RBF_ERR_INVALID;
     if (!d_params || !d_m || !d_v || !d_grad || t < 1) return rbf_fail(ctx, RBF_ERR_INVALID, "rbf_mlp_adam: bad argument");
-    const double b1 = 0.9, b2 = 0.999;
-    const float c1 = (float)(1.0 / (1.0 - pow(b1, t))), c2 = (float)(1.0 / (1.0 - pow(b2, t)));
-    k_adam<<<(NPAR + 255) / 256, 256, 0, ctx->stream>>>(d_params, d_m, d_v, d_grad, lr, (float)b1, (float)b2, c1, c2,
-                                                        1e-8f);
+    k_adam<<<(NPAR + 127) / 128, 128, 0, ctx->stream>>>(d_grad, adam_args(d_params, d_m, d_v, t, lr));
     RBF_LAUNCHED(ctx, "k_adam");
     return RBF_OK;
 }
@@ -389,8 +553,13 @@ extern "C" rbf_status rbf_mlp_train_step(rbf_ctx* ctx, float* d_params, float* d
                                          const float* d_x, const float* d_t, int batch, float* d_grad, float* h_loss) {
     if (!ctx) return RBF_ERR_INVALID;
     if (!d_grad) return rbf_fail(ctx, RBF_ERR_INVALID, "rbf_mlp_train_step: gradient buffer required");
-    RBF_TRY(mlp_grad_impl(ctx, d_params, d_x, d_t, batch, d_grad, h_loss));
-    return rbf_mlp_adam(ctx, d_params, d_m, d_v, d_grad, t, lr);
+    if (!d_m || !d_v || t < 1) {  // the update is refused after the gradient has been written
+        RBF_TRY(rbf_mlp_grad(ctx, d_params, d_x, d_t, batch, d_grad, h_loss));
+        return rbf_mlp_adam(ctx, d_params, d_m, d_v, d_grad, t, lr);
+    }
+    if (!d_params || !d_x || !d_t || batch < 1) return rbf_fail(ctx, RBF_ERR_INVALID, "rbf_mlp_grad: bad argument");
+    const AdamArgs o = adam_args(d_params, d_m, d_v, t, lr);
+    return mlp_grad_impl(ctx, d_params, d_x, d_t, batch, d_grad, h_loss, &o);
 }
 
 extern "C" rbf_status rbf_stop_features(rbf_ctx* ctx, const rbf_gkb_state* st, int j, const float* d_mean,
