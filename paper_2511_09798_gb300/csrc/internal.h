@@ -91,6 +91,10 @@ rbf_status rbf_many_slots(rbf_ctx* ctx, int count);
 rbf_status rbf_lanes_fork(rbf_ctx* ctx, int lanes);
 rbf_status rbf_lanes_join(rbf_ctx* ctx, int lanes);
 
+// Dynamic shared memory that needs no cudaFuncSetAttribute beside a kernel's few
+// hundred bytes of static shared memory (48 KB together).
+constexpr size_t SMEM_PLAIN = 40 * 1024;
+
 // ---- error helpers ---------------------------------------------------------
 rbf_status rbf_fail(rbf_ctx* ctx, rbf_status st, const char* fmt, ...);
 

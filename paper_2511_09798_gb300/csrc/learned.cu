@@ -139,7 +139,7 @@ extern "C" rbf_status rbf_hkt_error_table(rbf_ctx* ctx, const rbf_gkb_state* st,
     ProjDims d{n_ell, L, 0, d_ells};
     RBF_TRY(launch_projected_svd_batch(ctx, d, a_rep, b_rep, sigma, ftil, V, L, svd, nullptr, nullptr));
     const size_t smem = (size_t)2 * ET_Q * L * 8;
-    if (smem > 48 * 1024)
+    if (smem > SMEM_PLAIN)
         RBF_CUDA(ctx, cudaFuncSetAttribute(k_err_table, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     k_err_table<<<dim3((unsigned)((Jp + ET_Q - 1) / ET_Q), (unsigned)n_ell), ET_T, smem, ctx->stream>>>(
         d_ells, L, sigma, ftil, V, d_G, ldg, m, d_uref, J, ctx->opt.grid_t_lo, ctx->opt.grid_t_hi, t_stride, Jp,

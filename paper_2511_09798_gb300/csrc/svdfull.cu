@@ -972,7 +972,7 @@ rbf_status fsvd_bidiag(rbf_ctx* ctx, const rbf_operator* op, const double* f, Fs
     const int J = ctx->opt.grid_j;
     const int L = (int)n;
     const size_t smem = bd_smem(n, ctx->sm_count);
-    if (smem > 48 * 1024)
+    if (smem > SMEM_PLAIN)
         RBF_CUDA(ctx, cudaFuncSetAttribute(k_bidiag, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     F->G = coop_grid(ctx, (const void*)k_bidiag, BD_T, ctx->sm_count, &F->group, &F->bar_k, smem);
     const int G = F->G;

@@ -78,7 +78,8 @@ def test_projected_svd_edges(ctx, R, kind, l):
     assert abs(np.sum(ft.cpu().numpy() ** 2) - b[0] ** 2) <= 1e-11 * b[0] ** 2
 
 
-@pytest.mark.parametrize("n", [1823, 1825])  # the last size with 32 lanes per value on 152 SMs, the first with 8
+# the last size with 32 lanes per value on 152 SMs, the first with 8; shared tables of just under 48 KB
+@pytest.mark.parametrize("n", [1823, 1825, 2045])
 def test_singular_values_lane_split(ctx, R, n):
     g = torch.Generator(device="cuda").manual_seed(n)
     lda = R.padded_lda(n, R.RBF_FP64)
