@@ -43,6 +43,19 @@ __device__ __forceinline__ bool gkb_done(const int* done) {
     return done != nullptr && *(volatile const int*)done != 0;
 }
 
+// Programmatic dependent launch: returns when the kernel before this one in the
+// stream has completed and its writes are visible, then lets the kernel after
+// this one start its prologue (once every CTA of this one is past this point or
+// has ended).  In that order, so that when a kernel's prologue runs, everything
+// before the kernel it waits for has completed: a prologue may read what any
+// kernel but its predecessor writes.  Every path of a kernel launched with the
+// attribute passes here before it ends, so completion stays transitive along the
+// stream.  Without the attribute it does nothing.
+__device__ __forceinline__ void pdl_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Flat split of a row-major n x n matrix over W warps (the A z products):
 // warp w owns the elements [b_w, b_{w+1}) with b_w = floor(n^2 w / W), its
 // column rounded down to a multiple of FLAT_ALIGN (16-byte aligned vector

@@ -46,8 +46,10 @@ namespace {
 
 constexpr int FX_NONFINITE = 2047;
 constexpr int FXN_THREADS = 512;  // A z: 16 warps, the vector's limbs in shared memory
+constexpr int FXR_THREADS = 512;  // A z by rows: at most 16 warps
 constexpr int FXT_THREADS = 256;  // A^T w: 2 columns per thread, like the FP64 kernel
 constexpr int FXT_UNROLL = 8;     // rows of loads in flight per thread (A^T w)
+constexpr int FXT_LEAD = 4;       // rows loaded before the vector is converted (8 spill at 4 CTAs per SM)
 constexpr int FXE_THREADS = 256;  // exponent scan and conversion: 2 columns per thread
 
 __device__ __forceinline__ int fx_exp(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7FF); }
@@ -122,9 +124,9 @@ __device__ __forceinline__ double fx_scale_out(double v, int e_mat, int e_vec) {
 
 // Largest exponent field of x[i0 .. i1) over the CTA (every thread gets it).
 template <int NT>
-__device__ __forceinline__ int fx_block_max_exp(const double* __restrict__ x, int64_t i0, int64_t i1, int* red) {
+__device__ __forceinline__ int fx_block_max_exp(const double* x, int64_t i0, int64_t i1, int* red) {
     int em = 0;
-    for (int64_t i = i0 + threadIdx.x; i < i1; i += NT) em = max(em, fx_exp(__ldg(x + i)));
+    for (int64_t i = i0 + threadIdx.x; i < i1; i += NT) em = max(em, fx_exp(__ldcg(x + i)));
     em = __reduce_max_sync(RBF_FULL_MASK, em);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = em;
     __syncthreads();
@@ -272,6 +274,61 @@ __global__ void __launch_bounds__(FXN_THREADS) k_gemv_flat_fx(const long long* _
     }
 }
 
+// The same product for small n, one row per warp: no partial rows (part[0 .. n)
+// is A z) and no 64-bit divisions for the split; the CTA's warps share the
+// limbs of the vector.  Latency bounds both forms here (the matrix is in L2):
+// n = 1000 12.7 -> 9.2 us, n = 2161 21.6 -> 14.3 us, less what the programmatic
+// launch overlaps with the half-step before it (the row's first loads).
+__global__ void __launch_bounds__(FXR_THREADS) k_gemv_row_fx(const long long* __restrict__ NR, int64_t ld, int64_t n,
+                                                             const int* __restrict__ rowE,
+                                                             const double* x, double* __restrict__ part,
+                                                             const int* done) {
+    extern __shared__ int zs[];  // [3][nn] limbs of x
+    __shared__ int red[FXR_THREADS / 32];
+    const int nt = blockDim.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t nn = (n + 1) & ~(int64_t)1;
+    const int64_t r = (int64_t)blockIdx.x * (nt >> 5) + warp;
+    const longlong2* __restrict__ row = reinterpret_cast<const longlong2*>(NR + r * ld);
+    const int64_t nvec = r < n ? n >> 1 : 0;
+    // the first loads of the row go out before the vector is converted
+    longlong2 m[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) m[u] = lane + 32 * u < nvec ? __ldcs(row + lane + 32 * u) : make_longlong2(0, 0);
+    pdl_wait();
+    if (gkb_done(done)) return;
+    int em = 0;
+    for (int64_t i = threadIdx.x; i < n; i += nt) em = max(em, fx_exp(__ldcg(x + i)));
+    em = __reduce_max_sync(RBF_FULL_MASK, em);
+    if (lane == 0) red[warp] = em;
+    __syncthreads();
+    for (int w = 0; w < (nt >> 5); ++w) em = max(em, red[w]);
+    const int sz = 1084 - max(em, 1);
+    for (int64_t j = threadIdx.x; j < n; j += nt) {
+        const int4 l = fx_limbs_bal(fx_round(__ldcg(x + j), sz));
+        zs[j] = l.x;
+        zs[nn + j] = l.y;
+        zs[2 * nn + j] = l.z;
+    }
+    if (threadIdx.x == 0 && nn > n) zs[n] = zs[nn + n] = zs[2 * nn + n] = 0;
+    __syncthreads();
+    if (r >= n) return;
+    FxAcc acc;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+        if (lane + 32 * u < nvec) fx_pair(acc, m[u], zs, nn, 2 * (lane + 32 * u));
+    int64_t v = lane + 256;
+    for (; v + 224 < nvec; v += 256) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) m[u] = __ldcs(row + v + 32 * u);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) fx_pair(acc, m[u], zs, nn, 2 * (v + 32 * u));
+    }
+    for (; v < nvec; v += 32) fx_pair(acc, __ldcs(row + v), zs, nn, 2 * v);
+    if ((n & 1) && lane == 0) acc.add(NR[r * ld + n - 1], zs[n - 1], zs[nn + n - 1], zs[2 * nn + n - 1]);
+    const double s = warp_sum(acc.value());
+    if (lane == 0) part[r] = fx_scale_out(s, __ldg(rowE + r), em);
+}
+
 // ---------------------------------------------------------------------------
 // part[q][c] = sum over row chunk q of A_ic x_i, on NC: column panels x row
 // chunks as the FP64 kernel; each CTA rounds its chunk of x at the chunk's own
@@ -279,12 +336,10 @@ __global__ void __launch_bounds__(FXN_THREADS) k_gemv_flat_fx(const long long* _
 // no common scale) and keeps the limbs (int4 per row, read as a broadcast) in
 // shared memory.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(FXT_THREADS) k_gemv_t_fx(const long long* __restrict__ NC, int64_t ld, int64_t n,
-                                                           const int* __restrict__ colE,
-                                                           const double* __restrict__ x, int panel_cols, int chunks,
-                                                           int rows_max, double* __restrict__ part,
-                                                           const int* __restrict__ done) {
-    if (gkb_done(done)) return;
+__global__ void __launch_bounds__(FXT_THREADS, 4) k_gemv_t_fx(const long long* __restrict__ NC, int64_t ld, int64_t n,
+                                                           const int* __restrict__ colE, const double* x,
+                                                           int panel_cols, int chunks, int rows_max,
+                                                           double* __restrict__ part, const int* done) {
     extern __shared__ int4 xl[];  // [rows_max] limbs of the chunk of x
     __shared__ int red[FXT_THREADS / 32];
     const int q = blockIdx.x % chunks;
@@ -292,16 +347,33 @@ __global__ void __launch_bounds__(FXT_THREADS) k_gemv_t_fx(const long long* __re
     const int64_t i0 = n * (int64_t)q / chunks;
     int64_t i1 = n * (int64_t)(q + 1) / chunks;
     if (!RBF_IN_RANGE(i1 - i0, rows_max + 1)) i1 = i0 + rows_max;
+    const int64_t c = (int64_t)pnl * panel_cols + 2 * threadIdx.x;
+    const long long* __restrict__ base = NC + i0 * ld + c;
+    const int64_t rows = i1 - i0;
+    // the first rows of the matrix go out before the vector is waited for and converted
+    const bool lead = c < n && rows >= FXT_LEAD;
+    longlong2 ml[FXT_LEAD];
+#pragma unroll
+    for (int u = 0; u < FXT_LEAD; ++u)
+        ml[u] = lead ? __ldcs(reinterpret_cast<const longlong2*>(base + u * ld)) : make_longlong2(0, 0);
+    pdl_wait();
+    if (gkb_done(done)) return;
     const int ex = fx_block_max_exp<FXT_THREADS>(x, i0, i1, red);
     const int sx = 1084 - max(ex, 1);
-    for (int64_t i = i0 + threadIdx.x; i < i1; i += FXT_THREADS) xl[i - i0] = fx_limbs_bal(fx_round(__ldg(x + i), sx));
+    for (int64_t i = i0 + threadIdx.x; i < i1; i += FXT_THREADS) xl[i - i0] = fx_limbs_bal(fx_round(__ldcg(x + i), sx));
     __syncthreads();
-    const int64_t c = (int64_t)pnl * panel_cols + 2 * threadIdx.x;
     if (c >= n) return;
-    const long long* __restrict__ base = NC + i0 * ld + c;
     FxAcc ax, ay;
-    const int64_t rows = i1 - i0;
     int64_t r = 0;
+    if (lead) {
+#pragma unroll
+        for (int u = 0; u < FXT_LEAD; ++u) {
+            const int4 l = xl[u];
+            ax.add(ml[u].x, l.x, l.y, l.z);
+            ay.add(ml[u].y, l.x, l.y, l.z);
+        }
+        r = FXT_LEAD;
+    }
     for (; r + FXT_UNROLL - 1 < rows; r += FXT_UNROLL) {
         longlong2 m[FXT_UNROLL];
 #pragma unroll
@@ -314,10 +386,10 @@ __global__ void __launch_bounds__(FXT_THREADS) k_gemv_t_fx(const long long* __re
         }
     }
     for (; r < rows; ++r) {
-        const longlong2 m = __ldcs(reinterpret_cast<const longlong2*>(base + r * ld));
+        const longlong2 m0 = __ldcs(reinterpret_cast<const longlong2*>(base + r * ld));
         const int4 l = xl[r];
-        ax.add(m.x, l.x, l.y, l.z);
-        ay.add(m.y, l.x, l.y, l.z);
+        ax.add(m0.x, l.x, l.y, l.z);
+        ay.add(m0.y, l.x, l.y, l.z);
     }
     part[(int64_t)q * n + c] = fx_scale_out(ax.value(), __ldg(colE + c), ex);
     if (c + 1 < n) part[(int64_t)q * n + c + 1] = fx_scale_out(ay.value(), __ldg(colE + c + 1), ex);
@@ -363,9 +435,26 @@ void fxn_plan(const rbf_ctx* ctx, int64_t n, int* grid, int64_t* W, int* chunks)
     *grid = (int)((*W + FXN_THREADS / 32 - 1) / (FXN_THREADS / 32));
 }
 
-// A^T w plan (the FP64 kernel's panels and chunks) and its largest chunk.
-void fxt_plan(const rbf_ctx* ctx, int64_t n, int* panel_cols, int* panels, int* chunks, int* rows_max) {
+// One row per warp while the rows fit one wave of two CTAs of 16 warps per SM
+// (whole solves, rows against the flat split: n = 3000 5.13 and 5.47 ms, 4090 6.69
+// and 7.21, 4800 8.33 and 8.68; in two waves rows lose: 6400 19.4 and 19.0, 8000
+// 26.2 and 25.0): warps per CTA, or 0 for the flat split.
+int fxn_row_warps(const rbf_ctx* ctx, int64_t n) {
+    if (n > (int64_t)ctx->sm_count * 2 * (FXR_THREADS / 32)) return 0;
+    int w = 4;  // at least 4; as many as spread the rows over the SMs, at most 16
+    while (w < FXR_THREADS / 32 && (int64_t)w * ctx->sm_count < n) w *= 2;
+    return w;
+}
+
+// A^T w plan (the FP64 kernel's panels; its chunks, of FXT_MIN_ROWS rows or more:
+// shorter ones at small n cost the half-step more partials to add than they save
+// in the product) and its largest chunk.
+constexpr int FXT_MIN_ROWS = 32;
+void fxt_plan(const rbf_ctx* ctx, int64_t n, int* panel_cols, int* panels, int* chunks, int* rows_max,
+              int min_rows = FXT_MIN_ROWS) {
     plan_t(ctx, n, 2, panel_cols, panels, chunks);
+    const int64_t most = (n + min_rows - 1) / min_rows;
+    if (*chunks > most) *chunks = (int)most;
     int64_t rm = 0;
     for (int q = 0; q < *chunks; ++q) {
         const int64_t r = n * (int64_t)(q + 1) / *chunks - n * (int64_t)q / *chunks;
@@ -395,7 +484,14 @@ FxCopies fx_carve(WsCarve& wc, const rbf_operator* op) {
     return f;
 }
 
+int fx_t_chunks(const rbf_ctx* ctx, int64_t n) {
+    int pc, pn, ch, rows_max;
+    fxt_plan(ctx, n, &pc, &pn, &ch, &rows_max);
+    return ch;
+}
+
 int fx_n_chunks(const rbf_ctx* ctx, int64_t n) {
+    if (fxn_row_warps(ctx, n)) return 1;
     int g, ch;
     int64_t W;
     fxn_plan(ctx, n, &g, &W, &ch);
@@ -405,7 +501,7 @@ int fx_n_chunks(const rbf_ctx* ctx, int64_t n) {
 rbf_status launch_fx_prepare(rbf_ctx* ctx, const rbf_operator* op, const FxCopies& f) {
     const int64_t n = op->n;
     int pc, pn, ch, rows_max;
-    fxt_plan(ctx, n, &pc, &pn, &ch, &rows_max);
+    fxt_plan(ctx, n, &pc, &pn, &ch, &rows_max, 1);
     // the exponent scan and the conversion cover 2 * FXE_THREADS columns per panel
     if (pc != 2 * FXE_THREADS)
         return rbf_fail(ctx, RBF_ERR_INTERNAL, "fixed-point copies: panel of %d columns, kernels cover %d", pc,
@@ -413,7 +509,7 @@ rbf_status launch_fx_prepare(rbf_ctx* ctx, const rbf_operator* op, const FxCopie
     RBF_CUDA(ctx, cudaMemsetAsync(f.rowE, 0, (size_t)n * sizeof(int), ctx->stream));
     RBF_CUDA(ctx, cudaMemsetAsync(f.colE, 0, (size_t)n * sizeof(int), ctx->stream));
     const size_t smem = (size_t)rows_max * sizeof(int);
-    if (smem > 48 * 1024)
+    if (smem > SMEM_PLAIN)
         RBF_CUDA(ctx, cudaFuncSetAttribute((const void*)k_fx_exps, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)smem));
     k_fx_exps<<<pn * ch, FXE_THREADS, smem, ctx->stream>>>((const double*)op->d_A, op->lda, n, ch, rows_max,
@@ -426,7 +522,17 @@ rbf_status launch_fx_prepare(rbf_ctx* ctx, const rbf_operator* op, const FxCopie
 }
 
 rbf_status launch_fx_n(rbf_ctx* ctx, const rbf_operator* op, const FxCopies& f, const double* x, double* part,
-                       const int* done) {
+                       const int* done, bool pdl) {
+    if (const int w = fxn_row_warps(ctx, op->n)) {
+        const size_t smem = fxn_smem(op->n);
+        if (smem > SMEM_PLAIN)
+            RBF_CUDA(ctx, cudaFuncSetAttribute((const void*)k_gemv_row_fx, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)smem));
+        RBF_CUDA(ctx, rbf_launch_ex(ctx, k_gemv_row_fx, dim3((unsigned)((op->n + w - 1) / w)), dim3(w * 32), smem, pdl,
+                                    1, f.NR, op->lda, op->n, f.rowE, x, part, done));
+        RBF_LAUNCHED(ctx, "k_gemv_row_fx");
+        return RBF_OK;
+    }
     int g, ch;
     int64_t W;
     fxn_plan(ctx, op->n, &g, &W, &ch);
@@ -437,15 +543,15 @@ rbf_status launch_fx_n(rbf_ctx* ctx, const rbf_operator* op, const FxCopies& f, 
 }
 
 rbf_status launch_fx_t(rbf_ctx* ctx, const rbf_operator* op, const FxCopies& f, const double* x, double* part,
-                       const int* done) {
+                       const int* done, bool pdl) {
     int pc, pn, ch, rows_max;
     fxt_plan(ctx, op->n, &pc, &pn, &ch, &rows_max);
     const size_t smem = (size_t)rows_max * sizeof(int4);
-    if (smem > 48 * 1024)
+    if (smem > SMEM_PLAIN)
         RBF_CUDA(ctx, cudaFuncSetAttribute((const void*)k_gemv_t_fx, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)smem));
-    k_gemv_t_fx<<<pn * ch, FXT_THREADS, smem, ctx->stream>>>(f.NC, op->lda, op->n, f.colE, x, pc, ch, rows_max,
-                                                            part, done);
+    RBF_CUDA(ctx, rbf_launch_ex(ctx, k_gemv_t_fx, dim3(pn * ch), dim3(FXT_THREADS), smem, pdl, 1, f.NC, op->lda, op->n,
+                                f.colE, x, pc, ch, rows_max, part, done));
     RBF_LAUNCHED(ctx, "k_gemv_t_fx");
     return RBF_OK;
 }

@@ -20,6 +20,8 @@
 // order), so repeated runs are bitwise identical.  Grid barriers poll a bounded
 // number of times and report RBF_ERR_TIMEOUT instead of hanging.  Once a
 // breakdown is found a device flag makes every later kernel return at once.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cfloat>
 #include <vector>
@@ -169,13 +171,79 @@ struct HalfArgs {
     double* gpart;        // 2 x [mcount][barrier groups] group sums (by barrier parity)
     int64_t hpart_len;    // elements of hpart and of gpart (bounds-checked build)
     int64_t gpart_len;
-    double* npart;        // in: |q_raw|^2 partials; out: |v|^2 partials
+    double* npart;        // in: |q_raw|^2 partials; out: |v|^2 partials (one per CTA)
+    int np_in;            // partials in
     int rmax;             // slab rows held in shared memory (odd: conflict-free strides)
     unsigned* bar;        // barrier counters (see grid_reduce_sync)
     int bar_group;        // CTAs per barrier group
     unsigned epoch0;      // barriers completed on `bar` before this launch
     long long budget;
 };
+
+// Norm of q_raw from its sum of squares, its inverse and the breakdown test
+// (brk: 0 none, 1 alpha or beta_1, 2 beta; nonfinite: code 3), and what they
+// write to the run's state.
+struct HalfNorm {
+    double nrm, inv, ch_new;
+    int brk;
+    bool nonfinite;
+};
+
+// FAST: the square roots and the inverse from refined reciprocal square roots
+// (a third of the chain's latency, results within an ulp or two) where the sums
+// of squares are far from the ends of FP64's range.
+template <bool FAST>
+__device__ __forceinline__ HalfNorm half_norm(const HalfArgs& a, double acc) {
+    const double* sc = a.stt->scal;
+    const double eps = DBL_EPSILON;
+    auto mid = [](double x) { return x > 1e-200 && x < 1e200; };
+    HalfNorm h;
+    const bool fast = FAST && mid(acc);
+    const double rs = fast ? rsqrt_f64(acc) : 0.0;
+    h.nrm = fast ? acc * rs : sqrt(acc);
+    h.brk = 0;
+    // c_hat double buffer: the r-side of step j reads slot j&1, writes (j+1)&1;
+    // the p-side of step j reads slot (j+1)&1
+    const int rd = a.side == 0 ? (a.j & 1) : ((a.j + 1) & 1);
+    const double ch_old = sc[SC_CHAT0 + rd];
+    h.ch_new = ch_old;
+    if (a.resume) {
+        h.nrm = sc[SC_BETA];
+    } else if (a.side == 1) {
+        h.brk = h.nrm <= a.factor * (double)a.n * eps * fmax(ch_old, h.nrm) ? 1 : 0;
+    } else if (a.j == 1) {
+        h.brk = h.nrm > 0.0 ? 0 : 1;
+    } else {
+        const double al = a.alpha[a.j - 2], c2 = fma(al, al, acc);
+        h.ch_new = fmax(ch_old, fast && mid(c2) ? c2 * rsqrt_f64(c2) : hypot(al, h.nrm));
+        h.brk = h.nrm <= a.factor * (double)a.n * eps * h.ch_new ? 2 : 0;
+    }
+    // a norm that is not finite stops the run like a breakdown of the same
+    // side (code 3): NaN or Inf in f, the nodes or the operator
+    h.nonfinite = !isfinite(h.nrm);
+    if (h.nonfinite) h.brk = (a.side == 1 || a.j == 1) ? 1 : 2;
+    h.inv = a.resume ? 1.0 : (fast ? rs : 1.0 / h.nrm);
+    return h;
+}
+
+__device__ __forceinline__ void half_state(const HalfArgs& a, const HalfNorm& h) {
+    rbf_dev_state* stt = a.stt;
+    double* sc = stt->scal;
+    if (a.side == 0 && !a.resume && !h.nonfinite) sc[SC_CHAT0 + ((a.j + 1) & 1)] = h.ch_new;
+    if (h.brk) {
+        stt->info[IN_STEPS] = a.j - 1;
+        stt->info[IN_BREAK] = h.nonfinite ? 3 : h.brk;
+        if (h.brk == 2) a.beta[a.j - 1] = 0.0;
+        stt->info[IN_DONE] = 1;
+    } else if (a.side == 1) {
+        a.alpha[a.j - 1] = h.nrm;
+        sc[SC_ALPHA] = h.nrm;
+    } else {
+        a.beta[a.j - 1] = h.nrm;
+        sc[SC_BETA] = h.nrm;
+        stt->info[IN_STEPS] = a.j - 1;
+    }
+}
 
 // One half-step of Algorithm 1 after the product: finalize the norm of q_raw
 // (alpha_j or beta_j, breakdown test), form v, and reorthogonalize it twice
@@ -233,7 +301,7 @@ __global__ void __launch_bounds__(SL_THREADS) k_half(HalfArgs a) {
     // ---- |q_raw|^2 (every CTA sums the previous partials in the same order)
     if (warp == 0) {
         double acc = 0.0;
-        for (int b = lane; b < (int)gridDim.x; b += 32) acc += a.npart[b];
+        for (int b = lane; b < a.np_in; b += 32) acc += a.npart[b];
         acc = warp_sum(acc);
         if (lane == 0) {
             acc_s = acc;
@@ -244,47 +312,10 @@ __global__ void __launch_bounds__(SL_THREADS) k_half(HalfArgs a) {
     __syncthreads();
     // ---- norm, inverse and breakdown test: one thread of the last warp
     if (threadIdx.x == SL_THREADS - 32) {
-        double* sc = stt->scal;
-        const double eps = DBL_EPSILON;
-        double nrm = sqrt(acc_s);
-        int brk = 0;
-        // c_hat double buffer: the r-side of step j reads slot j&1, writes (j+1)&1;
-        // the p-side of step j reads slot (j+1)&1
-        const int rd = a.side == 0 ? (a.j & 1) : ((a.j + 1) & 1);
-        const double ch_old = sc[SC_CHAT0 + rd];
-        double ch_new = ch_old;
-        if (a.resume) {
-            nrm = sc[SC_BETA];
-        } else if (a.side == 1) {
-            brk = nrm <= a.factor * (double)a.n * eps * fmax(ch_old, nrm) ? 1 : 0;
-        } else if (a.j == 1) {
-            brk = nrm > 0.0 ? 0 : 1;
-        } else {
-            ch_new = fmax(ch_old, hypot(a.alpha[a.j - 2], nrm));
-            brk = nrm <= a.factor * (double)a.n * eps * ch_new ? 2 : 0;
-        }
-        // a norm that is not finite stops the run like a breakdown of the same
-        // side (code 3): NaN or Inf in f, the nodes or the operator
-        const bool nonfinite = !isfinite(nrm);
-        if (nonfinite) brk = (a.side == 1 || a.j == 1) ? 1 : 2;
-        inv_s = a.resume ? 1.0 : 1.0 / nrm;
-        brk_s = brk;
-        if (blockIdx.x == 0) {
-            if (a.side == 0 && !a.resume && !nonfinite) sc[SC_CHAT0 + ((a.j + 1) & 1)] = ch_new;
-            if (brk) {
-                stt->info[IN_STEPS] = a.j - 1;
-                stt->info[IN_BREAK] = nonfinite ? 3 : brk;
-                if (brk == 2) a.beta[a.j - 1] = 0.0;
-                stt->info[IN_DONE] = 1;
-            } else if (a.side == 1) {
-                a.alpha[a.j - 1] = nrm;
-                sc[SC_ALPHA] = nrm;
-            } else {
-                a.beta[a.j - 1] = nrm;
-                sc[SC_BETA] = nrm;
-                stt->info[IN_STEPS] = a.j - 1;
-            }
-        }
+        const HalfNorm h = half_norm<false>(a, acc_s);
+        inv_s = h.inv;
+        brk_s = h.brk;
+        if (blockIdx.x == 0) half_state(a, h);
     }
     // ---- R1: v' = (sum of partials) - fu u: FP64 partials split SPLIT ways;
     // FP32 slots added in order by a compensated (Neumaier) FP32 sum, hi + lo
@@ -407,6 +438,188 @@ __global__ void __launch_bounds__(SL_THREADS) k_half(HalfArgs a) {
     }
 }
 
+// The same half-step by one cluster of HC_CTAS CTAs, for small n mcount and FP64
+// operators: the slab of Q sits in shared memory (R rows x mcount) and the dot
+// products are added over the CTAs through distributed shared memory, so that a
+// reduction costs a hardware cluster barrier (under 1 us) instead of a grid
+// barrier's chain of L2 round trips (6.5 us); the FP64 work (4 n mcount FMAs)
+// runs on 16 of the SMs.  Sums in a fixed order; the state is written after the
+// first cluster barrier, when every CTA has read the done flag.
+// It is launched with programmatic stream serialization: the slab of Q, the norm
+// and the breakdown test are done while the product before it ends.  Per
+// half-step at n = 1000 (mcount up to 40) 22.4 -> 14.1 us, at n = 2161 (up to 120)
+// 26 -> 22.7, less what overlaps the product; a whole step at n = 1000 72 -> 37 us.
+constexpr int HC_CTAS = 16;
+constexpr int HC_T = 512;
+constexpr int HC_SPLIT = 16;  // most threads per basis vector in the dot products
+
+struct HalfClusterSmem {  // offsets in doubles
+    int q, v, scratch, hp, hs, total;
+};
+__host__ __device__ inline HalfClusterSmem half_cluster_smem(int mcount, int rmax) {
+    HalfClusterSmem o;
+    o.q = 0;
+    o.v = mcount * rmax;
+    o.scratch = o.v + rmax;
+    o.hp = o.scratch + 2 * HC_T;
+    o.hs = o.hp + 2 * mcount;
+    o.total = o.hs + mcount;
+    return o;
+}
+
+__global__ void __launch_bounds__(HC_T) k_half_cluster(HalfArgs a) {
+    namespace cg = cooperative_groups;
+    extern __shared__ double dsm[];
+    __shared__ double red[HC_T / 32];
+    __shared__ double acc_s;
+    __shared__ HalfNorm norm_s;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int M = a.mcount, RM = a.rmax;
+    const int64_t r0 = a.n * (int64_t)blockIdx.x / HC_CTAS;
+    int R = (int)(a.n * (int64_t)(blockIdx.x + 1) / HC_CTAS - r0);
+    if (!RBF_IN_RANGE(R, RM + 1)) R = RM;
+    const HalfClusterSmem o = half_cluster_smem(M, RM);
+    double* Qs = dsm + o.q;   // [M][RM]
+    double* vs = dsm + o.v;   // [RM]
+    double* sc = dsm + o.scratch;
+    double* hp = dsm + o.hp;  // [2][M] this CTA's dot products, by pass
+    double* hs = dsm + o.hs;  // [M]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // before the wait for the product: everything that the half-step before it
+    // left (the basis, q_raw, u, the norm partials, the done flag)
+    for (int m = warp; m < M; m += HC_T / 32)
+        for (int i = lane; i < R; i += 32) cp_async8(Qs + (size_t)m * RM + i, a.Q + (int64_t)m * a.ldq + r0 + i);
+    const int done = *(volatile int*)&a.stt->info[IN_DONE];  // set by an earlier launch: the same for every CTA
+    const double ui = a.u && threadIdx.x < R ? a.u[r0 + threadIdx.x] : 0.0;
+    const double qi = threadIdx.x < R ? a.q_raw[r0 + threadIdx.x] : 0.0;
+    if (warp == HC_T / 32 - 1) {
+        double acc = 0.0;
+        for (int b = lane; b < a.np_in; b += 32) acc += a.npart[b];
+        acc = warp_sum(acc);
+        if (lane == 0) {
+            acc_s = acc;
+            if (!done) norm_s = half_norm<true>(a, acc);
+        }
+    }
+    pdl_wait();
+    // ---- sums of the product partials: thread (row, group of chunks)
+    const int RP = max(32, (R + 31) & ~31);  // at most HC_T (n <= HC_MAX_N)
+    const int ng = HC_T / RP;
+    const int row = threadIdx.x % RP, grp = threadIdx.x / RP;
+    if (grp < ng) {
+        double t[4] = {0.0, 0.0, 0.0, 0.0};
+        if (row < R) {
+            const double* p = a.part + r0 + row;
+            int q = grp;
+            for (; q + 3 * ng < a.chunks; q += 4 * ng)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) t[u] += p[(int64_t)(q + u * ng) * a.n];
+            for (; q < a.chunks; q += ng) t[0] += p[(int64_t)q * a.n];
+        }
+        sc[grp * RP + row] = (t[0] + t[1]) + (t[2] + t[3]);
+    }
+    cp_async_wait_all();
+    if (done) return;
+    __syncthreads();
+    if (threadIdx.x < R) {
+        double v = 0.0;
+        for (int g = 0; g < ng; ++g) v += sc[g * RP + threadIdx.x];
+        if (a.u) v = fma(-(a.resume ? a.stt->scal[SC_BETA] : acc_s), ui, v);
+        vs[threadIdx.x] = v;
+    }
+    __syncthreads();
+    int split = 1;
+    while (split < HC_SPLIT && 2 * split * M <= HC_T) split *= 2;
+    for (int pass = 0; pass < 2 && M > 0; ++pass) {
+        for (int p = threadIdx.x; p < split * M; p += HC_T) {
+            const int k = p / M, m = p - k * M;
+            const double* q = Qs + (size_t)m * RM;
+            double c0 = 0.0, c1 = 0.0;
+            int i = k;
+            for (; i + split < R; i += 2 * split) {
+                c0 = fma(q[i], vs[i], c0);
+                c1 = fma(q[i + split], vs[i + split], c1);
+            }
+            if (i < R) c0 = fma(q[i], vs[i], c0);
+            sc[p] = c0 + c1;
+        }
+        __syncthreads();
+        for (int m = threadIdx.x; m < M; m += HC_T) {
+            double c0 = sc[m], c1 = 0.0;
+            int k = 1;
+            for (; k + 1 < split; k += 2) {
+                c1 += sc[k * M + m];
+                c0 += sc[(k + 1) * M + m];
+            }
+            if (k < split) c1 += sc[k * M + m];
+            hp[pass * M + m] = c0 + c1;
+        }
+        cluster.sync();
+        if (pass == 0) {
+            if (blockIdx.x == 0 && threadIdx.x == HC_T - 32) half_state(a, norm_s);
+            if (norm_s.brk) break;
+        }
+        for (int m = threadIdx.x; m < M; m += HC_T) {
+            double t[HC_CTAS];
+#pragma unroll
+            for (int r = 0; r < HC_CTAS; ++r) t[r] = cluster.map_shared_rank(hp, r)[pass * M + m];
+#pragma unroll
+            for (int w = HC_CTAS / 2; w > 0; w >>= 1)
+#pragma unroll
+                for (int r = 0; r < w; ++r) t[r] += t[r + w];
+            hs[m] = t[0];
+        }
+        __syncthreads();
+        if (grp < ng) {
+            double c0 = 0.0, c1 = 0.0;
+            if (row < R) {
+                int m = grp;
+                for (; m + ng < M; m += 2 * ng) {
+                    c0 = fma(Qs[(size_t)m * RM + row], hs[m], c0);
+                    c1 = fma(Qs[(size_t)(m + ng) * RM + row], hs[m + ng], c1);
+                }
+                if (m < M) c0 = fma(Qs[(size_t)m * RM + row], hs[m], c0);
+            }
+            sc[grp * RP + row] = c0 + c1;
+        }
+        __syncthreads();
+        if (threadIdx.x < R) {
+            double t = 0.0;
+            for (int g = 0; g < ng; ++g) t += sc[g * RP + threadIdx.x];
+            vs[threadIdx.x] -= t;
+        }
+        __syncthreads();
+    }
+    if (M == 0) {
+        cluster.sync();  // every CTA has read the done flag and the norm partials
+        if (blockIdx.x == 0 && threadIdx.x == HC_T - 32) half_state(a, norm_s);
+    }
+    const int brk = norm_s.brk;
+    if (brk) {
+        if (brk == 2 && a.basis_out && threadIdx.x < R) a.basis_out[r0 + threadIdx.x] = 0.0;
+    } else {
+        const double inv = norm_s.inv;
+        double acc = 0.0;
+        if (threadIdx.x < R) {
+            a.basis_out[r0 + threadIdx.x] = qi * inv;
+            const double t = vs[threadIdx.x] * inv;
+            a.v[r0 + threadIdx.x] = t;
+            acc = t * t;
+        }
+        if (threadIdx.x < RP) {
+            acc = warp_sum(acc);
+            if (lane == 0) red[warp] = acc;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double t = 0.0;
+            for (int w = 0; w < RP / 32; ++w) t += red[w];
+            a.npart[blockIdx.x] = t;
+        }
+    }
+    cluster.sync();  // no CTA leaves while another reads its dot products
+}
+
 __global__ void __launch_bounds__(SL_THREADS) k_norm_partials(int64_t n, const double* __restrict__ x,
                                                               double* __restrict__ npart,
                                                               double* __restrict__ copy,
@@ -476,6 +689,55 @@ static size_t half_smem_bytes(bool stage, int mcount, int chunks, int rmax, bool
     return ((stage ? (size_t)mcount * rmax : 0) + slots + (size_t)3 * rmax + scratch) * sizeof(double);
 }
 
+// The cluster half-step takes FP64 operators with n <= 8192 (512 rows per CTA) and
+// n mcount up to HC_WORK, or half of it above n = 4096, where the 16 SMs' FP64
+// time stays below that of the grid barriers saved (whole solves, cluster from
+// the first step to these limits against the grid kernel throughout: n = 1500,
+// 60 steps 3.15 and 4.63 ms, 3000 5.13 and 6.20, 4090 6.69 and 7.38; 4800, 100
+// steps 12.9 and 13.5, 6400 18.7 and 19.0, 8000 24.8 and 25.0; 256 K instead of
+// 416 K 1 % slower at n = 2161, the whole of it above 4096 2 % slower at 8000).
+// Mixed runs round their vectors to FP32 for the products and keep one order of
+// summation.
+// The rule depends on the problem and the context's options alone, so resumed and
+// concurrent runs take the same path.  A context with a wait budget far below
+// what a grid barrier takes asks for the timeout path, which only the grid
+// barriers have.
+constexpr int64_t HC_MAX_N = (int64_t)HC_CTAS * HC_T;
+constexpr int64_t HC_WORK = 416 * 1024;
+constexpr size_t HC_SMEM_MAX = 220 * 1024;
+constexpr long long HC_MIN_BUDGET = 4096;
+
+static bool half_cluster_takes(const rbf_ctx* ctx, int64_t n, int mcount, bool mixed) {
+    const int64_t work = n <= HC_MAX_N / 2 ? HC_WORK : HC_WORK / 2;
+    return !mixed && n <= HC_MAX_N && n * mcount <= work && ctx->opt.wait_budget >= HC_MIN_BUDGET;
+}
+
+// Whether this device runs the cluster half-step (one cluster of 16 CTAs with
+// the largest shared memory): asked once per context.
+static bool half_cluster_ready(rbf_ctx* ctx) {
+    if (ctx->half_cluster < 0) {
+        ctx->half_cluster = 0;
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim = {HC_CTAS, 1, 1};
+        cfg.gridDim = dim3(HC_CTAS);
+        cfg.blockDim = dim3(HC_T);
+        cfg.dynamicSmemBytes = HC_SMEM_MAX;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int clusters = 0;
+        if (cudaFuncSetAttribute(k_half_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+            cudaFuncSetAttribute(k_half_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)HC_SMEM_MAX) ==
+                cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&clusters, k_half_cluster, &cfg) == cudaSuccess && clusters > 0)
+            ctx->half_cluster = 1;
+        else
+            cudaGetLastError();
+    }
+    return ctx->half_cluster > 0;
+}
+
 static int slab_grid(const rbf_ctx* ctx, int64_t n) {
     int64_t g = ctx->sm_count;
     int64_t need = (n + SL_MAX_ROWS - 1) / SL_MAX_ROWS;
@@ -513,7 +775,7 @@ size_t gkb_ws_bytes(const rbf_ctx* ctx, int64_t n, int steps, int precision) {
     b += ws_align((size_t)(steps + 2) * G * 8);       // hpart
     b += ws_align((size_t)2 * (steps + 2) * G * 8);   // gpart (two buffers, at most G groups)
     b += ws_align((size_t)(G + 2) * BAR_STRIDE * 4);  // barrier counters
-    b += ws_align((size_t)G * 8);                     // npart
+    b += ws_align((size_t)std::max(G, HC_CTAS) * 8);  // npart
     return b + 4096;
 }
 
@@ -521,11 +783,12 @@ size_t gkb_ws_bytes(const rbf_ctx* ctx, int64_t n, int steps, int precision) {
 // fx: the run's fixed-point copies of A (FP64 assembled operators), or null.
 static rbf_status gkb_product(rbf_ctx* ctx, const rbf_operator* op, int trans, const double* q_raw,
                               const float* q32, const float* X32, const FxCopies* fx, double* part,
-                              const int* done) {
+                              const int* done, bool pdl) {
     const int slot = rbf_prod_begin(ctx, trans);
     rbf_status st;
     if (op->storage == RBF_MATRIX_FREE) st = launch_mf_partial(ctx, op, trans, q_raw, q32, X32, part, done);
-    else if (fx) st = trans ? launch_fx_t(ctx, op, *fx, q_raw, part, done) : launch_fx_n(ctx, op, *fx, q_raw, part, done);
+    else if (fx) st = trans ? launch_fx_t(ctx, op, *fx, q_raw, part, done, pdl)
+                     : launch_fx_n(ctx, op, *fx, q_raw, part, done, pdl);
     else if (trans) st = launch_gemv_t_partial(ctx, op, q_raw, q32, part, done);
     else st = launch_gemv_n(ctx, op, q_raw, q32, part, done);
     rbf_prod_end(ctx, trans, slot);
@@ -565,7 +828,13 @@ struct GkbRun {
     unsigned* bar = nullptr;
     const double* q_raw = nullptr;
     unsigned epochs = 0;  // barriers on `bar` since it was zeroed
+    int np = 0;           // |q_raw|^2 partials the last kernel wrote
+    bool after_cluster = false;  // the last half-step ran as a cluster
     bool mixed = false;
+    // programmatic dependent launches along the step: the fixed-point products
+    // and the cluster half-steps wait for the kernel before them on the device
+    // (not beside launch timing, whose events would sit between them)
+    bool pdl_ok = false;
 
     rbf_status begin(rbf_ctx* c, const rbf_operator* o, const double* f, int jb, rbf_gkb_state* s_) {
         ctx = c;
@@ -586,7 +855,7 @@ struct GkbRun {
             }
         }
         WsCarve wc(ctx->ws);
-        chT = product_chunks(ctx, op, 1);
+        chT = use_fx ? fx_t_chunks(ctx, n) : product_chunks(ctx, op, 1);
         chN = use_fx ? fx_n_chunks(ctx, n) : product_chunks(ctx, op, 0);
         f32slots = mf_slots_f32(ctx, op);
         slot_scale = op->form == RBF_FORM_EPS ? 1.0 / op->c : 1.0;
@@ -618,20 +887,22 @@ struct GkbRun {
             const size_t need = half_smem_bytes(false, st->capacity + 1, chmax, rmax, f32slots);
             if (need > HALF_SMEM_STAGE_MAX)
                 return rbf_fail(ctx, RBF_ERR_UNSUPPORTED, "half-step shared memory too large (%zu bytes)", need);
-            if (need > 48 * 1024)
+            if (need > SMEM_PLAIN)
                 RBF_CUDA(ctx, cudaFuncSetAttribute((const void*)k_half<false>,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need));
             RBF_CUDA(ctx, cudaFuncSetAttribute((const void*)k_half<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)HALF_SMEM_STAGE_MAX));
         }
-        npart = wc.take<double>((size_t)G);
+        npart = wc.take<double>((size_t)std::max(G, HC_CTAS));
         if (use_fx) {
             fx = fx_carve(wc, op);
             RBF_TRY(launch_fx_prepare(ctx, op, fx));
         }
         mixed = op->precision == RBF_MIXED;
+        pdl_ok = use_fx && !(ctx->opt.timing & 2) && !(ctx->owner && (ctx->owner->opt.timing & 2));
         rbf_dev_state* dst = ctx->d_state;
         epochs = 0;
+        np = G;
         // q_raw for the first r-side: f (fresh run) or the stored w_{j_begin} (resume)
         q_raw = vp;
         if (j_begin == 1) {
@@ -682,11 +953,29 @@ struct GkbRun {
         a.hpart_len = (int64_t)(st->capacity + 2) * G;
         a.gpart_len = (int64_t)2 * (st->capacity + 2) * G;
         a.npart = npart;
+        a.np_in = np;
         a.rmax = rmax;
         a.bar = bar;
         a.bar_group = bar_group;
         a.epoch0 = epochs;
         a.budget = ctx->opt.wait_budget;
+        if (half_cluster_takes(ctx, n, mcount, mixed) && half_cluster_ready(ctx)) {
+            a.rmax = (int)((n + HC_CTAS - 1) / HC_CTAS) | 1;
+            const size_t smem = sizeof(double) * (size_t)half_cluster_smem(mcount, a.rmax).total;
+            if (smem <= HC_SMEM_MAX) {
+                const int slot = rbf_prod_begin(ctx, 2);
+                const cudaError_t e = rbf_launch_ex(ctx, k_half_cluster, dim3(HC_CTAS), dim3(HC_T), smem, pdl_ok,
+                                                    HC_CTAS, a);
+                rbf_prod_end(ctx, 2, slot);
+                ctx->launches++;
+                if (e != cudaSuccess)
+                    return rbf_fail(ctx, RBF_ERR_CUDA, "launch of k_half_cluster failed: %s", cudaGetErrorString(e));
+                np = HC_CTAS;
+                after_cluster = true;
+                return RBF_OK;
+            }
+            a.rmax = rmax;
+        }
         void* args[] = {&a};
         const bool stage = half_smem_bytes(true, mcount, chunks, rmax, f32slots) <= half_stage_limit(ctx);
         const size_t smem = half_smem_bytes(stage, mcount, chunks, rmax, f32slots);
@@ -697,6 +986,8 @@ struct GkbRun {
         ctx->launches++;
         if (e != cudaSuccess)
             return rbf_fail(ctx, RBF_ERR_CUDA, "cooperative launch of k_half failed: %s", cudaGetErrorString(e));
+        np = G;
+        after_cluster = false;
         epochs += mcount > 0 ? 2 : 1;  // two reorthogonalization barriers, or one plain barrier
         return RBF_OK;
     }
@@ -707,11 +998,11 @@ struct GkbRun {
         double* Z = st->d_Z;
         const int64_t ldw = st->ldw, ldz = st->ldz;
         // ---------------- r-side: r = A^T w_j - beta_j z_{j-1} ----------------
-        RBF_TRY(gkb_product(ctx, op, 1, q_raw, vp32, X32, use_fx ? &fx : nullptr, part, done));
+        RBF_TRY(gkb_product(ctx, op, 1, q_raw, vp32, X32, use_fx ? &fx : nullptr, part, done, pdl_ok && after_cluster));
         RBF_TRY(half(0, j, (j == j_begin && j_begin > 1) ? 1 : 0, j >= 2 ? Z + (int64_t)(j - 2) * ldz : nullptr,
                      q_raw, W + (int64_t)(j - 1) * ldw, vr, mixed ? vr32 : nullptr, Z, ldz, j - 1, chT));
         // ---------------- p-side: p = A z_j - alpha_j w_j ----------------
-        RBF_TRY(gkb_product(ctx, op, 0, vr, vr32, X32, use_fx ? &fx : nullptr, part, done));
+        RBF_TRY(gkb_product(ctx, op, 0, vr, vr32, X32, use_fx ? &fx : nullptr, part, done, pdl_ok && after_cluster));
         RBF_TRY(half(1, j, 0, W + (int64_t)(j - 1) * ldw, vr, Z + (int64_t)(j - 1) * ldz, vp,
                      mixed ? vp32 : nullptr, W, ldw, j, chN));
         q_raw = vp;
@@ -722,7 +1013,7 @@ struct GkbRun {
         cudaStream_t s = ctx->stream;
         double* wl = st->d_W + (int64_t)j_end * st->ldw;
         // beta_{l+1} and w_{l+1}
-        k_finalize<<<1, 256, 0, s>>>(ctx->d_state, npart, G, 0, j_end + 1, n, ctx->opt.breakdown_factor,
+        k_finalize<<<1, 256, 0, s>>>(ctx->d_state, npart, np, 0, j_end + 1, n, ctx->opt.breakdown_factor,
                                      st->d_alpha, st->d_beta, wl, 1);
         RBF_LAUNCHED(ctx, "k_finalize");
         k_write_basis<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(ctx->d_state, n, SC_INV_BETA, vp, wl);
@@ -827,7 +1118,7 @@ extern "C" rbf_status rbf_gkb_many(rbf_ctx* ctx, int count, const rbf_operator* 
         const size_t need = half_smem_bytes(false, states[i].capacity + 1, chmax, rmax, mf_slots_f32(ctx, &ops[i]));
         if (need > HALF_SMEM_STAGE_MAX) continue;  // the run itself is refused with RBF_ERR_UNSUPPORTED below
         int per_sm = 0;
-        if (need > 48 * 1024)
+        if (need > SMEM_PLAIN)
             RBF_CUDA(ctx, cudaFuncSetAttribute((const void*)k_half<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)need));
         RBF_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)k_half<false>, SL_THREADS,

@@ -75,6 +75,7 @@ struct rbf_ctx {
     cudaEvent_t sync_ev = nullptr;   // fork (owner) or join (lane) event, no timing
     rbf_dev_state* h_many = nullptr; // pinned copies of the device state, one per run
     int h_many_cap = 0;
+    int half_cluster = -1;           // the cluster half-step runs on this device (-1: not asked yet)
 };
 void rbf_batch_state_free(rbf_ctx* ctx);
 cudaStream_t rbf_batch_stream(rbf_ctx* ctx);  // the batched driver's stream, or null
@@ -153,6 +154,34 @@ struct WsCarve {
 };
 inline size_t ws_align(size_t b) { return (b + 255) & ~(size_t)255; }
 
+// Launch of a kernel that calls pdl_wait, with programmatic stream serialization
+// (`pdl`) and as clusters of `cluster` CTAs (1: none).
+template <typename... KArgs, typename... Args>
+inline cudaError_t rbf_launch_ex(rbf_ctx* ctx, void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, bool pdl,
+                                 int cluster, Args... args) {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at[2];
+    int na = 0;
+    if (cluster > 1) {
+        at[na].id = cudaLaunchAttributeClusterDimension;
+        at[na].val.clusterDim.x = (unsigned)cluster;
+        at[na].val.clusterDim.y = at[na].val.clusterDim.z = 1;
+        ++na;
+    }
+    if (pdl) {
+        at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[na].val.programmaticStreamSerializationAllowed = 1;
+        ++na;
+    }
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = ctx->stream;
+    cfg.attrs = at;
+    cfg.numAttrs = na;
+    return cudaLaunchKernelEx(&cfg, k, static_cast<KArgs>(args)...);
+}
+
 // ---- timing ------------------------------------------------------------------
 // Launch timing (opt.timing bit 1) of kind 0 (A x), 1 (A^T x) or 2 (half-step
 // kernels), recorded on `s` (default: the context stream): returns the slot or -1.
@@ -201,11 +230,13 @@ bool fx_eligible(const rbf_ctx* ctx, const rbf_operator* op);
 size_t fx_ws_bytes(const rbf_operator* op);
 FxCopies fx_carve(WsCarve& wc, const rbf_operator* op);
 int fx_n_chunks(const rbf_ctx* ctx, int64_t n);  // partial rows of the fixed-point A z (<= 8)
+int fx_t_chunks(const rbf_ctx* ctx, int64_t n);  // and of A^T w
 rbf_status launch_fx_prepare(rbf_ctx* ctx, const rbf_operator* op, const FxCopies& f);
+// pdl: launched with programmatic stream serialization after the kernel before
 rbf_status launch_fx_n(rbf_ctx* ctx, const rbf_operator* op, const FxCopies& f, const double* x, double* part,
-                       const int* done);
+                       const int* done, bool pdl);
 rbf_status launch_fx_t(rbf_ctx* ctx, const rbf_operator* op, const FxCopies& f, const double* x, double* part,
-                       const int* done);
+                       const int* done, bool pdl);
 // mf.cu (matrix-free products, FP32 or FP64; partial sums over `mf_chunks` centre chunks)
 // Partial rows the consumer sums (mf_chunks) and rows the product writes
 // (mf_part_rows >= mf_chunks; the FP32 tile-pair product folds its slots).
