@@ -1,0 +1,249 @@
+// Reconstruction u(P_t) = sum_j coef_j Phi(|P_t - X_j|), Phi(r) = sqrt(r^2 + c^2)
+// (eq. u_reconstruction), for one or several coefficient vectors that share Phi.
+//
+// In FP64 a pair costs 12 FP64-pipe operations for Phi and an FMA per vector, at
+// 2 operations per clock per SM: 10.3 ms for 20 000 points and nodes (0.80 of the
+// pipe).  The pairs are therefore evaluated in 64-bit fixed point on the integer
+// and FP32 pipes (94 instructions per pair, 10 of them per vector, at 32
+// to 64 times the FP64 rate): 10.3 -> 1.70 ms.
+//
+//   - the coordinates and c are rounded at 2^-k, k such that the largest of them
+//     stays below 2^60: q = round(x 2^k) (exact for values within 2^7 of the
+//     largest, |error| <= 2^-61 of it otherwise);
+//   - with d = q_P - q_X = h 2^32 + l (l signed 32 bits), s = |P - X|^2 + c^2 in
+//     units of 2^(64-2k) is sum h^2 + (2 sum h l + (sum l^2 >> 32)) / 2^32, kept as 64
+//     integer and 32 fraction bits;
+//   - sqrt(s): FP32 estimate R0 = s rsqrt(s); with the exact residual e0 = s - R0^2,
+//     R1 = 2^12 R0 + round(2^12 e0 rsqrt(s) / 2); with the residual e1 = 2^24 s -
+//     R1^2, small enough to be taken modulo 2^64, N = 2^19 R1 + round(2^19 e1 rsqrt(s) /
+//     2^13): |N - 2^31 sqrt(s)| is under 9 units, 2^-57.8 of the largest Phi and 2^-53 of
+//     the smallest that the rule below admits;
+//   - the coefficients are rounded at 2^-62 of the largest of the CTA's chunk and
+//     the products N coef are added exactly in 21-bit limbs (fx_core.cuh), then
+//     rounded to FP64 once per chunk.
+// Every error is at most about 2^-58 of the largest Phi times the coefficients,
+// below the roundings of the FP64 form (an ulp or two per term and the sum's), so
+// long as c is not tiny beside the coordinates: an exponent at most 5 below the
+// largest (at 6 below the smallest Phi would carry 2^-51.4 relative).  Below
+// that, and with any Inf or NaN, a CTA takes the FP64 form (a first launch finds
+// the coordinates' largest exponent, the CTA its coefficients').
+#include "common.cuh"
+#include "fx_core.cuh"
+#include "internal.h"
+
+namespace {
+
+constexpr int EV_T = 128;           // points per CTA, one per thread; nodes per stage
+constexpr int EV_MAX_CHUNK = 1 << 19;  // nodes per CTA: the limb sums stay below 2^63
+constexpr int EX_CTAS = 64;         // partial maxima of the exponent scan
+
+// Largest exponent field of the nodes' and points' coordinates, one partial per CTA.
+__global__ void __launch_bounds__(256) k_eval_exps(const double* __restrict__ X, int64_t n3,
+                                                   const double* __restrict__ P, int64_t m3, int* __restrict__ out) {
+    __shared__ int red[8];
+    const int64_t t0 = (int64_t)blockIdx.x * 256 + threadIdx.x, step = (int64_t)gridDim.x * 256;
+    int ex = 0;
+    for (int64_t i = t0; i < n3; i += step) ex = max(ex, fx_exp(X[i]));
+    for (int64_t i = t0; i < m3; i += step) ex = max(ex, fx_exp(P[i]));
+    ex = __reduce_max_sync(RBF_FULL_MASK, ex);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ex;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 0; w < 8; ++w) ex = max(ex, red[w]);
+        out[blockIdx.x] = ex;
+    }
+}
+
+// 2^31 sqrt(s) for s = |d|^2 + c^2 from the fixed-point differences d = (hx, lx),
+// ..., and c's parts: hh0 = h_c^2, hl0 = h_c l_c + (l_c^2 >> 33).
+__device__ __forceinline__ long long eval_phi(long long dx, long long dy, long long dz, long long hh0, long long hl0) {
+    const int lx = (int)dx, ly = (int)dy, lz = (int)dz;
+    const int hx = (int)(dx >> 32) - (lx >> 31), hy = (int)(dy >> 32) - (ly >> 31), hz = (int)(dz >> 32) - (lz >> 31);
+    const long long hh = imad_wide(hx, hx, imad_wide(hy, hy, imad_wide(hz, hz, hh0)));
+    const long long hl = imad_wide(hx, lx, imad_wide(hy, ly, imad_wide(hz, lz, hl0)));
+    const unsigned long long ll = (unsigned long long)imad_wide(lx, lx, imad_wide(ly, ly, imad_wide(lz, lz, 0)));
+    const long long T = 2 * hl + (long long)(ll >> 32);
+    const long long s = hh + (T >> 32);  // >= 2^36
+    const unsigned frac = (unsigned)T, s0 = (unsigned)s, s1 = (unsigned)((unsigned long long)s >> 32);
+    const float sf = fmaf((float)s1, 4294967296.f, (float)s0);
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(sf));
+    const int R0 = (int)(sf * y);                           // < 2^30, within 2^8 of sqrt(s)
+    const long long e0 = imad_wide(-R0, R0, s);             // |e0| < 2^39
+    // d1 = 2^12 e0 y / 2, rounded to an integer by the addition of 1.5 2^23
+    const int b1 = __float_as_int(fmaf((float)(int)(e0 >> 9), y * 1048576.f, 12582912.f));
+    const long long R1 = (long long)R0 * 4096 + (b1 - 0x4B400000);
+    // e1 = 2^24 s - R1^2 modulo 2^64 (|e1| < 2^46)
+    const unsigned w0 = __funnelshift_l(frac, s0, 24), w1 = __funnelshift_l(s0, s1, 24);
+    const unsigned r0 = (unsigned)R1, r1 = (unsigned)((unsigned long long)R1 >> 32);
+    const unsigned long long sq = (unsigned long long)r0 * r0 + ((unsigned long long)(2u * r1 * r0) << 32);
+    const long long e1 = (long long)((((unsigned long long)w1 << 32) | w0) - sq);
+    const int b2 = __float_as_int(fmaf((float)(int)(e1 >> 15), y * 2097152.f, 12582912.f));  // 2^19 e1 y / 2^13
+    return (R1 << 19) + (b2 - 0x4B400000);
+}
+
+// Partials over the centre chunk blockIdx.y for the NC vectors blockIdx.z NC ..:
+// part[chunk][vector][t].
+template <int NC>
+__global__ void __launch_bounds__(EV_T) k_evaluate(const double* __restrict__ X, int64_t n,
+                                                   const double* __restrict__ coefs, int64_t ldc, int ncoef,
+                                                   const double* __restrict__ Pts, int64_t m, double c, double scale,
+                                                   int64_t chunk, const int* __restrict__ exps,
+                                                   double* __restrict__ part) {
+    __shared__ long long qx[EV_T], qy[EV_T], qz[EV_T];  // staged nodes (FP64 form: their bits)
+    __shared__ int4 qa[NC][EV_T];                       // staged coefficient limbs (FP64 form: values)
+    __shared__ int red[EV_T / 32][NC + 1];
+    const int64_t t = (int64_t)blockIdx.x * EV_T + threadIdx.x;
+    const bool active = t < m;
+    const int c0 = blockIdx.z * NC;
+    const int nc = min(NC, ncoef - c0);
+    const int64_t j0 = (int64_t)blockIdx.y * chunk;
+    const int64_t j1 = min(n, j0 + chunk);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const double px = active ? Pts[t] : 0.0, py = active ? Pts[m + t] : 0.0, pz = active ? Pts[2 * m + t] : 0.0;
+    // largest exponents: of all coordinates (ev[NC]), of the chunk's coefficients
+    int ev[NC + 1], ea = 0;
+    ev[NC] = threadIdx.x < EX_CTAS ? exps[threadIdx.x] : 0;
+#pragma unroll
+    for (int q = 0; q < NC; ++q) {
+        ev[q] = 0;
+        if (q < nc)
+            for (int64_t j = j0 + threadIdx.x; j < j1; j += EV_T)
+                ev[q] = max(ev[q], fx_exp(coefs[(int64_t)(c0 + q) * ldc + j]));
+    }
+#pragma unroll
+    for (int q = 0; q < NC + 1; ++q) {
+        ev[q] = __reduce_max_sync(RBF_FULL_MASK, ev[q]);
+        if (lane == 0) red[warp][q] = ev[q];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < NC + 1; ++q) {
+        for (int w = 0; w < EV_T / 32; ++w) ev[q] = max(ev[q], red[w][q]);
+        if (q < NC) ea = max(ea, ev[q]);
+    }
+    const int ec = fx_exp(c), es = max(max(ev[NC], ec), 1);
+    double res[NC];
+    if (es < FX_NONFINITE && ea < FX_NONFINITE && ec >= es - 5) {
+        const int k = 1082 - es;
+        const long long ux = fx_round(px, k), uy = fx_round(py, k), uz = fx_round(pz, k), qc = fx_round(c, k);
+        const int lc = (int)qc, hc = (int)(qc >> 32) - (lc >> 31);
+        const long long hh0 = imad_wide(hc, hc, 0), hl0 = imad_wide(hc, lc, imad_wide(lc, lc, 0) >> 33);
+        FxAcc acc[NC];
+        for (int64_t jb = j0; jb < j1; jb += EV_T) {
+            __syncthreads();
+            const int64_t j = jb + threadIdx.x;
+            const bool ok = j < j1;
+            qx[threadIdx.x] = ok ? fx_round(X[j], k) : 0;
+            qy[threadIdx.x] = ok ? fx_round(X[n + j], k) : 0;
+            qz[threadIdx.x] = ok ? fx_round(X[2 * n + j], k) : 0;
+#pragma unroll
+            for (int q = 0; q < NC; ++q)
+                qa[q][threadIdx.x] = ok && q < nc ? fx_limbs_bal(fx_round(coefs[(int64_t)(c0 + q) * ldc + j],
+                                                                          1084 - max(ev[q], 1)))
+                                                  : make_int4(0, 0, 0, 0);
+            __syncthreads();
+            const int cnt = (int)min((int64_t)EV_T, j1 - jb);
+#pragma unroll 2
+            for (int r = 0; r < cnt; ++r) {
+                const long long N = eval_phi(ux - qx[r], uy - qy[r], uz - qz[r], hh0, hl0);
+#pragma unroll
+                for (int q = 0; q < NC; ++q) {
+                    const int4 a = qa[q][r];
+                    acc[q].add(N, a.x, a.y, a.z);
+                }
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < NC; ++q) res[q] = ldexp(acc[q].value(), 43 - k - (1084 - max(ev[q], 1)));
+    } else {
+        const double c2 = c * c;
+        const bool far = ec < 1023 - 490 || es > 1023 + 490;  // s may leave the normal numbers
+        double* sx = (double*)qx;
+        double* sy = (double*)qy;
+        double* sz = (double*)qz;
+#pragma unroll
+        for (int q = 0; q < NC; ++q) res[q] = 0.0;
+        for (int64_t jb = j0; jb < j1; jb += EV_T) {
+            __syncthreads();
+            const int64_t j = jb + threadIdx.x;
+            const bool ok = j < j1;
+            sx[threadIdx.x] = ok ? X[j] : 0.0;
+            sy[threadIdx.x] = ok ? X[n + j] : 0.0;
+            sz[threadIdx.x] = ok ? X[2 * n + j] : 0.0;
+#pragma unroll
+            for (int q = 0; q < NC; ++q)
+                *(double*)&qa[q][threadIdx.x] = ok && q < nc ? coefs[(int64_t)(c0 + q) * ldc + j] : 0.0;
+            __syncthreads();
+            const int cnt = (int)min((int64_t)EV_T, j1 - jb);
+            for (int r = 0; r < cnt; ++r) {
+                const double dx = px - sx[r], dy = py - sy[r], dz = pz - sz[r];
+                const double s = fma(dx, dx, fma(dy, dy, fma(dz, dz, c2)));
+                const double ph = far ? sqrt(s) : s * rsqrt_f64(s);
+#pragma unroll
+                for (int q = 0; q < NC; ++q) res[q] = fma(*(const double*)&qa[q][r], ph, res[q]);
+            }
+        }
+    }
+    if (active)
+#pragma unroll
+        for (int q = 0; q < NC; ++q)
+            if (q < nc) part[((int64_t)blockIdx.y * ncoef + c0 + q) * m + t] = res[q] * scale;
+}
+
+rbf_status evaluate_vectors(rbf_ctx* ctx, const rbf_operator* op, const double* coefs, int64_t ldc, int ncoef,
+                            const double* pts, int64_t m, double* u) {
+    const int64_t n = op->n;
+    const int64_t tiles = (m + EV_T - 1) / EV_T;
+    // vectors per CTA: the smallest of 1, 2, 4, 8 that holds them all (8 beyond)
+    const int nc = ncoef <= 1 ? 1 : ncoef <= 2 ? 2 : ncoef <= 4 ? 4 : 8;
+    const int zs = (ncoef + nc - 1) / nc;
+    // one wave of resident CTAs, chunks of at least 256 nodes (the chains of a
+    // pair need all the warps that fit: 8 CTAs per SM 1.79, a full wave 1.70 ms at
+    // 20 000 points and nodes)
+    const void* kern = nc == 1 ? (const void*)k_evaluate<1> : nc == 2 ? (const void*)k_evaluate<2>
+                       : nc == 4 ? (const void*)k_evaluate<4> : (const void*)k_evaluate<8>;
+    int per_sm = 0;
+    RBF_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, EV_T, 0));
+    int64_t chunks = (int64_t)ctx->sm_count * per_sm / (tiles * zs);
+    chunks = chunks < 1 ? 1 : chunks;
+    if ((n + chunks - 1) / chunks < 256) chunks = (n + 255) / 256;
+    if ((n + chunks - 1) / chunks > EV_MAX_CHUNK) chunks = (n + EV_MAX_CHUNK - 1) / EV_MAX_CHUNK;
+    if (chunks > 65535) chunks = 65535;
+    const int64_t chunk = (n + chunks - 1) / chunks;
+    chunks = (n + chunk - 1) / chunk;
+    const int64_t total = m * ncoef;
+    RBF_TRY(rbf_ws_reserve(ctx, ws_align((size_t)chunks * total * sizeof(double)) + ws_align(EX_CTAS * sizeof(int))));
+    WsCarve wc(ctx->ws);
+    double* part = wc.take<double>((size_t)chunks * total);
+    int* exps = wc.take<int>(EX_CTAS);
+    k_eval_exps<<<EX_CTAS, 256, 0, ctx->stream>>>(op->d_nodes, 3 * n, pts, 3 * m, exps);
+    RBF_LAUNCHED(ctx, "k_eval_exps");
+    const double scale = op->form == RBF_FORM_EPS ? 1.0 / op->c : 1.0;
+    const dim3 grid((unsigned)tiles, (unsigned)chunks, (unsigned)zs);
+#define EV_LAUNCH(NC_)                                                                                            \
+    k_evaluate<NC_><<<grid, EV_T, 0, ctx->stream>>>(op->d_nodes, n, coefs, ldc, ncoef, pts, m, op->c, scale, chunk, \
+                                                    exps, part)
+    if (nc == 1) EV_LAUNCH(1);
+    else if (nc == 2) EV_LAUNCH(2);
+    else if (nc == 4) EV_LAUNCH(4);
+    else EV_LAUNCH(8);
+#undef EV_LAUNCH
+    RBF_LAUNCHED(ctx, "k_evaluate");
+    return launch_reduce_partials(ctx, total, (int)chunks, part, u);
+}
+
+}  // namespace
+
+rbf_status launch_evaluate(rbf_ctx* ctx, const rbf_operator* op, const double* coef, const double* pts, int64_t m,
+                           double* u) {
+    return evaluate_vectors(ctx, op, coef, op->n, 1, pts, m, u);
+}
+
+extern "C" rbf_status rbf_evaluate_many(rbf_ctx* ctx, const rbf_operator* op, const double* d_coefs, int64_t ldc,
+                                        int ncoef, const double* d_points, int64_t m, double* d_u) {
+    if (!ctx) return RBF_ERR_INVALID;
+    if (!op || !d_coefs || !d_points || !d_u || m < 1 || ncoef < 1 || ldc < op->n)
+        return rbf_fail(ctx, RBF_ERR_INVALID, "rbf_evaluate_many: bad argument");
+    return evaluate_vectors(ctx, op, d_coefs, ldc, ncoef, d_points, m, d_u);
+}

@@ -198,6 +198,7 @@ rbf_status launch_assemble(rbf_ctx* ctx, const rbf_operator* op);
 // launch_assemble calls.
 bool assemble_pairable(const rbf_operator* a, const rbf_operator* b);
 rbf_status launch_assemble_pair(rbf_ctx* ctx, const rbf_operator* a, const rbf_operator* b);
+// evaluate.cu
 rbf_status launch_evaluate(rbf_ctx* ctx, const rbf_operator* op, const double* coef,
                            const double* pts, int64_t m, double* u);
 // gemv.cu

@@ -1,6 +1,6 @@
 // Stopping / lambda network (20 -> 128 -> 128 -> 2, exact-erf GELU, FP32) with
 // forward, backward and Adam kernels; the features it reads from the first GKB
-// steps; a multi-vector reconstruction used to build its training labels.
+// steps.
 //
 // A training step is three launches: forward and activation gradients of a few
 // samples per CTA with W2 in shared memory (k_mlp_pass), partial weight
@@ -396,59 +396,6 @@ __global__ void k_stop_features_batch(const double* __restrict__ alpha, const do
     stop_features_one(alpha + (size_t)b * L, beta + (size_t)b * (L + 1), sigma + (size_t)b * L, j, mean, stdv, out);
 }
 
-// u[c][t] = sum_j coef[c][j] Phi(|P_t - X_j|) for 8 coefficient vectors per
-// grid.z slice (partials over centre chunks in grid.y).
-// EM_C coefficient vectors per CTA share each Phi(|P_t - X_j|): 12 FP64-pipe
-// operations for Phi plus one FMA per vector.
-constexpr int EM_T = 128;
-template <int EM_C>
-__global__ void __launch_bounds__(EM_T) k_evaluate_many(const double* __restrict__ X, int64_t n,
-                                                       const double* __restrict__ coefs, int64_t ldc, int ncoef,
-                                                       const double* __restrict__ Pts, int64_t m, double c,
-                                                       double scale, int64_t chunk, double* __restrict__ part) {
-    __shared__ double sx[EM_T], sy[EM_T], sz[EM_T], sa[EM_C][EM_T];
-    const int64_t t = (int64_t)blockIdx.x * EM_T + threadIdx.x;
-    const bool active = t < m;
-    const double px = active ? Pts[t] : 0.0, py = active ? Pts[m + t] : 0.0, pz = active ? Pts[2 * m + t] : 0.0;
-    const int c0 = blockIdx.z * EM_C;
-    const int nc = min(EM_C, ncoef - c0);
-    const int64_t j0 = (int64_t)blockIdx.y * chunk;
-    const int64_t j1 = min(n, j0 + chunk);
-    const double c2 = c * c;
-    double acc[EM_C];
-#pragma unroll
-    for (int q = 0; q < EM_C; ++q) acc[q] = 0.0;
-    for (int64_t jb = j0; jb < j1; jb += EM_T) {
-        __syncthreads();
-        const int64_t j = jb + threadIdx.x;
-        const bool ok = j < j1;
-        sx[threadIdx.x] = ok ? X[j] : 0.0;
-        sy[threadIdx.x] = ok ? X[n + j] : 0.0;
-        sz[threadIdx.x] = ok ? X[2 * n + j] : 0.0;
-#pragma unroll
-        for (int q = 0; q < EM_C; ++q) sa[q][threadIdx.x] = (ok && q < nc) ? coefs[(int64_t)(c0 + q) * ldc + j] : 0.0;
-        __syncthreads();
-        const int cnt = (int)min((int64_t)EM_T, j1 - jb);
-        for (int r = 0; r < cnt; ++r) {
-            const double dx = px - sx[r], dy = py - sy[r], dz = pz - sz[r];
-            const double s = fma(dx, dx, fma(dy, dy, fma(dz, dz, c2)));
-            const double ph = s * rsqrt_f64(s);
-#pragma unroll
-            for (int q = 0; q < EM_C; ++q) acc[q] = fma(sa[q][r], ph, acc[q]);
-        }
-    }
-    if (active)
-        for (int q = 0; q < nc; ++q) part[((int64_t)blockIdx.y * ncoef + c0 + q) * m + t] = acc[q] * scale;
-}
-
-__global__ void k_reduce_many(const double* __restrict__ part, int chunks, int64_t total, double* __restrict__ out) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= total) return;
-    double s = 0.0;
-    for (int q = 0; q < chunks; ++q) s += part[(int64_t)q * total + i];
-    out[i] = s;
-}
-
 }  // namespace
 
 // ---------------------------------------------------------------------------
@@ -587,44 +534,5 @@ rbf_status launch_stop_features_batch(rbf_ctx* ctx, const double* alpha, const d
                                       float* feat) {
     k_stop_features_batch<<<B, 32, 0, ctx->stream>>>(alpha, beta, sigma, L, d_l, j, mean, stdv, feat);
     RBF_LAUNCHED(ctx, "k_stop_features_batch");
-    return RBF_OK;
-}
-
-extern "C" rbf_status rbf_evaluate_many(rbf_ctx* ctx, const rbf_operator* op, const double* d_coefs, int64_t ldc,
-                                        int ncoef, const double* d_points, int64_t m, double* d_u) {
-    if (!ctx) return RBF_ERR_INVALID;
-    if (!op || !d_coefs || !d_points || !d_u || m < 1 || ncoef < 1 || ldc < op->n)
-        return rbf_fail(ctx, RBF_ERR_INVALID, "rbf_evaluate_many: bad argument");
-    const int64_t n = op->n;
-    const int64_t tiles = (m + EM_T - 1) / EM_T;
-    // vectors per CTA: the smallest of 1, 2, 4, 8 that holds them all (8 beyond)
-    const int em_c = ncoef <= 1 ? 1 : ncoef <= 2 ? 2 : ncoef <= 4 ? 4 : 8;
-    const int zs = (ncoef + em_c - 1) / em_c;
-    int64_t chunks = ((int64_t)ctx->sm_count * 8 + tiles * zs - 1) / (tiles * zs);
-    if (chunks < 1) chunks = 1;
-    if ((n + chunks - 1) / chunks < 256) chunks = (n + 255) / 256;
-    if (chunks < 1) chunks = 1;
-    const int64_t chunk = (n + chunks - 1) / chunks;
-    chunks = (n + chunk - 1) / chunk;
-    const int64_t total = m * ncoef;
-    RBF_TRY(rbf_ws_reserve(ctx, ws_align((size_t)chunks * total * 8)));
-    double* part = (double*)ctx->ws;
-    const double scale = op->form == RBF_FORM_EPS ? 1.0 / op->c : 1.0;
-    const dim3 grid((unsigned)tiles, (unsigned)chunks, (unsigned)zs);
-    if (em_c == 1)
-        k_evaluate_many<1><<<grid, EM_T, 0, ctx->stream>>>(op->d_nodes, n, d_coefs, ldc, ncoef, d_points, m, op->c,
-                                                           scale, chunk, part);
-    else if (em_c == 2)
-        k_evaluate_many<2><<<grid, EM_T, 0, ctx->stream>>>(op->d_nodes, n, d_coefs, ldc, ncoef, d_points, m, op->c,
-                                                           scale, chunk, part);
-    else if (em_c == 4)
-        k_evaluate_many<4><<<grid, EM_T, 0, ctx->stream>>>(op->d_nodes, n, d_coefs, ldc, ncoef, d_points, m, op->c,
-                                                           scale, chunk, part);
-    else
-        k_evaluate_many<8><<<grid, EM_T, 0, ctx->stream>>>(op->d_nodes, n, d_coefs, ldc, ncoef, d_points, m, op->c,
-                                                           scale, chunk, part);
-    RBF_LAUNCHED(ctx, "k_evaluate_many");
-    k_reduce_many<<<(unsigned)((total + 255) / 256), 256, 0, ctx->stream>>>(part, (int)chunks, total, d_u);
-    RBF_LAUNCHED(ctx, "k_reduce_many");
     return RBF_OK;
 }
