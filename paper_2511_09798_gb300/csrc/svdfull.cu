@@ -25,6 +25,8 @@
 #include <cfloat>
 #include <vector>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "grid_sync.cuh"
 #include "internal.h"
@@ -415,8 +417,8 @@ __device__ __forceinline__ Refl reflector(double x0, double ss) {
 // vectors u, x and v sit in shared memory, and the norms come from one partial
 // per CTA instead of a pass over the vector in every CTA.  The FP64 pipe bounds
 // it (4 n^3 / 3 FMAs: 57 ms at n = 3001, 2.1 ms at 1000) together with the two
-// barriers and reflector chains per step.  n = 1000: 26.5 -> 20.5 ms, n =
-// 3001: 244 -> 137 ms.
+// barriers and reflector chains per step.  n = 1000: 26.5 -> 17.8 ms, n =
+// 3001: 244 -> 130 ms.
 constexpr int BD_T = 512;
 constexpr int BD_W = BD_T / 32;
 constexpr int BD_ROWS = 256;  // rows of a column piece (8 per lane)
@@ -427,10 +429,8 @@ struct BidiagArgs {
     int64_t n, ld;
     double *dg, *eg, *taur, *scaler;
     double *y, *r, *x, *a;  // [n+1] y' and r by column, x' and column k + 1 of A by row
-    double* part;           // [3][G] |r|^2, y.r (columns past k + 1), |a|^2 (rows past k + 1)
+    ulonglong2* slot;       // [3][G to][G from] |r|^2, y.r (columns past k + 1), |a|^2 (rows past k + 1), with epochs
     rbf_dev_state* stt;
-    unsigned* bar;
-    int group;
     long long budget;
 };
 
@@ -443,11 +443,70 @@ inline size_t bd_smem(int64_t n, int G) {
     return sizeof(double) * (size_t)(3 * n + bd_cols(n, G) * (bd_pieces(n) + 1) + bd_blocks(n, G) * BD_W * BD_RB);
 }
 
-// sum of G partials, in every lane of the calling warp (fixed order)
-__device__ __forceinline__ double bd_sum(const double* p, int G, int lane) {
-    double s = 0.0;
-    for (int b = lane; b < G; b += 32) s += __ldcg(p + b);
-    return warp_sum(s);
+// Grid barrier that carries its own reduction: a CTA sends its partial sum and
+// the barrier's number as one 128-bit word to a slot of its own in every CTA's
+// row of slots, and one warp of each CTA polls that CTA's row and adds the values
+// (in a fixed order).  One store and one load across the L2, where arriving at a
+// counter, polling it and then loading the partials takes three trips: the whole
+// solve 24.2 -> 21.5 ms at n = 1000 and 157 -> 150 ms at 3001 (with the loads
+// ahead of the barriers below).  All CTAs polling one shared row of slots: 22.9
+// and 154.5 ms, its lines are too hot; one load after the other: 27.4 and 166.
+__device__ __forceinline__ void bd_fence() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+__device__ __forceinline__ void bd_publish(ulonglong2* slot, double v, unsigned long long epoch) {
+    asm volatile("{\n .reg .b128 t;\n mov.b128 t, {%1, %2};\n st.relaxed.gpu.global.b128 [%0], t;\n}" ::"l"(slot),
+                 "l"(__double_as_longlong(v)), "l"(epoch)
+                 : "memory");
+}
+__device__ __forceinline__ ulonglong2 bd_peek(const ulonglong2* slot) {
+    ulonglong2 r;
+    asm volatile("{\n .reg .b128 t;\n ld.relaxed.gpu.global.b128 t, [%2];\n mov.b128 {%0, %1}, t;\n}"
+                 : "=l"(r.x), "=l"(r.y)
+                 : "l"(slot)
+                 : "memory");
+    return r;
+}
+
+// The calling warp waits until all G slots of each of NS sums carry `epoch` and
+// adds their values; all loads of a lane are in flight together.  Bounded: false
+// after `budget` polls (the run is then stopped).
+constexpr int BD_SLOTS = 5;  // slots per lane and sum in flight: 160 CTAs in one go
+template <int NS>
+__device__ __forceinline__ bool bd_collect(const ulonglong2* slot, int G, unsigned long long epoch, long long budget,
+                                           int lane, double* sum) {
+    bool ok = true;
+#pragma unroll
+    for (int e = 0; e < NS; ++e) sum[e] = 0.0;
+    for (int b0 = lane; b0 < G; b0 += 32 * BD_SLOTS) {
+        ulonglong2 v[NS][BD_SLOTS];
+        for (long long it = 0;; ++it) {
+            bool all = true;
+#pragma unroll
+            for (int e = 0; e < NS; ++e)
+#pragma unroll
+                for (int q = 0; q < BD_SLOTS; ++q)
+                    v[e][q] = b0 + 32 * q < G ? bd_peek(slot + (int64_t)e * G * G + b0 + 32 * q)
+                                              : make_ulonglong2(0, epoch);
+#pragma unroll
+            for (int e = 0; e < NS; ++e)
+#pragma unroll
+                for (int q = 0; q < BD_SLOTS; ++q) all = all && v[e][q].y == epoch;
+            if (all) break;
+            if (it > budget) {
+                ok = false;
+                break;
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < NS; ++e) {
+            double d[BD_SLOTS];
+#pragma unroll
+            for (int q = 0; q < BD_SLOTS; ++q) d[q] = __longlong_as_double((long long)v[e][q].x);
+            sum[e] += ((d[0] + d[1]) + (d[2] + d[3])) + d[4];
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < NS; ++e) sum[e] = warp_sum(sum[e]);
+    return __all_sync(RBF_FULL_MASK, ok);
 }
 
 __global__ void __launch_bounds__(BD_T) k_bidiag(BidiagArgs g) {
@@ -464,7 +523,32 @@ __global__ void __launch_bounds__(BD_T) k_bidiag(BidiagArgs g) {
     double* pd = sm + 3 * n;                 // [columns][pieces] partial dots
     double* sk = pd + bd_cols(n, G) * pmax;  // [columns] row k of the updated columns
     double* rp = sk + bd_cols(n, G);         // [row blocks][warps][rows]
-    unsigned epoch = 0;
+    __shared__ int go;
+    unsigned long long epoch = 1;
+    const ulonglong2* mine = g.slot + (int64_t)cta * G;
+    // warp 0 sends v (the same in every lane) to all CTAs
+    auto publish = [&](int e, double v) {
+        for (int b = lane; b < G; b += 32) bd_publish(g.slot + ((int64_t)e * G + b) * G + cta, v, epoch);
+    };
+    // a collected barrier: warp 0 waits; false stops the CTA
+    double sums[2] = {0.0, 0.0};  // (warp 0)
+    auto collect = [&](auto two) -> bool {
+        if (warp == 0) {
+            const bool ok = two ? bd_collect<2>(mine, G, epoch, g.budget, lane, sums)
+                                : bd_collect<1>(mine + 2 * (int64_t)G * G, G, epoch, g.budget, lane, sums);
+            bd_fence();  // the others' stores, made before they published, are visible from here on
+            if (lane == 0) {
+                go = ok;
+                if (!ok) {
+                    atomicExch(&g.stt->info[IN_ERR], (int)RBF_ERR_TIMEOUT);
+                    atomicExch(&g.stt->info[IN_DONE], 1);
+                }
+            }
+        }
+        ++epoch;
+        __syncthreads();
+        return go != 0;
+    };
     // column 0 and its norm
     {
         double ss = 0.0;
@@ -475,15 +559,40 @@ __global__ void __launch_bounds__(BD_T) k_bidiag(BidiagArgs g) {
             if (i > 0) ss = fma(v, v, ss);
         }
         ss = block_sum1<BD_W>(ss, pd);
-        if (threadIdx.x == 0) g.part[2 * G + cta] = ss;
         for (int64_t i = threadIdx.x; i < n; i += BD_T) uo[i] = 0.0;
-        if (!grid_reduce_sync(g.stt, g.bar, g.group, g.budget, ++epoch, nullptr, nullptr, nullptr, 0, 0)) return;
+        __syncthreads();
+        if (warp == 0) {
+            bd_fence();
+            publish(2, ss);
+        }
     }
     double vscale = 0.0;  // 1 once a right reflector is pending
     for (int64_t k = 0; k < n; ++k) {
+        // the columns of pass A and the values they need were written by this CTA:
+        // the first piece is loaded ahead of the barrier
+        const int64_t j0 = k + 1 + (((int64_t)cta - (k + 1)) % G + G) % G;  // first own column past k
+        const int nc = j0 <= n ? (int)((n - j0) / G) + 1 : 0;
+        const int64_t base = k & ~(int64_t)31;
+        const int np = (int)((n - base + BD_ROWS - 1) / BD_ROWS);
+        double v[8], yj = 0.0, vj = 0.0;
+        auto load = [&](int u, double* v, double* yj, double* vj) {
+            const int c = u / np, piece = u - c * np;
+            const int64_t j = j0 + (int64_t)c * G;
+            const double* col = W + j * ld;
+            const int64_t i0 = base + (int64_t)piece * BD_ROWS + lane;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int64_t i = i0 + 32 * q;
+                v[q] = i >= k && i < n ? __ldcg(col + i) : 0.0;
+            }
+            *yj = k > 0 ? __ldcg(g.y + j) : 0.0;
+            *vj = j < n && vscale != 0.0 ? __ldcg(g.r + j) : 0.0;
+        };
+        if (warp < nc * np) load(warp, v, &yj, &vj);
+        if (!collect(std::false_type{})) return;
         // ---- left reflector of column k
         if (warp == 0) {
-            const Refl h = reflector(__ldcg(g.a + k), bd_sum(g.part + 2 * G, G, lane));
+            const Refl h = reflector(__ldcg(g.a + k), sums[0]);
             if (lane == 0) {
                 sc[0] = h.t;
                 sc[1] = h.w0;
@@ -501,23 +610,13 @@ __global__ void __launch_bounds__(BD_T) k_bidiag(BidiagArgs g) {
         __syncthreads();
         const double t1 = sc[0], uk = sc[1], xk = sc[2];
         // ---- pass A
-        const int64_t j0 = k + 1 + (((int64_t)cta - (k + 1)) % G + G) % G;  // first own column past k
-        const int nc = j0 <= n ? (int)((n - j0) / G) + 1 : 0;
-        const int64_t base = k & ~(int64_t)31;
-        const int np = (int)((n - base + BD_ROWS - 1) / BD_ROWS);
         for (int u = warp; u < nc * np; u += BD_W) {
             const int c = u / np, piece = u - c * np;
             const int64_t j = j0 + (int64_t)c * G;
             double* col = W + j * ld;
-            const double yj = k > 0 ? __ldcg(g.y + j) : 0.0;
-            const double vj = j < n && vscale != 0.0 ? __ldcg(g.r + j) : 0.0;
             const int64_t i0 = base + (int64_t)piece * BD_ROWS + lane;
-            double v[8], dot = 0.0, dot1 = 0.0;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const int64_t i = i0 + 32 * q;
-                v[q] = i >= k && i < n ? __ldcg(col + i) : 0.0;
-            }
+            double vn[8], yn = 0.0, rn = 0.0, dot = 0.0, dot1 = 0.0;
+            if (u + BD_W < nc * np) load(u + BD_W, vn, &yn, &rn);  // the next piece while this one is updated
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
                 const int64_t i = i0 + 32 * q;
@@ -534,11 +633,15 @@ __global__ void __launch_bounds__(BD_T) k_bidiag(BidiagArgs g) {
             }
             dot = warp_sum(dot + dot1);
             if (lane == 0) pd[(int64_t)c * pmax + piece] = dot;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[q] = vn[q];
+            yj = yn;
+            vj = rn;
         }
         __syncthreads();
-        if (warp < 2) {
+        if (warp == 0) {
             double rr = 0.0, yr = 0.0;
-            for (int c = threadIdx.x; c < nc; c += 64) {
+            for (int c = lane; c < nc; c += 32) {
                 const int64_t j = j0 + (int64_t)c * G;
                 double d = 0.0;
                 for (int q = 0; q < np; ++q) d += pd[(int64_t)c * pmax + q];
@@ -554,33 +657,42 @@ __global__ void __launch_bounds__(BD_T) k_bidiag(BidiagArgs g) {
             }
             rr = warp_sum(rr);
             yr = warp_sum(yr);
-            if (lane == 0) {
-                rp[2 * warp] = rr;
-                rp[2 * warp + 1] = yr;
+            __syncwarp();
+            if (k < n - 1) {  // (the other warps' stores came before the barrier above)
+                bd_fence();
+                publish(0, rr);
+                publish(1, yr);
             }
         }
         if (k == n - 1) break;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            g.part[cta] = rp[0] + rp[2];
-            g.part[G + cta] = rp[1] + rp[3];
+        if (!collect(std::true_type{})) return;
+        // the first entries of pass B, ahead of the reflector
+        const int64_t rbase = (k + 1) & ~(int64_t)(BD_RB - 1);
+        const int64_t nblk = (n - rbase + BD_RB - 1) / BD_RB;
+        const int rl = lane & (BD_RB - 1), cl = lane / BD_RB;
+        constexpr int CPW = 32 / BD_RB, CW = BD_W * CPW;  // columns of a warp step, of a CTA step
+        const int64_t jb = k + 1 + warp * CPW + cl;
+        double first[4];
+        {
+            const int64_t i = rbase + (int64_t)cta * BD_RB + rl;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                first[q] = cta < nblk && i > k && i < n && jb + q * CW < n ? __ldcg(W + i + (jb + q * CW) * ld) : 0.0;
         }
-        if (!grid_reduce_sync(g.stt, g.bar, g.group, g.budget, ++epoch, nullptr, nullptr, nullptr, 0, 0)) return;
         // ---- right reflector of row k
         if (warp == 0) {
-            const double ss = bd_sum(g.part, G, lane), yr = bd_sum(g.part + G, G, lane);
             const double x0 = __ldcg(g.r + k + 1);
-            const Refl h = reflector(x0, ss);
+            const Refl h = reflector(x0, sums[0]);
             if (lane == 0) {
                 sc[0] = h.t;
-                sc[1] = fma(__ldcg(g.y + k + 1), h.w0, yr);  // y'^T v'
+                sc[1] = fma(__ldcg(g.y + k + 1), h.w0, sums[1]);  // y'^T v'
                 xs[k + 1] = h.w0;
                 sc[2] = __ldcg(g.y + k + 1);
                 sc[3] = h.w0;
                 if (cta == 0) {
                     g.eg[k] = h.beta;
-                    g.taur[k] = h.t * h.w0 * h.w0;
-                    g.scaler[k] = h.t != 0.0 ? 1.0 / h.w0 : 0.0;
+                    g.taur[k] = h.t;  // (k_bidiag_ab turns the two into tau and 1 / w_0)
+                    g.scaler[k] = h.w0;
                 }
             }
         }
@@ -588,10 +700,6 @@ __global__ void __launch_bounds__(BD_T) k_bidiag(BidiagArgs g) {
         __syncthreads();
         const double t2 = sc[0], yv = sc[1], y1 = sc[2], v1 = sc[3];
         // ---- pass B
-        const int64_t rbase = (k + 1) & ~(int64_t)(BD_RB - 1);
-        const int64_t nblk = (n - rbase + BD_RB - 1) / BD_RB;
-        const int rl = lane & (BD_RB - 1), cl = lane / BD_RB;
-        constexpr int CPW = 32 / BD_RB, CW = BD_W * CPW;  // columns of a warp step, of a CTA step
         int nb = 0;
         for (int64_t rb = cta; rb < nblk; rb += G, ++nb) {
             const int64_t i = rbase + rb * BD_RB + rl;
@@ -599,7 +707,14 @@ __global__ void __launch_bounds__(BD_T) k_bidiag(BidiagArgs g) {
             double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
             if (ok) {
                 const double* p = W + i;
-                int64_t j = k + 1 + warp * CPW + cl;
+                int64_t j = jb;
+                if (nb == 0) {
+                    if (j < n) a0 = first[0] * xs[j];
+                    if (j + CW < n) a1 = first[1] * xs[j + CW];
+                    if (j + 2 * CW < n) a2 = first[2] * xs[j + 2 * CW];
+                    if (j + 3 * CW < n) a3 = first[3] * xs[j + 3 * CW];
+                    j += 4 * CW;
+                }
                 for (; j + 3 * CW < n; j += 4 * CW) {
                     const double s0 = __ldcg(p + j * ld), s1 = __ldcg(p + (j + CW) * ld);
                     const double s2 = __ldcg(p + (j + 2 * CW) * ld), s3 = __ldcg(p + (j + 3 * CW) * ld);
@@ -617,7 +732,7 @@ __global__ void __launch_bounds__(BD_T) k_bidiag(BidiagArgs g) {
         }
         __syncthreads();
         double ss = 0.0;
-        for (int e = threadIdx.x; e < nb * BD_RB; e += BD_T) {
+        for (int e = threadIdx.x; warp == 0 && e < nb * BD_RB; e += 32) {
             const int q = e / BD_RB, rr = e - q * BD_RB;
             const int64_t i = rbase + ((int64_t)cta + (int64_t)q * G) * BD_RB + rr;
             if (i <= k || i >= n) continue;
@@ -633,18 +748,12 @@ __global__ void __launch_bounds__(BD_T) k_bidiag(BidiagArgs g) {
             g.a[i] = ai;
             if (i > k + 1) ss = fma(ai, ai, ss);
         }
-        const int nw = min(BD_W, (nb * BD_RB + 31) / 32);  // warps that hold rows
-        if (warp < nw) {
+        if (warp == 0) {
             ss = warp_sum(ss);
-            if (lane == 0) pd[warp] = ss;
+            __syncwarp();
+            bd_fence();
+            publish(2, ss);
         }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double t = 0.0;
-            for (int w = 0; w < nw; ++w) t += pd[w];
-            g.part[2 * G + cta] = t;
-        }
-        if (!grid_reduce_sync(g.stt, g.bar, g.group, g.budget, ++epoch, nullptr, nullptr, nullptr, 0, 0)) return;
         double* t = uo;
         uo = un;
         un = t;
@@ -653,10 +762,17 @@ __global__ void __launch_bounds__(BD_T) k_bidiag(BidiagArgs g) {
 }
 
 // alpha / beta of C = [B^T; 0] for the tridiagonal SVD: alpha = dg, beta =
-// (1, eg, 0); beta_1 only scales f~, which is not used here.
+// (1, eg, 0); beta_1 only scales f~, which is not used here.  The right
+// reflectors (t, w_0) become (t w_0^2, 1 / w_0): I - tau w' w'^T with w'_0 = 1.
 __global__ void k_bidiag_ab(const double* __restrict__ dg, const double* __restrict__ eg, int64_t n,
-                            double* __restrict__ alpha, double* __restrict__ beta) {
+                            double* __restrict__ alpha, double* __restrict__ beta, double* __restrict__ taur,
+                            double* __restrict__ scaler) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n - 1) {
+        const double t = taur[i], w0 = scaler[i];
+        taur[i] = t * w0 * w0;
+        scaler[i] = t != 0.0 ? 1.0 / w0 : 0.0;
+    }
     if (i < n) alpha[i] = dg[i];
     if (i <= n) beta[i] = i == 0 ? 1.0 : (i < n ? eg[i - 1] : 0.0);
 }
@@ -982,9 +1098,9 @@ rbf_status fsvd_bidiag(rbf_ctx* ctx, const rbf_operator* op, const double* f, Fs
     const size_t need = ws_align((size_t)F->ldw * (n + 1) * 8) + ws_align((size_t)n * n * 8) +
                         ws_align((size_t)(n + 1) * n * 8) + 14 * ws_align((size_t)(n + 2) * 8) +
                         ws_align((size_t)(J > n ? J : n) * 8) + ws_align(8) + ws_align(4) +
-                        ws_align((size_t)3 * G * 8) + ws_align((size_t)3 * QB * G * 8) +
+                        ws_align((size_t)3 * G * G * sizeof(ulonglong2)) + ws_align((size_t)3 * QB * G * 8) +
                         ws_align((size_t)(qchunk + 1) * qblk * QB * QB * 8) + ws_align((size_t)2 * QB * G * 8) +
-                        2 * ws_align((size_t)(F->bar_k + 2) * BAR_STRIDE * 4) + svd_ws_bytes(L) + 4096;
+                        ws_align((size_t)(F->bar_k + 2) * BAR_STRIDE * 4) + svd_ws_bytes(L) + 4096;
     RBF_TRY(rbf_ws_reserve(ctx, need));
     WsCarve wc(ctx->ws);
     F->tgk = true;
@@ -1008,17 +1124,16 @@ rbf_status fsvd_bidiag(rbf_ctx* ctx, const rbf_operator* op, const double* f, Fs
     F->curve = wc.take<double>((size_t)(J > n ? J : n));
     F->sperp = wc.take<double>(1);
     F->r = wc.take<int>(1);
-    double* part = wc.take<double>((size_t)3 * G);
+    ulonglong2* slot = wc.take<ulonglong2>((size_t)3 * G * G);
     F->hpart = wc.take<double>((size_t)QB * G);
     F->gpart = wc.take<double>((size_t)2 * QB * G);
     F->gram_part = wc.take<double>((size_t)qchunk * qblk * QB * QB);
     F->gram = wc.take<double>((size_t)qblk * QB * QB);
-    unsigned* bar = wc.take<unsigned>((size_t)(F->bar_k + 2) * BAR_STRIDE);
     F->bar = wc.take<unsigned>((size_t)(F->bar_k + 2) * BAR_STRIDE);
     void* svd = (void*)wc.take<char>(svd_ws_bytes(L));
     cudaStream_t s = ctx->stream;
     const size_t bar_bytes = (size_t)(F->bar_k + 2) * BAR_STRIDE * sizeof(unsigned);
-    RBF_CUDA(ctx, cudaMemsetAsync(bar, 0, bar_bytes, s));
+    RBF_CUDA(ctx, cudaMemsetAsync(slot, 0, (size_t)3 * G * G * sizeof(ulonglong2), s));
     RBF_CUDA(ctx, cudaMemsetAsync(F->bar, 0, bar_bytes, s));
     RBF_CUDA(ctx, cudaMemsetAsync(&ctx->d_state->info[IN_ERR], 0, 2 * sizeof(int), s));
     RBF_CUDA(ctx, cudaMemsetAsync(F->taur, 0, sizeof(double) * (n + 2), s));
@@ -1031,7 +1146,7 @@ rbf_status fsvd_bidiag(rbf_ctx* ctx, const rbf_operator* op, const double* f, Fs
     else RBF_CUDA(ctx, cudaMemsetAsync(g, 0, sizeof(double) * n, s));
     {
         BidiagArgs a{F->Wb, n,      F->ldw, dg,     eg,   F->taur,      F->scaler, vec[0], vec[1],
-                     vec[2], vec[3], part,   ctx->d_state, bar, F->group, ctx->opt.wait_budget};
+                     vec[2], vec[3], slot,   ctx->d_state, ctx->opt.wait_budget};
         void* args[] = {&a};
         RBF_CUDA(ctx, cudaLaunchCooperativeKernel((const void*)k_bidiag, dim3(G), dim3(BD_T), args, smem, s));
         ctx->launches++;
@@ -1040,7 +1155,7 @@ rbf_status fsvd_bidiag(rbf_ctx* ctx, const rbf_operator* op, const double* f, Fs
     RBF_CUDA(ctx, cudaMemcpyAsync(&err, &ctx->d_state->info[IN_ERR], sizeof(int), cudaMemcpyDeviceToHost, s));
     RBF_CUDA(ctx, cudaStreamSynchronize(s));
     if (err) return rbf_fail(ctx, (rbf_status)err, "a bounded grid barrier of the bidiagonalization gave up");
-    k_bidiag_ab<<<(unsigned)((n + 256) / 256), 256, 0, s>>>(dg, eg, n, alpha, beta);
+    k_bidiag_ab<<<(unsigned)((n + 256) / 256), 256, 0, s>>>(dg, eg, n, alpha, beta, F->taur, F->scaler);
     RBF_LAUNCHED(ctx, "k_bidiag_ab");
     ProjDims dd{1, L, L, nullptr};
     RBF_TRY(launch_projected_svd_batch(ctx, dd, alpha, beta, F->sig, ftil, F->Vt, n, svd, nullptr, nullptr, F->Ut,
