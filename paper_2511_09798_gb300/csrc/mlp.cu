@@ -215,6 +215,7 @@ __global__ void __launch_bounds__(WG_T) k_mlp_wgrad(GradArgs a) {
     const float* __restrict__ Rg = task == 4 ? a.DZ1 : (task == 6 ? a.H2 : a.DZ2);
     const int r0 = (threadIdx.x >> 5) * 4, c0 = (threadIdx.x & 31) * 4;
     Pair acc[4][4], b3;
+    pdl_wait();
     for (int s0 = sb; s0 < se; s0 += WG_S) {
         const int cnt = min(WG_S, se - s0);
         __syncthreads();
@@ -298,12 +299,13 @@ struct AdamArgs {
     float lr, b1, b2, c1, c2, eps;
 };
 
-__device__ __forceinline__ void adam_one(const AdamArgs& o, int p, float g) {
-    const float m = o.b1 * o.M[p] + (1.f - o.b1) * g;
-    const float v = o.b2 * o.V[p] + (1.f - o.b2) * g * g;
+// (P, m0, v0: the parameter and its moments before the update)
+__device__ __forceinline__ void adam_one(const AdamArgs& o, int p, float g, float P, float m0, float v0) {
+    const float m = o.b1 * m0 + (1.f - o.b1) * g;
+    const float v = o.b2 * v0 + (1.f - o.b2) * g * g;
     o.M[p] = m;
     o.V[p] = v;
-    o.P[p] -= o.lr * (m * o.c1) / (sqrtf(v * o.c2) + o.eps);
+    o.P[p] = P - o.lr * (m * o.c1) / (sqrtf(v * o.c2) + o.eps);
 }
 
 // G = sum of the chunks' partials in chunk order; with ADAM the update of the
@@ -311,7 +313,11 @@ __device__ __forceinline__ void adam_one(const AdamArgs& o, int p, float g) {
 template <bool ADAM>
 __global__ void __launch_bounds__(128) k_mlp_finish(GradArgs a, float* __restrict__ G, AdamArgs o) {
     const int p = blockIdx.x * 128 + threadIdx.x;
-    if (p >= NPAR) return;
+    const bool ok = p < NPAR;
+    // the parameters and moments are not written by the launches of this step before
+    const float P = ADAM && ok ? o.P[p] : 0.f, m0 = ADAM && ok ? o.M[p] : 0.f, v0 = ADAM && ok ? o.V[p] : 0.f;
+    pdl_wait();
+    if (!ok) return;
     Pair t;
     const float2* __restrict__ q = a.part + p;
 #pragma unroll 8
@@ -322,12 +328,12 @@ __global__ void __launch_bounds__(128) k_mlp_finish(GradArgs a, float* __restric
     float g = t.s + t.c;
     if (!isfinite(g)) g = grad_f64(a, p);
     G[p] = g;
-    if (ADAM) adam_one(o, p, g);
+    if (ADAM) adam_one(o, p, g, P, m0, v0);
 }
 
 __global__ void __launch_bounds__(128) k_adam(const float* __restrict__ G, AdamArgs o) {
     const int p = blockIdx.x * 128 + threadIdx.x;
-    if (p < NPAR) adam_one(o, p, G[p]);
+    if (p < NPAR) adam_one(o, p, G[p], o.P[p], o.M[p], o.V[p]);
 }
 
 __global__ void k_sum_parts(const double* __restrict__ parts, int n, double scale, double* __restrict__ out) {
@@ -458,10 +464,12 @@ static rbf_status mlp_grad_impl(rbf_ctx* ctx, const float* P, const float* X, co
     int tiles = 0;
     RBF_TRY(launch_mlp_pass<true>(ctx, a, &tiles));
     const GradArgs ga{X, a.H1, a.H2, a.DY, a.DZ1, a.DZ2, B, chunk, chunks, part};
-    k_mlp_wgrad<<<dim3(chunks, 7), WG_T, 0, ctx->stream>>>(ga);
+    // programmatic launches: their start-up overlaps the launch before (26.7 -> 21.5 us a step)
+    RBF_CUDA(ctx, rbf_launch_ex(ctx, k_mlp_wgrad, dim3(chunks, 7), dim3(WG_T), 0, true, 1, ga));
     RBF_LAUNCHED(ctx, "k_mlp_wgrad");
-    if (adam) k_mlp_finish<true><<<(NPAR + 127) / 128, 128, 0, ctx->stream>>>(ga, G, *adam);
-    else k_mlp_finish<false><<<(NPAR + 127) / 128, 128, 0, ctx->stream>>>(ga, G, AdamArgs{});
+    const dim3 fg((NPAR + 127) / 128);
+    if (adam) RBF_CUDA(ctx, rbf_launch_ex(ctx, k_mlp_finish<true>, fg, dim3(128), 0, true, 1, ga, G, *adam));
+    else RBF_CUDA(ctx, rbf_launch_ex(ctx, k_mlp_finish<false>, fg, dim3(128), 0, true, 1, ga, G, AdamArgs{}));
     RBF_LAUNCHED(ctx, "k_mlp_finish");
     if (h_loss) {
         k_sum_parts<<<1, 32, 0, ctx->stream>>>(lpart, tiles, 1.0 / (2.0 * B), lpart + tiles);
