@@ -31,26 +31,33 @@ __global__ void k_replicate(const double* __restrict__ alpha, const double* __re
     }
 }
 
-constexpr int ET_Q = 8, ET_T = 256;
+// The error table in two launches, so that the work of an l is spread over the
+// SMs by lambda and by points, the largest l first when they ascend.  One CTA per
+// l and 8 lambdas took 301 us for 15 values of l up to 150 and 500 points, the
+// largest l on 11 SMs; now 58 + 165 us (the FMAs alone: 93 us of the FP64 pipe).
+//   k_err_coef  y = V~ diag(s~ f~ / (s~^2 + lambda^2)) for YQ lambdas of an l
+//   k_err_table max_t |G_l y - uref| / max |uref| for EQ lambdas and ET points,
+//               merged over the point tiles by an integer maximum of the bits
+//               (non-negative doubles order like their bits)
+constexpr int YQ = 4, YT = 256;
+constexpr int EQ = 8, ET = 128;
 
-__global__ void __launch_bounds__(ET_T) k_err_table(const int* __restrict__ ells, int L,
-                                                    const double* __restrict__ sigma_all,
-                                                    const double* __restrict__ ftil_all,
-                                                    const double* __restrict__ V_all, const double* __restrict__ G,
-                                                    int64_t ldg, int64_t m, const double* __restrict__ uref, int J,
-                                                    double t_lo, double t_hi, int tstride, int Jp,
-                                                    double* __restrict__ err) {
-    extern __shared__ double sm[];
-    __shared__ double red[ET_T / 32][ET_Q + 1];
-    const int e = blockIdx.y;
+__global__ void __launch_bounds__(YT) k_err_coef(const int* __restrict__ ells, int L,
+                                                 const double* __restrict__ sigma_all,
+                                                 const double* __restrict__ ftil_all,
+                                                 const double* __restrict__ V_all, int64_t m,
+                                                 const double* __restrict__ uref, int J, double t_lo, double t_hi,
+                                                 int tstride, int Jp, double* __restrict__ y_all,
+                                                 double* __restrict__ umax, double* __restrict__ err) {
+    extern __shared__ double cv[];  // [YQ][L]
+    __shared__ double red[YT / 32];
+    const int e = gridDim.y - 1 - blockIdx.y, q0 = blockIdx.x * YQ;
     const int l = ells[e];
     const double* sigma = sigma_all + (size_t)e * L;
     const double* ftil = ftil_all + (size_t)e * (L + 1);
     const double* V = V_all + (size_t)e * L * L;
-    const int q0 = blockIdx.x * ET_Q;
-    double* cv = sm;
-    double* y = sm + ET_Q * L;
-    for (int idx = threadIdx.x; idx < ET_Q * l; idx += ET_T) {
+    if (threadIdx.x < YQ && q0 + (int)threadIdx.x < Jp) err[(size_t)e * Jp + q0 + threadIdx.x] = 0.0;
+    for (int idx = threadIdx.x; idx < YQ * l; idx += YT) {
         const int q = idx / l, i = idx - q * l;
         double v = 0.0;
         if (q0 + q < Jp) {
@@ -61,47 +68,78 @@ __global__ void __launch_bounds__(ET_T) k_err_table(const int* __restrict__ ells
         cv[q * L + i] = v;
     }
     __syncthreads();
-    for (int idx = threadIdx.x; idx < ET_Q * l; idx += ET_T) {
+    for (int r = threadIdx.x; r < l; r += YT) {
+        double acc[YQ];
+#pragma unroll
+        for (int q = 0; q < YQ; ++q) acc[q] = 0.0;
+#pragma unroll 8
+        for (int i = 0; i < l; ++i) {
+            const double v = V[(int64_t)i * L + r];
+#pragma unroll
+            for (int q = 0; q < YQ; ++q) acc[q] = fma(v, cv[q * L + i], acc[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < YQ; ++q)
+            if (q0 + q < Jp) y_all[((size_t)e * Jp + q0 + q) * L + r] = acc[q];
+    }
+    if (blockIdx.x != 0 || blockIdx.y != 0) return;
+    double u = 0.0;
+    for (int64_t t = threadIdx.x; t < m; t += YT) u = fmax(u, fabs(uref[t]));
+    for (int o = 16; o > 0; o >>= 1) u = fmax(u, __shfl_xor_sync(RBF_FULL_MASK, u, o));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = u;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 0; w < YT / 32; ++w) u = fmax(u, red[w]);
+        *umax = u;
+    }
+}
+
+__global__ void __launch_bounds__(ET) k_err_table(const int* __restrict__ ells, int L, const double* __restrict__ y_all,
+                                                  const double* __restrict__ umax, const double* __restrict__ G,
+                                                  int64_t ldg, int64_t m, const double* __restrict__ uref, int Jp,
+                                                  double* __restrict__ err) {
+    extern __shared__ double y[];  // [l][EQ]
+    __shared__ double red[ET / 32][EQ];
+    const int e = gridDim.y - 1 - blockIdx.y, q0 = blockIdx.x * EQ;
+    const int l = ells[e];
+    for (int idx = threadIdx.x; idx < EQ * l; idx += ET) {
         const int q = idx / l, r = idx - q * l;
-        double acc = 0.0;
-        for (int i = 0; i < l; ++i) acc = fma(V[(int64_t)i * L + r], cv[q * L + i], acc);
-        y[q * L + r] = acc;
+        y[r * EQ + q] = q0 + q < Jp ? y_all[((size_t)e * Jp + q0 + q) * L + r] : 0.0;
     }
     __syncthreads();
-    double mx[ET_Q];
+    double mx[EQ];
 #pragma unroll
-    for (int q = 0; q < ET_Q; ++q) mx[q] = 0.0;
-    double umax = 0.0;
-    for (int64_t t = threadIdx.x; t < m; t += ET_T) {
-        double acc[ET_Q];
+    for (int q = 0; q < EQ; ++q) mx[q] = 0.0;
+    // uref all zero: 0/0 of one tile must not hide x/0 of another, so one CTA takes all tiles
+    const bool flat = *umax == 0.0;
+    if (flat && blockIdx.z != 0) return;
+    const int64_t step = (flat ? 1 : (int64_t)gridDim.z) * ET;
+    for (int64_t t = (int64_t)blockIdx.z * ET + threadIdx.x; t < m; t += step) {
+        double acc[EQ];
 #pragma unroll
-        for (int q = 0; q < ET_Q; ++q) acc[q] = 0.0;
+        for (int q = 0; q < EQ; ++q) acc[q] = 0.0;
+#pragma unroll 4
         for (int r = 0; r < l; ++r) {
             const double g = G[(int64_t)r * ldg + t];
 #pragma unroll
-            for (int q = 0; q < ET_Q; ++q) acc[q] = fma(g, y[q * L + r], acc[q]);
+            for (int q = 0; q < EQ; ++q) acc[q] = fma(g, y[r * EQ + q], acc[q]);
         }
         const double ur = uref[t];
-        umax = fmax(umax, fabs(ur));
 #pragma unroll
-        for (int q = 0; q < ET_Q; ++q) mx[q] = fmax(mx[q], fabs(acc[q] - ur));
+        for (int q = 0; q < EQ; ++q) mx[q] = fmax(mx[q], fabs(acc[q] - ur));
     }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
-    for (int q = 0; q <= ET_Q; ++q) {
-        double v = q < ET_Q ? mx[q] : umax;
-        for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(RBF_FULL_MASK, v, o));
-        if (lane == 0) red[warp][q] = v;
+    for (int q = 0; q < EQ; ++q) {
+        for (int o = 16; o > 0; o >>= 1) mx[q] = fmax(mx[q], __shfl_xor_sync(RBF_FULL_MASK, mx[q], o));
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][q] = mx[q];
     }
     __syncthreads();
-    if (threadIdx.x <= ET_Q) {
+    if (threadIdx.x < EQ && q0 + (int)threadIdx.x < Jp) {
         double v = 0.0;
-        for (int w = 0; w < ET_T / 32; ++w) v = fmax(v, red[w][threadIdx.x]);
-        red[0][threadIdx.x] = v;
+        for (int w = 0; w < ET / 32; ++w) v = fmax(v, red[w][threadIdx.x]);
+        atomicMax((unsigned long long*)(err + (size_t)e * Jp + q0 + threadIdx.x),
+                  (unsigned long long)__double_as_longlong(v / *umax));
     }
-    __syncthreads();
-    if (threadIdx.x < ET_Q && q0 + (int)threadIdx.x < Jp)
-        err[(size_t)e * Jp + q0 + threadIdx.x] = red[0][threadIdx.x] / red[0][ET_Q];
 }
 
 }  // namespace
@@ -123,7 +161,8 @@ extern "C" rbf_status rbf_hkt_error_table(rbf_ctx* ctx, const rbf_gkb_state* st,
     const int Jp = (J - 1) / t_stride + 1;
     const size_t B = (size_t)n_ell;
     const size_t need = ws_align(B * 4) + ws_align(B * L * 8) + 2 * ws_align(B * (L + 1) * 8) +
-                        ws_align(B * L * 8) + ws_align(B * L * L * 8) + svd_ws_bytes_batch(L, n_ell);
+                        ws_align(B * L * 8) + ws_align(B * L * L * 8) + ws_align(B * Jp * L * 8) + ws_align(8) +
+                        svd_ws_bytes_batch(L, n_ell);
     RBF_TRY(rbf_ws_reserve(ctx, need));
     WsCarve wc(ctx->ws);
     int* d_ells = wc.take<int>(B);
@@ -132,18 +171,25 @@ extern "C" rbf_status rbf_hkt_error_table(rbf_ctx* ctx, const rbf_gkb_state* st,
     double* ftil = wc.take<double>(B * (L + 1));
     double* sigma = wc.take<double>(B * L);
     double* V = wc.take<double>(B * L * L);
+    double* y = wc.take<double>(B * Jp * L);
+    double* umax = wc.take<double>(1);
     void* svd = (void*)wc.take<char>(svd_ws_bytes_batch(L, n_ell));
     RBF_CUDA(ctx, cudaMemcpyAsync(d_ells, h_ells, B * 4, cudaMemcpyHostToDevice, ctx->stream));
     k_replicate<<<n_ell, 256, 0, ctx->stream>>>(st->d_alpha, st->d_beta, L, a_rep, b_rep);
     RBF_LAUNCHED(ctx, "k_replicate");
     ProjDims d{n_ell, L, 0, d_ells};
     RBF_TRY(launch_projected_svd_batch(ctx, d, a_rep, b_rep, sigma, ftil, V, L, svd, nullptr, nullptr));
-    const size_t smem = (size_t)2 * ET_Q * L * 8;
-    if (smem > SMEM_PLAIN)
-        RBF_CUDA(ctx, cudaFuncSetAttribute(k_err_table, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_err_table<<<dim3((unsigned)((Jp + ET_Q - 1) / ET_Q), (unsigned)n_ell), ET_T, smem, ctx->stream>>>(
-        d_ells, L, sigma, ftil, V, d_G, ldg, m, d_uref, J, ctx->opt.grid_t_lo, ctx->opt.grid_t_hi, t_stride, Jp,
-        d_err);
+    const size_t smem_y = (size_t)YQ * L * 8, smem_e = (size_t)EQ * L * 8;
+    if (smem_y > SMEM_PLAIN)
+        RBF_CUDA(ctx, cudaFuncSetAttribute(k_err_coef, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_y));
+    if (smem_e > SMEM_PLAIN)
+        RBF_CUDA(ctx, cudaFuncSetAttribute(k_err_table, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_e));
+    k_err_coef<<<dim3((unsigned)((Jp + YQ - 1) / YQ), (unsigned)n_ell), YT, smem_y, ctx->stream>>>(
+        d_ells, L, sigma, ftil, V, m, d_uref, J, ctx->opt.grid_t_lo, ctx->opt.grid_t_hi, t_stride, Jp, y, umax, d_err);
+    RBF_LAUNCHED(ctx, "k_err_coef");
+    const int64_t zt = (m + ET - 1) / ET;
+    k_err_table<<<dim3((unsigned)((Jp + EQ - 1) / EQ), (unsigned)n_ell, (unsigned)(zt < 64 ? zt : 64)), ET, smem_e,
+                  ctx->stream>>>(d_ells, L, y, umax, d_G, ldg, m, d_uref, Jp, d_err);
     RBF_LAUNCHED(ctx, "k_err_table");
     // the host array of l values must outlive the copy
     RBF_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
