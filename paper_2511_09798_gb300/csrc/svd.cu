@@ -508,43 +508,39 @@ __global__ void __launch_bounds__(VEC_WARPS * 32)
 // Clusters of close singular values: inverse iteration (3 steps) with the
 // stored LDL^T factors of T - s_a I, all members in parallel lanes, then
 // modified Gram-Schmidt in order.  One block per instance, one warp per cluster.
-constexpr int CL_WARPS = 8;
+constexpr int CL_WARPS = 4;  // one per FP64 unit of an SM
 constexpr int CL_MAX = 32;
 constexpr int CL_BLK = 8;  // steps of a triangular solve whose operands are loaded together
 
 // One lane: v[k] += -f[k - 1] v[k - 1] for k = 1 .. nt - 1 (forward), or
-// v[k] += -f[k] v[k + 1] for k = nt - 2 .. 0 (backward).
-__device__ __forceinline__ void solve_fwd(double* v, const double* f, int nt) {
-    double c = v[0];
-    int k = 1;
-    for (; k + CL_BLK <= nt; k += CL_BLK) {
-        double a[CL_BLK], y[CL_BLK];
+// v[k] += -f[k] v[k + 1] for k = nt - 2 .. 0 (backward).  The operands of a block
+// are loaded while the block before it is in its chain.
+template <int DIR>
+__device__ __forceinline__ void solve_chain(double* v, const double* f, int nt) {
+    double* x = DIR > 0 ? v : v + nt - 1;
+    const double* g = DIR > 0 ? f : f + nt - 2;
+    double c = x[0];
+    double a[2][CL_BLK], y[2][CL_BLK];
+    auto load = [&](int k, double* a, double* y) {
 #pragma unroll
         for (int u = 0; u < CL_BLK; ++u) {
-            a[u] = f[k + u - 1];
-            y[u] = v[k + u];
+            const bool in = k + u < nt;
+            a[u] = in ? g[DIR * (k + u - 1)] : 0.0;
+            y[u] = in ? x[DIR * (k + u)] : 0.0;
         }
+    };
+    auto chain = [&](int k, const double* a, const double* y) {
 #pragma unroll
-        for (int u = 0; u < CL_BLK; ++u) v[k + u] = c = fma(-a[u], c, y[u]);
+        for (int u = 0; u < CL_BLK; ++u)
+            if (k + u < nt) x[DIR * (k + u)] = c = fma(-a[u], c, y[u]);
+    };
+    load(1, a[0], y[0]);
+    for (int k = 1; k < nt; k += 2 * CL_BLK) {
+        load(k + CL_BLK, a[1], y[1]);
+        chain(k, a[0], y[0]);
+        load(k + 2 * CL_BLK, a[0], y[0]);
+        chain(k + CL_BLK, a[1], y[1]);
     }
-    for (; k < nt; ++k) v[k] = c = fma(-f[k - 1], c, v[k]);
-}
-__device__ __forceinline__ void solve_bwd(double* v, const double* f, const double* invd, int nt) {
-    double c = v[nt - 1] * invd[nt - 1];
-    v[nt - 1] = c;
-    int k = nt - 2;
-    for (; k - CL_BLK + 1 >= 0; k -= CL_BLK) {
-        double a[CL_BLK], y[CL_BLK], w[CL_BLK];
-#pragma unroll
-        for (int u = 0; u < CL_BLK; ++u) {
-            a[u] = f[k - u];
-            y[u] = v[k - u];
-            w[u] = invd[k - u];
-        }
-#pragma unroll
-        for (int u = 0; u < CL_BLK; ++u) v[k - u] = c = fma(-a[u], c, y[u] * w[u]);
-    }
-    for (; k >= 0; --k) v[k] = c = fma(-f[k], c, v[k] * invd[k]);
 }
 
 // Grid (B, gy): CTA y takes the clusters of index y CL_WARPS .. y CL_WARPS +
@@ -600,12 +596,14 @@ __global__ void k_tgk_clusters(ProjDims d, const double* __restrict__ sigma_all,
     __syncwarp();
     for (int it = 0; it < 3; ++it) {
         // lane a solves (T - s_a I) x = y_a:  L D L^T with L_{k+1,k} = rp_k
-        if (lane < mcnt) {
-            double* v = y + (size_t)lane * NT;
-            const double* f = rp_all + row0 + (size_t)lane * NT;
-            solve_fwd(v, f, nt);
-            solve_bwd(v, f, invdp_all + row0 + (size_t)lane * NT, nt);
-        }
+        // (a lane's warp instruction takes the FP64 unit as long as a full warp's: the
+        // scaling by the inverse pivots runs over the lanes, not in the chain)
+        if (lane < mcnt) solve_chain<1>(y + (size_t)lane * NT, rp_all + row0 + (size_t)lane * NT, nt);
+        __syncwarp();
+        for (int a = 0; a < mcnt; ++a)
+            for (int k = lane; k < nt; k += 32) y[(size_t)a * NT + k] *= invdp_all[row0 + (size_t)a * NT + k];
+        __syncwarp();
+        if (lane < mcnt) solve_chain<-1>(y + (size_t)lane * NT, rp_all + row0 + (size_t)lane * NT, nt);
         __syncwarp();
         // modified Gram-Schmidt in member order
         for (int a = 0; a < mcnt; ++a) {
