@@ -34,6 +34,7 @@
 namespace {
 
 constexpr int EV_T = 128;           // points per CTA, one per thread; nodes per stage
+constexpr int EV_MIN_CHUNK = 64;     // nodes per CTA
 constexpr int EV_MAX_CHUNK = 1 << 19;  // nodes per CTA: the limb sums stay below 2^63
 constexpr int EX_CTAS = 64;         // partial maxima of the exponent scan
 
@@ -198,7 +199,7 @@ rbf_status evaluate_vectors(rbf_ctx* ctx, const rbf_operator* op, const double* 
     // vectors per CTA: the smallest of 1, 2, 4, 8 that holds them all (8 beyond)
     const int nc = ncoef <= 1 ? 1 : ncoef <= 2 ? 2 : ncoef <= 4 ? 4 : 8;
     const int zs = (ncoef + nc - 1) / nc;
-    // one wave of resident CTAs, chunks of at least 256 nodes (the chains of a
+    // one wave of resident CTAs, chunks of at least 64 nodes (the chains of a
     // pair need all the warps that fit: 8 CTAs per SM 1.79, a full wave 1.70 ms at
     // 20 000 points and nodes)
     const void* kern = nc == 1 ? (const void*)k_evaluate<1> : nc == 2 ? (const void*)k_evaluate<2>
@@ -207,7 +208,7 @@ rbf_status evaluate_vectors(rbf_ctx* ctx, const rbf_operator* op, const double* 
     RBF_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, EV_T, 0));
     int64_t chunks = (int64_t)ctx->sm_count * per_sm / (tiles * zs);
     chunks = chunks < 1 ? 1 : chunks;
-    if ((n + chunks - 1) / chunks < 256) chunks = (n + 255) / 256;
+    if ((n + chunks - 1) / chunks < EV_MIN_CHUNK) chunks = (n + EV_MIN_CHUNK - 1) / EV_MIN_CHUNK;
     if ((n + chunks - 1) / chunks > EV_MAX_CHUNK) chunks = (n + EV_MAX_CHUNK - 1) / EV_MAX_CHUNK;
     if (chunks > 65535) chunks = 65535;
     const int64_t chunk = (n + chunks - 1) / chunks;
