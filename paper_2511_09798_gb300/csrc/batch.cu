@@ -39,7 +39,7 @@ struct BInst {
     int chunks;         // product: partial slots = blocks of the tile-pair product
     int64_t poff;       // product partials offset (chunks * n doubles)
     int cfirst, ncta;   // half-step CTAs whose slabs intersect the instance
-    int64_t hoff;       // dot partials offset ((L+2) * ncta doubles)
+    int64_t hoff;       // dot partials offset ([pass][ncta][L+2] doubles)
     int noff;           // norm partials offset (ncta doubles)
 };
 
@@ -52,6 +52,12 @@ constexpr int DG_LOG = 2;
 constexpr int DG = 1 << DG_LOG;  // basis vectors per warp in the half-step's dot products
 constexpr int HB_WARPS = HB_THREADS / 32;
 constexpr int SEGMAX = 16;       // instances intersecting one slab
+// Instances on at most this many CTAs: every CTA sums the dot partials of its own
+// instances, one barrier per pass.  Beyond, each sum is taken once and passed on
+// across a second barrier: G CTAs that read L partials of G CTAs each would move
+// more through the L2 (118 MB for one instance on 608 CTAs and 40 vectors) than
+// the barrier costs.
+constexpr int HB_DIRECT = 128;
 constexpr int UPD_ROWS_B = 64;
 constexpr int UPD_GROUPS_B = HB_THREADS / UPD_ROWS_B;
 
@@ -150,6 +156,7 @@ struct HalfBArgs {
     int bar_group;
     long long budget;
     int rmax;
+    int direct;              // every CTA sums its instances' partials itself
 };
 
 __global__ void __launch_bounds__(HB_THREADS, 4) k_half_batch(HalfBArgs a) {
@@ -343,27 +350,42 @@ __global__ void __launch_bounds__(HB_THREADS, 4) k_half_batch(HalfBArgs a) {
                 const int m = m0 + ((lane >> (5 - DG_LOG)) & (DG - 1));  // the vector lane holds
                 if ((lane & ((32 >> DG_LOG) - 1)) == 0 && m < M && RBF_IN_RANGE(cslot, I.ncta) &&
                     RBF_IN_RANGE(m, L + 2))
-                    a.hpart_all[I.hoff + (int64_t)m * I.ncta + cslot] = t;
+                    a.hpart_all[I.hoff + ((int64_t)pass * I.ncta + cslot) * (L + 2) + m] = t;
             }
         }
         if (!grid_sync_b(a.stt, a.bar, a.bar_group, a.budget)) return;
-        // distributed reduction over all (instance, m) pairs
-        {
+        // sum of an instance's partials, in the order of its CTAs; 8 loads in flight
+        auto total = [&](const BInst& I, int m) {
+            const double* hp = a.hpart_all + I.hoff + (int64_t)pass * I.ncta * (L + 2) + m;
+            double acc = 0.0;
+            int s = 0;
+            for (; s + 8 <= I.ncta; s += 8) {
+                double t[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) t[u] = __ldcg(hp + (int64_t)(s + u) * (L + 2));
+#pragma unroll
+                for (int u = 0; u < 8; ++u) acc += t[u];
+            }
+            for (; s < I.ncta; ++s) acc += __ldcg(hp + (int64_t)s * (L + 2));
+            return acc;
+        };
+        if (a.direct) {
+            for (int e = threadIdx.x; e < nseg * M; e += HB_THREADS) {
+                const int sx = e / M, m = e - sx * M;
+                if (seg_act[sx]) hs[sx * (L + 2) + m] = total(a.inst[seg_b[sx]], m);
+            }
+        } else {
+            // distributed over all (instance, m) pairs
             const int64_t P = (int64_t)a.B * M;
             for (int64_t p = (int64_t)blockIdx.x * HB_THREADS + threadIdx.x; p < P; p += (int64_t)G * HB_THREADS) {
                 const int b = (int)(p / M), m = (int)(p % M);
-                if (a.done_in[b]) continue;
-                const BInst I = a.inst[b];
-                const double* hp = a.hpart_all + I.hoff + (int64_t)m * I.ncta;
-                double acc = 0.0;
-                for (int s = 0; s < I.ncta; ++s) acc += __ldcg(hp + s);
-                a.h_all[(size_t)b * (L + 2) + m] = acc;
+                if (!a.done_in[b]) a.h_all[(size_t)b * (L + 2) + m] = total(a.inst[b], m);
             }
+            if (!grid_sync_b(a.stt, a.bar, a.bar_group, a.budget)) return;
+            for (int sx = 0; sx < nseg; ++sx)
+                for (int m = threadIdx.x; m < M; m += HB_THREADS)
+                    hs[sx * (L + 2) + m] = __ldcg(a.h_all + (size_t)seg_b[sx] * (L + 2) + m);
         }
-        if (!grid_sync_b(a.stt, a.bar, a.bar_group, a.budget)) return;
-        for (int sx = 0; sx < nseg; ++sx)
-            for (int m = threadIdx.x; m < M; m += HB_THREADS)
-                hs[sx * (L + 2) + m] = __ldcg(a.h_all + (size_t)seg_b[sx] * (L + 2) + m);
         __syncthreads();
         // v -= Q h over the slab rows: thread (row, group of basis vectors)
         const int row = threadIdx.x % UPD_ROWS_B;
@@ -515,7 +537,7 @@ void launch_mf_cand(int c, int items, cudaStream_t s, const MfItem* it, const BI
 
 // Host-side description of one batch shape and its device tables.
 struct BatchPlan {
-    int B = 0, L = 0, G = 0, rmax = 0, bar_group = 0, bar_k = 0;
+    int B = 0, L = 0, G = 0, rmax = 0, bar_group = 0, bar_k = 0, ncta_max = 0;
     int64_t T = 0;
     std::vector<BInst> inst;
     std::vector<int64_t> offs;
@@ -614,6 +636,7 @@ static rbf_status plan_batch(rbf_ctx* ctx, const rbf_batch* bt, int form, BatchP
     P->bar_k = (P->G + P->bar_group - 1) / P->bar_group;
     P->inst.resize(B);
     int64_t poff = 0, hoff = 0;  // (partials: set_blocks)
+    P->ncta_max = 0;
     int noff = 0;
     for (int b = 0; b < B; ++b) {
         BInst& I = P->inst[b];
@@ -634,7 +657,8 @@ static rbf_status plan_batch(rbf_ctx* ctx, const rbf_batch* bt, int form, BatchP
         I.cfirst = c0;
         I.ncta = c1 - c0 + 1;
         I.hoff = hoff;
-        hoff += (int64_t)(P->L + 2) * I.ncta;
+        hoff += 2 * (int64_t)(P->L + 2) * I.ncta;
+        P->ncta_max = std::max(P->ncta_max, I.ncta);
         I.noff = noff;
         noff += I.ncta;
     }
@@ -800,6 +824,7 @@ extern "C" rbf_status rbf_batch_gkb(rbf_ctx* ctx, rbf_batch* bt, int steps, int 
     a.part_all = w.part;
     a.hpart_all = w.hpart;
     a.h_all = w.h;
+    a.direct = P.ncta_max <= HB_DIRECT;
     a.npart_all = w.npart;
     a.binfo = w.binfo;
     a.chat_all = w.chat;
@@ -878,7 +903,7 @@ extern "C" rbf_status rbf_batch_gkb(rbf_ctx* ctx, rbf_batch* bt, int steps, int 
     put(a.inst); put(a.offs); put(a.B); put(a.T); put(a.L); put(a.factor);
     put(a.alpha_all); put(a.beta_all); put(a.W_all); put(a.Z_all); put(a.part_all); put(a.hpart_all);
     put(a.h_all); put(a.npart_all); put(a.binfo); put(a.limit); put(a.chat_all); put(a.stt); put(a.bar);
-    put(a.bar_group); put(a.budget); put(a.rmax);
+    put(a.bar_group); put(a.budget); put(a.rmax); put(a.direct);
     put(bt->d_nodes); put(bt->d_f); put(w.items); put(w.part); put(w.X32); put(w.vr); put(w.vp); put(w.vr32); put(w.vp32);
     put(nit); put(cand); put(P.G); put(hsmem); put(steps); put(form); put(s);
     // per-launch timing (opt.timing bit 1): the loop is launched directly, each
