@@ -18,7 +18,7 @@
 //     2^13): |N - 2^31 sqrt(s)| is under 9 units, 2^-57.8 of the largest Phi and 2^-53 of
 //     the smallest that the rule below admits;
 //   - the coefficients are rounded at 2^-62 of the largest of the CTA's chunk and
-//     the products N coef are added in 64-bit integers (EvAcc), then rounded to
+//     the products N coef are added in 64-bit integers (FxAcc32), then rounded to
 //     FP64 once per chunk.
 // Every error is at most about 2^-58 of the largest Phi times the coefficients,
 // below the roundings of the FP64 form (an ulp or two per term and the sum's), so
@@ -82,44 +82,6 @@ __device__ __forceinline__ long long eval_phi(long long dx, long long dy, long l
     return (R1 << 19) + (b2 - 0x4B400000);
 }
 
-// Sum of products N Z in units of 2^64, N = n1 2^32 + n0 in [0, 2^61), |Z| = |z1
-// 2^32 + z0| < 2^62 (signed 32-bit low parts, so |n1| <= 2^29 and |z1| <= 2^30).
-// n1 z1 goes to c, which holds EV_FOLD terms of at most 2^59 + 2^32 before it is
-// folded; the cross products, below 2^62 together and made positive by EV_BIAS,
-// add their upper word to c and carry their lower word into the next term.  n0 z0
-// (under a quarter of a unit, either sign) is left out: an error of at most n / 4
-// units of 2^-59 of the largest term.  Three wide products per term; 21-bit limbs
-// that accumulate without folds took six, which bound the form for 8 vectors (the
-// pipe of the wide products 63 % busy): 816 -> 608 us for 150 vectors, 8000 nodes and
-// 500 points, 1.70 -> 1.59 ms for one vector and 20 000 nodes and points.  (16
-// vectors per CTA, so that Phi is shared by more: no gain, 12 warps per SM.)
-constexpr int EV_FOLD = 8;
-constexpr unsigned EV_BIAS = 1u << 30;  // in the upper word
-
-struct EvAcc {
-    long long c = 0, hi = 0, lo = 0;  // value c + hi 2^32 + lo
-    unsigned rem = 0;
-    __device__ __forceinline__ void add(int n1, int n0, int z1, int z0) {
-        const long long x =
-            imad_wide(n0, z1, imad_wide(n1, z0, (long long)(((unsigned long long)EV_BIAS << 32) | rem)));
-        rem = (unsigned)x;
-        c = imad_wide(n1, z1, c) + (long long)((unsigned long long)x >> 32);
-    }
-    __device__ __forceinline__ void fold() {
-        hi += c >> 32;
-        lo += (long long)((unsigned long long)c & 0xffffffffu);
-        c = 0;
-    }
-    __device__ __forceinline__ double value(int64_t terms) const {
-        return fma((double)hi, 0x1p32, (double)(lo - terms * (long long)EV_BIAS));
-    }
-};
-
-__device__ __forceinline__ int2 ev_split(long long v) {  // (low, high) with a signed low part
-    const int l = (int)v;
-    return make_int2(l, (int)(v >> 32) - (l >> 31));
-}
-
 // Partials over the centre chunk blockIdx.y for the NC vectors blockIdx.z NC ..:
 // part[chunk][vector][t].
 template <int NC>
@@ -167,7 +129,7 @@ __global__ void __launch_bounds__(EV_T) k_evaluate(const double* __restrict__ X,
         const long long ux = fx_round(px, k), uy = fx_round(py, k), uz = fx_round(pz, k), qc = fx_round(c, k);
         const int lc = (int)qc, hc = (int)(qc >> 32) - (lc >> 31);
         const long long hh0 = imad_wide(hc, hc, 0), hl0 = imad_wide(hc, lc, imad_wide(lc, lc, 0) >> 33);
-        EvAcc acc[NC];
+        FxAcc32 acc[NC];
         for (int64_t jb = j0; jb < j1; jb += EV_T) {
             __syncthreads();
             const int64_t j = jb + threadIdx.x;
@@ -177,16 +139,16 @@ __global__ void __launch_bounds__(EV_T) k_evaluate(const double* __restrict__ X,
             qz[threadIdx.x] = ok ? fx_round(X[2 * n + j], k) : 0;
 #pragma unroll
             for (int q = 0; q < NC; ++q)
-                qa[q][threadIdx.x] = ok && q < nc ? ev_split(fx_round(coefs[(int64_t)(c0 + q) * ldc + j],
+                qa[q][threadIdx.x] = ok && q < nc ? fx_split(fx_round(coefs[(int64_t)(c0 + q) * ldc + j],
                                                                       1084 - max(ev[q], 1)))
                                                   : make_int2(0, 0);
             __syncthreads();
             const int cnt = (int)min((int64_t)EV_T, j1 - jb);
-            for (int rb = 0; rb < cnt; rb += EV_FOLD) {
-                const int re = min(rb + EV_FOLD, cnt);
+            for (int rb = 0; rb < cnt; rb += FX_FOLD) {
+                const int re = min(rb + FX_FOLD, cnt);
 #pragma unroll 2
                 for (int r = rb; r < re; ++r) {
-                    const int2 N = ev_split(eval_phi(ux - qx[r], uy - qy[r], uz - qz[r], hh0, hl0));
+                    const int2 N = fx_split(eval_phi(ux - qx[r], uy - qy[r], uz - qz[r], hh0, hl0));
 #pragma unroll
                     for (int q = 0; q < NC; ++q) {
                         const int2 a = qa[q][r];
@@ -198,7 +160,7 @@ __global__ void __launch_bounds__(EV_T) k_evaluate(const double* __restrict__ X,
             }
         }
 #pragma unroll
-        for (int q = 0; q < NC; ++q) res[q] = ldexp(acc[q].value(j1 - j0), 65 - k - (1084 - max(ev[q], 1)));
+        for (int q = 0; q < NC; ++q) res[q] = ldexp(FxAcc32::value(acc[q].pair(j1 - j0)), 65 - k - (1084 - max(ev[q], 1)));
     } else {
         const double c2 = c * c;
         const bool far = ec < 1023 - 490 || es > 1023 + 490;  // s may leave the normal numbers
@@ -242,7 +204,7 @@ rbf_status evaluate_vectors(rbf_ctx* ctx, const rbf_operator* op, const double* 
     const int nc = ncoef <= 1 ? 1 : ncoef <= 2 ? 2 : ncoef <= 4 ? 4 : 8;
     const int zs = (ncoef + nc - 1) / nc;
     // one wave of resident CTAs, chunks of at least 64 nodes (the chains of a
-    // pair need all the warps that fit: 8 CTAs per SM 1.79, a full wave 1.70 ms at
+    // pair need all the warps that fit: 8 CTAs per SM took 5 % longer than a full wave at
     // 20 000 points and nodes)
     const void* kern = nc == 1 ? (const void*)k_evaluate<1> : nc == 2 ? (const void*)k_evaluate<2>
                        : nc == 4 ? (const void*)k_evaluate<4> : (const void*)k_evaluate<8>;

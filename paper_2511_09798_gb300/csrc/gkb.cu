@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "fx_core.cuh"
 #include "internal.h"
 #include "grid_sync.cuh"
 
@@ -452,9 +453,18 @@ __global__ void __launch_bounds__(SL_THREADS) k_half(HalfArgs a) {
 constexpr int HC_CTAS = 16;
 constexpr int HC_T = 512;
 constexpr int HC_SPLIT = 16;  // most threads per basis vector in the dot products
+// Slabs of Q of at least this many entries: the dot products and updates in
+// 64-bit fixed point (fx_core.cuh) on the integer pipes instead of 2 FP64 FMAs per
+// clock on each of the 16 SMs.  Q is rounded at 2^-61 (its columns have norm 1;
+// below 2^-53 of a typical entry), v and the products h at 2^-61 of their largest; sums are
+// exact to 2^-59 of the largest term.  The conversions and scales cost 2 us per
+// half-step, what about 2800 entries cost in FP64: 1000 rows and up to 40 vectors
+// 14.1 us in FP64, 16.1 in fixed point; 2161 rows and 140 steps, a solve 10.08 -> 9.22 ms.
+// FP64 also where an entry of Q is 2 or more (a caller's own basis).
+constexpr int HC_FX_MIN = 4096;
 
 struct HalfClusterSmem {  // offsets in doubles
-    int q, v, scratch, hp, hs, total;
+    int q, v, scratch, hp, hs, vx, hx, total;
 };
 __host__ __device__ inline HalfClusterSmem half_cluster_smem(int mcount, int rmax) {
     HalfClusterSmem o;
@@ -463,7 +473,9 @@ __host__ __device__ inline HalfClusterSmem half_cluster_smem(int mcount, int rma
     o.scratch = o.v + rmax;
     o.hp = o.scratch + 2 * HC_T;
     o.hs = o.hp + 2 * mcount;
-    o.total = o.hs + mcount;
+    o.vx = o.hs + mcount;
+    o.hx = o.vx + rmax;
+    o.total = o.hx + mcount;
     return o;
 }
 
@@ -471,6 +483,7 @@ __global__ void __launch_bounds__(HC_T) k_half_cluster(HalfArgs a) {
     namespace cg = cooperative_groups;
     extern __shared__ double dsm[];
     __shared__ double red[HC_T / 32];
+    __shared__ int rede[HC_T / 32];
     __shared__ double acc_s;
     __shared__ HalfNorm norm_s;
     cg::cluster_group cluster = cg::this_cluster();
@@ -484,6 +497,10 @@ __global__ void __launch_bounds__(HC_T) k_half_cluster(HalfArgs a) {
     double* sc = dsm + o.scratch;
     double* hp = dsm + o.hp;  // [2][M] this CTA's dot products, by pass
     double* hs = dsm + o.hs;  // [M]
+    int2* Qx = (int2*)Qs;           // fixed-point form: Q at 2^-60, split
+    int2* vx = (int2*)(dsm + o.vx);  // [RM] v, split
+    int2* hx = (int2*)(dsm + o.hx);  // [M] hs, split
+    long long* sch = (long long*)sc;  // [HC_T] high, [HC_T] low parts of partial sums
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // before the wait for the product: everything that the half-step before it
     // left (the basis, q_raw, u, the norm partials, the done flag)
@@ -501,6 +518,19 @@ __global__ void __launch_bounds__(HC_T) k_half_cluster(HalfArgs a) {
             if (!done) norm_s = half_norm<true>(a, acc);
         }
     }
+    // the basis in fixed point (a thread converts what it copied)
+    cp_async_wait_all();
+    const bool large = M * RM >= HC_FX_MIN && M <= HC_T;
+    int big = large ? 0 : 2047;
+    for (int m = warp; large && m < M; m += HC_T / 32)
+        for (int i = lane; i < R; i += 32) big = max(big, fx_exp(Qs[(size_t)m * RM + i]));
+    const bool fx = !__syncthreads_or(big > 1023);  // |q| < 2, finite
+    if (fx)
+        for (int m = warp; m < M; m += HC_T / 32)
+            for (int i = lane; i < R; i += 32) {
+                const size_t e = (size_t)m * RM + i;
+                Qx[e] = fx_split(fx_round(Qs[e], 60));
+            }
     pdl_wait();
     // ---- sums of the product partials: thread (row, group of chunks)
     const int RP = max(32, (R + 31) & ~31);  // at most HC_T (n <= HC_MAX_N)
@@ -518,8 +548,43 @@ __global__ void __launch_bounds__(HC_T) k_half_cluster(HalfArgs a) {
         }
         sc[grp * RP + row] = (t[0] + t[1]) + (t[2] + t[3]);
     }
-    cp_async_wait_all();
     if (done) return;
+    // x (a row's or a basis vector's value, 0 elsewhere) in fixed point at the largest
+    // exponent: every thread gets the scale s (x 2^s), FX_NONFINITE when a value is not finite
+    auto to_fixed = [&](double x, int2* out, int cnt) -> int {
+        int e = __reduce_max_sync(RBF_FULL_MASK, fx_exp(x));
+        if (lane == 0) rede[warp] = e;
+        __syncthreads();
+        e = 1;
+#pragma unroll
+        for (int w = 0; w < HC_T / 32; ++w) e = max(e, rede[w]);
+        if (e < FX_NONFINITE && threadIdx.x < cnt) out[threadIdx.x] = fx_split(fx_round(x, 1083 - e));
+        __syncthreads();
+        return e < FX_NONFINITE ? 1083 - e : FX_NONFINITE;  // (s <= 1082)
+    };
+    // one term of a sum at a time, folded every FX_FOLD; the pair goes to sch[slot]
+    auto fixed_sum = [&](const int2* n, int n_step, const int2* z, int z_step, int cnt, int slot) {
+        FxAcc32 acc;
+        for (int i0 = 0; i0 < cnt; i0 += FX_FOLD) {
+            const int i1 = min(i0 + FX_FOLD, cnt);
+            for (int i = i0; i < i1; ++i) {
+                const int2 N = n[(size_t)i * n_step], Z = z[(size_t)i * z_step];
+                acc.add(N.y, N.x, Z.y, Z.x);
+            }
+            acc.fold();
+        }
+        const longlong2 p = acc.pair(cnt);
+        sch[slot] = p.x;
+        sch[HC_T + slot] = p.y;
+    };
+    auto fixed_total = [&](int slot, int step, int cnt, int s) -> double {
+        longlong2 p = make_longlong2(0, 0);
+        for (int k = 0; k < cnt; ++k) {
+            p.x += sch[slot + k * step];
+            p.y += sch[HC_T + slot + k * step];
+        }
+        return s == FX_NONFINITE ? fx_nan() : ldexp(FxAcc32::value(p), 4 - s);
+    };
     __syncthreads();
     if (threadIdx.x < R) {
         double v = 0.0;
@@ -531,28 +596,39 @@ __global__ void __launch_bounds__(HC_T) k_half_cluster(HalfArgs a) {
     int split = 1;
     while (split < HC_SPLIT && 2 * split * M <= HC_T) split *= 2;
     for (int pass = 0; pass < 2 && M > 0; ++pass) {
-        for (int p = threadIdx.x; p < split * M; p += HC_T) {
-            const int k = p / M, m = p - k * M;
-            const double* q = Qs + (size_t)m * RM;
-            double c0 = 0.0, c1 = 0.0;
-            int i = k;
-            for (; i + split < R; i += 2 * split) {
-                c0 = fma(q[i], vs[i], c0);
-                c1 = fma(q[i + split], vs[i + split], c1);
+        if (fx) {
+            const int sv = to_fixed(threadIdx.x < R ? vs[threadIdx.x] : 0.0, vx, R);
+            if (threadIdx.x < split * M) {
+                const int k = threadIdx.x / M, m = threadIdx.x - k * M;
+                fixed_sum(vx + k, split, Qx + (size_t)m * RM + k, split,
+                          sv == FX_NONFINITE || k >= R ? 0 : (R - k + split - 1) / split, threadIdx.x);
             }
-            if (i < R) c0 = fma(q[i], vs[i], c0);
-            sc[p] = c0 + c1;
-        }
-        __syncthreads();
-        for (int m = threadIdx.x; m < M; m += HC_T) {
-            double c0 = sc[m], c1 = 0.0;
-            int k = 1;
-            for (; k + 1 < split; k += 2) {
-                c1 += sc[k * M + m];
-                c0 += sc[(k + 1) * M + m];
+            __syncthreads();
+            if (threadIdx.x < M) hp[pass * M + threadIdx.x] = fixed_total(threadIdx.x, M, split, sv);
+        } else {
+            for (int p = threadIdx.x; p < split * M; p += HC_T) {
+                const int k = p / M, m = p - k * M;
+                const double* q = Qs + (size_t)m * RM;
+                double c0 = 0.0, c1 = 0.0;
+                int i = k;
+                for (; i + split < R; i += 2 * split) {
+                    c0 = fma(q[i], vs[i], c0);
+                    c1 = fma(q[i + split], vs[i + split], c1);
+                }
+                if (i < R) c0 = fma(q[i], vs[i], c0);
+                sc[p] = c0 + c1;
             }
-            if (k < split) c1 += sc[k * M + m];
-            hp[pass * M + m] = c0 + c1;
+            __syncthreads();
+            for (int m = threadIdx.x; m < M; m += HC_T) {
+                double c0 = sc[m], c1 = 0.0;
+                int k = 1;
+                for (; k + 1 < split; k += 2) {
+                    c1 += sc[k * M + m];
+                    c0 += sc[(k + 1) * M + m];
+                }
+                if (k < split) c1 += sc[k * M + m];
+                hp[pass * M + m] = c0 + c1;
+            }
         }
         cluster.sync();
         if (pass == 0) {
@@ -570,6 +646,16 @@ __global__ void __launch_bounds__(HC_T) k_half_cluster(HalfArgs a) {
             hs[m] = t[0];
         }
         __syncthreads();
+        if (fx) {
+            const int sh = to_fixed(threadIdx.x < M ? hs[threadIdx.x] : 0.0, hx, M);
+            if (grp < ng)
+                fixed_sum(hx + grp, ng, Qx + (size_t)grp * RM + row, ng * RM,
+                          sh == FX_NONFINITE || row >= R || grp >= M ? 0 : (M - grp + ng - 1) / ng, grp * RP + row);
+            __syncthreads();
+            if (threadIdx.x < R) vs[threadIdx.x] -= fixed_total(threadIdx.x, RP, ng, sh);
+            __syncthreads();
+            continue;
+        }
         if (grp < ng) {
             double c0 = 0.0, c1 = 0.0;
             if (row < R) {
