@@ -358,9 +358,11 @@ rbf_status rbf_tsvd(rbf_ctx* ctx, const rbf_operator* op, const double* d_f, int
 /* ---- reconstruction (eq. u_reconstruction) --------------------------- */
 
 /* d_u[m] = sum_j d_coef[j] Phi(|P_t - X_j|) at the m points d_points (FP64 SoA
- * [3][m]).  Always FP64 (also for RBF_MIXED operators): the coefficients of an
- * ill-conditioned collocation system cancel, so FP32 basis values would lose
- * the reconstruction.  Uses the operator's form (c or eps). */
+ * [3][m]).  To FP64 accuracy also for RBF_MIXED operators: the coefficients of
+ * an ill-conditioned collocation system cancel, so FP32 basis values would lose
+ * the reconstruction.  Evaluated in 64-bit fixed point where c is within 2^5 of
+ * the largest coordinate and every value is finite, else in FP64.  Uses the
+ * operator's form (c or eps). */
 rbf_status rbf_evaluate(rbf_ctx* ctx, const rbf_operator* op, const double* d_coef,
                         const double* d_points, int64_t m, double* d_u);
 
