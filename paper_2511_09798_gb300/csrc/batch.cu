@@ -15,7 +15,8 @@
 //                   norm finalisation and breakdown test, then classical
 //                   Gram-Schmidt applied twice against each instance's basis,
 //                   with per-instance dot partials reduced across the CTAs that
-//                   share the instance (bounded grid barriers)
+//                   share the instance (one bounded grid barrier
+//                   per pass; two for instances on more than 128 CTAs)
 //   k_mf_batch<0>, k_half_batch   the same for the p-side
 // The whole step loop is captured into one CUDA graph and launched once.  The
 // block size of the batched product (4 or 8 rows per lane: blocks of 128 or

@@ -448,8 +448,9 @@ __global__ void __launch_bounds__(SL_THREADS) k_half(HalfArgs a) {
 // first cluster barrier, when every CTA has read the done flag.
 // It is launched with programmatic stream serialization: the slab of Q, the norm
 // and the breakdown test are done while the product before it ends.  Per
-// half-step at n = 1000 (mcount up to 40) 22.4 -> 14.1 us, at n = 2161 (up to 120)
-// 26 -> 22.7, less what overlaps the product; a whole step at n = 1000 72 -> 37 us.
+// half-step at n = 1000 (mcount up to 40) 22.4 -> 14.1 us, less what overlaps the
+// product; a whole step at n = 1000 72 -> 37 us, at n = 2161 (mcount up to 140)
+// 102 -> 64 us.
 constexpr int HC_CTAS = 16;
 constexpr int HC_T = 512;
 constexpr int HC_SPLIT = 16;  // most threads per basis vector in the dot products
@@ -781,7 +782,9 @@ static size_t half_smem_bytes(bool stage, int mcount, int chunks, int rmax, bool
 // the first step to these limits against the grid kernel throughout: n = 1500,
 // 60 steps 3.15 and 4.63 ms, 3000 5.13 and 6.20, 4090 6.69 and 7.38; 4800, 100
 // steps 12.9 and 13.5, 6400 18.7 and 19.0, 8000 24.8 and 25.0; 256 K instead of
-// 416 K 1 % slower at n = 2161, the whole of it above 4096 2 % slower at 8000).
+// 416 K 1 % slower at n = 2161, the whole of it above 4096 2 % slower at 8000; these
+// with the sums in FP64.  With the fixed-point form, half of it above 4096 and the
+// whole: n = 4500, 140 steps 18.0 and 18.5 ms; 6000, 40 steps 7.46 and 7.50).
 // Mixed runs round their vectors to FP32 for the products and keep one order of
 // summation.
 // The rule depends on the problem and the context's options alone, so resumed and
