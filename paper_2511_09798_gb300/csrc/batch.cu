@@ -614,7 +614,7 @@ static rbf_status plan_batch(rbf_ctx* ctx, const rbf_batch* bt, int form, BatchP
     // cooperative grid: up to 4 co-resident CTAs per SM (measured on the 96-instance
     // sweep: 0.663 ms per half-step against 0.691 with 8 and 0.728 with 2), at least 64 rows per
     // CTA; the shared memory depends on the slab size, so iterate to a fixed point
-    cudaFuncSetAttribute(k_half_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    RBF_CUDA(ctx, smem_limit<k_half_batch>(ctx, SIZE_MAX));  // the occupancy of several sizes is asked below
     int64_t G = (int64_t)ctx->sm_count * 4;
     for (int it = 0; it < 6; ++it) {
         if (G > P->T / 64) G = P->T / 64;
@@ -887,8 +887,7 @@ extern "C" rbf_status rbf_batch_gkb(rbf_ctx* ctx, rbf_batch* bt, int steps, int 
     RBF_CUDA(ctx, cudaMemcpyAsync(w.items, items.data(), sizeof(MfItem) * items.size(), cudaMemcpyHostToDevice, s));
     const int nit = (int)items.size();
     const size_t hsmem = ((size_t)P.rmax + (size_t)SEGMAX * (P.L + 2)) * sizeof(double);
-    if (hsmem > 48 * 1024)
-        RBF_CUDA(ctx, cudaFuncSetAttribute(k_half_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hsmem));
+    RBF_CUDA(ctx, smem_limit<k_half_batch>(ctx, hsmem));
 
     // ---- the step loop, captured into one graph.  A cached graph is reused only
     // when every value it bakes in is the same, compared byte for byte: the

@@ -337,23 +337,18 @@ constexpr int64_t FX_MAX_N = 16384;  // the vector's limbs of A z fit in shared 
 size_t fxn_smem(int64_t n) { return (size_t)3 * ((n + 1) & ~(int64_t)1) * sizeof(int); }
 
 // CTAs of k_gemv_flat_fx resident per SM at this n (cached per device for the
-// last n asked; the shared-memory limit is raised once to the largest size).
+// last n asked).
 // Contexts on different host threads share the cache, hence the mutex.
 int fxn_per_sm(const rbf_ctx* ctx, int64_t n) {
     static std::mutex mu;
     static int64_t last_n[64] = {0};
     static int last_per[64] = {0};
-    static bool raised[64] = {false};
     std::lock_guard<std::mutex> lock(mu);
     const int dev = ctx->device >= 0 && ctx->device < 64 ? ctx->device : 0;
     if (last_n[dev] == n && last_per[dev] > 0) return last_per[dev];
-    if (!raised[dev]) {
-        if (cudaFuncSetAttribute((const void*)k_gemv_flat_fx, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)fxn_smem(FX_MAX_N)) != cudaSuccess) {
-            cudaGetLastError();
-            return 0;
-        }
-        raised[dev] = true;
+    if (smem_limit<k_gemv_flat_fx>(ctx, fxn_smem(n)) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
     }
     int a = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_gemv_flat_fx, FXN_THREADS, fxn_smem(n)) != cudaSuccess) {
@@ -446,9 +441,7 @@ rbf_status launch_fx_prepare(rbf_ctx* ctx, const rbf_operator* op, const FxCopie
     RBF_CUDA(ctx, cudaMemsetAsync(f.rowE, 0, (size_t)n * sizeof(int), ctx->stream));
     RBF_CUDA(ctx, cudaMemsetAsync(f.colE, 0, (size_t)n * sizeof(int), ctx->stream));
     const size_t smem = (size_t)rows_max * sizeof(int);
-    if (smem > SMEM_PLAIN)
-        RBF_CUDA(ctx, cudaFuncSetAttribute((const void*)k_fx_exps, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)smem));
+    RBF_CUDA(ctx, smem_limit<k_fx_exps>(ctx, smem));
     k_fx_exps<<<pn * ch, FXE_THREADS, smem, ctx->stream>>>((const double*)op->d_A, op->lda, n, ch, rows_max,
                                                            f.rowE, f.colE);
     RBF_LAUNCHED(ctx, "k_fx_exps");
@@ -462,9 +455,7 @@ rbf_status launch_fx_n(rbf_ctx* ctx, const rbf_operator* op, const FxCopies& f, 
                        const int* done, bool pdl) {
     if (const int w = fxn_row_warps(ctx, op->n)) {
         const size_t smem = fxn_smem(op->n);
-        if (smem > SMEM_PLAIN)
-            RBF_CUDA(ctx, cudaFuncSetAttribute((const void*)k_gemv_row_fx, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)smem));
+        RBF_CUDA(ctx, smem_limit<k_gemv_row_fx>(ctx, smem));
         RBF_CUDA(ctx, rbf_launch_ex(ctx, k_gemv_row_fx, dim3((unsigned)((op->n + w - 1) / w)), dim3(w * 32), smem, pdl,
                                     1, f.NR, op->lda, op->n, f.rowE, x, part, done));
         RBF_LAUNCHED(ctx, "k_gemv_row_fx");
@@ -484,9 +475,7 @@ rbf_status launch_fx_t(rbf_ctx* ctx, const rbf_operator* op, const FxCopies& f, 
     int pc, pn, ch, rows_max;
     fxt_plan(ctx, op->n, &pc, &pn, &ch, &rows_max);
     const size_t smem = (size_t)rows_max * sizeof(int4);
-    if (smem > SMEM_PLAIN)
-        RBF_CUDA(ctx, cudaFuncSetAttribute((const void*)k_gemv_t_fx, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)smem));
+    RBF_CUDA(ctx, smem_limit<k_gemv_t_fx>(ctx, smem));
     RBF_CUDA(ctx, rbf_launch_ex(ctx, k_gemv_t_fx, dim3(pn * ch), dim3(FXT_THREADS), smem, pdl, 1, f.NC, op->lda, op->n,
                                 f.colE, x, pc, ch, rows_max, part, done));
     RBF_LAUNCHED(ctx, "k_gemv_t_fx");

@@ -817,8 +817,7 @@ static bool half_cluster_ready(rbf_ctx* ctx) {
         cfg.numAttrs = 1;
         int clusters = 0;
         if (cudaFuncSetAttribute(k_half_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-            cudaFuncSetAttribute(k_half_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)HC_SMEM_MAX) ==
-                cudaSuccess &&
+            smem_raise((const void*)k_half_cluster) == cudaSuccess &&
             cudaOccupancyMaxActiveClusters(&clusters, k_half_cluster, &cfg) == cudaSuccess && clusters > 0)
             ctx->half_cluster = 1;
         else
@@ -976,11 +975,8 @@ struct GkbRun {
             const size_t need = half_smem_bytes(false, st->capacity + 1, chmax, rmax, f32slots);
             if (need > HALF_SMEM_STAGE_MAX)
                 return rbf_fail(ctx, RBF_ERR_UNSUPPORTED, "half-step shared memory too large (%zu bytes)", need);
-            if (need > SMEM_PLAIN)
-                RBF_CUDA(ctx, cudaFuncSetAttribute((const void*)k_half<false>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need));
-            RBF_CUDA(ctx, cudaFuncSetAttribute((const void*)k_half<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)HALF_SMEM_STAGE_MAX));
+            RBF_CUDA(ctx, smem_limit<k_half<false>>(ctx, need));
+            RBF_CUDA(ctx, smem_limit<k_half<true>>(ctx, HALF_SMEM_STAGE_MAX));
         }
         npart = wc.take<double>((size_t)std::max(G, HC_CTAS));
         if (use_fx) {
@@ -1207,9 +1203,7 @@ extern "C" rbf_status rbf_gkb_many(rbf_ctx* ctx, int count, const rbf_operator* 
         const size_t need = half_smem_bytes(false, states[i].capacity + 1, chmax, rmax, mf_slots_f32(ctx, &ops[i]));
         if (need > HALF_SMEM_STAGE_MAX) continue;  // the run itself is refused with RBF_ERR_UNSUPPORTED below
         int per_sm = 0;
-        if (need > SMEM_PLAIN)
-            RBF_CUDA(ctx, cudaFuncSetAttribute((const void*)k_half<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)need));
+        RBF_CUDA(ctx, smem_limit<k_half<false>>(ctx, need));
         RBF_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)k_half<false>, SL_THREADS,
                                                                     need));
         const int64_t fit = (int64_t)per_sm * ctx->sm_count / G;

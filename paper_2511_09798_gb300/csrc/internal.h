@@ -5,6 +5,7 @@
 #include <nvtx3/nvToolsExt.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <cstdarg>
 #include <cstdio>
 
@@ -92,10 +93,6 @@ rbf_status rbf_many_slots(rbf_ctx* ctx, int count);
 rbf_status rbf_lanes_fork(rbf_ctx* ctx, int lanes);
 rbf_status rbf_lanes_join(rbf_ctx* ctx, int lanes);
 
-// Dynamic shared memory that needs no cudaFuncSetAttribute beside a kernel's few
-// hundred bytes of static shared memory (48 KB together).
-constexpr size_t SMEM_PLAIN = 40 * 1024;
-
 // ---- error helpers ---------------------------------------------------------
 rbf_status rbf_fail(rbf_ctx* ctx, rbf_status st, const char* fmt, ...);
 
@@ -153,6 +150,41 @@ struct WsCarve {
     }
 };
 inline size_t ws_align(size_t b) { return (b + 255) & ~(size_t)255; }
+
+// ---- shared-memory limits -----------------------------------------------------
+// Dynamic shared memory that needs no raised limit beside a kernel's few hundred
+// bytes of static shared memory (48 KB together).
+constexpr size_t SMEM_PLAIN = 40 * 1024;
+
+// The kernel's dynamic shared-memory limit, raised to all that its static shared
+// memory leaves.
+inline cudaError_t smem_raise(const void* kernel) {
+    int dev = 0, most = 0;
+    cudaFuncAttributes fa{};
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes);
+    return e;
+}
+
+// Makes K ready for launches with `bytes` of dynamic shared memory.  The limit
+// belongs to the function on the device, not to the context, and contexts on
+// several host threads launch the same kernels at different sizes: a limit set to
+// one call's size could be lowered by another thread between its setting and its
+// launch.  So it is raised once per device, to the most there is, and never
+// lowered (two threads that raise it at once set the same value).
+template <auto K>
+inline cudaError_t smem_limit(const rbf_ctx* ctx, size_t bytes) {
+    static std::atomic<uint64_t> raised{0};
+    if (bytes <= SMEM_PLAIN) return cudaSuccess;
+    const uint64_t bit = ctx->device >= 0 && ctx->device < 64 ? (uint64_t)1 << ctx->device : 0;
+    if (raised.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    const cudaError_t e = smem_raise((const void*)K);
+    if (e == cudaSuccess) raised.fetch_or(bit, std::memory_order_release);
+    return e;
+}
 
 // Launch of a kernel that calls pdl_wait, with programmatic stream serialization
 // (`pdl`) and as clusters of `cluster` CTAs (1: none).

@@ -180,10 +180,8 @@ extern "C" rbf_status rbf_hkt_error_table(rbf_ctx* ctx, const rbf_gkb_state* st,
     ProjDims d{n_ell, L, 0, d_ells};
     RBF_TRY(launch_projected_svd_batch(ctx, d, a_rep, b_rep, sigma, ftil, V, L, svd, nullptr, nullptr));
     const size_t smem_y = (size_t)YQ * L * 8, smem_e = (size_t)EQ * L * 8;
-    if (smem_y > SMEM_PLAIN)
-        RBF_CUDA(ctx, cudaFuncSetAttribute(k_err_coef, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_y));
-    if (smem_e > SMEM_PLAIN)
-        RBF_CUDA(ctx, cudaFuncSetAttribute(k_err_table, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_e));
+    RBF_CUDA(ctx, smem_limit<k_err_coef>(ctx, smem_y));
+    RBF_CUDA(ctx, smem_limit<k_err_table>(ctx, smem_e));
     k_err_coef<<<dim3((unsigned)((Jp + YQ - 1) / YQ), (unsigned)n_ell), YT, smem_y, ctx->stream>>>(
         d_ells, L, sigma, ftil, V, m, d_uref, J, ctx->opt.grid_t_lo, ctx->opt.grid_t_hi, t_stride, Jp, y, umax, d_err);
     RBF_LAUNCHED(ctx, "k_err_coef");

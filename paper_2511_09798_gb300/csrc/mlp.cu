@@ -412,9 +412,9 @@ static rbf_status launch_mlp_pass(rbf_ctx* ctx, const PassArgs& a, int* tiles) {
     const bool small = (int64_t)a.B <= (int64_t)ctx->sm_count * 48;
     const int ts = small ? 4 : 8;
     *tiles = (a.B + ts - 1) / ts;
-    const void* k = small ? (const void*)k_mlp_pass<4, TRAIN> : (const void*)k_mlp_pass<8, TRAIN>;
     const size_t smem = small ? mlp_smem<4>() : mlp_smem<8>();
-    RBF_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (small) RBF_CUDA(ctx, (smem_limit<k_mlp_pass<4, TRAIN>>(ctx, smem)));
+    else RBF_CUDA(ctx, (smem_limit<k_mlp_pass<8, TRAIN>>(ctx, smem)));
     if (small) k_mlp_pass<4, TRAIN><<<*tiles, MP_T, smem, ctx->stream>>>(a);
     else k_mlp_pass<8, TRAIN><<<*tiles, MP_T, smem, ctx->stream>>>(a);
     RBF_LAUNCHED(ctx, "k_mlp_pass");

@@ -762,13 +762,10 @@ rbf_status launch_projected_svd_batch(rbf_ctx* ctx, ProjDims d, const double* al
     const bool wide = (int64_t)L * B <= (int64_t)ctx->sm_count * 12;
     const int warps = L > 4096 ? 2 * BS_WARPS : BS_WARPS;  // one CTA per SM holds the tables above 4096
     const int per_cta = warps * (wide ? 1 : 4);
-    if (sh_b > SMEM_PLAIN) {
-        RBF_CUDA(ctx, cudaFuncSetAttribute(wide ? k_tgk_bisect<32> : k_tgk_bisect<8>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_b));
-        RBF_CUDA(ctx, cudaFuncSetAttribute(k_tgk_vectors, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_v));
-    }
-    if (sh_f > SMEM_PLAIN)
-        RBF_CUDA(ctx, cudaFuncSetAttribute(k_tgk_finalize, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_f));
+    if (wide) RBF_CUDA(ctx, smem_limit<k_tgk_bisect<32>>(ctx, sh_b));
+    else RBF_CUDA(ctx, smem_limit<k_tgk_bisect<8>>(ctx, sh_b));
+    RBF_CUDA(ctx, smem_limit<k_tgk_vectors>(ctx, sh_v));
+    RBF_CUDA(ctx, smem_limit<k_tgk_finalize>(ctx, sh_f));
     const dim3 gb((L + per_cta - 1) / per_cta, B);
     if (wide) k_tgk_bisect<32><<<gb, warps * 32, sh_b, s>>>(d, alpha, beta, sigma, bound);
     else k_tgk_bisect<8><<<gb, warps * 32, sh_b, s>>>(d, alpha, beta, sigma, bound);

@@ -1088,8 +1088,7 @@ rbf_status fsvd_bidiag(rbf_ctx* ctx, const rbf_operator* op, const double* f, Fs
     const int J = ctx->opt.grid_j;
     const int L = (int)n;
     const size_t smem = bd_smem(n, ctx->sm_count);
-    if (smem > SMEM_PLAIN)
-        RBF_CUDA(ctx, cudaFuncSetAttribute(k_bidiag, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    RBF_CUDA(ctx, smem_limit<k_bidiag>(ctx, smem));
     F->G = coop_grid(ctx, (const void*)k_bidiag, BD_T, ctx->sm_count, &F->group, &F->bar_k, smem);
     const int G = F->G;
     if (G != ctx->sm_count) return rbf_fail(ctx, RBF_ERR_INTERNAL, "bidiagonalization grid of %d CTAs", G);
@@ -1179,6 +1178,7 @@ rbf_status fsvd_apply_qr(rbf_ctx* ctx, const Fsvd* F, double* z) {
     QrArgs a{F->Wb, n, F->ldw, F->taur, F->scaler, F->gram, z, F->hpart, F->gpart, ctx->d_state, F->bar, F->group,
              ctx->opt.wait_budget};
     void* args[] = {&a};
+    RBF_CUDA(ctx, smem_limit<k_qr_apply>(ctx, smem));
     RBF_CUDA(ctx, cudaLaunchCooperativeKernel((const void*)k_qr_apply, dim3(F->G), dim3(QA_T), args, smem, s));
     ctx->launches++;
     return RBF_OK;
