@@ -790,7 +790,8 @@ __global__ void __launch_bounds__(BT) k_vt_g(const double* __restrict__ Vt, int6
 
 // x[row] = sum_i U~[row][i] d_i over the first n rows of U~ (ld n+1): 32 rows x
 // 32 column groups per CTA, four chains each (one thread per row: 1.45 ms at n =
-// 3001, latency of n dependent FMAs)
+// 3001, latency of n dependent FMAs).  Columns with d_i = 0 (beyond the rank) are
+// left out: the vector of a zero singular value may have no u part to normalise.
 __global__ void __launch_bounds__(1024) k_u_d(const double* __restrict__ Ut, int64_t n, const double* __restrict__ d,
                                               double* __restrict__ x) {
     __shared__ double red[32][33];
@@ -800,10 +801,14 @@ __global__ void __launch_bounds__(1024) k_u_d(const double* __restrict__ Ut, int
     if (row < n) {
         const double* p = Ut + row;
         int64_t i = grp;
+        auto add = [&](int64_t c, double& acc) {
+            const double dc = d[c], t = fma(p[c * ldu], dc, acc);
+            acc = dc != 0.0 ? t : acc;
+        };
         for (; i + 96 < n; i += 128)
 #pragma unroll
-            for (int u = 0; u < 4; ++u) a[u] = fma(p[(i + 32 * u) * ldu], d[i + 32 * u], a[u]);
-        for (; i < n; i += 32) a[0] = fma(p[i * ldu], d[i], a[0]);
+            for (int u = 0; u < 4; ++u) add(i + 32 * u, a[u]);
+        for (; i < n; i += 32) add(i, a[0]);
     }
     red[grp][lane] = (a[0] + a[1]) + (a[2] + a[3]);
     __syncthreads();
