@@ -23,36 +23,45 @@ namespace {
 
 __device__ __forceinline__ int sel_l(const ProjDims& d, int b) { return d.l_arr ? d.l_arr[b] : d.l; }
 
-// One warp per grid point, lanes along the singular values (one thread per
-// point spent its time in a chain of l IEEE divisions: 82 -> 10 us at l = 150).
+// LPP lanes per grid point, along the singular values.  A point costs an exp10 and
+// two logarithms besides a division per value, and an FP64 instruction takes the
+// FP64 unit as long for one lane as for 32: many lanes per point shorten the chain
+// of one run (a thread per point 82 us at l = 150, a warp 10), few lanes waste
+// less where many instances fill the units (300 runs of l = 10: a warp per point
+// 757 us, a thread 50).
 constexpr int GT_WARPS = 4;
 
+template <int LPP>
 __global__ void __launch_bounds__(GT_WARPS * 32)
     k_grid_terms(ProjDims d, const double* __restrict__ sigma_all, const double* __restrict__ ftil_all, int J,
                  double t_lo, double t_hi, double* __restrict__ gcv_all, double* __restrict__ xr_all,
                  double* __restrict__ ye_all) {
     const int b = blockIdx.y;
     const int l = sel_l(d, b);
-    const int t = blockIdx.x * GT_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (t >= J || l < 1) return;
+    const int t = (blockIdx.x * (GT_WARPS * 32) + threadIdx.x) / LPP, g = threadIdx.x % LPP;
+    if (l < 1 || __all_sync(RBF_FULL_MASK, t >= J)) return;
     const double* sigma = sigma_all + (size_t)b * d.L;
     const double* ftil = ftil_all + (size_t)b * (d.L + 1);
-    const double lam = sigma[0] * exp10(grid_t(t, J, t_lo, t_hi));
+    const double lam = sigma[0] * exp10(grid_t(min(t, J - 1), J, t_lo, t_hi));
     const double lam2 = lam * lam;
     double rho2 = 0.0, eta2 = 0.0, den = 0.0;
-    for (int i = lane; i < l; i += 32) {
+    for (int i = g; i < l; i += LPP) {
         const double s = sigma[i], f = ftil[i];
         const double inv = 1.0 / fma(s, s, lam2);
         const double q = lam2 * inv;
-        const double g = s * f * inv;
-        rho2 = fma(q * q, f * f, rho2);
+        const double r = q * f, g = s * f * inv;
+        rho2 = fma(r, r, rho2);
         eta2 = fma(g, g, eta2);
         den += q;
     }
-    rho2 = warp_sum(rho2);
-    eta2 = warp_sum(eta2);
-    den = 1.0 + warp_sum(den);
-    if (lane == 0) {
+#pragma unroll
+    for (int o = LPP / 2; o > 0; o >>= 1) {
+        rho2 += __shfl_xor_sync(RBF_FULL_MASK, rho2, o);
+        eta2 += __shfl_xor_sync(RBF_FULL_MASK, eta2, o);
+        den += __shfl_xor_sync(RBF_FULL_MASK, den, o);
+    }
+    den += 1.0;
+    if (g == 0 && t < J) {
         rho2 = fma(ftil[l], ftil[l], rho2);
         gcv_all[(size_t)b * J + t] = rho2 / (den * den);
         xr_all[(size_t)b * J + t] = 0.5 * log(rho2);
@@ -343,6 +352,30 @@ __global__ void __launch_bounds__(CM_GROUPS * 32)
 
 size_t select_ws_bytes(const rbf_ctx* ctx, int l) { return select_ws_bytes_batch(ctx, l, 1); }
 
+using GridTermsFn = void (*)(ProjDims, const double*, const double*, int, double, double, double*, double*, double*);
+
+// Lanes per grid point: the smallest of (warps per FP64 unit) x (FP64 instructions
+// of a warp, in terms of a sum of about 15 each: 9 for the exp10 and the logarithms
+// and one per value of a lane); the most lanes on ties.  Whole batched choices with
+// 32 lanes, 1 lane and the rule's (321 points): 1 run of l = 150 466, 540 and 468 us (32),
+// 12 of 40 168, 158 and 144 (4), 24 of 40 233, 183 and 172 (2), 300 of 10 911, 208 and 209 (1).
+static GridTermsFn grid_terms_lanes(const rbf_ctx* ctx, int L, int B, int J, int* lpp) {
+    const GridTermsFn kern[6] = {k_grid_terms<1>, k_grid_terms<2>,  k_grid_terms<4>,
+                                 k_grid_terms<8>, k_grid_terms<16>, k_grid_terms<32>};
+    int best = 5;
+    int64_t least = INT64_MAX;
+    for (int q = 5; q >= 0; --q) {
+        const int64_t warps = ((int64_t)J * B * (1 << q) + 31) / 32, units = 4 * (int64_t)ctx->sm_count;
+        const int64_t cost = (warps + units - 1) / units * (9 + (L + (1 << q) - 1) / (1 << q));
+        if (cost < least) {
+            least = cost;
+            best = q;
+        }
+    }
+    *lpp = 1 << best;
+    return kern[best];
+}
+
 rbf_status launch_select_batch(rbf_ctx* ctx, ProjDims d, int method, int rule, double lambda_in, int rank,
                                const double* alpha, const double* beta, const double* Z, LiftDims ld,
                                double* coef, double* curve, void* ws, double* lam_out, int* idx_out,
@@ -367,7 +400,10 @@ rbf_status launch_select_batch(rbf_ctx* ctx, ProjDims d, int method, int rule, d
     rbf_timer_start(ctx);
     if (method == 0) {
         if (rule == RBF_GCV || rule == RBF_LCURVE || rule_arr) {
-            k_grid_terms<<<dim3((J + GT_WARPS - 1) / GT_WARPS, B), GT_WARPS * 32, 0, s>>>(d, sigma, ftil, J, tlo, thi, gcv, xr, ye);
+            int lpp;
+            const GridTermsFn kern = grid_terms_lanes(ctx, L, B, J, &lpp);
+            const int per_cta = GT_WARPS * 32 / lpp;
+            kern<<<dim3((J + per_cta - 1) / per_cta, B), GT_WARPS * 32, 0, s>>>(d, sigma, ftil, J, tlo, thi, gcv, xr, ye);
             RBF_LAUNCHED(ctx, "k_grid_terms");
         }
         k_choose_lambda<<<B, CH_T, 0, s>>>(d, sigma, ftil, J, tlo, thi, rule, lambda_in, rule_arr, lam_arr, gcv, xr,
