@@ -25,8 +25,6 @@
 #include <cfloat>
 #include <vector>
 
-#include <type_traits>
-
 #include "common.cuh"
 #include "grid_sync.cuh"
 #include "internal.h"
@@ -409,16 +407,20 @@ __device__ __forceinline__ Refl reflector(double x0, double ss) {
 //      apply that update, write S, and take u'^T s_j with the new left reflector
 //      u' in the same pass: y'_j = t u'^T s_j, row k: r_j = s_kj - u'_k y'_j
 //   -- barrier --  right reflector v' from r
-//   B  (blocks of 4 rows over all columns): x'_i = t' (sum_j S_ij v'_j - u'_i
-//      y'^T v'), and column k + 1 of A with its norm: the next left reflector
+//   B  (blocks of 4 rows over all columns): x'_i = t' sum_j (S_ij - u'_i y'_j)
+//      v'_j, and column k + 1 of A with its norm: the next left reflector
 //   -- barrier --
 // so S is read twice and written once per step (a pass for the products and one
 // for the update of each reflector read it four times and wrote it twice), the
 // vectors u, x and v sit in shared memory, and the norms come from one partial
-// per CTA instead of a pass over the vector in every CTA.  The FP64 pipe bounds
-// it (4 n^3 / 3 FMAs: 57 ms at n = 3001, 2.1 ms at 1000) together with the two
-// barriers and reflector chains per step.  n = 1000: 26.5 -> 17.8 ms, n =
-// 3001: 244 -> 130 ms.
+// per CTA instead of a pass over the vector in every CTA.  Pass B applies u' to
+// the entries first: sum_j S_ij v'_j - u'_i y'^T v' saves an FMA per entry, but
+// its difference cancels, and Tikhonov solutions of collocation matrices (singular
+// values that fall off fast) come out 2.4 times as far off (n = 1000; n = 500
+// 1.6 times).  The FP64 pipe bounds it (5 n^3 / 3 FMAs: 71 ms at n = 3001, 2.7 ms
+// at 1000) together with the two barriers and reflector chains per step.  Whole GCV
+// Tikhonov solves 46.5 -> 21.1 ms at n = 1000, 386 -> 161 ms at 3001 (21.2 and
+// 148 with the cancelling difference).
 constexpr int BD_T = 512;
 constexpr int BD_W = BD_T / 32;
 constexpr int BD_ROWS = 256;  // rows of a column piece (8 per lane)
@@ -429,7 +431,7 @@ struct BidiagArgs {
     int64_t n, ld;
     double *dg, *eg, *taur, *scaler;
     double *y, *r, *x, *a;  // [n+1] y' and r by column, x' and column k + 1 of A by row
-    ulonglong2* slot;       // [3][G to][G from] |r|^2, y.r (columns past k + 1), |a|^2 (rows past k + 1), with epochs
+    ulonglong2* slot;       // [2][G to][G from] |r|^2 (columns past k + 1), |a|^2 (rows past k + 1), with epochs
     rbf_dev_state* stt;
     long long budget;
 };
@@ -449,8 +451,9 @@ inline size_t bd_smem(int64_t n, int G) {
 // (in a fixed order).  One store and one load across the L2, where arriving at a
 // counter, polling it and then loading the partials takes three trips: the whole
 // solve 24.2 -> 21.5 ms at n = 1000 and 157 -> 150 ms at 3001 (with the loads
-// ahead of the barriers below).  All CTAs polling one shared row of slots: 22.9
-// and 154.5 ms, its lines are too hot; one load after the other: 27.4 and 166.
+// ahead of the barriers below and one FMA less per entry in pass B).  All CTAs
+// polling one shared row of slots: 22.9 and 154.5 ms, its lines are too hot; one
+// load after the other: 27.4 and 166.
 __device__ __forceinline__ void bd_fence() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 __device__ __forceinline__ void bd_publish(ulonglong2* slot, double v, unsigned long long epoch) {
     asm volatile("{\n .reg .b128 t;\n mov.b128 t, {%1, %2};\n st.relaxed.gpu.global.b128 [%0], t;\n}" ::"l"(slot),
@@ -466,46 +469,35 @@ __device__ __forceinline__ ulonglong2 bd_peek(const ulonglong2* slot) {
     return r;
 }
 
-// The calling warp waits until all G slots of each of NS sums carry `epoch` and
-// adds their values; all loads of a lane are in flight together.  Bounded: false
-// after `budget` polls (the run is then stopped).
-constexpr int BD_SLOTS = 5;  // slots per lane and sum in flight: 160 CTAs in one go
-template <int NS>
+// The calling warp waits until all G slots carry `epoch` and adds their values;
+// all loads of a lane are in flight together.  Bounded: false after `budget` polls
+// (the run is then stopped).
+constexpr int BD_SLOTS = 5;  // slots per lane in flight: 160 CTAs in one go
 __device__ __forceinline__ bool bd_collect(const ulonglong2* slot, int G, unsigned long long epoch, long long budget,
                                            int lane, double* sum) {
     bool ok = true;
-#pragma unroll
-    for (int e = 0; e < NS; ++e) sum[e] = 0.0;
+    double t = 0.0;
     for (int b0 = lane; b0 < G; b0 += 32 * BD_SLOTS) {
-        ulonglong2 v[NS][BD_SLOTS];
+        ulonglong2 v[BD_SLOTS];
         for (long long it = 0;; ++it) {
             bool all = true;
 #pragma unroll
-            for (int e = 0; e < NS; ++e)
+            for (int q = 0; q < BD_SLOTS; ++q)
+                v[q] = b0 + 32 * q < G ? bd_peek(slot + b0 + 32 * q) : make_ulonglong2(0, epoch);
 #pragma unroll
-                for (int q = 0; q < BD_SLOTS; ++q)
-                    v[e][q] = b0 + 32 * q < G ? bd_peek(slot + (int64_t)e * G * G + b0 + 32 * q)
-                                              : make_ulonglong2(0, epoch);
-#pragma unroll
-            for (int e = 0; e < NS; ++e)
-#pragma unroll
-                for (int q = 0; q < BD_SLOTS; ++q) all = all && v[e][q].y == epoch;
+            for (int q = 0; q < BD_SLOTS; ++q) all = all && v[q].y == epoch;
             if (all) break;
             if (it > budget) {
                 ok = false;
                 break;
             }
         }
+        double d[BD_SLOTS];
 #pragma unroll
-        for (int e = 0; e < NS; ++e) {
-            double d[BD_SLOTS];
-#pragma unroll
-            for (int q = 0; q < BD_SLOTS; ++q) d[q] = __longlong_as_double((long long)v[e][q].x);
-            sum[e] += ((d[0] + d[1]) + (d[2] + d[3])) + d[4];
-        }
+        for (int q = 0; q < BD_SLOTS; ++q) d[q] = __longlong_as_double((long long)v[q].x);
+        t += ((d[0] + d[1]) + (d[2] + d[3])) + d[4];
     }
-#pragma unroll
-    for (int e = 0; e < NS; ++e) sum[e] = warp_sum(sum[e]);
+    *sum = warp_sum(t);
     return __all_sync(RBF_FULL_MASK, ok);
 }
 
@@ -516,7 +508,7 @@ __global__ void __launch_bounds__(BD_T) k_bidiag(BidiagArgs g) {
     const int G = gridDim.x, cta = blockIdx.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double* W = g.W;
-    double* uo = sm;          // left reflector of the step before
+    double* uo = sm;          // left reflector of the step before, then y' of this step
     double* un = sm + n;      // left reflector of this step
     double* xs = sm + 2 * n;  // x of the step before, then v' of this step
     const int pmax = (int)bd_pieces(n);
@@ -531,11 +523,10 @@ __global__ void __launch_bounds__(BD_T) k_bidiag(BidiagArgs g) {
         for (int b = lane; b < G; b += 32) bd_publish(g.slot + ((int64_t)e * G + b) * G + cta, v, epoch);
     };
     // a collected barrier: warp 0 waits; false stops the CTA
-    double sums[2] = {0.0, 0.0};  // (warp 0)
-    auto collect = [&](auto two) -> bool {
+    double sum = 0.0;  // (warp 0)
+    auto collect = [&](int e) -> bool {
         if (warp == 0) {
-            const bool ok = two ? bd_collect<2>(mine, G, epoch, g.budget, lane, sums)
-                                : bd_collect<1>(mine + 2 * (int64_t)G * G, G, epoch, g.budget, lane, sums);
+            const bool ok = bd_collect(mine + (int64_t)e * G * G, G, epoch, g.budget, lane, &sum);
             bd_fence();  // the others' stores, made before they published, are visible from here on
             if (lane == 0) {
                 go = ok;
@@ -563,7 +554,7 @@ __global__ void __launch_bounds__(BD_T) k_bidiag(BidiagArgs g) {
         __syncthreads();
         if (warp == 0) {
             bd_fence();
-            publish(2, ss);
+            publish(1, ss);
         }
     }
     double vscale = 0.0;  // 1 once a right reflector is pending
@@ -589,10 +580,10 @@ __global__ void __launch_bounds__(BD_T) k_bidiag(BidiagArgs g) {
             *vj = j < n && vscale != 0.0 ? __ldcg(g.r + j) : 0.0;
         };
         if (warp < nc * np) load(warp, v, &yj, &vj);
-        if (!collect(std::false_type{})) return;
+        if (!collect(1)) return;
         // ---- left reflector of column k
         if (warp == 0) {
-            const Refl h = reflector(__ldcg(g.a + k), sums[0]);
+            const Refl h = reflector(__ldcg(g.a + k), sum);
             if (lane == 0) {
                 sc[0] = h.t;
                 sc[1] = h.w0;
@@ -640,7 +631,7 @@ __global__ void __launch_bounds__(BD_T) k_bidiag(BidiagArgs g) {
         }
         __syncthreads();
         if (warp == 0) {
-            double rr = 0.0, yr = 0.0;
+            double rr = 0.0;
             for (int c = lane; c < nc; c += 32) {
                 const int64_t j = j0 + (int64_t)c * G;
                 double d = 0.0;
@@ -650,22 +641,17 @@ __global__ void __launch_bounds__(BD_T) k_bidiag(BidiagArgs g) {
                 g.y[j] = yj;
                 g.r[j] = r;
                 W[j * ld + k] = r;
-                if (j > k + 1 && j < n) {
-                    rr = fma(r, r, rr);
-                    yr = fma(yj, r, yr);
-                }
+                if (j > k + 1 && j < n) rr = fma(r, r, rr);
             }
             rr = warp_sum(rr);
-            yr = warp_sum(yr);
             __syncwarp();
             if (k < n - 1) {  // (the other warps' stores came before the barrier above)
                 bd_fence();
                 publish(0, rr);
-                publish(1, yr);
             }
         }
         if (k == n - 1) break;
-        if (!collect(std::true_type{})) return;
+        if (!collect(0)) return;
         // the first entries of pass B, ahead of the reflector
         const int64_t rbase = (k + 1) & ~(int64_t)(BD_RB - 1);
         const int64_t nblk = (n - rbase + BD_RB - 1) / BD_RB;
@@ -682,13 +668,10 @@ __global__ void __launch_bounds__(BD_T) k_bidiag(BidiagArgs g) {
         // ---- right reflector of row k
         if (warp == 0) {
             const double x0 = __ldcg(g.r + k + 1);
-            const Refl h = reflector(x0, sums[0]);
+            const Refl h = reflector(x0, sum);
             if (lane == 0) {
                 sc[0] = h.t;
-                sc[1] = fma(__ldcg(g.y + k + 1), h.w0, sums[1]);  // y'^T v'
                 xs[k + 1] = h.w0;
-                sc[2] = __ldcg(g.y + k + 1);
-                sc[3] = h.w0;
                 if (cta == 0) {
                     g.eg[k] = h.beta;
                     g.taur[k] = h.t;  // (k_bidiag_ab turns the two into tau and 1 / w_0)
@@ -696,9 +679,12 @@ __global__ void __launch_bounds__(BD_T) k_bidiag(BidiagArgs g) {
                 }
             }
         }
-        for (int64_t j = k + 2 + threadIdx.x; j < n; j += BD_T) xs[j] = __ldcg(g.r + j);
+        for (int64_t j = k + 1 + threadIdx.x; j < n; j += BD_T) {
+            if (j > k + 1) xs[j] = __ldcg(g.r + j);
+            uo[j] = __ldcg(g.y + j);
+        }
         __syncthreads();
-        const double t2 = sc[0], yv = sc[1], y1 = sc[2], v1 = sc[3];
+        const double t2 = sc[0], y1 = uo[k + 1], v1 = xs[k + 1];
         // ---- pass B
         int nb = 0;
         for (int64_t rb = cta; rb < nblk; rb += G, ++nb) {
@@ -707,23 +693,25 @@ __global__ void __launch_bounds__(BD_T) k_bidiag(BidiagArgs g) {
             double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
             if (ok) {
                 const double* p = W + i;
+                const double ui = un[i];
+                auto add = [&](double s, int64_t j, double& acc) { acc = fma(fma(-ui, uo[j], s), xs[j], acc); };
                 int64_t j = jb;
                 if (nb == 0) {
-                    if (j < n) a0 = first[0] * xs[j];
-                    if (j + CW < n) a1 = first[1] * xs[j + CW];
-                    if (j + 2 * CW < n) a2 = first[2] * xs[j + 2 * CW];
-                    if (j + 3 * CW < n) a3 = first[3] * xs[j + 3 * CW];
+                    if (j < n) add(first[0], j, a0);
+                    if (j + CW < n) add(first[1], j + CW, a1);
+                    if (j + 2 * CW < n) add(first[2], j + 2 * CW, a2);
+                    if (j + 3 * CW < n) add(first[3], j + 3 * CW, a3);
                     j += 4 * CW;
                 }
                 for (; j + 3 * CW < n; j += 4 * CW) {
                     const double s0 = __ldcg(p + j * ld), s1 = __ldcg(p + (j + CW) * ld);
                     const double s2 = __ldcg(p + (j + 2 * CW) * ld), s3 = __ldcg(p + (j + 3 * CW) * ld);
-                    a0 = fma(s0, xs[j], a0);
-                    a1 = fma(s1, xs[j + CW], a1);
-                    a2 = fma(s2, xs[j + 2 * CW], a2);
-                    a3 = fma(s3, xs[j + 3 * CW], a3);
+                    add(s0, j, a0);
+                    add(s1, j + CW, a1);
+                    add(s2, j + 2 * CW, a2);
+                    add(s3, j + 3 * CW, a3);
                 }
-                for (; j < n; j += CW) a0 = fma(__ldcg(p + j * ld), xs[j], a0);
+                for (; j < n; j += CW) add(__ldcg(p + j * ld), j, a0);
             }
             a0 = (a0 + a1) + (a2 + a3);
 #pragma unroll
@@ -742,7 +730,7 @@ __global__ void __launch_bounds__(BD_T) k_bidiag(BidiagArgs g) {
                 z0 += rp[((int64_t)q * BD_W + w) * BD_RB + rr];
                 z1 += rp[((int64_t)q * BD_W + w + 1) * BD_RB + rr];
             }
-            const double xi = t2 * fma(-un[i], yv, z0 + z1);
+            const double xi = t2 * (z0 + z1);
             const double ai = fma(-xi, v1, fma(-un[i], y1, __ldcg(W + (k + 1) * ld + i)));
             g.x[i] = xi;
             g.a[i] = ai;
@@ -752,7 +740,7 @@ __global__ void __launch_bounds__(BD_T) k_bidiag(BidiagArgs g) {
             ss = warp_sum(ss);
             __syncwarp();
             bd_fence();
-            publish(2, ss);
+            publish(1, ss);
         }
         double* t = uo;
         uo = un;
@@ -1102,7 +1090,7 @@ rbf_status fsvd_bidiag(rbf_ctx* ctx, const rbf_operator* op, const double* f, Fs
     const size_t need = ws_align((size_t)F->ldw * (n + 1) * 8) + ws_align((size_t)n * n * 8) +
                         ws_align((size_t)(n + 1) * n * 8) + 14 * ws_align((size_t)(n + 2) * 8) +
                         ws_align((size_t)(J > n ? J : n) * 8) + ws_align(8) + ws_align(4) +
-                        ws_align((size_t)3 * G * G * sizeof(ulonglong2)) + ws_align((size_t)3 * QB * G * 8) +
+                        ws_align((size_t)2 * G * G * sizeof(ulonglong2)) + ws_align((size_t)3 * QB * G * 8) +
                         ws_align((size_t)(qchunk + 1) * qblk * QB * QB * 8) + ws_align((size_t)2 * QB * G * 8) +
                         ws_align((size_t)(F->bar_k + 2) * BAR_STRIDE * 4) + svd_ws_bytes(L) + 4096;
     RBF_TRY(rbf_ws_reserve(ctx, need));
@@ -1128,7 +1116,7 @@ rbf_status fsvd_bidiag(rbf_ctx* ctx, const rbf_operator* op, const double* f, Fs
     F->curve = wc.take<double>((size_t)(J > n ? J : n));
     F->sperp = wc.take<double>(1);
     F->r = wc.take<int>(1);
-    ulonglong2* slot = wc.take<ulonglong2>((size_t)3 * G * G);
+    ulonglong2* slot = wc.take<ulonglong2>((size_t)2 * G * G);
     F->hpart = wc.take<double>((size_t)QB * G);
     F->gpart = wc.take<double>((size_t)2 * QB * G);
     F->gram_part = wc.take<double>((size_t)qchunk * qblk * QB * QB);
@@ -1137,7 +1125,7 @@ rbf_status fsvd_bidiag(rbf_ctx* ctx, const rbf_operator* op, const double* f, Fs
     void* svd = (void*)wc.take<char>(svd_ws_bytes(L));
     cudaStream_t s = ctx->stream;
     const size_t bar_bytes = (size_t)(F->bar_k + 2) * BAR_STRIDE * sizeof(unsigned);
-    RBF_CUDA(ctx, cudaMemsetAsync(slot, 0, (size_t)3 * G * G * sizeof(ulonglong2), s));
+    RBF_CUDA(ctx, cudaMemsetAsync(slot, 0, (size_t)2 * G * G * sizeof(ulonglong2), s));
     RBF_CUDA(ctx, cudaMemsetAsync(F->bar, 0, bar_bytes, s));
     RBF_CUDA(ctx, cudaMemsetAsync(&ctx->d_state->info[IN_ERR], 0, 2 * sizeof(int), s));
     RBF_CUDA(ctx, cudaMemsetAsync(F->taur, 0, sizeof(double) * (n + 2), s));
