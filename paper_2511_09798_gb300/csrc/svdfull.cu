@@ -365,9 +365,10 @@ __device__ __forceinline__ double block_sum1(double v, double* red) {
 // Householder reflector of x = [x0; rest], ss = |rest|^2, in the unnormalised
 // form H = I - t w w^T, w = [x0 - beta; rest], H x = beta e_1: t = 1 / (nrm (nrm
 // + |x0|)) with nrm = |x| and beta = -sign(x0) nrm; t = 0 (w_0 = 0, beta = x0)
-// when the rest is zero.  One reciprocal square root and one reciprocal, each
-// an estimate refined to FP64 rounding; out-of-range sums of squares take the
-// library's square root and division.
+// when the rest is zero or |x|^2 no normal number (|x| < 2^-511, what a matrix of
+// low rank leaves after several steps: t would overflow).  One reciprocal square
+// root and one reciprocal, each an estimate refined to FP64 rounding;
+// out-of-range sums of squares take the library's square root and division.
 struct Refl {
     double t, w0, beta;
 };
@@ -382,8 +383,9 @@ __device__ __forceinline__ double rcp_f64(double x) {
 }
 
 __device__ __forceinline__ Refl reflector(double x0, double ss) {
-    if (ss == 0.0) return Refl{0.0, 0.0, x0};
     const double q = fma(x0, x0, ss), ax = fabs(x0);
+    const int qh = __double2hiint(q);  // (integer tests: a comparison would take its turn in the FP64 chain)
+    if (qh < 0x00100000 || (__double2hiint(ss) | __double2loint(ss)) == 0) return Refl{0.0, 0.0, x0};
     double nrm, t;
     if (q > 1e-140 && q < 1e140) {
         nrm = q * rsqrt_f64(q);

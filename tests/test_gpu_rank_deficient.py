@@ -77,3 +77,32 @@ def _check(ctx, R, A):
                                   "diagonal, last zero", "bidiagonal", "equal columns"])
 def test_zero_singular_values(ctx, R, kind, n):
     _check(ctx, R, _matrix(kind, n))
+
+
+@pytest.mark.parametrize("n", [33, 160, 300])
+def test_reflectors_of_roundings(ctx, R, n):
+    """Rank 1 exactly: every step divides what is left by another 1e16, down to
+    columns whose squares underflow."""
+    _check(ctx, R, np.ones((n, n)))
+    _check(ctx, R, np.outer(1.0 + np.arange(n) % 3, 2.0 ** (np.arange(n) % 5)))
+
+
+@pytest.mark.parametrize("k", [-505, -470, 470, 500])
+def test_ends_of_the_range(ctx, R, k):
+    """Norms near the square roots of the smallest and the largest double."""
+    g = np.random.default_rng(2).normal(size=(40, 40))
+    n = 40
+    lda = R.padded_lda(n, R.RBF_FP64)
+    out = []
+    for scale in (1.0, 2.0**k):
+        D = torch.zeros((n, lda), dtype=torch.float64, device="cuda")
+        D[:, :n] = torch.as_tensor(g * scale, device="cuda")
+        op = ctx.rbf_operator_init(torch.zeros((3, n), dtype=torch.float64, device="cuda"), n, n // 2, 1.0, 1.0, A=D,
+                                   lda=lda)
+        sig = torch.empty(n, dtype=torch.float64, device="cuda")
+        V = torch.empty((n, n), dtype=torch.float64, device="cuda")
+        ctx.rbf_svd_full(op, sig, None, None, V)
+        V = V.cpu().numpy()
+        assert np.max(np.abs(V @ V.T - np.eye(n))) <= 40 * n * EPS / 1e-3
+        out.append(sig.cpu().numpy() / scale)
+    assert np.max(np.abs(out[0] - out[1])) <= 8 * n * EPS * out[0][0]
