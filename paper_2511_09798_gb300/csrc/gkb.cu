@@ -190,18 +190,11 @@ struct HalfNorm {
     bool nonfinite;
 };
 
-// FAST: the square roots and the inverse from refined reciprocal square roots
-// (a third of the chain's latency, results within an ulp or two) where the sums
-// of squares are far from the ends of FP64's range.
-template <bool FAST>
 __device__ __forceinline__ HalfNorm half_norm(const HalfArgs& a, double acc) {
     const double* sc = a.stt->scal;
     const double eps = DBL_EPSILON;
-    auto mid = [](double x) { return x > 1e-200 && x < 1e200; };
     HalfNorm h;
-    const bool fast = FAST && mid(acc);
-    const double rs = fast ? rsqrt_f64(acc) : 0.0;
-    h.nrm = fast ? acc * rs : sqrt(acc);
+    h.nrm = sqrt(acc);
     h.brk = 0;
     // c_hat double buffer: the r-side of step j reads slot j&1, writes (j+1)&1;
     // the p-side of step j reads slot (j+1)&1
@@ -215,15 +208,14 @@ __device__ __forceinline__ HalfNorm half_norm(const HalfArgs& a, double acc) {
     } else if (a.j == 1) {
         h.brk = h.nrm > 0.0 ? 0 : 1;
     } else {
-        const double al = a.alpha[a.j - 2], c2 = fma(al, al, acc);
-        h.ch_new = fmax(ch_old, fast && mid(c2) ? c2 * rsqrt_f64(c2) : hypot(al, h.nrm));
+        h.ch_new = fmax(ch_old, hypot(a.alpha[a.j - 2], h.nrm));
         h.brk = h.nrm <= a.factor * (double)a.n * eps * h.ch_new ? 2 : 0;
     }
     // a norm that is not finite stops the run like a breakdown of the same
     // side (code 3): NaN or Inf in f, the nodes or the operator
     h.nonfinite = !isfinite(h.nrm);
     if (h.nonfinite) h.brk = (a.side == 1 || a.j == 1) ? 1 : 2;
-    h.inv = a.resume ? 1.0 : (fast ? rs : 1.0 / h.nrm);
+    h.inv = a.resume ? 1.0 : 1.0 / h.nrm;
     return h;
 }
 
@@ -313,7 +305,7 @@ __global__ void __launch_bounds__(SL_THREADS) k_half(HalfArgs a) {
     __syncthreads();
     // ---- norm, inverse and breakdown test: one thread of the last warp
     if (threadIdx.x == SL_THREADS - 32) {
-        const HalfNorm h = half_norm<false>(a, acc_s);
+        const HalfNorm h = half_norm(a, acc_s);
         inv_s = h.inv;
         brk_s = h.brk;
         if (blockIdx.x == 0) half_state(a, h);
@@ -516,7 +508,7 @@ __global__ void __launch_bounds__(HC_T) k_half_cluster(HalfArgs a) {
         acc = warp_sum(acc);
         if (lane == 0) {
             acc_s = acc;
-            if (!done) norm_s = half_norm<true>(a, acc);
+            if (!done) norm_s = half_norm(a, acc);
         }
     }
     // the basis in fixed point (a thread converts what it copied)
