@@ -15,17 +15,20 @@
 //   - sqrt(s): FP32 estimate R0 = s rsqrt(s); with the exact residual e0 = s - R0^2,
 //     R1 = 2^12 R0 + round(2^12 e0 rsqrt(s) / 2); with the residual e1 = 2^24 s -
 //     R1^2, small enough to be taken modulo 2^64, N = 2^19 R1 + round(2^19 e1 rsqrt(s) /
-//     2^13): |N - 2^31 sqrt(s)| is under 9 units, 2^-57.8 of the largest Phi and 2^-53 of
-//     the smallest that the rule below admits;
-//   - the coefficients are rounded at 2^-62 of the largest of the CTA's chunk and
-//     the products N coef are added in 64-bit integers (FxAcc32), then rounded to
-//     FP64 once per chunk.
-// Every error is at most about 2^-58 of the largest Phi times the coefficients,
-// below the roundings of the FP64 form (an ulp or two per term and the sum's), so
-// long as c is not tiny beside the coordinates: an exponent at most 5 below the
-// largest (at 6 below the smallest Phi would carry 2^-51.4 relative).  Below
-// that, and with any Inf or NaN, a CTA takes the FP64 form (a first launch finds
-// the coordinates' largest exponent, the CTA its coefficients').
+//     2^13): |N - 2^31 sqrt(s)| is at most 1 unit (0.8 from N = 2^54 on, 0.3 in the root
+//     mean square) wherever the rule below admits;
+//   - the coefficients are rounded at 2^-62 of the largest of a stage of 128 nodes
+//     and the products N coef are added in 64-bit integers (FxAcc32), then
+//     rounded to FP64 once per stage (one scale for all the nodes of a CTA loses more
+//     of the small coefficients, and its sums live through the whole kernel: 1.59 ms at
+//     20 000 points and nodes instead of 1.53).
+// What that is relative to Phi depends on the smallest N, 2^53 where c is smallest
+// beside the coordinates: Phi is good to 2^-53 there, to 2^-61 where it is as large
+// as they are; a stage's sum to FxAcc32's error.  c may be smaller than the
+// largest coordinate by an exponent of at most 5 (at 6 Phi would be good to 2^-51.4).
+// Below that, and with any Inf or NaN, a CTA takes the FP64 form (a first launch
+// finds the coordinates' largest exponent, the CTA whether its coefficients are
+// finite).
 #include "common.cuh"
 #include "fx_core.cuh"
 #include "internal.h"
@@ -34,7 +37,6 @@ namespace {
 
 constexpr int EV_T = 128;           // points per CTA, one per thread; nodes per stage
 constexpr int EV_MIN_CHUNK = 64;     // nodes per CTA
-constexpr int EV_MAX_CHUNK = 1 << 19;  // nodes per CTA: the folded sums stay below 2^52
 constexpr int EX_CTAS = 64;         // partial maxima of the exponent scan
 
 // Largest exponent field of the nodes' and points' coordinates, one partial per CTA.
@@ -128,20 +130,33 @@ __global__ void __launch_bounds__(EV_T) k_evaluate(const double* __restrict__ X,
         const int k = 1082 - es;
         const long long ux = fx_round(px, k), uy = fx_round(py, k), uz = fx_round(pz, k), qc = fx_round(c, k);
         const int lc = (int)qc, hc = (int)(qc >> 32) - (lc >> 31);
+        auto stage_exp = [&](int q) {
+            int e = 1;
+#pragma unroll
+            for (int w = 0; w < EV_T / 32; ++w) e = max(e, red[w][q]);
+            return e;
+        };
         const long long hh0 = imad_wide(hc, hc, 0), hl0 = imad_wide(hc, lc, imad_wide(lc, lc, 0) >> 33);
-        FxAcc32 acc[NC];
+#pragma unroll
+        for (int q = 0; q < NC; ++q) res[q] = 0.0;
         for (int64_t jb = j0; jb < j1; jb += EV_T) {
+            FxAcc32 acc[NC];
             __syncthreads();
             const int64_t j = jb + threadIdx.x;
             const bool ok = j < j1;
             qx[threadIdx.x] = ok ? fx_round(X[j], k) : 0;
             qy[threadIdx.x] = ok ? fx_round(X[n + j], k) : 0;
             qz[threadIdx.x] = ok ? fx_round(X[2 * n + j], k) : 0;
+            double cf[NC];
 #pragma unroll
-            for (int q = 0; q < NC; ++q)
-                qa[q][threadIdx.x] = ok && q < nc ? fx_split(fx_round(coefs[(int64_t)(c0 + q) * ldc + j],
-                                                                      1084 - max(ev[q], 1)))
-                                                  : make_int2(0, 0);
+            for (int q = 0; q < NC; ++q) {
+                cf[q] = ok && q < nc ? coefs[(int64_t)(c0 + q) * ldc + j] : 0.0;
+                const int e = __reduce_max_sync(RBF_FULL_MASK, fx_exp(cf[q]));
+                if (lane == 0) red[warp][q] = e;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < NC; ++q) qa[q][threadIdx.x] = fx_split(fx_round(cf[q], 1084 - stage_exp(q)));
             __syncthreads();
             const int cnt = (int)min((int64_t)EV_T, j1 - jb);
             for (int rb = 0; rb < cnt; rb += FX_FOLD) {
@@ -158,9 +173,10 @@ __global__ void __launch_bounds__(EV_T) k_evaluate(const double* __restrict__ X,
 #pragma unroll
                 for (int q = 0; q < NC; ++q) acc[q].fold();
             }
-        }
 #pragma unroll
-        for (int q = 0; q < NC; ++q) res[q] = ldexp(FxAcc32::value(acc[q].pair(j1 - j0)), 65 - k - (1084 - max(ev[q], 1)));
+            for (int q = 0; q < NC; ++q)
+                res[q] += ldexp(FxAcc32::value(acc[q].pair(cnt)), 65 - k - (1084 - stage_exp(q)));
+        }
     } else {
         const double c2 = c * c;
         const bool far = ec < 1023 - 490 || es > 1023 + 490;  // s may leave the normal numbers
@@ -213,7 +229,6 @@ rbf_status evaluate_vectors(rbf_ctx* ctx, const rbf_operator* op, const double* 
     int64_t chunks = (int64_t)ctx->sm_count * per_sm / (tiles * zs);
     chunks = chunks < 1 ? 1 : chunks;
     if ((n + chunks - 1) / chunks < EV_MIN_CHUNK) chunks = (n + EV_MIN_CHUNK - 1) / EV_MIN_CHUNK;
-    if ((n + chunks - 1) / chunks > EV_MAX_CHUNK) chunks = (n + EV_MAX_CHUNK - 1) / EV_MAX_CHUNK;
     if (chunks > 65535) chunks = 65535;
     const int64_t chunk = (n + chunks - 1) / chunks;
     chunks = (n + chunk - 1) / chunk;
