@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(EV_T) k_evaluate(const double* __restrict__ X,
             }
 #pragma unroll
             for (int q = 0; q < NC; ++q)
-                res[q] += ldexp(FxAcc32::value(acc[q].pair(cnt)), 65 - k - (1084 - stage_exp(q)));
+                res[q] += ldexp(FxAcc32::value(acc[q].pair(cnt)), FX_UNIT + 1 - k - (1084 - stage_exp(q)));
         }
     } else {
         const double c2 = c * c;

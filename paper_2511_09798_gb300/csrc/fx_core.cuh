@@ -71,19 +71,24 @@ struct FxAcc {
     }
 };
 
-// Sum of products N Z in units of 2^64, both split into a high and a signed 32-bit
-// low part, |N| < 2^61 and |Z| < 2^62 (so |n1| <= 2^29 and |z1| <= 2^30).  n1 z1
-// goes to c, which holds FX_FOLD terms of at most 2^59 + 2^32 before it is folded;
-// the cross products, below 2^62 together and made positive by FX_BIAS, add their
-// upper word to c and carry their lower word into the next term.  n0 z0 (under a
-// quarter of a unit, either sign) is left out: an error of at most n / 4 units of
-// 2^-59 of the largest term.  Three wide products per term where 21-bit limbs
-// that accumulate without folds take six: those bound the reconstruction of 8
-// vectors (the pipe of the wide products 63 % busy): 816 -> 608 us for 150
-// vectors, 8000 nodes and 500 points, 1.70 -> 1.59 ms for one vector and 20 000
-// nodes and points.  (16 vectors per CTA: no gain, 12 warps per SM.)
+// Sum of products N Z, both split into a high and a signed 32-bit low part, |N| <
+// 2^61 and |Z| < 2^62 (so |n1| <= 2^29 and |z1| <= 2^30).  n1 z1 goes to c (units of
+// 2^64), which holds FX_FOLD terms of at most 2^59 + 2^32 before it is folded; the
+// cross products, below 2^62 together and made positive by FX_BIAS, add their
+// upper word to c and carry their lower word into the next term and, after the
+// last, into the result.  n0 z0 is left out: an error of at most a quarter of a
+// unit of 2^64 per term, of either sign (a twelfth in the root mean square).  What
+// that is relative to a term depends on how large N and Z are: 2^-61 for N = 2^61
+// and Z = 2^62, 2^-52 for N = 2^53 and Z = 2^61.  Three wide
+// products per term where 21-bit limbs that accumulate without folds take six:
+// those bound the reconstruction of 8 vectors (the pipe of the wide products 63 %
+// busy): 816 -> 608 us for 150 vectors, 8000 nodes and 500 points, 1.70 -> 1.59 ms
+// for one vector and 20 000 nodes and points (a fourth for the upper half of n0 z0
+// 1.68 ms, and a solve with 2161 rows and 140 steps 8.94 -> 9.28 ms).  (16 vectors
+// per CTA: no gain, 12 warps per SM.)
 constexpr int FX_FOLD = 8;
 constexpr unsigned FX_BIAS = 1u << 30;  // in the upper word
+constexpr int FX_UNIT = 44;             // the result's low part is in units of 2^FX_UNIT
 
 struct FxAcc32 {
     long long c = 0, hi = 0, lo = 0;  // value c + hi 2^32 + lo
@@ -99,12 +104,13 @@ struct FxAcc32 {
         lo += (long long)((unsigned long long)c & 0xffffffffu);
         c = 0;
     }
-    // (folded) the value as h 2^32 + l; such pairs add
+    // (folded) the sum of up to 2^12 terms as h 2^96 + l 2^FX_UNIT; such pairs add
     __device__ __forceinline__ longlong2 pair(int64_t terms) const {
-        return make_longlong2(hi, lo - terms * (long long)FX_BIAS);
+        return make_longlong2(hi, ((lo - terms * (long long)FX_BIAS) << (64 - FX_UNIT)) | (rem >> (FX_UNIT - 32)));
     }
+    // a pair in units of 2^FX_UNIT
     static __device__ __forceinline__ double value(longlong2 p) {
-        return fma((double)p.x, 0x1p32, (double)p.y);
+        return fma((double)p.x, 0x1p52, (double)p.y);
     }
 };
 

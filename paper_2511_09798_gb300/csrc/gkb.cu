@@ -576,7 +576,7 @@ __global__ void __launch_bounds__(HC_T) k_half_cluster(HalfArgs a) {
             p.x += sch[slot + k * step];
             p.y += sch[HC_T + slot + k * step];
         }
-        return s == FX_NONFINITE ? fx_nan() : ldexp(FxAcc32::value(p), 4 - s);
+        return s == FX_NONFINITE ? fx_nan() : ldexp(FxAcc32::value(p), FX_UNIT - 60 - s);
     };
     __syncthreads();
     if (threadIdx.x < R) {

@@ -61,3 +61,30 @@ def test_small_coefficients_beside_cancelling_ones(ctx, R):
     phi = np.sqrt((d * d).sum(-1) + L(0.2) * L(0.2))
     ref, mag = phi @ co[128:].astype(L), phi @ np.abs(co[128:]).astype(L)
     assert np.all(np.abs(u[:200].cpu().numpy() - ref) <= 4 * 2.0**-53 * mag)
+
+
+@pytest.mark.parametrize("n", [1, 2, 63])
+@pytest.mark.parametrize("ratio", [2.0**-4.99, 2.0**-4, 0.4])
+def test_one_term(ctx, R, n, ratio):
+    """One coefficient of 1 (the others zero): the term itself, and no more roundings
+    than those of the stage and of the sum over the partials."""
+    rng = np.random.default_rng(2)
+    X = rng.uniform(-0.9, 0.9, (n, 3))
+    X[-1] = 0.9
+    P = X[-1] + 1e-3 * rng.normal(size=(500, 3))
+    co = np.zeros(n)
+    co[-1] = 1.0
+    c = 0.5 * ratio  # the coordinates are in [0.5, 1)
+    u, ref, _ = _eval(ctx, R, X, P, co, c)
+    edge = 2.0**-5 / ratio  # 2^53 / N0
+    assert np.all(np.abs(u - ref) <= 2.0**-53 * (1 + 3 * edge) * ref)
+
+
+@pytest.mark.parametrize("where,size,c", [(10.0, 0.5, 0.5), (1.0, 0.01, 1 / 32), (-3.0, 1.0, 0.13)])
+def test_domain_off_the_origin(ctx, R, where, size, c):
+    rng = np.random.default_rng(3)
+    X, P = where + size * rng.uniform(-1, 0, (3000, 3)), where + size * rng.uniform(-1, 0, (140, 3))
+    u, ref, mag = _eval(ctx, R, X, P, rng.normal(size=3000), c)
+    # per term the bound at the edge of the rule, a rounding per stage and per partial
+    # of sums that are well below the sum of magnitudes
+    assert np.all(np.abs(u - ref) <= 2.0**-53 * 4 * mag)
