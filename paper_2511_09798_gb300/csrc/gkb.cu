@@ -448,12 +448,18 @@ constexpr int HC_T = 512;
 constexpr int HC_SPLIT = 16;  // most threads per basis vector in the dot products
 // Slabs of Q of at least this many entries: the dot products and updates in
 // 64-bit fixed point (fx_core.cuh) on the integer pipes instead of 2 FP64 FMAs per
-// clock on each of the 16 SMs.  Q is rounded at 2^-61 (its columns have norm 1;
-// below 2^-53 of a typical entry), v and the products h at 2^-61 of their largest; sums are
-// exact to 2^-59 of the largest term.  The conversions and scales cost 2 us per
-// half-step, what about 2800 entries cost in FP64: 1000 rows and up to 40 vectors
-// 14.1 us in FP64, 16.1 in fixed point; 2161 rows and 140 steps, a solve 10.08 -> 9.22 ms.
-// FP64 also where an entry of Q is 2 or more (a caller's own basis).
+// clock on each of the 16 SMs.  Q is rounded at 2^-62 of the largest entry of each
+// row, v (times that entry's power of two) and the products h at 2^-61 of their
+// largest, and FxAcc32 leaves out up to 2^-59: a term is off by at most 2^-58 of the
+// largest |Q_im v_i| of the CTA in a dot product, of the largest |Q_im h_m| of its row in
+// an update (2^-60 in the root mean square, signs random), where every FMA rounds at
+// 2^-53 of its sum.  The scale by rows keeps rows of different size apart as FP64
+// does.  Over 48 problems each the basis and the coefficients are half as far from
+// extended precision as with the FP64 grid form (n = 2161, 140 steps: W 0.47, alpha 0.51
+// of its error; 2000, 60: 0.53 and 0.68; geometric means, standard errors 1.13).  The
+// conversions and scales cost 2 us per half-step, what about 2800 entries cost in
+// FP64: 1000 rows and up to 40 vectors 14.1 us in FP64, 16.1 in fixed point; 2161 rows
+// and 140 steps, a solve 10.08 -> 8.92 ms.  FP64 also where an entry of Q is not finite.
 constexpr int HC_FX_MIN = 4096;
 
 struct HalfClusterSmem {  // offsets in doubles
@@ -477,6 +483,7 @@ __global__ void __launch_bounds__(HC_T) k_half_cluster(HalfArgs a) {
     extern __shared__ double dsm[];
     __shared__ double red[HC_T / 32];
     __shared__ int rede[HC_T / 32];
+    __shared__ int rowe[HC_T];  // largest exponent of each row of Q
     __shared__ double acc_s;
     __shared__ HalfNorm norm_s;
     cg::cluster_group cluster = cg::this_cluster();
@@ -511,24 +518,27 @@ __global__ void __launch_bounds__(HC_T) k_half_cluster(HalfArgs a) {
             if (!done) norm_s = half_norm(a, acc);
         }
     }
-    // the basis in fixed point (a thread converts what it copied)
-    cp_async_wait_all();
-    const bool large = M * RM >= HC_FX_MIN && M <= HC_T;
-    int big = large ? 0 : 2047;
-    for (int m = warp; large && m < M; m += HC_T / 32)
-        for (int i = lane; i < R; i += 32) big = max(big, fx_exp(Qs[(size_t)m * RM + i]));
-    const bool fx = !__syncthreads_or(big > 1023);  // |q| < 2, finite
-    if (fx)
-        for (int m = warp; m < M; m += HC_T / 32)
-            for (int i = lane; i < R; i += 32) {
-                const size_t e = (size_t)m * RM + i;
-                Qx[e] = fx_split(fx_round(Qs[e], 60));
-            }
-    pdl_wait();
-    // ---- sums of the product partials: thread (row, group of chunks)
     const int RP = max(32, (R + 31) & ~31);  // at most HC_T (n <= HC_MAX_N)
     const int ng = HC_T / RP;
     const int row = threadIdx.x % RP, grp = threadIdx.x / RP;
+    // the basis in fixed point, each row at its largest exponent
+    const bool large = M * RM >= HC_FX_MIN && M <= HC_T;
+    rowe[threadIdx.x] = 1;
+    cp_async_wait_all();
+    __syncthreads();
+    int big = large ? 1 : FX_NONFINITE;
+    if (large && row < R)
+        for (int m = grp; m < M; m += ng) big = max(big, fx_exp(Qs[(size_t)m * RM + row]));
+    if (large && row < R && grp < ng) atomicMax(&rowe[row], big);
+    const bool fx = !__syncthreads_or(big == FX_NONFINITE);
+    const int sq = 1084 - rowe[row];  // Q's row 2^sq is below 2^62
+    if (fx && row < R && grp < ng)
+        for (int m = grp; m < M; m += ng) {
+            const size_t e = (size_t)m * RM + row;
+            Qx[e] = fx_split(fx_round(Qs[e], sq));
+        }
+    pdl_wait();
+    // ---- sums of the product partials: thread (row, group of chunks)
     if (grp < ng) {
         double t[4] = {0.0, 0.0, 0.0, 0.0};
         if (row < R) {
@@ -570,13 +580,14 @@ __global__ void __launch_bounds__(HC_T) k_half_cluster(HalfArgs a) {
         sch[slot] = p.x;
         sch[HC_T + slot] = p.y;
     };
-    auto fixed_total = [&](int slot, int step, int cnt, int s) -> double {
+    // (e: the exponent of the sums' unit)
+    auto fixed_total = [&](int slot, int step, int cnt, int s, int e) -> double {
         longlong2 p = make_longlong2(0, 0);
         for (int k = 0; k < cnt; ++k) {
             p.x += sch[slot + k * step];
             p.y += sch[HC_T + slot + k * step];
         }
-        return s == FX_NONFINITE ? fx_nan() : ldexp(FxAcc32::value(p), FX_UNIT - 60 - s);
+        return s == FX_NONFINITE ? fx_nan() : ldexp(FxAcc32::value(p), e - s);
     };
     __syncthreads();
     if (threadIdx.x < R) {
@@ -590,14 +601,16 @@ __global__ void __launch_bounds__(HC_T) k_half_cluster(HalfArgs a) {
     while (split < HC_SPLIT && 2 * split * M <= HC_T) split *= 2;
     for (int pass = 0; pass < 2 && M > 0; ++pass) {
         if (fx) {
-            const int sv = to_fixed(threadIdx.x < R ? vs[threadIdx.x] : 0.0, vx, R);
+            // v times the powers of two of its rows of Q: 2^(61 - sq)
+            const int sv =
+                to_fixed(threadIdx.x < R ? vs[threadIdx.x] * __hiloint2double((1084 - sq) << 20, 0) : 0.0, vx, R);
             if (threadIdx.x < split * M) {
                 const int k = threadIdx.x / M, m = threadIdx.x - k * M;
                 fixed_sum(vx + k, split, Qx + (size_t)m * RM + k, split,
                           sv == FX_NONFINITE || k >= R ? 0 : (R - k + split - 1) / split, threadIdx.x);
             }
             __syncthreads();
-            if (threadIdx.x < M) hp[pass * M + threadIdx.x] = fixed_total(threadIdx.x, M, split, sv);
+            if (threadIdx.x < M) hp[pass * M + threadIdx.x] = fixed_total(threadIdx.x, M, split, sv, FX_UNIT - 61);
         } else {
             for (int p = threadIdx.x; p < split * M; p += HC_T) {
                 const int k = p / M, m = p - k * M;
@@ -645,7 +658,7 @@ __global__ void __launch_bounds__(HC_T) k_half_cluster(HalfArgs a) {
                 fixed_sum(hx + grp, ng, Qx + (size_t)grp * RM + row, ng * RM,
                           sh == FX_NONFINITE || row >= R || grp >= M ? 0 : (M - grp + ng - 1) / ng, grp * RP + row);
             __syncthreads();
-            if (threadIdx.x < R) vs[threadIdx.x] -= fixed_total(threadIdx.x, RP, ng, sh);
+            if (threadIdx.x < R) vs[threadIdx.x] -= fixed_total(threadIdx.x, RP, ng, sh, FX_UNIT - sq);
             __syncthreads();
             continue;
         }
