@@ -422,6 +422,8 @@ int fx_t_chunks(const rbf_ctx* ctx, int64_t n) {
     return ch;
 }
 
+bool fx_n_by_rows(const rbf_ctx* ctx, int64_t n) { return fxn_row_warps(ctx, n) > 0; }
+
 int fx_n_chunks(const rbf_ctx* ctx, int64_t n) {
     if (fxn_row_warps(ctx, n)) return 1;
     int g, ch;

@@ -483,7 +483,6 @@ __global__ void __launch_bounds__(HC_T) k_half_cluster(HalfArgs a) {
     extern __shared__ double dsm[];
     __shared__ double red[HC_T / 32];
     __shared__ int rede[HC_T / 32];
-    __shared__ int rowe[HC_T];  // largest exponent of each row of Q
     __shared__ double acc_s;
     __shared__ HalfNorm norm_s;
     cg::cluster_group cluster = cg::this_cluster();
@@ -523,16 +522,20 @@ __global__ void __launch_bounds__(HC_T) k_half_cluster(HalfArgs a) {
     const int row = threadIdx.x % RP, grp = threadIdx.x / RP;
     // the basis in fixed point, each row at its largest exponent
     const bool large = M * RM >= HC_FX_MIN && M <= HC_T;
-    rowe[threadIdx.x] = 1;
+    int* rowe = (int*)vs;  // [R] its exponents, until v takes the place
+    if (threadIdx.x < R) rowe[threadIdx.x] = 1;
     cp_async_wait_all();
     __syncthreads();
     int big = large ? 1 : FX_NONFINITE;
-    if (large && row < R)
+    if (large && row < R) {
+#pragma unroll 8
         for (int m = grp; m < M; m += ng) big = max(big, fx_exp(Qs[(size_t)m * RM + row]));
-    if (large && row < R && grp < ng) atomicMax(&rowe[row], big);
+        if (grp < ng) atomicMax(&rowe[row], big);
+    }
     const bool fx = !__syncthreads_or(big == FX_NONFINITE);
-    const int sq = 1084 - rowe[row];  // Q's row 2^sq is below 2^62
+    const int sq = row < R ? 1084 - rowe[row] : 0;  // Q's row 2^sq is below 2^62
     if (fx && row < R && grp < ng)
+#pragma unroll 4
         for (int m = grp; m < M; m += ng) {
             const size_t e = (size_t)m * RM + row;
             Qx[e] = fx_split(fx_round(Qs[e], sq));
@@ -799,6 +802,12 @@ static size_t half_smem_bytes(bool stage, int mcount, int chunks, int rmax, bool
 constexpr int64_t HC_MAX_N = (int64_t)HC_CTAS * HC_T;
 constexpr int64_t HC_WORK = 416 * 1024;
 constexpr size_t HC_SMEM_MAX = 220 * 1024;
+// Least shared memory of a cluster where A z runs by the flat split (n above about
+// 4900, up to 98 KB per CTA): enough that none of another lane's CTAs of that product
+// joins it on its SMs.  Six runs of 100 steps with and without: n = 6000 64.7 and 66.7
+// ms, 7000 (80 steps) 65.8 and 67.0, 8000 102.6 and 104.2 (26 steps alone 27.7 and 27.2);
+// 5000 48.7 and 48.9.  Below, sharing is the better one: 4000, 60 steps 18.6 and 18.1.
+constexpr size_t HC_SMEM_APART = 140 * 1024;
 constexpr long long HC_MIN_BUDGET = 4096;
 
 static bool half_cluster_takes(const rbf_ctx* ctx, int64_t n, int mcount, bool mixed) {
@@ -1051,8 +1060,9 @@ struct GkbRun {
         a.budget = ctx->opt.wait_budget;
         if (half_cluster_takes(ctx, n, mcount, mixed) && half_cluster_ready(ctx)) {
             a.rmax = (int)((n + HC_CTAS - 1) / HC_CTAS) | 1;
-            const size_t smem = sizeof(double) * (size_t)half_cluster_smem(mcount, a.rmax).total;
+            size_t smem = sizeof(double) * (size_t)half_cluster_smem(mcount, a.rmax).total;
             if (smem <= HC_SMEM_MAX) {
+                if (use_fx && !fx_n_by_rows(ctx, n)) smem = std::max(smem, HC_SMEM_APART);
                 const int slot = rbf_prod_begin(ctx, 2);
                 const cudaError_t e = rbf_launch_ex(ctx, k_half_cluster, dim3(HC_CTAS), dim3(HC_T), smem, pdl_ok,
                                                     HC_CTAS, a);

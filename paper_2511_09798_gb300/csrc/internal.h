@@ -264,6 +264,7 @@ size_t fx_ws_bytes(const rbf_operator* op);
 FxCopies fx_carve(WsCarve& wc, const rbf_operator* op);
 int fx_n_chunks(const rbf_ctx* ctx, int64_t n);  // partial rows of the fixed-point A z (<= 8)
 int fx_t_chunks(const rbf_ctx* ctx, int64_t n);  // and of A^T w
+bool fx_n_by_rows(const rbf_ctx* ctx, int64_t n);  // A z by rows instead of the flat split
 rbf_status launch_fx_prepare(rbf_ctx* ctx, const rbf_operator* op, const FxCopies& f);
 // pdl: launched with programmatic stream serialization after the kernel before
 rbf_status launch_fx_n(rbf_ctx* ctx, const rbf_operator* op, const FxCopies& f, const double* x, double* part,
