@@ -84,6 +84,29 @@ __device__ __forceinline__ long long eval_phi(long long dx, long long dy, long l
     return (R1 << 19) + (b2 - 0x4B400000);
 }
 
+// u = sum of the chunks' partials, from 16 on in eight chains (a serial sum rounds once
+// per chunk at the size of a large early partial).
+__global__ void __launch_bounds__(256) k_eval_reduce(int64_t total, int chunks, const double* __restrict__ part,
+                                                     double* __restrict__ u) {
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (i >= total) return;
+    if (chunks < 16) {
+        double s = 0.0;
+        for (int q = 0; q < chunks; ++q) s += part[(int64_t)q * total + i];
+        u[i] = s;
+        return;
+    }
+    double t[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    int q = 0;
+    for (; q + 7 < chunks; q += 8)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) t[e] += part[(int64_t)(q + e) * total + i];
+#pragma unroll
+    for (int e = 0; e < 7; ++e)
+        if (q + e < chunks) t[e] += part[(int64_t)(q + e) * total + i];
+    u[i] = ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
+}
+
 // Partials over the centre chunk blockIdx.y for the NC vectors blockIdx.z NC ..:
 // part[chunk][vector][t].
 template <int NC>
@@ -212,6 +235,31 @@ __global__ void __launch_bounds__(EV_T) k_evaluate(const double* __restrict__ X,
             if (q < nc) part[((int64_t)blockIdx.y * ncoef + c0 + q) * m + t] = res[q] * scale;
 }
 
+// Centre chunks for `ctas` CTAs per chunk.  At most one wave of resident CTAs (the
+// chains of a pair need all the warps that fit: 8 CTAs per SM took 5 % longer than a
+// full wave at 20 000 points and nodes) and at least 64 nodes each; among these down to
+// 3/4 as many (up to eight per point tile where one wave holds a single one), the number that fills
+// the SMs most evenly: ceil(CTAs per SM) times a CTA's nodes and its fixed part,
+// about 24 nodes.  One full wave against this, 8000 nodes: 500 points and 150 vectors 612
+// and 551 us, 8 vectors 70 and 60 (in FP64 199 and 171), 20 000 points and 17 vectors 4.69 and
+// 3.13 ms (21.4 and 17.3).
+int64_t eval_chunks(int64_t n, int64_t ctas, int64_t sms, int64_t per_sm) {
+    int64_t top = sms * per_sm / ctas;
+    if (top < 2) top = 8;
+    const int64_t most = (n + EV_MIN_CHUNK - 1) / EV_MIN_CHUNK;
+    if (top > most) top = most;
+    int64_t low = sms * per_sm / ctas < 2 ? 1 : (3 * top + 3) / 4;
+    int64_t best = top, least = INT64_MAX;
+    for (int64_t c = top; c >= low; --c) {
+        const int64_t cost = (ctas * c + sms - 1) / sms * ((n + c - 1) / c + 24);
+        if (cost < least) {
+            least = cost;
+            best = c;
+        }
+    }
+    return best;
+}
+
 rbf_status evaluate_vectors(rbf_ctx* ctx, const rbf_operator* op, const double* coefs, int64_t ldc, int ncoef,
                             const double* pts, int64_t m, double* u) {
     const int64_t n = op->n;
@@ -219,16 +267,11 @@ rbf_status evaluate_vectors(rbf_ctx* ctx, const rbf_operator* op, const double* 
     // vectors per CTA: the smallest of 1, 2, 4, 8 that holds them all (8 beyond)
     const int nc = ncoef <= 1 ? 1 : ncoef <= 2 ? 2 : ncoef <= 4 ? 4 : 8;
     const int zs = (ncoef + nc - 1) / nc;
-    // one wave of resident CTAs, chunks of at least 64 nodes (the chains of a
-    // pair need all the warps that fit: 8 CTAs per SM took 5 % longer than a full wave at
-    // 20 000 points and nodes)
     const void* kern = nc == 1 ? (const void*)k_evaluate<1> : nc == 2 ? (const void*)k_evaluate<2>
                        : nc == 4 ? (const void*)k_evaluate<4> : (const void*)k_evaluate<8>;
     int per_sm = 0;
     RBF_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, EV_T, 0));
-    int64_t chunks = (int64_t)ctx->sm_count * per_sm / (tiles * zs);
-    chunks = chunks < 1 ? 1 : chunks;
-    if ((n + chunks - 1) / chunks < EV_MIN_CHUNK) chunks = (n + EV_MIN_CHUNK - 1) / EV_MIN_CHUNK;
+    int64_t chunks = eval_chunks(n, tiles * zs, ctx->sm_count, per_sm);
     if (chunks > 65535) chunks = 65535;
     const int64_t chunk = (n + chunks - 1) / chunks;
     chunks = (n + chunk - 1) / chunk;
@@ -250,7 +293,9 @@ rbf_status evaluate_vectors(rbf_ctx* ctx, const rbf_operator* op, const double* 
     else EV_LAUNCH(8);
 #undef EV_LAUNCH
     RBF_LAUNCHED(ctx, "k_evaluate");
-    return launch_reduce_partials(ctx, total, (int)chunks, part, u);
+    k_eval_reduce<<<(unsigned)((total + 255) / 256), 256, 0, ctx->stream>>>(total, (int)chunks, part, u);
+    RBF_LAUNCHED(ctx, "k_eval_reduce");
+    return RBF_OK;
 }
 
 }  // namespace

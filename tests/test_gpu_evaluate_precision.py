@@ -88,3 +88,21 @@ def test_domain_off_the_origin(ctx, R, where, size, c):
     # per term the bound at the edge of the rule, a rounding per stage and per partial
     # of sums that are well below the sum of magnitudes
     assert np.all(np.abs(u - ref) <= 2.0**-53 * 4 * mag)
+
+
+@pytest.mark.parametrize("n,m,q", [(1, 70000, 1), (65, 70000, 9), (515, 70000, 17), (20001, 3, 1), (1025, 257, 2)])
+def test_chunks(ctx, R, n, m, q):
+    """Both ends of the rule for the centre chunks: more CTAs than one wave holds, and
+    hundreds of chunks for a few points."""
+    rng = np.random.default_rng(n)
+    X, P, co = rng.uniform(0, 1, (n, 3)), rng.uniform(0, 1, (m, 3)), rng.normal(size=(q, n))
+    op = ctx.rbf_operator_init(_dev(X.T), n, n // 2, 0.2, 1.0, R.RBF_MATRIX_FREE, R.RBF_MIXED)
+    u = torch.full((q, m), float("nan"), dtype=torch.float64, device="cuda")
+    ctx.rbf_evaluate_many(op, _dev(co), n, q, _dev(P.T), m, u)
+    assert torch.isfinite(u).all()
+    at = rng.choice(m, min(m, 40), replace=False)
+    L = np.longdouble
+    d = P[at][:, None, :].astype(L) - X[None].astype(L)
+    phi = np.sqrt((d * d).sum(-1) + L(0.2) * L(0.2))
+    ref, mag = co.astype(L) @ phi.T, np.abs(co).astype(L) @ phi.T
+    assert np.all(np.abs(u.cpu().numpy()[:, at] - ref) <= 4 * 2.0**-53 * mag)
