@@ -23,15 +23,15 @@ __device__ __forceinline__ float gelu_grad_f(float z) {
     return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * expf(-0.5f * z * z) * 0.39894228040143268f;
 }
 
-// Forward pass and, with TRAIN, the activation gradients of TS samples per CTA
-// of 256 threads: thread (half, j) owns hidden unit j for the samples [half TS /
+// Forward pass and, with TRAIN, the activation gradients of TS samples at a time by
+// CTAs of 256 threads: thread (half, j) owns hidden unit j for the samples [half TS /
 // 2, (half + 1) TS / 2).  W2 sits in shared memory for both directions (rows of
-// W2_LD floats: conflict-free reads along a row by 16 bytes and down a column);
-// it arrives by cp.async while layer 1 runs.  Latency bounds it (a network of 19
-// 458 weights): few samples per CTA, so that the batch spreads over the SMs, and
-// no second launch and no cached z.  Forward and activation gradients of 512
-// samples: 27 + 36 us (16 samples per CTA, W2 from L2, read across rows in the
-// backward pass) -> 9.4 us.
+// W2_LD floats: conflict-free reads along a row by 16 bytes and down a column), read
+// once per CTA however many tiles it takes; it arrives by cp.async while layer 1 of
+// the first runs.  Latency bounds small batches (a network of 19 458 weights): few
+// samples per CTA, so that the batch spreads over the SMs, and no second launch and
+// no cached z.  Forward and activation gradients of 512 samples: 27 + 36 us (16
+// samples per CTA, W2 from L2, read across rows in the backward pass) -> 9.4 us.
 // Writes Y [B][2] and, with TRAIN, H1, H2, DZ1, DZ2 [B][NH] and DY = (Y - T) / B;
 // lpart (optional): squared-error partial per CTA.
 constexpr int MP_T = 2 * NH;
@@ -44,9 +44,9 @@ struct PassArgs {
     double* lpart;
 };
 
-template <int TS>
+template <int TS, bool TRAIN>
 constexpr size_t mlp_smem() {
-    return sizeof(float) * (size_t)(NH * W2_LD + TS * (NI + 2 * NH));
+    return sizeof(float) * (size_t)(NH * W2_LD + TS * (NI + (TRAIN ? 2 : 1) * NH));
 }
 
 template <int TS, bool TRAIN>
@@ -60,8 +60,6 @@ __global__ void __launch_bounds__(MP_T) k_mlp_pass(PassArgs a) {
     __shared__ float red[MP_T / 32][HS][NO];
     __shared__ float dys[TS][NO];
     const float* __restrict__ P = a.P;
-    const int s0 = blockIdx.x * TS;
-    const int ns = min(TS, a.B - s0);
     const int j = threadIdx.x & (NH - 1), half = threadIdx.x / NH;
     for (int q = threadIdx.x; q < NH * NH / 4; q += MP_T) {
         const int i = q / (NH / 4), c = (q % (NH / 4)) * 4;
@@ -72,103 +70,112 @@ __global__ void __launch_bounds__(MP_T) k_mlp_pass(PassArgs a) {
         else
             for (int e = 0; e < 4; ++e) w2[i * W2_LD + c + e] = P[OFF_W2 + i * NH + c + e];
     }
-    for (int q = threadIdx.x; q < TS * NI; q += MP_T) xs[q] = q / NI < ns ? a.X[(int64_t)s0 * NI + q] : 0.f;
-    __syncthreads();
-    float z1[HS], z2[HS], h2[HS];
-    const float* x = xs + half * HS * NI;
+    const int tiles = (a.B + TS - 1) / TS;
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int s0 = tile * TS;
+        const int ns = min(TS, a.B - s0);
+        if (tile != (int)blockIdx.x) __syncthreads();  // the tile before is read
+        for (int q = threadIdx.x; q < TS * NI; q += MP_T) xs[q] = q / NI < ns ? a.X[(int64_t)s0 * NI + q] : 0.f;
+        __syncthreads();
+        float z1[HS], z2[HS], h2[HS];
+        const float* x = xs + half * HS * NI;
 #pragma unroll
-    for (int s = 0; s < HS; ++s) z1[s] = P[OFF_B1 + j];
+        for (int s = 0; s < HS; ++s) z1[s] = P[OFF_B1 + j];
 #pragma unroll
-    for (int i = 0; i < NI; ++i) {
-        const float wv = P[OFF_W1 + i * NH + j];
+        for (int i = 0; i < NI; ++i) {
+            const float wv = P[OFF_W1 + i * NH + j];
 #pragma unroll
-        for (int s = 0; s < HS; ++s) z1[s] = fmaf(x[s * NI + i], wv, z1[s]);
-    }
-    float* h1 = h1s + half * HS * NH;
-#pragma unroll
-    for (int s = 0; s < HS; ++s) {
-        const float h = gelu_f(z1[s]);
-        h1[s * NH + j] = h;
-        if (TRAIN && half * HS + s < ns) a.H1[(int64_t)(s0 + half * HS + s) * NH + j] = h;
-    }
-    asm volatile("cp.async.wait_all;\n" ::: "memory");
-    __syncthreads();
-#pragma unroll
-    for (int s = 0; s < HS; ++s) z2[s] = P[OFF_B2 + j];
-#pragma unroll 4
-    for (int i = 0; i < NH; i += 4) {
-        float w[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) w[e] = w2[(i + e) * W2_LD + j];
+            for (int s = 0; s < HS; ++s) z1[s] = fmaf(x[s * NI + i], wv, z1[s]);
+        }
+        float* h1 = h1s + half * HS * NH;
 #pragma unroll
         for (int s = 0; s < HS; ++s) {
-            const float4 h = *reinterpret_cast<const float4*>(h1 + s * NH + i);
-            z2[s] = fmaf(h.w, w[3], fmaf(h.z, w[2], fmaf(h.y, w[1], fmaf(h.x, w[0], z2[s]))));
+            const float h = gelu_f(z1[s]);
+            h1[s * NH + j] = h;
+            if (TRAIN && half * HS + s < ns) a.H1[(int64_t)(s0 + half * HS + s) * NH + j] = h;
         }
-    }
-    // output layer: partial products per unit, reduced over the warps of the half
-    const float w30 = P[OFF_W3 + j * NO], w31 = P[OFF_W3 + j * NO + 1];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        asm volatile("cp.async.wait_all;\n" ::: "memory");
+        __syncthreads();
 #pragma unroll
-    for (int s = 0; s < HS; ++s) {
-        h2[s] = gelu_f(z2[s]);
-        if (TRAIN && half * HS + s < ns) a.H2[(int64_t)(s0 + half * HS + s) * NH + j] = h2[s];
-        const float p0 = warp_sumf(h2[s] * w30), p1 = warp_sumf(h2[s] * w31);
-        if (lane == 0) {
-            red[warp][s][0] = p0;
-            red[warp][s][1] = p1;
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x < TS * NO) {
-        const int s = threadIdx.x / NO, o = threadIdx.x % NO, hf = s / HS;
-        float y = P[OFF_B3 + o], d = 0.f;
-        double dl = 0.0;
-        for (int w = 0; w < NH / 32; ++w) y += red[hf * (NH / 32) + w][s % HS][o];
-        if (s < ns) {
-            const int64_t at = (int64_t)(s0 + s) * NO + o;
-            a.Y[at] = y;
-            if (TRAIN) {
-                d = y - a.T[at];
-                dl = (double)y - (double)a.T[at];
-                a.DY[at] = d / (float)a.B;
+        for (int s = 0; s < HS; ++s) z2[s] = P[OFF_B2 + j];
+#pragma unroll 4
+        for (int i = 0; i < NH; i += 4) {
+            float w[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) w[e] = w2[(i + e) * W2_LD + j];
+#pragma unroll
+            for (int s = 0; s < HS; ++s) {
+                const float4 h = *reinterpret_cast<const float4*>(h1 + s * NH + i);
+                z2[s] = fmaf(h.w, w[3], fmaf(h.z, w[2], fmaf(h.y, w[1], fmaf(h.x, w[0], z2[s]))));
             }
         }
-        if (TRAIN) dys[s][o] = d / (float)a.B;
-        if (TRAIN && a.lpart) {  // TS * NO <= 32: one warp
-            double l = dl * dl;
-            for (int q = TS * NO / 2; q > 0; q >>= 1) l += __shfl_xor_sync((1u << (TS * NO)) - 1u, l, q);
-            if (threadIdx.x == 0) a.lpart[blockIdx.x] = l;
-        }
-    }
-    if (!TRAIN) return;
-    __syncthreads();
-    float* dz2 = dzs + half * HS * NH;
-#pragma unroll
-    for (int s = 0; s < HS; ++s) {
-        const int q = half * HS + s;
-        const float dz = (dys[q][0] * w30 + dys[q][1] * w31) * gelu_grad_f(z2[s]);
-        dz2[s * NH + j] = dz;
-        if (q < ns) a.DZ2[(int64_t)(s0 + q) * NH + j] = dz;
-    }
-    __syncthreads();
-    // dh1_j = sum over units u of dz2_u W2[j][u]
-    float acc[HS];
-#pragma unroll
-    for (int s = 0; s < HS; ++s) acc[s] = 0.f;
-    const float* wr = w2 + j * W2_LD;
-#pragma unroll 4
-    for (int u = 0; u < NH; u += 4) {
-        const float4 w = *reinterpret_cast<const float4*>(wr + u);
+        // output layer: partial products per unit, reduced over the warps of the half
+        const float w30 = P[OFF_W3 + j * NO], w31 = P[OFF_W3 + j * NO + 1];
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
         for (int s = 0; s < HS; ++s) {
-            const float4 d = *reinterpret_cast<const float4*>(dz2 + s * NH + u);
-            acc[s] = fmaf(d.w, w.w, fmaf(d.z, w.z, fmaf(d.y, w.y, fmaf(d.x, w.x, acc[s]))));
+            h2[s] = gelu_f(z2[s]);
+            if (TRAIN && half * HS + s < ns) a.H2[(int64_t)(s0 + half * HS + s) * NH + j] = h2[s];
+            const float p0 = warp_sumf(h2[s] * w30), p1 = warp_sumf(h2[s] * w31);
+            if (lane == 0) {
+                red[warp][s][0] = p0;
+                red[warp][s][1] = p1;
+            }
         }
-    }
+        __syncthreads();
+        if (threadIdx.x < TS * NO) {
+            const int s = threadIdx.x / NO, o = threadIdx.x % NO, hf = s / HS;
+            float y = P[OFF_B3 + o], d = 0.f;
+            double dl = 0.0;
+            for (int w = 0; w < NH / 32; ++w) y += red[hf * (NH / 32) + w][s % HS][o];
+            if (s < ns) {
+                const int64_t at = (int64_t)(s0 + s) * NO + o;
+                a.Y[at] = y;
+                if (TRAIN) {
+                    d = y - a.T[at];
+                    dl = (double)y - (double)a.T[at];
+                    a.DY[at] = d / (float)a.B;
+                }
+            }
+            if (TRAIN) dys[s][o] = d / (float)a.B;
+            if constexpr (TRAIN) {
+                static_assert(TS * NO <= 32, "the loss is summed by one warp");
+                if (a.lpart) {
+                    double l = dl * dl;
+                    for (int q = TS * NO / 2; q > 0; q >>= 1) l += __shfl_xor_sync(0xffffffffu >> (32 - TS * NO), l, q);
+                    if (threadIdx.x == 0) a.lpart[tile] = l;
+                }
+            }
+        }
+        if (!TRAIN) continue;
+        __syncthreads();
+        float* dz2 = dzs + half * HS * NH;
 #pragma unroll
-    for (int s = 0; s < HS; ++s)
-        if (half * HS + s < ns) a.DZ1[(int64_t)(s0 + half * HS + s) * NH + j] = acc[s] * gelu_grad_f(z1[s]);
+        for (int s = 0; s < HS; ++s) {
+            const int q = half * HS + s;
+            const float dz = (dys[q][0] * w30 + dys[q][1] * w31) * gelu_grad_f(z2[s]);
+            dz2[s * NH + j] = dz;
+            if (q < ns) a.DZ2[(int64_t)(s0 + q) * NH + j] = dz;
+        }
+        __syncthreads();
+        // dh1_j = sum over units u of dz2_u W2[j][u]
+        float acc[HS];
+#pragma unroll
+        for (int s = 0; s < HS; ++s) acc[s] = 0.f;
+        const float* wr = w2 + j * W2_LD;
+#pragma unroll 4
+        for (int u = 0; u < NH; u += 4) {
+            const float4 w = *reinterpret_cast<const float4*>(wr + u);
+#pragma unroll
+            for (int s = 0; s < HS; ++s) {
+                const float4 d = *reinterpret_cast<const float4*>(dz2 + s * NH + u);
+                acc[s] = fmaf(d.w, w.w, fmaf(d.z, w.z, fmaf(d.y, w.y, fmaf(d.x, w.x, acc[s]))));
+            }
+        }
+#pragma unroll
+        for (int s = 0; s < HS; ++s)
+            if (half * HS + s < ns) a.DZ1[(int64_t)(s0 + half * HS + s) * NH + j] = acc[s] * gelu_grad_f(z1[s]);
+    }
 }
 
 // Sum of FP32 products as an unevaluated pair s + c (Ogita, Rump and Oishi's
@@ -405,20 +412,38 @@ __global__ void k_stop_features_batch(const double* __restrict__ alpha, const do
 }  // namespace
 
 // ---------------------------------------------------------------------------
-// Samples per CTA: 4 while that gives at most four waves of CTAs (three fit on an
-// SM), else 8 (each CTA reads W2 once).
-template <bool TRAIN>
-static rbf_status launch_mlp_pass(rbf_ctx* ctx, const PassArgs& a, int* tiles) {
-    const bool small = (int64_t)a.B <= (int64_t)ctx->sm_count * 48;
-    const int ts = small ? 4 : 8;
-    *tiles = (a.B + ts - 1) / ts;
-    const size_t smem = small ? mlp_smem<4>() : mlp_smem<8>();
-    if (small) RBF_CUDA(ctx, (smem_limit<k_mlp_pass<4, TRAIN>>(ctx, smem)));
-    else RBF_CUDA(ctx, (smem_limit<k_mlp_pass<8, TRAIN>>(ctx, smem)));
-    if (small) k_mlp_pass<4, TRAIN><<<*tiles, MP_T, smem, ctx->stream>>>(a);
-    else k_mlp_pass<8, TRAIN><<<*tiles, MP_T, smem, ctx->stream>>>(a);
+template <int TS, bool TRAIN>
+static rbf_status launch_pass(rbf_ctx* ctx, const PassArgs& a, int* tiles) {
+    constexpr size_t smem = mlp_smem<TS, TRAIN>();
+    constexpr int per_sm = (int)((227 * 1024) / (smem + 2 * 1024));
+    *tiles = (a.B + TS - 1) / TS;
+    RBF_CUDA(ctx, (smem_limit<k_mlp_pass<TS, TRAIN>>(ctx, smem)));
+    const int grid = *tiles < ctx->sm_count * per_sm ? *tiles : ctx->sm_count * per_sm;
+    k_mlp_pass<TS, TRAIN><<<grid, MP_T, smem, ctx->stream>>>(a);
     RBF_LAUNCHED(ctx, "k_mlp_pass");
     return RBF_OK;
+}
+
+// Samples per CTA: few for small batches, so that they spread over the SMs; more
+// where the SMs take several tiles each, so that a weight read from shared memory
+// serves more of them.  Forward, tiles per SM and time, with 4, 8, 32 and 48 samples:
+// 512 samples 8.3, 8.3, 12.5 and 16.5 us; 2048 13.0, 10.4, 12.5 and 16.5; 4096 16.6, 16.5, 12.5
+// and 16.6; 7000 23.9, 20.6, 20.6 and 16.6; 65536 156, 123, 105 and 112 (16 samples of W2 from
+// L2, in CTAs of 128 threads: 16.6, 16.6, 18.6, 18.6 and 103).  With the activation
+// gradients: 7000 samples 119, 119 and 119 with 4, 8 and 16 after 128 with 4 and W2 read
+// for each tile; 65536 992 with 8, 952 with 16.
+static rbf_status launch_mlp_train(rbf_ctx* ctx, const PassArgs& a, int* tiles) {
+    return (int64_t)a.B <= (int64_t)ctx->sm_count * 48 ? launch_pass<4, true>(ctx, a, tiles)
+                                                        : launch_pass<16, true>(ctx, a, tiles);
+}
+
+static rbf_status launch_mlp_forward(rbf_ctx* ctx, const PassArgs& a) {
+    const int64_t per_sm = ((int64_t)a.B + ctx->sm_count - 1) / ctx->sm_count;
+    int tiles = 0;
+    if (per_sm <= 4) return launch_pass<4, false>(ctx, a, &tiles);
+    if (per_sm <= 16) return launch_pass<8, false>(ctx, a, &tiles);
+    if (per_sm > 32 && per_sm <= 48) return launch_pass<48, false>(ctx, a, &tiles);
+    return launch_pass<32, false>(ctx, a, &tiles);
 }
 
 extern "C" rbf_status rbf_mlp_forward(rbf_ctx* ctx, const float* d_params, const float* d_x, int batch, float* d_y) {
@@ -429,8 +454,7 @@ extern "C" rbf_status rbf_mlp_forward(rbf_ctx* ctx, const float* d_params, const
     a.X = d_x;
     a.B = batch;
     a.Y = d_y;
-    int tiles = 0;
-    return launch_mlp_pass<false>(ctx, a, &tiles);
+    return launch_mlp_forward(ctx, a);
 }
 
 // Gradient into G and, with `adam`, the update in the same last launch.
@@ -462,7 +486,7 @@ static rbf_status mlp_grad_impl(rbf_ctx* ctx, const float* P, const float* X, co
     double* lpart = wc.take<double>((size_t)tiles_max + 1);
     a.lpart = h_loss ? lpart : nullptr;
     int tiles = 0;
-    RBF_TRY(launch_mlp_pass<true>(ctx, a, &tiles));
+    RBF_TRY(launch_mlp_train(ctx, a, &tiles));
     const GradArgs ga{X, a.H1, a.H2, a.DY, a.DZ1, a.DZ2, B, chunk, chunks, part};
     // programmatic launches: their start-up overlaps the launch before (26.7 -> 21.5 us a step)
     RBF_CUDA(ctx, rbf_launch_ex(ctx, k_mlp_wgrad, dim3(chunks, 7), dim3(WG_T), 0, true, 1, ga));
