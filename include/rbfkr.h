@@ -443,8 +443,8 @@ rbf_status rbf_get_tuning(const rbf_ctx* ctx, rbf_tuning* out);
  * first 10 GKB steps, the stopping index l and log10 lambda, so that GKB can
  * end early and the selection sweep is skipped.  The network is not in the
  * paper: a 20 -> 128 -> 128 -> 2 perceptron with exact (erf) GELU after both
- * hidden layers, FP32 parameters and arithmetic (gradients accumulated in
- * twice FP32's precision).  Parameters are one FP32 vector of RBF_MLP_PARAMS elements laid out
+ * hidden layers, FP32 parameters and arithmetic (gradients accumulated
+ * as exactly as FP64 would).  Parameters are one FP32 vector of RBF_MLP_PARAMS elements laid out
  * as W1 [20][128] (row-major, input index first), b1 [128], W2 [128][128],
  * b2 [128], W3 [128][2], b3 [2]; the layer computes h_out = h_in W + b.
  * Inputs d_x are [batch][20] row-major, outputs and targets [batch][2]. */
@@ -459,10 +459,10 @@ rbf_status rbf_mlp_forward(rbf_ctx* ctx, const float* d_params, const float* d_x
 
 /* Gradient of the loss sum_(s,o) (y_so - t_so)^2 / (2 batch) with respect to
  * the parameters, written to d_grad (RBF_MLP_PARAMS floats, same layout as the
- * parameters; each element summed over the batch in a fixed order in twice
- * FP32's precision, so the result is deterministic).  When h_loss is not NULL
- * the loss is written there and the stream is synchronised.  Uses the context
- * workspace (about 2 KiB per sample and up to 10 MB of partial sums). */
+ * parameters; each element summed over the batch in a fixed order, to the
+ * precision of an FP64 sum, so the result is deterministic).  When h_loss is
+ * not NULL the loss is written there and the stream is synchronised.  Uses the
+ * context workspace (about 2 KiB per sample and up to 15 MB of partial sums). */
 rbf_status rbf_mlp_grad(rbf_ctx* ctx, const float* d_params, const float* d_x, const float* d_t, int batch,
                         float* d_grad, float* h_loss);
 

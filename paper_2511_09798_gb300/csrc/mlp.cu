@@ -178,21 +178,39 @@ __global__ void __launch_bounds__(MP_T) k_mlp_pass(PassArgs a) {
     }
 }
 
-// Sum of FP32 products as an unevaluated pair s + c (Ogita, Rump and Oishi's
-// Dot2: the product's and the sum's rounding errors, both exact in FP32, are
-// carried in c): the result of a sum in twice FP32's precision.
+// a + b and its rounding error (Knuth's TwoSum).
+__device__ __forceinline__ float two_sum(float a, float b, float& err) {
+    const float t = __fadd_rn(a, b), z = __fsub_rn(t, a);
+    err = __fadd_rn(__fsub_rn(a, __fsub_rn(t, z)), __fsub_rn(b, z));
+    return t;
+}
+
+// Sums in FP32 as unevaluated pairs s + c and triples s + c + d (Ogita, Rump and Oishi's
+// Dot2 and SumK with K = 3: the rounding errors of a product and of an addition,
+// both exact in FP32, are added to the next word).  A stage of 16 samples is summed in
+// pairs, whose own roundings are about 2^-49 of the stage's sum; stages and chunks in
+// triples, 2^-70.  A sum of the exact products in FP64 rounds at 2^-54 of its partial sum
+// once per sample: for 512 samples the two come to the same 2^-50.
 struct Pair {
     float s = 0.f, c = 0.f;
-    __device__ __forceinline__ void two_sum(float p, float e) {
-        const float t = __fadd_rn(s, p), b = __fsub_rn(t, s);
-        const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(p, b));
-        s = t;
-        c = __fadd_rn(c, __fadd_rn(err, e));
-    }
     __device__ __forceinline__ void dot(float a, float b) {
         const float p = __fmul_rn(a, b);
-        two_sum(p, __fmaf_rn(a, b, -p));
+        float e;
+        s = two_sum(s, p, e);
+        c = __fadd_rn(c, __fadd_rn(e, __fmaf_rn(a, b, -p)));
     }
+};
+
+struct Triple {
+    float s = 0.f, c = 0.f, d = 0.f;
+    __device__ __forceinline__ void add(float p, float e) {
+        float q, r, u;
+        s = two_sum(s, p, q);
+        e = two_sum(e, q, r);
+        c = two_sum(c, e, u);
+        d = __fadd_rn(d, __fadd_rn(r, u));
+    }
+    __device__ __forceinline__ double value() const { return (double)s + ((double)c + (double)d); }
 };
 
 // Weight-gradient partials over the samples [chunk c, chunk (c + 1)) of chunk c =
@@ -201,16 +219,17 @@ struct Pair {
 // X and 1, R = DZ1); 5 b2 (L = 1, R = DZ2); 6 W3 transposed (L = DY, R = H2) and b3.
 // An FP64 sum of the products (exact in FP64) runs at 1/64 of the FP32 rate: 10
 // M FP64 FMAs of a 512-sample step are 16 us at best; ten FP32 operations per
-// product in Dot2 give the same FP32 gradients (its error, 2^-47 of the sum of
-// magnitudes, is far below their rounding).  One thread per weight with an FP64
-// chain over the batch: 127 us -> 13.0, and 6.4 for the sum of the partials with the update.
+// product and 22 per stage give its precision (triples throughout, 24 operations per
+// product: 33 us for a step of 512 samples; this, 27; pairs throughout, 24, but errors
+// 8 times as large at 4096 samples).  One thread per weight with an FP64 chain over the
+// batch took 127 us, a step 162.
 constexpr int WG_T = 256;
 constexpr int WG_S = 16;  // samples staged at a time
 
 struct GradArgs {
     const float *X, *H1, *H2, *DY, *DZ1, *DZ2;
     int B, chunk, chunks;
-    float2* part;  // [chunks][NPAR]
+    float* part;  // [chunks][3][NPAR]
 };
 
 __global__ void __launch_bounds__(WG_T) k_mlp_wgrad(GradArgs a) {
@@ -221,7 +240,7 @@ __global__ void __launch_bounds__(WG_T) k_mlp_wgrad(GradArgs a) {
     const int rows = task < 4 ? 32 : (task == 4 ? NI + 1 : (task == 5 ? 1 : NO));
     const float* __restrict__ Rg = task == 4 ? a.DZ1 : (task == 6 ? a.H2 : a.DZ2);
     const int r0 = (threadIdx.x >> 5) * 4, c0 = (threadIdx.x & 31) * 4;
-    Pair acc[4][4], b3;
+    Triple acc[4][4], b3;
     pdl_wait();
     for (int s0 = sb; s0 < se; s0 += WG_S) {
         const int cnt = min(WG_S, se - s0);
@@ -241,6 +260,7 @@ __global__ void __launch_bounds__(WG_T) k_mlp_wgrad(GradArgs a) {
         }
         __syncthreads();
         if (r0 < rows) {
+            Pair run[4][4];
 #pragma unroll 2
             for (int s = 0; s < cnt; ++s) {
                 const float4 l = *reinterpret_cast<const float4*>(&Ls[s][r0]);
@@ -249,14 +269,23 @@ __global__ void __launch_bounds__(WG_T) k_mlp_wgrad(GradArgs a) {
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
 #pragma unroll
-                    for (int v = 0; v < 4; ++v) acc[u][v].dot(lv[u], rv[v]);
+                    for (int v = 0; v < 4; ++v) run[u][v].dot(lv[u], rv[v]);
             }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v < 4; ++v) acc[u][v].add(run[u][v].s, run[u][v].c);
         }
         if (task == 6 && threadIdx.x >= 32 && threadIdx.x < 32 + NO)
-            for (int s = 0; s < cnt; ++s) b3.two_sum(Ls[s][threadIdx.x - 32], 0.f);
+            for (int s = 0; s < cnt; ++s) b3.add(Ls[s][threadIdx.x - 32], 0.f);
     }
-    float2* out = a.part + (int64_t)blockIdx.x * NPAR;
-    if (task == 6 && threadIdx.x >= 32 && threadIdx.x < 32 + NO) out[OFF_B3 + threadIdx.x - 32] = make_float2(b3.s, b3.c);
+    float* out = a.part + (int64_t)blockIdx.x * 3 * NPAR;
+    auto put = [&](int at, const Triple& t) {
+        out[at] = t.s;
+        out[NPAR + at] = t.c;
+        out[2 * NPAR + at] = t.d;
+    };
+    if (task == 6 && threadIdx.x >= 32 && threadIdx.x < 32 + NO) put(OFF_B3 + threadIdx.x - 32, b3);
     if (r0 >= rows) return;
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
@@ -269,34 +298,39 @@ __global__ void __launch_bounds__(WG_T) k_mlp_wgrad(GradArgs a) {
             if (task < 4) at = OFF_W2 + (task * 32 + r) * NH + c;
             else if (task == 4) at = r < NI ? OFF_W1 + r * NH + c : OFF_B1 + c;
             else at = task == 5 ? OFF_B2 + c : OFF_W3 + c * NO + r;
-            out[at] = make_float2(acc[u][v].s, acc[u][v].c);
+            put(at, acc[u][v]);
         }
     }
 }
 
-// Gradient of one parameter in FP64 over the whole batch: where the paired sum
-// left FP32's range (an infinite or NaN product or sum).
-__device__ float grad_f64(const GradArgs& a, int p) {
+// The factors of sample s in the gradient of parameter p.
+__device__ __forceinline__ float2 grad_factors(const GradArgs& a, int p, int64_t s) {
+    if (p < OFF_B1) return make_float2(a.X[s * NI + p / NH], a.DZ1[s * NH + p % NH]);
+    if (p < OFF_W2) return make_float2(1.f, a.DZ1[s * NH + p - OFF_B1]);
+    if (p < OFF_B2) return make_float2(a.H1[s * NH + (p - OFF_W2) / NH], a.DZ2[s * NH + (p - OFF_W2) % NH]);
+    if (p < OFF_W3) return make_float2(1.f, a.DZ2[s * NH + p - OFF_B2]);
+    if (p < OFF_B3) return make_float2(a.H2[s * NH + (p - OFF_W3) / NO], a.DY[s * NO + (p - OFF_W3) % NO]);
+    return make_float2(1.f, a.DY[s * NO + p - OFF_B3]);
+}
+
+// Gradient of one parameter where the paired sum left FP32's range.  A product below
+// 2^-102 has lost part of its rounding error, at most 2^-149 per sample: where the
+// sum is below B 2^-100 (a unit without response, for one) it is taken again with the
+// second factors times 2^96, exactly, which leaves 2^-245.  An infinite or NaN product
+// or sum: in FP64, whose products are exact.
+__device__ __noinline__ float grad_again(const GradArgs& a, int p) {
+    Triple t;
+    for (int64_t s = 0; s < a.B; ++s) {
+        const float2 f = grad_factors(a, p, s);
+        const float r = f.y * 0x1p96f, q = __fmul_rn(f.x, r);
+        t.add(q, __fmaf_rn(f.x, r, -q));
+    }
+    const double g = t.value() * 0x1p-96;
+    if (isfinite(g)) return (float)g;
     double acc = 0.0;
     for (int64_t s = 0; s < a.B; ++s) {
-        double l = 1.0, r;
-        if (p < OFF_B1) {
-            l = a.X[s * NI + p / NH];
-            r = a.DZ1[s * NH + p % NH];
-        } else if (p < OFF_W2) {
-            r = a.DZ1[s * NH + p - OFF_B1];
-        } else if (p < OFF_B2) {
-            l = a.H1[s * NH + (p - OFF_W2) / NH];
-            r = a.DZ2[s * NH + (p - OFF_W2) % NH];
-        } else if (p < OFF_W3) {
-            r = a.DZ2[s * NH + p - OFF_B2];
-        } else if (p < OFF_B3) {
-            l = a.H2[s * NH + (p - OFF_W3) / NO];
-            r = a.DY[s * NO + (p - OFF_W3) % NO];
-        } else {
-            r = a.DY[s * NO + p - OFF_B3];
-        }
-        acc += l * r;
+        const float2 f = grad_factors(a, p, s);
+        acc += (double)f.x * (double)f.y;
     }
     return (float)acc;
 }
@@ -325,15 +359,15 @@ __global__ void __launch_bounds__(128) k_mlp_finish(GradArgs a, float* __restric
     const float P = ADAM && ok ? o.P[p] : 0.f, m0 = ADAM && ok ? o.M[p] : 0.f, v0 = ADAM && ok ? o.V[p] : 0.f;
     pdl_wait();
     if (!ok) return;
-    Pair t;
-    const float2* __restrict__ q = a.part + p;
+    Triple t;
+    const float* __restrict__ q = a.part + p;
 #pragma unroll 8
-    for (int c = 0; c < a.chunks; ++c) {
-        const float2 v = q[(int64_t)c * NPAR];
-        t.two_sum(v.x, v.y);
+    for (int c = 0; c < a.chunks; ++c, q += 3 * NPAR) {
+        t.add(q[0], q[NPAR]);
+        t.d = __fadd_rn(t.d, q[2 * NPAR]);
     }
-    float g = t.s + t.c;
-    if (!isfinite(g)) g = grad_f64(a, p);
+    float g = (float)t.value();
+    if (!(fabsf(g) >= (float)a.B * 0x1p-100f && fabsf(g) <= FLT_MAX)) g = grad_again(a, p);
     G[p] = g;
     if (ADAM) adam_one(o, p, g, P, m0, v0);
 }
@@ -461,14 +495,14 @@ extern "C" rbf_status rbf_mlp_forward(rbf_ctx* ctx, const float* d_params, const
 static rbf_status mlp_grad_impl(rbf_ctx* ctx, const float* P, const float* X, const float* T, int B, float* G,
                                 float* h_loss, const AdamArgs* adam) {
     // chunks of the batch: 16 samples each (32 x 7 CTAs at 512 samples), longer
-    // ones past 64 chunks, where the partials (156 KB per chunk) would cost more
+    // ones past 64 chunks, where the partials (234 KB per chunk) would cost more
     // than the shorter sums save
     int chunk = WG_S;
     while ((B + chunk - 1) / chunk > 64) chunk += WG_S;
     const int chunks = (B + chunk - 1) / chunk;
     const int tiles_max = (B + 3) / 4;
     const size_t need = 4 * ws_align((size_t)B * NH * 4) + 2 * ws_align((size_t)B * NO * 4) +
-                        ws_align((size_t)chunks * NPAR * sizeof(float2)) + ws_align((size_t)(tiles_max + 1) * 8);
+                        ws_align((size_t)chunks * 3 * NPAR * sizeof(float)) + ws_align((size_t)(tiles_max + 1) * 8);
     RBF_TRY(rbf_ws_reserve(ctx, need));
     WsCarve wc(ctx->ws);
     PassArgs a{};
@@ -482,7 +516,7 @@ static rbf_status mlp_grad_impl(rbf_ctx* ctx, const float* P, const float* X, co
     a.DZ2 = wc.take<float>((size_t)B * NH);
     a.Y = wc.take<float>((size_t)B * NO);
     a.DY = wc.take<float>((size_t)B * NO);
-    float2* part = wc.take<float2>((size_t)chunks * NPAR);
+    float* part = wc.take<float>((size_t)chunks * 3 * NPAR);
     double* lpart = wc.take<double>((size_t)tiles_max + 1);
     a.lpart = h_loss ? lpart : nullptr;
     int tiles = 0;
