@@ -47,11 +47,12 @@ __global__ void __launch_bounds__(YT) k_err_coef(const int* __restrict__ ells, i
                                                  const double* __restrict__ ftil_all,
                                                  const double* __restrict__ V_all, int64_t m,
                                                  const double* __restrict__ uref, int J, double t_lo, double t_hi,
-                                                 int tstride, int Jp, double* __restrict__ y_all,
-                                                 double* __restrict__ umax, double* __restrict__ err) {
+                                                 int tstride, int Jp, int first, int slice,
+                                                 double* __restrict__ y_all, double* __restrict__ umax,
+                                                 double* __restrict__ err) {
     extern __shared__ double cv[];  // [YQ][L]
     __shared__ double red[YT / 32];
-    const int e = gridDim.y - 1 - blockIdx.y, q0 = blockIdx.x * YQ;
+    const int e = gridDim.y - 1 - blockIdx.y, q0 = first + blockIdx.x * YQ;
     const int l = ells[e];
     const double* sigma = sigma_all + (size_t)e * L;
     const double* ftil = ftil_all + (size_t)e * (L + 1);
@@ -80,7 +81,7 @@ __global__ void __launch_bounds__(YT) k_err_coef(const int* __restrict__ ells, i
         }
 #pragma unroll
         for (int q = 0; q < YQ; ++q)
-            if (q0 + q < Jp) y_all[((size_t)e * Jp + q0 + q) * L + r] = acc[q];
+            if (q0 + q < Jp) y_all[((size_t)e * slice + q0 - first + q) * L + r] = acc[q];
     }
     if (blockIdx.x != 0 || blockIdx.y != 0) return;
     double u = 0.0;
@@ -97,14 +98,14 @@ __global__ void __launch_bounds__(YT) k_err_coef(const int* __restrict__ ells, i
 __global__ void __launch_bounds__(ET) k_err_table(const int* __restrict__ ells, int L, const double* __restrict__ y_all,
                                                   const double* __restrict__ umax, const double* __restrict__ G,
                                                   int64_t ldg, int64_t m, const double* __restrict__ uref, int Jp,
-                                                  double* __restrict__ err) {
+                                                  int first, int slice, double* __restrict__ err) {
     extern __shared__ double y[];  // [l][EQ]
     __shared__ double red[ET / 32][EQ];
-    const int e = gridDim.y - 1 - blockIdx.y, q0 = blockIdx.x * EQ;
+    const int e = gridDim.y - 1 - blockIdx.y, q0 = first + blockIdx.x * EQ;
     const int l = ells[e];
     for (int idx = threadIdx.x; idx < EQ * l; idx += ET) {
         const int q = idx / l, r = idx - q * l;
-        y[r * EQ + q] = q0 + q < Jp ? y_all[((size_t)e * Jp + q0 + q) * L + r] : 0.0;
+        y[r * EQ + q] = q0 + q < Jp ? y_all[((size_t)e * slice + q0 - first + q) * L + r] : 0.0;
     }
     __syncthreads();
     double mx[EQ];
@@ -161,8 +162,7 @@ extern "C" rbf_status rbf_hkt_error_table(rbf_ctx* ctx, const rbf_gkb_state* st,
     const int Jp = (J - 1) / t_stride + 1;
     const size_t B = (size_t)n_ell;
     const size_t need = ws_align(B * 4) + ws_align(B * L * 8) + 2 * ws_align(B * (L + 1) * 8) +
-                        ws_align(B * L * 8) + ws_align(B * L * L * 8) + ws_align(B * Jp * L * 8) + ws_align(8) +
-                        svd_ws_bytes_batch(L, n_ell);
+                        ws_align(B * L * 8) + ws_align(B * L * L * 8) + svd_ws_bytes_batch(L, n_ell);
     RBF_TRY(rbf_ws_reserve(ctx, need));
     WsCarve wc(ctx->ws);
     int* d_ells = wc.take<int>(B);
@@ -171,9 +171,13 @@ extern "C" rbf_status rbf_hkt_error_table(rbf_ctx* ctx, const rbf_gkb_state* st,
     double* ftil = wc.take<double>(B * (L + 1));
     double* sigma = wc.take<double>(B * L);
     double* V = wc.take<double>(B * L * L);
-    double* y = wc.take<double>(B * Jp * L);
-    double* umax = wc.take<double>(1);
     void* svd = (void*)wc.take<char>(svd_ws_bytes_batch(L, n_ell));
+    // y takes the place of the SVD's scratch, which holds at least 8 lambdas of every l
+    // (4 (2 L + 1) of them): in slices of lambdas where it does not hold them all
+    double* umax = (double*)svd;
+    double* y = umax + 32;
+    const size_t fit = (svd_ws_bytes_batch(L, n_ell) - 256) / (B * L * 8) / EQ * EQ;
+    const int slice = fit < (size_t)Jp ? (int)fit : Jp;
     RBF_CUDA(ctx, cudaMemcpyAsync(d_ells, h_ells, B * 4, cudaMemcpyHostToDevice, ctx->stream));
     k_replicate<<<n_ell, 256, 0, ctx->stream>>>(st->d_alpha, st->d_beta, L, a_rep, b_rep);
     RBF_LAUNCHED(ctx, "k_replicate");
@@ -182,13 +186,17 @@ extern "C" rbf_status rbf_hkt_error_table(rbf_ctx* ctx, const rbf_gkb_state* st,
     const size_t smem_y = (size_t)YQ * L * 8, smem_e = (size_t)EQ * L * 8;
     RBF_CUDA(ctx, smem_limit<k_err_coef>(ctx, smem_y));
     RBF_CUDA(ctx, smem_limit<k_err_table>(ctx, smem_e));
-    k_err_coef<<<dim3((unsigned)((Jp + YQ - 1) / YQ), (unsigned)n_ell), YT, smem_y, ctx->stream>>>(
-        d_ells, L, sigma, ftil, V, m, d_uref, J, ctx->opt.grid_t_lo, ctx->opt.grid_t_hi, t_stride, Jp, y, umax, d_err);
-    RBF_LAUNCHED(ctx, "k_err_coef");
     const int64_t zt = (m + ET - 1) / ET;
-    k_err_table<<<dim3((unsigned)((Jp + EQ - 1) / EQ), (unsigned)n_ell, (unsigned)(zt < 64 ? zt : 64)), ET, smem_e,
-                  ctx->stream>>>(d_ells, L, y, umax, d_G, ldg, m, d_uref, Jp, d_err);
-    RBF_LAUNCHED(ctx, "k_err_table");
+    for (int first = 0; first < Jp; first += slice) {
+        const int cnt = Jp - first < slice ? Jp - first : slice;
+        k_err_coef<<<dim3((unsigned)((cnt + YQ - 1) / YQ), (unsigned)n_ell), YT, smem_y, ctx->stream>>>(
+            d_ells, L, sigma, ftil, V, m, d_uref, J, ctx->opt.grid_t_lo, ctx->opt.grid_t_hi, t_stride, Jp,
+            first, slice, y, umax, d_err);
+        RBF_LAUNCHED(ctx, "k_err_coef");
+        k_err_table<<<dim3((unsigned)((cnt + EQ - 1) / EQ), (unsigned)n_ell, (unsigned)(zt < 64 ? zt : 64)), ET,
+                      smem_e, ctx->stream>>>(d_ells, L, y, umax, d_G, ldg, m, d_uref, Jp, first, slice, d_err);
+        RBF_LAUNCHED(ctx, "k_err_table");
+    }
     // the host array of l values must outlive the copy
     RBF_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     return RBF_OK;
