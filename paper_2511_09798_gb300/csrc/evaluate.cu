@@ -273,10 +273,17 @@ rbf_status evaluate_vectors(rbf_ctx* ctx, const rbf_operator* op, const double* 
     RBF_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, EV_T, 0));
     int64_t chunks = eval_chunks(n, tiles * zs, ctx->sm_count, per_sm);
     if (chunks > 65535) chunks = 65535;
-    const int64_t chunk = (n + chunks - 1) / chunks;
-    chunks = (n + chunk - 1) / chunk;
     const int64_t total = m * ncoef;
-    RBF_TRY(rbf_ws_reserve(ctx, ws_align((size_t)chunks * total * sizeof(double)) + ws_align(EX_CTAS * sizeof(int))));
+    int64_t chunk;
+    for (;;) {  // fewer chunks where the partials of so many do not fit the workspace cap
+        chunk = (n + chunks - 1) / chunks;
+        chunks = (n + chunk - 1) / chunk;
+        const rbf_status st = rbf_ws_reserve(ctx, ws_align((size_t)chunks * total * sizeof(double)) +
+                                                      ws_align(EX_CTAS * sizeof(int)));
+        if (st == RBF_OK) break;
+        if (chunks == 1) return st;
+        chunks = (chunks + 1) / 2;
+    }
     WsCarve wc(ctx->ws);
     double* part = wc.take<double>((size_t)chunks * total);
     int* exps = wc.take<int>(EX_CTAS);
