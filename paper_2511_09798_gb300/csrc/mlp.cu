@@ -499,11 +499,18 @@ static rbf_status mlp_grad_impl(rbf_ctx* ctx, const float* P, const float* X, co
     // than the shorter sums save
     int chunk = WG_S;
     while ((B + chunk - 1) / chunk > 64) chunk += WG_S;
-    const int chunks = (B + chunk - 1) / chunk;
     const int tiles_max = (B + 3) / 4;
-    const size_t need = 4 * ws_align((size_t)B * NH * 4) + 2 * ws_align((size_t)B * NO * 4) +
-                        ws_align((size_t)chunks * 3 * NPAR * sizeof(float)) + ws_align((size_t)(tiles_max + 1) * 8);
-    RBF_TRY(rbf_ws_reserve(ctx, need));
+    int chunks;
+    for (;;) {  // fewer chunks where the partials of so many do not fit the workspace cap
+        chunks = (B + chunk - 1) / chunk;
+        const size_t need = 4 * ws_align((size_t)B * NH * 4) + 2 * ws_align((size_t)B * NO * 4) +
+                            ws_align((size_t)chunks * 3 * NPAR * sizeof(float)) +
+                            ws_align((size_t)(tiles_max + 1) * 8);
+        const rbf_status st = rbf_ws_reserve(ctx, need);
+        if (st == RBF_OK) break;
+        if (chunks == 1) return st;
+        chunk *= 2;
+    }
     WsCarve wc(ctx->ws);
     PassArgs a{};
     a.P = P;

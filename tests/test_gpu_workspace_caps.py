@@ -31,3 +31,18 @@ def test_evaluate(R):
         ctx.close()
     # another order of the same sum: n roundings of at most the sum of magnitudes (|co| < 5, Phi < 2)
     assert (out[0] - out[1]).abs().max() <= n * 2.0**-53 * 10 * n
+
+
+def test_gradient(R):
+    g = torch.Generator(device="cuda").manual_seed(1)
+    p = 0.1 * torch.randn(19458, generator=g, device="cuda")
+    x, y = torch.randn((512, 20), generator=g, device="cuda"), torch.randn((512, 2), generator=g, device="cuda")
+    out = []
+    for c in (0, 1700 * 1024):
+        ctx = R.Context(0, workspace_cap=c)
+        grad = torch.empty_like(p)
+        ctx.rbf_mlp_grad(p, x, y, 512, grad)
+        out.append(grad)
+        ctx.close()
+    # both are exact sums but for one FP32 rounding
+    assert (out[0] - out[1]).abs().max() <= 2.0**-23 * out[0].abs().max()
