@@ -22,6 +22,7 @@
 //
 // Both: numerical rank r = #{sigma_i > N eps sigma_1}, s_perp = sum_{i>r}
 // f^_i^2, the GCV grid (Tikhonov) or rank curve (TSVD), the solution alpha.
+#include <algorithm>
 #include <cfloat>
 #include <vector>
 
@@ -1073,12 +1074,16 @@ rbf_status fsvd_bidiag(rbf_ctx* ctx, const rbf_operator* op, const double* f, Fs
     if (G != ctx->sm_count) return rbf_fail(ctx, RBF_ERR_INTERNAL, "bidiagonalization grid of %d CTAs", G);
     const int64_t qblk = (n - 1 + QB - 1) / QB, qchunk = (n + QG_ROWS - 1) / QG_ROWS;
     F->ldw = (n + 3) & ~(int64_t)3;
+    // the bidiagonalization's vectors and slots are needed before the tridiagonal SVD's
+    // scratch is, the dot products and Gram matrices of Q_R after it: one place for all
+    const size_t early = 4 * ws_align((size_t)(n + 2) * 8) + ws_align((size_t)2 * G * G * sizeof(ulonglong2));
+    const size_t late = 2 * ws_align((size_t)2 * QB * G * 8) + ws_align((size_t)qchunk * qblk * QB * QB * 8) +
+                        ws_align((size_t)qblk * QB * QB * 8);
+    const size_t scratch = std::max(svd_ws_bytes(L), std::max(early, late));
     const size_t need = ws_align((size_t)F->ldw * (n + 1) * 8) + ws_align((size_t)n * n * 8) +
-                        ws_align((size_t)(n + 1) * n * 8) + 14 * ws_align((size_t)(n + 2) * 8) +
+                        ws_align((size_t)(n + 1) * n * 8) + 10 * ws_align((size_t)(n + 2) * 8) +
                         ws_align((size_t)(J > n ? J : n) * 8) + ws_align(8) + ws_align(4) +
-                        ws_align((size_t)2 * G * G * sizeof(ulonglong2)) + ws_align((size_t)3 * QB * G * 8) +
-                        ws_align((size_t)(qchunk + 1) * qblk * QB * QB * 8) + ws_align((size_t)2 * QB * G * 8) +
-                        ws_align((size_t)(F->bar_k + 2) * BAR_STRIDE * 4) + svd_ws_bytes(L) + 4096;
+                        ws_align((size_t)(F->bar_k + 2) * BAR_STRIDE * 4) + ws_align(scratch);
     RBF_TRY(rbf_ws_reserve(ctx, need));
     WsCarve wc(ctx->ws);
     F->tgk = true;
@@ -1097,18 +1102,19 @@ rbf_status fsvd_bidiag(rbf_ctx* ctx, const rbf_operator* op, const double* f, Fs
     F->sig = wc.take<double>((size_t)n + 2);
     F->fhat = wc.take<double>((size_t)n + 2);
     F->d = wc.take<double>((size_t)n + 2);
-    double* vec[4];
-    for (double*& v : vec) v = wc.take<double>((size_t)n + 2);
     F->curve = wc.take<double>((size_t)(J > n ? J : n));
     F->sperp = wc.take<double>(1);
     F->r = wc.take<int>(1);
-    ulonglong2* slot = wc.take<ulonglong2>((size_t)2 * G * G);
-    F->hpart = wc.take<double>((size_t)QB * G);
-    F->gpart = wc.take<double>((size_t)2 * QB * G);
-    F->gram_part = wc.take<double>((size_t)qchunk * qblk * QB * QB);
-    F->gram = wc.take<double>((size_t)qblk * QB * QB);
     F->bar = wc.take<unsigned>((size_t)(F->bar_k + 2) * BAR_STRIDE);
-    void* svd = (void*)wc.take<char>(svd_ws_bytes(L));
+    void* svd = (void*)wc.take<char>(scratch);
+    WsCarve before(svd), after(svd);
+    double* vec[4];
+    for (double*& v : vec) v = before.take<double>((size_t)n + 2);
+    ulonglong2* slot = before.take<ulonglong2>((size_t)2 * G * G);
+    F->hpart = after.take<double>((size_t)QB * G);
+    F->gpart = after.take<double>((size_t)2 * QB * G);
+    F->gram_part = after.take<double>((size_t)qchunk * qblk * QB * QB);
+    F->gram = after.take<double>((size_t)qblk * QB * QB);
     cudaStream_t s = ctx->stream;
     const size_t bar_bytes = (size_t)(F->bar_k + 2) * BAR_STRIDE * sizeof(unsigned);
     RBF_CUDA(ctx, cudaMemsetAsync(slot, 0, (size_t)2 * G * G * sizeof(ulonglong2), s));

@@ -46,3 +46,21 @@ def test_gradient(R):
         ctx.close()
     # both are exact sums but for one FP32 rounding
     assert (out[0] - out[1]).abs().max() <= 2.0**-23 * out[0].abs().max()
+
+
+def test_full_svd(R):
+    n = 1000
+    rng = np.random.default_rng(2)
+    D = torch.zeros((n, R.padded_lda(n, R.RBF_FP64)), dtype=torch.float64, device="cuda")
+    D[:, :n] = torch.as_tensor(rng.normal(size=(n, n)), device="cuda")
+    f = torch.as_tensor(rng.normal(size=n), device="cuda")
+    out = []
+    for c in (0, 88_200_000):
+        ctx = R.Context(0, workspace_cap=c)
+        op = ctx.rbf_operator_init(torch.zeros((3, n), dtype=torch.float64, device="cuda"), n, n // 2, 1.0, 1.0, A=D,
+                                   lda=D.shape[1])
+        coef = torch.empty(n, dtype=torch.float64, device="cuda")
+        ctx.rbf_tikhonov(op, f, R.RBF_GCV, 0.0, coef)
+        out.append(coef)
+        ctx.close()
+    assert torch.equal(out[0], out[1])
