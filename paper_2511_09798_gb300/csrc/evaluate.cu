@@ -84,27 +84,24 @@ __device__ __forceinline__ long long eval_phi(long long dx, long long dy, long l
     return (R1 << 19) + (b2 - 0x4B400000);
 }
 
-// u = sum of the chunks' partials, from 16 on in eight chains (a serial sum rounds once
-// per chunk at the size of a large early partial).
+// u = sum of the chunks' partials: eight chains over the chunks, one per warp of a
+// CTA of 32 outputs (a serial sum rounds once per chunk at the size of a large early
+// partial, and its loads wait for one another: 20 000 nodes and 100 points, 304 chunks, 54
+// -> 31 us in all).
 __global__ void __launch_bounds__(256) k_eval_reduce(int64_t total, int chunks, const double* __restrict__ part,
                                                      double* __restrict__ u) {
-    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    if (i >= total) return;
-    if (chunks < 16) {
-        double s = 0.0;
-        for (int q = 0; q < chunks; ++q) s += part[(int64_t)q * total + i];
-        u[i] = s;
-        return;
-    }
-    double t[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    int q = 0;
-    for (; q + 7 < chunks; q += 8)
-#pragma unroll
-        for (int e = 0; e < 8; ++e) t[e] += part[(int64_t)(q + e) * total + i];
-#pragma unroll
-    for (int e = 0; e < 7; ++e)
-        if (q + e < chunks) t[e] += part[(int64_t)(q + e) * total + i];
-    u[i] = ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
+    __shared__ double t[8][32];
+    const int lane = threadIdx.x & 31, e = threadIdx.x >> 5;
+    const int64_t i = (int64_t)blockIdx.x * 32 + lane;
+    double s = 0.0;
+    if (i < total)
+#pragma unroll 8
+        for (int q = e; q < chunks; q += 8) s += part[(int64_t)q * total + i];
+    t[e][lane] = s;
+    __syncthreads();
+    if (e == 0 && i < total)
+        u[i] = ((t[0][lane] + t[1][lane]) + (t[2][lane] + t[3][lane])) +
+               ((t[4][lane] + t[5][lane]) + (t[6][lane] + t[7][lane]));
 }
 
 // Partials over the centre chunk blockIdx.y for the NC vectors blockIdx.z NC ..:
@@ -241,7 +238,7 @@ __global__ void __launch_bounds__(EV_T) k_evaluate(const double* __restrict__ X,
 // 3/4 as many (up to eight per point tile where one wave holds a single one), the number that fills
 // the SMs most evenly: ceil(CTAs per SM) times a CTA's nodes and its fixed part,
 // about 24 nodes.  One full wave against this, 8000 nodes: 500 points and 150 vectors 612
-// and 551 us, 8 vectors 70 and 60 (in FP64 199 and 171), 20 000 points and 17 vectors 4.69 and
+// and 549 us, 8 vectors 69 and 49 (in FP64 198 and 160), 20 000 points and 17 vectors 4.69 and
 // 3.13 ms (21.4 and 17.3).
 int64_t eval_chunks(int64_t n, int64_t ctas, int64_t sms, int64_t per_sm) {
     int64_t top = sms * per_sm / ctas;
@@ -300,7 +297,8 @@ rbf_status evaluate_vectors(rbf_ctx* ctx, const rbf_operator* op, const double* 
     else EV_LAUNCH(8);
 #undef EV_LAUNCH
     RBF_LAUNCHED(ctx, "k_evaluate");
-    k_eval_reduce<<<(unsigned)((total + 255) / 256), 256, 0, ctx->stream>>>(total, (int)chunks, part, u);
+    if (chunks < 16) return launch_reduce_partials(ctx, total, (int)chunks, part, u);
+    k_eval_reduce<<<(unsigned)((total + 31) / 32), 256, 0, ctx->stream>>>(total, (int)chunks, part, u);
     RBF_LAUNCHED(ctx, "k_eval_reduce");
     return RBF_OK;
 }
