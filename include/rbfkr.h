@@ -95,7 +95,12 @@ typedef struct {
                                 gives up: the run stops and the call returns
                                 RBF_ERR_TIMEOUT instead of waiting for ever (default
                                 2^23, several seconds; a tiny value forces the timeout
-                                path, which leaves the context usable) */
+                                path, which leaves the context usable).  Small FP64
+                                runs (n <= 8192, few basis vectors) take their
+                                half-steps in one cluster, whose hardware barriers it
+                                does not bound, with sums in another order; a value
+                                below 4096 keeps them on the grid barriers that it
+                                bounds */
     int fma_products;        /* FP64 assembled operators, n <= 16384: GKB (and LSQR on
                                 its state) computes A z and A^T w in exact integer
                                 fixed point from two int64 copies of A made at the

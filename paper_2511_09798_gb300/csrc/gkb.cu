@@ -440,9 +440,9 @@ __global__ void __launch_bounds__(SL_THREADS) k_half(HalfArgs a) {
 // first cluster barrier, when every CTA has read the done flag.
 // It is launched with programmatic stream serialization: the slab of Q, the norm
 // and the breakdown test are done while the product before it ends.  Per
-// half-step at n = 1000 (mcount up to 40) 22.4 -> 14.1 us, less what overlaps the
-// product; a whole step at n = 1000 72 -> 37 us, at n = 2161 (mcount up to 140)
-// 102 -> 64 us.
+// half-step at n = 1000 (mcount up to 40) the kernel takes 14.4 us by itself, where the
+// grid form takes 22.4, less what overlaps the product; a whole step at n = 1000 72 ->
+// 37 us, at n = 2161 (mcount up to 140; 25.5 us a kernel) 102 -> 64 us.
 constexpr int HC_CTAS = 16;
 constexpr int HC_T = 512;
 constexpr int HC_SPLIT = 16;  // most threads per basis vector in the dot products
@@ -455,10 +455,10 @@ constexpr int HC_SPLIT = 16;  // most threads per basis vector in the dot produc
 // an update (2^-60 in the root mean square, signs random), where every FMA rounds at
 // 2^-53 of its sum.  The scale by rows keeps rows of different size apart as FP64
 // does.  Over 48 problems each the basis and the coefficients are half as far from
-// extended precision as with the FP64 grid form (n = 2161, 140 steps: W 0.47, alpha 0.51
+// extended precision as with the FP64 grid form (n = 2161, 140 steps: W 0.45, alpha 0.50
 // of its error; 2000, 60: 0.53 and 0.68; geometric means, standard errors 1.13).  The
 // conversions and scales cost 2 us per half-step, what about 2800 entries cost in
-// FP64: 1000 rows and up to 40 vectors 14.1 us in FP64, 16.1 in fixed point; 2161 rows
+// FP64: 1000 rows and up to 40 vectors 14.4 us in FP64, 16.3 in fixed point; 2161 rows
 // and 140 steps, a solve 10.08 -> 8.92 ms.  FP64 also where an entry of Q is not finite.
 constexpr int HC_FX_MIN = 4096;
 

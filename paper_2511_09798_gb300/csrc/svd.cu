@@ -25,7 +25,8 @@
 //  4. k_tgk_finalize split into u~ and v~, normalise, f~_i = beta_1 u~_i[0];
 //     f~_{l+1} = beta_1 / |u| with u the null vector of C^T (u_1 = 1,
 //     u_{j+1} = -alpha_j u_j / beta_{j+1}), accumulated in log space.
-// Everything is FP64.
+// Every result is FP64; the FP32 counts, secant roots and square roots only place the
+// points at which the FP64 counts are taken.
 #include <cfloat>
 
 #include "common.cuh"
@@ -207,8 +208,8 @@ __device__ __forceinline__ int sturm_count_f32(const float* __restrict__ e2, int
 //     little, an even multisection.
 // The FP64 counts bound the kernel: 2 n_t FP64 instructions of 64 cycles per
 // round and warp.  About 4 FP64 rounds with 32 lanes (6 with 8) replace the 12
-// to 14 of an even multisection of the whole range: l = 150 668 -> 148 us, l =
-// 3001 84.5 -> 5.7 ms.  LPV = 32 takes the fewest rounds, 8 the fewest counts (the
+// to 14 of an even multisection of the whole range (kernel times): l = 150 668 -> 147
+// us, l = 3001 84.5 -> 5.7 ms.  LPV = 32 takes the fewest rounds, 8 the fewest counts (the
 // launcher chooses by the number of values).
 constexpr int BI_ROUNDS = 64;
 
@@ -757,8 +758,8 @@ rbf_status launch_projected_svd_batch(rbf_ctx* ctx, ProjDims d, const double* al
     const size_t sh_v = 2 * (size_t)L * sizeof(double);
     const size_t sh_f = ((size_t)L + 1) * sizeof(double);
     // 32 lanes per value up to three warps per SM scheduler, 8 lanes beyond, where
-    // the number of counts bounds it (32 and 8 lanes: l = 150 0.172 and 0.254 ms,
-    // l = 1000 1.44 and 1.64, 15 runs of l = 150 0.240 and 0.236, l = 3001 11.2 and 6.2)
+    // the number of counts bounds it (kernel times with 32 and 8 lanes: l = 150 0.147 and
+    // 0.219 ms, l = 1000 1.32 and 1.40, 15 runs of up to l = 150 0.240 and 0.218, l = 3001 10.6 and 5.7)
     const bool wide = (int64_t)L * B <= (int64_t)ctx->sm_count * 12;
     const int warps = L > 4096 ? 2 * BS_WARPS : BS_WARPS;  // one CTA per SM holds the tables above 4096
     const int per_cta = warps * (wide ? 1 : 4);
